@@ -239,8 +239,7 @@ struct PtMacArgs {
   const u64* pt[16];
   int count;
 };
-__global__ void k_pt_mac_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ r64s, PtMacArgs A,
-                                u64* __restrict__ out, size_t os, int n_parts, int limbs, int log_n, int q_count,
+__global__ void k_pt_mac_kernel(const PrimeDev* __restrict__ pr, PtMacArgs A, u64* __restrict__ out, size_t os, int n_parts, int limbs, int log_n, int q_count,
                                 int p_first) {
   const size_t per = (size_t)limbs << log_n, total = n_parts * per;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
@@ -249,7 +248,7 @@ __global__ void k_pt_mac_kernel(const PrimeDev* __restrict__ pr, const u64* __re
     const int li = (int)(r >> log_n), i = li < q_count ? li : p_first + (li - q_count);
     Acc128 s{0, 0};
     for (int b = 0; b < A.count; ++b) mac128(s, A.ct[b][p * A.cs[b] + r], A.pt[b][r]);
-    out[p * os + r] = reduce128(s, pr[i], r64s[2 * i], r64s[2 * i + 1]);
+    out[p * os + r] = reduce128(s, pr[i]);
   }
 }
 
@@ -397,7 +396,7 @@ static std::unique_ptr<Ct> lt_apply(Ctx& C, const Ct& v, const LTGroup& G, Plain
       ProfScope prof_(PROF_ELEMENTWISE, C.stream, (1.5 * A.count + 1.0) * v.parts() * ext * C.N * 8);
       prof_count_launches(1);
       k_pt_mac_kernel<<<grid_for((size_t)v.parts() * ext * C.N, 256), 256, 0, C.stream>>>(
-          C.tab.pr, C.d_r64.p, A, sum.p, qp_stride, v.parts(), ext, C.log_n, l + 1, C.n_q);
+          C.tab.pr, A, sum.p, qp_stride, v.parts(), ext, C.log_n, l + 1, C.n_q);
       HEDAP_LAUNCH_CHECK();
     }
     auto inner = ct_alloc(C, l, v.batch);

@@ -130,17 +130,17 @@ API hedap_status hedap_export_key(hedap_ctx* ctx, uint64_t g, uint32_t digit, ui
     need((int)digit < C.dnum(C.L()), "digit out of range");
     const size_t part = (size_t)C.total_primes() * C.N;
     const uint64_t* base = C.keys.at(g).p + (size_t)digit * 2 * part;
-    HEDAP_CUDA(cudaMemcpyAsync(b, base, part * 8, cudaMemcpyDeviceToHost, C.stream));
-    HEDAP_CUDA(cudaMemcpyAsync(a, base + part, part * 8, cudaMemcpyDeviceToHost, C.stream));
+    std::vector<uint64_t> stored(2 * part);
+    HEDAP_CUDA(cudaMemcpyAsync(stored.data(), base, 2 * part * 8, cudaMemcpyDeviceToHost, C.stream));
     HEDAP_CUDA(cudaStreamSynchronize(C.stream));
-    // the key as defined, without the conversion factors folded into its stored limbs
+    // the key as defined: in order, without the conversion factors folded into its stored limbs
     const int T = C.total_primes();
     for (int t = 0; t < T; ++t) {
       const uint64_t u = C.key_unscale[(size_t)digit * T + t], pt = C.primes[t];
-      if (u == 1) continue;
       for (size_t n = 0; n < C.N; ++n) {
-        b[(size_t)t * C.N + n] = hedap::h_mulmod(b[(size_t)t * C.N + n], u, pt);
-        a[(size_t)t * C.N + n] = hedap::h_mulmod(a[(size_t)t * C.N + n], u, pt);
+        const size_t at = (size_t)t * C.N + 2 * hedap::key_pair(n / 2) + n % 2;
+        b[(size_t)t * C.N + n] = u == 1 ? stored[at] : hedap::h_mulmod(stored[at], u, pt);
+        a[(size_t)t * C.N + n] = u == 1 ? stored[part + at] : hedap::h_mulmod(stored[part + at], u, pt);
       }
     }
   });
@@ -318,17 +318,21 @@ API hedap_status hedap_ntt(hedap_ctx* ctx, uint64_t* limbs, size_t n_limbs, uint
     const size_t words = n_limbs * C.N;
     hedap::DevBuf tmp;
     uint64_t* d = limbs;
-    if (!on_device) {
+    // the transforms load and store 16 bytes: words at an 8-byte boundary go through a buffer
+    const bool staged = !on_device || ((uintptr_t)limbs & 15);
+    if (staged) {
       tmp = hedap::DevBuf(words, C.stream);
-      HEDAP_CUDA(cudaMemcpyAsync(tmp.p, limbs, words * 8, cudaMemcpyHostToDevice, C.stream));
+      HEDAP_CUDA(cudaMemcpyAsync(tmp.p, limbs, words * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                                 C.stream));
       d = tmp.p;
     }
     hedap::LimbSet S{d, 0, 1, 0, (int)n_limbs, INT_MAX, (int)first_prime, 0};
     if (inverse) hedap::ntt_inverse(C.tab, S, C.stream);
     else hedap::ntt_forward(C.tab, S, C.stream);
-    if (!on_device) {
-      HEDAP_CUDA(cudaMemcpyAsync(limbs, tmp.p, words * 8, cudaMemcpyDeviceToHost, C.stream));
-      HEDAP_CUDA(cudaStreamSynchronize(C.stream));
+    if (staged) {
+      HEDAP_CUDA(cudaMemcpyAsync(limbs, tmp.p, words * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                                 C.stream));
+      if (!on_device) HEDAP_CUDA(cudaStreamSynchronize(C.stream));
     }
   });
 }
@@ -588,17 +592,21 @@ API hedap_status hedap_ntt_batch(hedap_ctx* ctx, uint64_t* limbs, size_t n_limbs
     const size_t words = n_polys * n_limbs * C.N;
     hedap::DevBuf tmp;
     uint64_t* d = limbs;
-    if (!on_device) {
+    // the transforms load and store 16 bytes: words at an 8-byte boundary go through a buffer
+    const bool staged = !on_device || ((uintptr_t)limbs & 15);
+    if (staged) {
       tmp = hedap::DevBuf(words, C.stream);
-      HEDAP_CUDA(cudaMemcpyAsync(tmp.p, limbs, words * 8, cudaMemcpyHostToDevice, C.stream));
+      HEDAP_CUDA(cudaMemcpyAsync(tmp.p, limbs, words * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                                 C.stream));
       d = tmp.p;
     }
     hedap::LimbSet S{d, n_limbs * C.N, (int)n_polys, 0, (int)n_limbs, INT_MAX, (int)first_prime, 0};
     if (inverse) hedap::ntt_inverse(C.tab, S, C.stream);
     else hedap::ntt_forward(C.tab, S, C.stream);
-    if (!on_device) {
-      HEDAP_CUDA(cudaMemcpyAsync(limbs, tmp.p, words * 8, cudaMemcpyDeviceToHost, C.stream));
-      HEDAP_CUDA(cudaStreamSynchronize(C.stream));
+    if (staged) {
+      HEDAP_CUDA(cudaMemcpyAsync(limbs, tmp.p, words * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                                 C.stream));
+      if (!on_device) HEDAP_CUDA(cudaStreamSynchronize(C.stream));
     }
   });
 }

@@ -59,9 +59,21 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
   const int T = C->total_primes();
   const size_t N = C->N;
 
-  // NTT tables: psi^bitrev(i), psi^-bitrev(i) and Shoup companions
-  std::vector<u64> psi2(2 * T * N), ipsi2(2 * T * N), ninv(T), ninv_sh(T), r64(2 * T);
+  // NTT tables: (w 2^32, w 2^64) mod q of w = psi^bitrev(i) and psi^-bitrev(i), in the transforms' order (Tables)
+  const int l1 = C->log_n / 2, l2 = C->log_n - l1;
+  const size_t TS = tw_stride(l1, l2);
+  std::vector<u64> psi2(2 * T * TS), ipsi2(2 * T * TS), ninv(T), ninv_sh(T);
   std::vector<u64> pw(N), ipw(N);
+  std::vector<uint32_t> slot(N);  // place of twiddle index i = 2^s + r
+  for (uint32_t i = 1; i < N; ++i) {
+    const int s = 31 - __builtin_clz(i), sl = s - l1;
+    if (sl < 0) {
+      slot[i] = tw_slot(l1, i);
+    } else {
+      const uint32_t r = i - (1u << s);
+      slot[i] = (1u << l1) + ((r >> sl) << l2) + tw_slot(l2, (1u << sl) + (r & ((1u << sl) - 1)));
+    }
+  }
   for (int t = 0; t < T; ++t) {
     const u64 q = C->primes[t];
     C->pdev.push_back(h_prime_dev(q));
@@ -71,17 +83,16 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
       pw[k] = h_mulmod(pw[k - 1], w, q);
       ipw[k] = h_mulmod(ipw[k - 1], wi, q);
     }
-    for (size_t i = 0; i < N; ++i) {
+    for (size_t i = 1; i < N; ++i) {
       const uint32_t r = h_bitrev((uint32_t)i, C->log_n);
-      psi2[2 * (t * N + i)] = pw[r];
-      psi2[2 * (t * N + i) + 1] = h_shoup(pw[r], q);
-      ipsi2[2 * (t * N + i)] = ipw[r];
-      ipsi2[2 * (t * N + i) + 1] = h_shoup(ipw[r], q);
+      const size_t at = 2 * (t * TS + slot[i]);
+      psi2[at] = h_mont(pw[r], q);
+      psi2[at + 1] = h_mont(psi2[at], q);
+      ipsi2[at] = h_mont(ipw[r], q);
+      ipsi2[at + 1] = h_mont(ipsi2[at], q);
     }
     ninv[t] = h_invmod(N % q, q);
     ninv_sh[t] = h_shoup(ninv[t], q);
-    r64[2 * t] = (u64)(((u128)1 << 64) % q);
-    r64[2 * t + 1] = h_shoup(r64[2 * t], q);
   }
   {
     std::vector<u64> pd(T * sizeof(PrimeDev) / 8);
@@ -92,7 +103,6 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
   upload(*C, C->d_ipsi2, ipsi2);
   upload(*C, C->d_ninv, ninv);
   upload(*C, C->d_ninv_sh, ninv_sh);
-  upload(*C, C->d_r64, r64);
   C->tab = Tables{(const PrimeDev*)C->d_primes.p, (const ulonglong2*)C->d_psi2.p, (const ulonglong2*)C->d_ipsi2.p,
                   C->d_ninv.p, C->d_ninv_sh.p, C->log_n, 3, 3, 3, 3};
 
@@ -138,7 +148,7 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
   md.insert(md.end(), pinv_sh.begin(), pinv_sh.end());
   md.insert(md.end(), halfq.begin(), halfq.end());
   // fused ModDown: the special-prime iNTT ends with N^-1 phinv_k, the conversion adds
-  // c_k = floor(P/2) phinv_k and multiplies by phat_q with Shoup companions
+  // c_k = floor(P/2) phinv_k and multiplies by phat_q
   std::vector<u64> md2;
   for (int k = 0; k < K; ++k) {
     const u64 pk = p_of(k), w = h_mulmod(h_invmod(N % pk, pk), phinv[k], pk);
@@ -146,9 +156,18 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
     md2.push_back(h_shoup(w, pk));
   }
   for (int k = 0; k < K; ++k) md2.push_back(h_mulmod(halfP_mod(p_of(k)), phinv[k], p_of(k)));
-  for (int k = 0; k < K; ++k)
-    for (int i = 0; i < nq; ++i) md2.push_back(h_shoup(md[3 * K + (size_t)k * nq + i], C->primes[i]));
   for (int k = 0; k < K; ++k) md2.push_back(p_of(k));
+  for (int word = 0; word < 2; ++word)
+    for (int k = 0; k < K; ++k)
+      for (int i = 0; i < nq; ++i) {
+        const u64 a = h_mont(md[3 * K + (size_t)k * nq + i], C->primes[i]);
+        md2.push_back(word ? h_mont(a, C->primes[i]) : a);
+      }
+  for (int word = 0; word < 2; ++word)
+    for (int i = 0; i < nq; ++i) {
+      const u64 a = h_mont(pinv[i], C->primes[i]);
+      md2.push_back(word ? h_mont(a, C->primes[i]) : a);
+    }
   upload(*C, C->d_moddown, md);
   upload(*C, C->d_moddown2, md2);
   // ModDown fused with a rescale: the conversion scaled by P^-1, i.e. phat_k P^-1 = p_k^-1 mod q_i and
@@ -157,8 +176,8 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
   for (int k = 0; k < K; ++k)
     for (int i = 0; i < nq; ++i) {
       const u64 qi = C->primes[i], f = h_invmod(p_of(k) % qi, qi);
-      mdr[(size_t)k * nq + i] = f;
-      mdr[(size_t)(K + k) * nq + i] = h_shoup(f, qi);
+      mdr[(size_t)k * nq + i] = h_mont(f, qi);
+      mdr[(size_t)(K + k) * nq + i] = h_mont(h_mont(f, qi), qi);
     }
   for (int i = 0; i < nq; ++i) mdr[(size_t)2 * K * nq + i] = h_mulmod(halfq[i], pinv[i], C->primes[i]);
   upload(*C, C->d_mdr, mdr);
@@ -221,7 +240,7 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
 void gen_switch_key(Ctx& C, u64 g, const u64* sp, const u64* s_to) {
   const int T = C.total_primes(), nq = C.n_q, dn = C.dnum(C.L());
   const size_t N = C.N;
-  DevBuf key((size_t)dn * 2 * T * N, C.stream);
+  DevBuf key((size_t)dn * 2 * T * N, C.stream), digit((size_t)2 * T * N, C.stream);
   std::vector<u64> ah(T * N), eh(T * N);
   std::vector<i64> e(N);
   for (int j = 0; j < dn; ++j) {
@@ -232,16 +251,17 @@ void gen_switch_key(Ctx& C, u64 g, const u64* sp, const u64* s_to) {
     for (size_t i = 0; i < N; ++i) e[i] = draw_cbd21(se);
     for (int t = 0; t < T; ++t)
       for (size_t i = 0; i < N; ++i) eh[t * N + i] = h_smod(e[i], C.primes[t]);
-    u64* b = key.p + (size_t)j * 2 * T * N;
+    u64* b = digit.p;
     u64* a = b + (size_t)T * N;
+    u64* to = key.p + (size_t)j * 2 * T * N;
     HEDAP_CUDA(cudaMemcpyAsync(b, eh.data(), T * N * 8, cudaMemcpyHostToDevice, C.stream));
     HEDAP_CUDA(cudaMemcpyAsync(a, ah.data(), T * N * 8, cudaMemcpyHostToDevice, C.stream));
     ntt_forward(C.tab, LimbSet{b, 0, 1, 0, T, nq, 0, nq}, C.stream);
     const int lo = j * C.alpha, hi = std::min(lo + C.alpha, nq);
     k_keygen_combine(C, b, a, s_to, sp, C.d_pmod.p, lo, hi);
     const u64* f = C.d_key_scale.p + (size_t)2 * j * T;  // the folded conversion factors (Ctx::key_scale)
-    k_scale_limbs(C, b, T, f);
-    k_scale_limbs(C, a, T, f);
+    k_key_store(C, b, to, T, f);
+    k_key_store(C, a, to + (size_t)T * N, T, f);
     HEDAP_CUDA(cudaStreamSynchronize(C.stream));  // host buffers are reused
   }
   C.keys[g] = std::move(key);

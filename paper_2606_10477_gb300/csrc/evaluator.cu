@@ -129,9 +129,9 @@ const LevelConsts& level_consts(Ctx& C, int l) {
   }
   L->modup = DevBuf(v.size(), C.stream);
   HEDAP_CUDA(cudaMemcpyAsync(L->modup.p, v.data(), v.size() * 8, cudaMemcpyHostToDevice, C.stream));
-  // the key switch's fused ModUp: every factor divided by the key's scale (Ctx::key_scale); the factor
-  // of the folded limb becomes 1 and is marked by a Shoup companion 0
-  std::vector<u64> vk(v);
+  // the key switch's fused ModUp: every factor divided by the key's scale (Ctx::key_scale), as pairs for
+  // mont_mul_lazy; the factor of the folded limb becomes 1 and is marked by a second word 0
+  std::vector<u64> vk(2 * nb, 0);
   double products = 0;
   const int T = C.total_primes();
   for (int j = 0; j < dn; ++j) {
@@ -143,10 +143,11 @@ const LevelConsts& level_consts(Ctx& C, int l) {
       const int i0 = C.key_scale_i0[(size_t)j * T + gt];
       for (int i = lo; i < hi; ++i) {
         const size_t at = 2 * (l + 1) + ((size_t)j * a + (i - lo)) * ext + t;
+        const size_t to = at - 2 * (l + 1);
         const u64 f = h_mulmod(v[at], un, pt);
-        vk[at] = f;
-        vk[at + nb] = (i == i0 && f == 1) ? 0 : h_shoup(f, pt);
-        products += vk[at + nb] ? 1 : 0;
+        vk[to] = h_mont(f, pt);
+        vk[to + nb] = (i == i0 && f == 1) ? 0 : h_mont(vk[to], pt);
+        products += vk[to + nb] ? 1 : 0;
       }
     }
   }
@@ -171,8 +172,8 @@ const LevelConsts& level_consts(Ctx& C, int l) {
       L->rescale.inv[i] = h_invmod(ql % q[i], q[i]);
       L->rescale.inv_sh[i] = h_shoup(L->rescale.inv[i], q[i]);
       r[i] = L->rescale.ql_mod[i];
-      r[l + i] = L->rescale.inv[i];
-      r[2 * l + i] = L->rescale.inv_sh[i];
+      r[l + i] = h_mont(L->rescale.inv[i], q[i]);
+      r[2 * l + i] = h_mont(r[l + i], q[i]);
     }
     L->d_rescale = DevBuf(r.size(), C.stream);
     HEDAP_CUDA(cudaMemcpyAsync(L->d_rescale.p, r.data(), r.size() * 8, cudaMemcpyHostToDevice, C.stream));
@@ -185,8 +186,8 @@ const LevelConsts& level_consts(Ctx& C, int l) {
     };
     std::vector<u64> w(2 * (size_t)l);
     for (int i = 0; i < l; ++i) {
-      w[i] = h_mulmod(h_invmod(P_mod(q[i]), q[i]), L->rescale.inv[i], q[i]);
-      w[l + i] = h_shoup(w[i], q[i]);
+      w[i] = h_mont(h_mulmod(h_invmod(P_mod(q[i]), q[i]), L->rescale.inv[i], q[i]), q[i]);
+      w[l + i] = h_mont(w[i], q[i]);
     }
     L->d_mdr = DevBuf(w.size(), C.stream);
     HEDAP_CUDA(cudaMemcpyAsync(L->d_mdr.p, w.data(), w.size() * 8, cudaMemcpyHostToDevice, C.stream));
@@ -244,8 +245,8 @@ static DevBuf ks_modup(Ctx& C, const u64* d, size_t d_stride, int batch, int l, 
   up.own_limit = l + 1;
   up.z = dc.p;
   up.z_stride = nl * N;
-  up.bconv = LC.modup_ks.p + 2 * nl;  // factors divided by the key's folded ones
-  up.bconv_sh_offset = (size_t)dn * C.alpha * ext;
+  up.bconv = LC.modup_ks.p;  // factors divided by the key's folded ones
+  up.bconv_b_offset = (size_t)dn * C.alpha * ext;
   up.ext = ext;
   up.z_products = LC.modup_products * batch * (double)N;
   ntt_forward(C.tab, LimbSet{y.p, (size_t)ext * N, batch * dn, 0, ext, l + 1, 0, C.n_q}, C.stream, &up, fuse);
@@ -274,17 +275,17 @@ static void ks_moddown(Ctx& C, const DevBuf& acc, int batch, int l, u64* out, si
   ntt_inverse(C.tab, LimbSet{acc.p, (size_t)ext * N, 2 * batch, l + 1, K, l + 1, 0, C.n_q}, C.stream, &inv);
   DevBuf v((size_t)batch * 2 * nl * N, C.stream);
   if (!fuse) k_moddown_spread(C, acc.p, v.p, 2 * batch, l);
-  const u64* Pinv = C.d_moddown.p + 3 * K + (size_t)K * C.n_q;
+  const u64* Pinv = C.d_moddown2.p + 4 * K + 2 * (size_t)K * C.n_q;
   NttAux fw{};
   if (fuse) {
     fw.pconv = acc.p + nl * N;
     fw.pconv_stride = (size_t)ext * N;
     fw.pconv_K = K;
     fw.pconv_ld = C.n_q;
-    fw.pconv_q = C.d_moddown2.p + 3 * K + (size_t)K * C.n_q;
+    fw.pconv_q = C.d_moddown2.p + 3 * K;
     fw.pconv_c = C.d_moddown2.p + 2 * K;
-    fw.pconv_phat = C.d_moddown.p + 3 * K;
-    fw.pconv_phat_sh = C.d_moddown2.p + 3 * K;
+    fw.pconv_phat = C.d_moddown2.p + 4 * K;
+    fw.pconv_phat_b = C.d_moddown2.p + 4 * K + (size_t)K * C.n_q;
     fw.pconv_half = C.d_moddown.p + 3 * K + (size_t)K * C.n_q + 2 * (size_t)C.n_q;
   }
   fw.fin_dst = out;
@@ -292,7 +293,7 @@ static void ks_moddown(Ctx& C, const DevBuf& acc, int batch, int l, u64* out, si
   fw.fin_c = acc.p;
   fw.fin_c_stride = (size_t)ext * N;
   fw.fin_w = Pinv;
-  fw.fin_wsh = Pinv + C.n_q;
+  fw.fin_wb = Pinv + C.n_q;
   fw.fin_acc_even = acc0 ? 1 : 0;
   fw.fin_acc_odd = acc1 ? 1 : 0;
   ntt_forward(C.tab, qset(v.p, nl * N, 2 * batch, 0, l + 1), C.stream, &fw);
@@ -323,7 +324,6 @@ static DevBuf ks_inner(Ctx& C, const u64* d, size_t d_stride, int batch, int l, 
   F.key_a_offset = (size_t)T * C.N;
   F.acc = acc.p;
   F.acc_part_stride = (size_t)(l + 1 + C.n_p) * C.N;
-  F.r64 = C.d_r64.p;
   F.batch = batch;
   ks_modup(C, d, d_stride, batch, l, &F);  // its column-phase buffer is released stream-ordered
   return acc;
@@ -364,10 +364,10 @@ static void ks_moddown_rescale(Ctx& C, const DevBuf& acc, int batch, int l, cons
   fw.pconv_stride = (size_t)ext * N;
   fw.pconv_K = K;
   fw.pconv_ld = nq;
-  fw.pconv_q = C.d_moddown2.p + 3 * K + (size_t)K * nq;
+  fw.pconv_q = C.d_moddown2.p + 3 * K;
   fw.pconv_c = C.d_moddown2.p + 2 * K;
   fw.pconv_phat = C.d_mdr.p;
-  fw.pconv_phat_sh = C.d_mdr.p + (size_t)K * nq;
+  fw.pconv_phat_b = C.d_mdr.p + (size_t)K * nq;
   fw.pconv_half = C.d_mdr.p + 2 * (size_t)K * nq;
   fw.spread = x.p;
   fw.spread_stride = N;
@@ -378,11 +378,11 @@ static void ks_moddown_rescale(Ctx& C, const DevBuf& acc, int batch, int l, cons
   fw.fin_c = acc.p;
   fw.fin_c_stride = (size_t)ext * N;
   fw.fin_w = LC.d_mdr.p;
-  fw.fin_wsh = LC.d_mdr.p + l;
+  fw.fin_wb = LC.d_mdr.p + l;
   fw.fin_e = e;
   fw.fin_e_stride = e_stride;
   fw.fin_w2 = LC.d_rescale.p + l;
-  fw.fin_w2sh = LC.d_rescale.p + 2 * l;
+  fw.fin_w2b = LC.d_rescale.p + 2 * l;
   fw.fin_neg = negate ? 1 : 0;
   ntt_forward(C.tab, qset(v.p, (size_t)l * N, 2 * batch, 0, l), C.stream, &fw);
 }
@@ -467,7 +467,7 @@ std::unique_ptr<Ct> ev_rescale(Ctx& C, const Ct& a) {
   fw.fin_c = a.part(0);
   fw.fin_c_stride = a.part_stride();
   fw.fin_w = LC.d_rescale.p + l;
-  fw.fin_wsh = LC.d_rescale.p + 2 * l;
+  fw.fin_wb = LC.d_rescale.p + 2 * l;
   ntt_forward(C.tab, qset(tmp.p, (size_t)l * N, P, 0, l), C.stream, &fw);
   return o;
 }

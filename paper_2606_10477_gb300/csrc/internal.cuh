@@ -42,6 +42,7 @@ bool h_is_prime(u64 n);
 std::vector<u64> h_prime_chain(int log_n, const std::vector<int>& bits);
 u64 h_find_psi(u64 q, int log_n);
 u64 h_shoup(u64 w, u64 q);  // floor(w * 2^64 / q)
+u64 h_mont(u64 w, u64 q);   // w 2^32 mod q: (h_mont(w), h_mont(h_mont(w))) is mont_mul_lazy's pair for w
 PrimeDev h_prime_dev(u64 q);
 uint32_t h_bitrev(uint32_t x, int bits);
 u64 h_smod(i64 v, u64 q);
@@ -80,10 +81,23 @@ struct DevBuf {
 };
 
 // ------------------------------------------------------------------ tables and limb sets
+// Twiddles of one prime, N = 2^(L1+L2), L1 = floor(log2 N / 2): first the column phase's (stages 0 .. L1-1), then
+// a run of 2^L2 for each of the 2^L1 blocks of the row phase.  Within a phase of L stages the twiddle of stage s,
+// sub-block r has tree index 2^s + r; tw_slot gives its place, so that the lanes of a warp, one group each,
+// read consecutive pairs: the first K0 = ceil(L/2) stages in tree order, then entry by entry (stage K0 + u, sub-block
+// mm of a group) over the 2^K0 groups.  Slot 0 of a run is unused.
+__host__ __device__ constexpr size_t tw_stride(int l1, int l2) { return ((size_t)1 << (l1 + l2)) + ((size_t)1 << l1); }
+inline uint32_t tw_slot(int l, uint32_t tree) {
+  const int k0 = (l + 1) / 2;
+  if (tree < (1u << k0)) return tree;
+  const int s = 31 - __builtin_clz(tree), u = s - k0;
+  const uint32_t r = tree - (1u << s);
+  return (1u << k0) + (((1u << u) - 1 + (r & ((1u << u) - 1))) << k0) + (r >> u);
+}
 struct Tables {
   const PrimeDev* pr;        // [n_primes]
-  const ulonglong2* psi2;    // [n_primes][N] (psi^bitrev(i), Shoup companion)
-  const ulonglong2* ipsi2;   // [n_primes][N] (psi^-bitrev(i), Shoup companion)
+  const ulonglong2* psi2;    // [n_primes][tw_stride] (w 2^32, w 2^64) mod q of w = psi^bitrev(i)
+  const ulonglong2* ipsi2;   // the same of psi^-bitrev(i)
   const u64* ninv;           // [n_primes] N^-1
   const u64* ninv_sh;
   int log_n;
@@ -95,7 +109,7 @@ struct Tables {
   int ntt_modup_variant;
   int ntt_fin_variant;
 };
-constexpr int kNttVariants = 8;
+constexpr int kNttVariants = 8, kNttShapes = 2;  // variants v and v + kNttShapes are one launch shape
 enum NttRole { NTT_ROLE_FORWARD = 0, NTT_ROLE_INVERSE = 1, NTT_ROLE_MODUP = 2, NTT_ROLE_FINISH = 3 };
 int& ntt_role_variant(Tables& T, int role);
 
@@ -136,8 +150,8 @@ struct NttAux {
   // from z (limb stride N, member stride z_stride) instead of reading limb li
   const u64* z = nullptr;
   size_t z_stride = 0;
-  const u64* bconv = nullptr;  // [dn][alpha][ext]; their Shoup companions at bconv + bconv_sh_offset
-  size_t bconv_sh_offset = 0;  // a companion 0 marks a factor 1: z is added without a product
+  const u64* bconv = nullptr;  // [dn][alpha][ext]: f 2^32; f 2^64 at bconv + bconv_b_offset (mont_mul_lazy's pairs)
+  size_t bconv_b_offset = 0;   // a second word 0 marks a factor 1: z is added without a product
   int ext = 0;
   double z_products = -1;  // products of the whole launch's conversion (word x term), for the profiler
   // forward only: the first phase loads the centred residue of one coefficient-domain limb (the
@@ -156,18 +170,18 @@ struct NttAux {
   int pconv_ld = 0;                   // row length of the per-target tables
   const u64* pconv_q = nullptr;       // [K] the special moduli s_k
   const u64* pconv_c = nullptr;       // [K] floor(S/2) shat_k^-1 mod s_k
-  const u64* pconv_phat = nullptr;    // [K][ld] (S / s_k) mod q_i
-  const u64* pconv_phat_sh = nullptr; // their Shoup companions
+  const u64* pconv_phat = nullptr;    // [K][ld] (S / s_k) 2^32 mod q_i
+  const u64* pconv_phat_b = nullptr;  // [K][ld] (S / s_k) 2^64 mod q_i
   const u64* pconv_half = nullptr;    // [ld] floor(S/2) mod q_i
   // forward only: the second phase does not store the transform v; it writes
   //   fin_dst[part][li] = (fin_c[part][li] - v) * fin_w[li]  (+ fin_dst[part][li] when the part's
-  //   parity bit is set), Shoup factors fin_w / fin_wsh per limb, canonical residues
+  //   parity bit is set), factors as mont_mul_lazy's pairs fin_w / fin_wb per limb, canonical residues
   u64* fin_dst = nullptr;
   size_t fin_dst_stride = 0;
   const u64* fin_c = nullptr;
   size_t fin_c_stride = 0;
   const u64* fin_w = nullptr;
-  const u64* fin_wsh = nullptr;
+  const u64* fin_wb = nullptr;
   int fin_acc_even = 0, fin_acc_odd = 0;
   // with fin_e: a key switch's ModDown fused with the rescale that follows it (see ks_moddown_rescale):
   //   fin_dst[part][li] = fin_c[part][li] * fin_w[li] + (fin_e[part][li] - v) * fin_w2[li]
@@ -176,22 +190,28 @@ struct NttAux {
   const u64* fin_e = nullptr;
   size_t fin_e_stride = 0;
   const u64* fin_w2 = nullptr;
-  const u64* fin_w2sh = nullptr;
+  const u64* fin_w2b = nullptr;
   int fin_neg = 0;  // with fin_e: store the negated residues
 };
 // Forward only: the second phase of the ModUp transform of a key switch fused with the key inner
 // product (k_ntt_fwd_rows_ksk): the transformed digits are multiplied by the switching key and summed
 // over the digits instead of being stored.  The LimbSet's parts are (ciphertext k, digit j) = k dn + j
 // (dn = NttAux::own_dn), its limbs the extended limbs t; a digit's own limbs are read from d.
+// Switching keys are stored with the word pairs of each 256-word run permuted: pair p (words 2 p, 2 p + 1) sits at pair
+// key_pair(p), so that a warp whose lanes own 8 consecutive words each reads 512 consecutive bytes per
+// load (k_ntt_fwd_rows_ksk), and one whose lanes own consecutive pairs reads whole 128-byte lines
+// (k_ksk_inner_kernel).  Exported keys are put back in order.
+__host__ __device__ constexpr size_t key_pair(size_t p) {
+  return (p & ~(size_t)127) + (p & 3) * 32 + ((p >> 2) & 31);
+}
 struct KskFuse {
   const u64* d = nullptr;        // NTT-domain inputs: ciphertext k's limb t at d + k d_stride + t N
   size_t d_stride = 0;
-  const u64* key = nullptr;      // switching key [dn][2][n_q + n_p][N] (digit j: b then a)
+  const u64* key = nullptr;      // switching key [dn][2][n_q + n_p][N] (digit j: b then a), see key_pair
   size_t key_digit_stride = 0;   // 2 (n_q + n_p) N
   size_t key_a_offset = 0;       // (n_q + n_p) N
   u64* acc = nullptr;            // output: part p of ciphertext k, limb t at acc + (2k + p) acc_part_stride + t N
   size_t acc_part_stride = 0;
-  const u64* r64 = nullptr;      // per prime: 2^64 mod q and its Shoup companion
   int batch = 0;
 };
 void ntt_forward(const Tables& T, const LimbSet& S, cudaStream_t st, const NttAux* aux = nullptr,
@@ -250,13 +270,13 @@ struct MdrLast {
 };
 struct LevelConsts {  // device constants for one level (evaluator.cu)
   DevBuf modup;       // qhat_inv (+shoup) per Q prime, qhat mod target per digit (+shoup)
-  DevBuf modup_ks;    // the same with every factor divided by the key's scale (key_scale); a factor 1
-                      // folded into the key has Shoup companion 0 (the load adds z without a product)
+  DevBuf modup_ks;    // qhat mod target per digit divided by the key's scale (key_scale), as mont_mul_lazy's pairs
+                      // [f 2^32][f 2^64]; a factor 1 folded into the key has second word 0 (z added as it is)
   double modup_products = 0;  // products per word of one ciphertext's fused ModUp (folded terms excluded)
   DevBuf intt_post;   // per Q prime i <= l: N^-1 qhat_i^-1 mod q_i and its Shoup companion
-  DevBuf d_rescale;   // [ql_mod l][inv l][inv_sh l] (the rescale constants below, on the device)
+  DevBuf d_rescale;   // [q_l mod q_i] and mont_mul_lazy's pair of q_l^-1 mod q_i, [first words][second words], i < l
   RescaleConsts rescale;
-  DevBuf d_mdr;       // ModDown fused with the rescale: [(P q_l)^-1 mod q_i][its Shoup companion], i < l
+  DevBuf d_mdr;       // ModDown fused with the rescale: mont_mul_lazy's pair of (P q_l)^-1 mod q_i, i < l
   MdrLast mdr_last;   // ... and the constants of its last limb (prime q_l)
 };
 
@@ -287,15 +307,15 @@ struct Ctx {
   std::vector<PrimeDev> pdev;
   DevBuf d_primes, d_psi2, d_ipsi2, d_ninv, d_ninv_sh;
   DevBuf d_moddown;   // level-independent ModDown constants
-  DevBuf d_moddown2;  // fused ModDown: [N^-1 phinv_k, Shoup][K] pairs, c_k [K], phat_q Shoup [K][n_q], p_k [K]
-  DevBuf d_mdr;       // ModDown scaled by P^-1 (fused with a rescale): p_k^-1 mod q_i [K][n_q], their Shoup
-                      // companions [K][n_q], floor(P/2) P^-1 mod q_i [n_q]
-  DevBuf d_r64;       // per prime: 2^64 mod q and its Shoup companion
+  DevBuf d_moddown2;  // fused ModDown: [N^-1 phinv_k, Shoup][K] pairs, c_k [K], p_k [K], then mont_mul_lazy's pairs of
+                      // phat_q, [K][n_q] first words and [K][n_q] second words, and of P^-1 mod q_i, [n_q] and [n_q]
+  DevBuf d_mdr;       // ModDown scaled by P^-1 (fused with a rescale): mont_mul_lazy's pairs of p_k^-1 mod q_i, [K][n_q]
+                      // first and [K][n_q] second words, then floor(P/2) P^-1 mod q_i [n_q]
   DevBuf d_pmod;      // per prime: P mod q_t (key generation)
   Tables tab{};
   std::vector<i64> sk;
   DevBuf d_sk;        // [n_q+n_p][N] NTT domain
-  std::map<u64, DevBuf> keys;  // galois (0 = relinearisation; 2, 4 encapsulation) -> [dnum][2][n_q+n_p][N]
+  std::map<u64, DevBuf> keys;  // galois (0 = relinearisation; 2, 4 encapsulation) -> [dnum][2][n_q+n_p][N], see key_pair
   // Limb t of key digit j, t outside the digit, is stored multiplied by key_scale[j][t]: the conversion
   // factor qhat_{i0} mod p_t of one digit limb i0 = key_scale_i0[j][t] (-1 and factor 1 where none is
   // folded), so that the ModUp conversion adds z_{i0} without a product (see ks_modup).  Exported keys

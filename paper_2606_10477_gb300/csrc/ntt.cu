@@ -5,24 +5,29 @@
 
 namespace hedap {
 
-void ntt_launch_10_11(int log_n, int v, const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse,
-                      const NttAux& A, const KskFuse* F);
-void ntt_launch_12_13(int log_n, int v, const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse,
-                      const NttAux& A, const KskFuse* F);
-void ntt_launch_14_15(int log_n, int v, const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse,
-                      const NttAux& A, const KskFuse* F);
-void ntt_launch_16(int log_n, int v, const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse,
-                   const NttAux& A, const KskFuse* F);
-void ntt_launch_17(int log_n, int v, const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse,
-                   const NttAux& A, const KskFuse* F);
+#define HEDAP_DECLARE(n)                                                                                        \
+  void ntt_launch_##n(int v, const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse, const NttAux& A, \
+                      const KskFuse* F);
+HEDAP_DECLARE(10)
+HEDAP_DECLARE(11)
+HEDAP_DECLARE(12)
+HEDAP_DECLARE(13)
+HEDAP_DECLARE(14)
+HEDAP_DECLARE(15)
+HEDAP_DECLARE(16)
+HEDAP_DECLARE(17)
+#undef HEDAP_DECLARE
 void ntt_launch(int log_n, int v, const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse,
                 const NttAux& A, const KskFuse* F) {
   switch (log_n) {
-    case 10: case 11: ntt_launch_10_11(log_n, v, S, T, st, inverse, A, F); break;
-    case 12: case 13: ntt_launch_12_13(log_n, v, S, T, st, inverse, A, F); break;
-    case 14: case 15: ntt_launch_14_15(log_n, v, S, T, st, inverse, A, F); break;
-    case 16: ntt_launch_16(log_n, v, S, T, st, inverse, A, F); break;
-    case 17: ntt_launch_17(log_n, v, S, T, st, inverse, A, F); break;
+    case 10: ntt_launch_10(v, S, T, st, inverse, A, F); break;
+    case 11: ntt_launch_11(v, S, T, st, inverse, A, F); break;
+    case 12: ntt_launch_12(v, S, T, st, inverse, A, F); break;
+    case 13: ntt_launch_13(v, S, T, st, inverse, A, F); break;
+    case 14: ntt_launch_14(v, S, T, st, inverse, A, F); break;
+    case 15: ntt_launch_15(v, S, T, st, inverse, A, F); break;
+    case 16: ntt_launch_16(v, S, T, st, inverse, A, F); break;
+    case 17: ntt_launch_17(v, S, T, st, inverse, A, F); break;
     default: throw Error(HEDAP_ERR_ARG, "log_n must lie in [10, 17]");
   }
 }
@@ -31,20 +36,20 @@ static void dispatch(const Tables& T, const LimbSet& S, cudaStream_t st, bool in
                      const KskFuse* F = nullptr) {
   if (S.n_parts * S.n_limbs == 0) return;
   const NttAux A = aux ? *aux : NttAux{};
-  if (F && (inverse || !A.own_alpha || !A.z || A.fin_dst || !F->d || !F->key || !F->acc || !F->r64 ||
+  if (F && (inverse || !A.own_alpha || !A.z || A.fin_dst || !F->d || !F->key || !F->acc ||
             F->batch < 1 || S.n_parts != F->batch * A.own_dn))
     throw Error(HEDAP_ERR_ARG, "NTT: bad key inner product fusion");
   if (A.own_alpha && (A.own_dn < 1 || A.own_alpha > 8)) throw Error(HEDAP_ERR_ARG, "NTT: bad digit layout");
-  if (A.z && (inverse || !A.own_alpha || !A.bconv || !A.bconv_sh_offset)) throw Error(HEDAP_ERR_ARG, "NTT: bad ModUp fusion");
+  if (A.z && (inverse || !A.own_alpha || !A.bconv || !A.bconv_b_offset)) throw Error(HEDAP_ERR_ARG, "NTT: bad ModUp fusion");
   if (A.post && !inverse) throw Error(HEDAP_ERR_ARG, "NTT: post factors apply to the inverse only");
   if ((A.spread || A.fin_dst || A.pconv) && inverse)
     throw Error(HEDAP_ERR_ARG, "NTT: fused rescale / ModDown applies to the forward only");
   if (A.pconv && (A.pconv_K < 1 || A.pconv_K > 8 || A.z || A.src || (A.spread && !A.fin_e)))
     throw Error(HEDAP_ERR_ARG, "NTT: bad ModDown fusion");
-  if (A.fin_e && (!A.fin_dst || !A.fin_w2 || !A.fin_w2sh || !A.pconv || !A.spread))
+  if (A.fin_e && (!A.fin_dst || !A.fin_w2 || !A.fin_w2b || !A.pconv || !A.spread))
     throw Error(HEDAP_ERR_ARG, "NTT: bad ModDown-rescale fusion");
   if (A.spread && (A.z || A.src || !A.spread_sub)) throw Error(HEDAP_ERR_ARG, "NTT: bad spread fusion");
-  if (A.fin_dst && (!A.fin_c || !A.fin_w || !A.fin_wsh)) throw Error(HEDAP_ERR_ARG, "NTT: bad epilogue fusion");
+  if (A.fin_dst && (!A.fin_c || !A.fin_w || !A.fin_wb)) throw Error(HEDAP_ERR_ARG, "NTT: bad epilogue fusion");
   const int v = inverse ? T.ntt_inv_variant
                         : A.z ? T.ntt_modup_variant
                               : (A.pconv || A.spread || A.fin_dst) ? T.ntt_fin_variant : T.ntt_fwd_variant;
@@ -75,21 +80,21 @@ void ntt_inverse(const Tables& T, const LimbSet& S, cudaStream_t st, const NttAu
 }
 
 // Register-only loop of the transform's butterfly (the rate the integer pipes allow without any
-// memory or shared-memory traffic): each thread runs `iters` rounds (even, alternating the even-
-// and odd-stage forms) of 4 independent lazy Cooley-Tukey butterflies on 8 residues of the
-// context's first prime and stores one word.
+// memory or shared-memory traffic): each thread runs `iters` rounds of 4 independent lazy Cooley-Tukey
+// butterflies (the small primes' form) on 8 words with the context's first prime and stores one word.
 __global__ void k_butterfly_loop(const Tables T, u64* out, int iters) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const u64 q = T.pr[0].q;
+  const uint32_t nqi = T.pr[0].nqi;
   const ulonglong2 w = T.psi2[1 + (threadIdx.x & 63)];
   u64 v[8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) v[m] = ((u64)i * 8 + m) % q;
   for (int it = 0; it < iters; it += 2) {  // an even and an odd stage
 #pragma unroll
-    for (int m = 0; m < 4; ++m) ct_bfly<true>(v[m], v[m + 4], w, q);
+    for (int m = 0; m < 4; ++m) ct_bfly<true, true>(v[m], v[m + 4], w, q, nqi);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) ct_bfly<false>(v[m], v[m + 4], w, q);
+    for (int m = 0; m < 4; ++m) ct_bfly<true, false>(v[m], v[m + 4], w, q, nqi);
   }
   u64 s = 0;
 #pragma unroll
@@ -161,10 +166,12 @@ void ntt_tune(Ctx& C, int limbs, int reps, std::vector<float>* fwd_ms, std::vect
   for (int dir = 0; dir < 2; ++dir) {
     float best = 1e30f;
     int best_v = 0;
+    float shape_ms[kNttShapes];
     for (int v = 0; v < kNttVariants; ++v) {
       Tables T = C.tab;
       T.ntt_fwd_variant = T.ntt_inv_variant = v;
-      const float ms = best_of([&] { dispatch(T, S, C.stream, dir == 1, nullptr); });
+      if (v < kNttShapes) shape_ms[v] = best_of([&] { dispatch(T, S, C.stream, dir == 1, nullptr); });
+      const float ms = shape_ms[v % kNttShapes];
       if (dir == 0 && fwd_ms) fwd_ms->push_back(ms);
       if (dir == 1 && inv_ms) inv_ms->push_back(ms);
       if (ms < best) { best = ms; best_v = v; }
@@ -181,7 +188,7 @@ void ntt_tune(Ctx& C, int limbs, int reps, std::vector<float>* fwd_ms, std::vect
       int& slot = ntt_role_variant(C.tab, role);
       float best = 1e30f;
       int best_v = slot;
-      for (int v = 0; v < kNttVariants; ++v) {
+      for (int v = 0; v < kNttShapes; ++v) {
         slot = v;
         const float ms = best_of([&] { ev_mul(C, *ct, *ct); });
         if (ms < best) { best = ms; best_v = v; }

@@ -6,761 +6,982 @@
 // Gentleman-Sande stages with psi^-bitrev, then N^-1.
 //
 // N = 2^(L1+L2) is split in two launches.  The first L1 forward stages only
-// couple elements whose index agrees modulo 2^L2, so each CTA loads C such
-// "columns" (rows of C consecutive words, coalesced) into shared memory and
-// runs those stages there; the last L2 stages couple only elements inside
-// blocks of 2^L2 consecutive words, so the second launch stages whole blocks.
-// Inside a launch every thread takes groups of 2^RL elements through RL stages
-// in registers between shared-memory exchanges (RL = 4: two passes per
-// 256-point phase; RL = 3: three).  For a group with elements at c = high*2^(S+K) + m*2^S + low (or the
-// mirrored forward form), the twiddle of every butterfly has a closed-form index
-// in (high, m, u), so no per-element index arithmetic is needed.  Twiddles are
-// (w, floor(w 2^64 / q)) pairs; every CTA stages the twiddles it uses in shared
-// memory with its data (the column phase's 2^L1, the row phase's contiguous
-// per-stage ranges for its blocks), both copied with cp.async so that all of a
-// tile's copies are in flight at once.  Optional fusions (NttAux):
-// the first phase may read another buffer (out of place) or compute its input as
-// the fast basis conversion of a key-switching digit (ModUp fused into the load),
-// the inverse may end with a per-limb factor other than N^-1, a digit's own
-// limbs may be skipped, and a rescale, a ModDown or both (one transform, see
-// ks_moddown_rescale) may be fused around a forward transform (conversion and
-// spread into the first phase's load, the finish into the second phase's store).  Butterflies keep residues
-// lazily (Harvey 2014): forward below 8q with the first operand reduced at every
-// other stage, inverse in [0, 2q); the final launch writes canonical residues.
+// couple elements whose index agrees modulo 2^L2 ("columns", 2^L1 words 2^L2 apart);
+// the last L2 stages couple only elements inside blocks of 2^L2 consecutive words.
+// What bounds a transform is instruction issue on the integer pipes (32-bit multiply-adds at half
+// rate, 64-bit products at a quarter), not memory: so the layout spends as few instructions per
+// butterfly as it can.
+//  * A phase of L stages is two register passes of K0 = ceil(L / 2) and K1 = floor(L / 2) stages
+//    (radix 16 twice for L = 8) with one exchange through shared memory between them, every thread
+//    holding 2^K0 words of a column or a block.  The 2^K1 threads of one block lie in one warp: the row phase
+//    has no CTA barrier.
+//  * The first pass of the column phase and the last one read and write global memory from
+//    registers (8 adjacent columns a CTA: whole 32-byte sectors).
+//  * Twiddles are (w 2^32, w 2^64) mod q pairs (mont_mul_lazy), stored per phase and block in the
+//    order in which the lanes of a warp read them (tw_slot): every load is coalesced and
+//    free of bank conflicts, and a block's twiddles are one run of 2^L2 pairs.
+//  * Residues stay lazy (Harvey 2014).  For 1.5 2^32 <= q < 2^57 the forward stages reduce nothing: the first load adds a
+//    multiple of q that keeps every difference non-negative, and the last store reduces (below 112q < 2^64);
+//    other primes reduce the first operand at every other stage (below 12q).  Inverse: for 1.5 2^32 <= q < 2^55
+//    bounds double unreduced through a phase.
+// GB300, N = 2^16, against Shoup butterflies in radix-8 passes with a CTA barrier each: forward of 384 limbs
+// 304 -> 222 us, HMult with rescale of 8 ciphertexts at level 23 3.28 -> 2.37 ms.  The big kernels then issue
+// 0.45 - 0.47 instructions a cycle with the multiply pipe 68 - 78% busy, as the register loop of the
+// butterfly itself does (0.48 and 82%): what is left is their instruction count.
+// Optional fusions (NttAux): the first phase may read another buffer (out of place) or compute its
+// input as the fast basis conversion of a key-switching digit (ModUp fused into the load),
+// the inverse may end with a per-limb factor other than N^-1, a digit's own limbs may be skipped,
+// and a rescale, a ModDown or both (one transform, see ks_moddown_rescale) may be fused around a
+// forward transform (conversion and spread into the first phase's load, the finish into the second
+// phase's store).
 #pragma once
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.cuh"
 #include "profiler.cuh"
 
 namespace hedap {
 
-// Forward (Cooley-Tukey) butterfly on lazy residues.  Every stage adds at most 2q to the bound
-// (t < 2q), so the first operand is brought from [0, 8q) into [0, 4q) only at even stages
-// (REDUCE): an even stage leaves values below 6q, the odd stage after it below 8q (< 2^64 for
-// q < 2^61), and the next even stage starts again from [0, 4q).
-template <bool REDUCE>
-__device__ __forceinline__ void ct_bfly(u64& x, u64& y, const ulonglong2 w, u64 q) {
-  if constexpr (REDUCE) {
-    const u64 q4 = q << 2;
-    if (x >= q4) x -= q4;
-  }
-  const u64 t = shoup_mul_lazy(y, w.x, w.y, q);  // [0, 2q)
-  const u64 q2 = q << 1;
-  y = x + q2 - t;
+// ---------------------------------------------------------------- butterflies
+// mont_mul_lazy returns less than 3q.  Forward (Cooley-Tukey), small primes (1.5 2^32 <= q < 2^57): x + t and x - t
+// as they are; a stage lowers and raises the bounds by 3q, so the first load adds 3 log2(N) q and the words stay
+// within [0, (9.2 + 6 log2(N)) q) < 2^64.  Seven products and eight additions, 32.9 cycles of a scheduler per warp
+// in a register loop, against 40.3 with x + 3q - t and 37.2 of a Shoup butterfly that reduces x every other stage.
+// Large primes: x + 3q - t, and x brought from [0, 12q) to [0, 6q] at even stages: 9q after an even
+// stage, 12q < 2^64 after the odd one (and 2^32 more, see sub_if_above).
+template <bool SMALL, bool EVEN>
+__device__ __forceinline__ void ct_bfly(u64& x, u64& y, const ulonglong2 w, u64 q, uint32_t nqi) {
+  if constexpr (!SMALL && EVEN) x = sub_if_above(x, q * 6);
+  const u64 t = mont_mul_lazy(y, w.x, w.y, q, nqi);  // [0, 3q)
+  y = SMALL ? x - t : x + q * 3 - t;
   x = x + t;
 }
-// stage `s` of the forward transform (global index)
-__device__ __forceinline__ void ct_bfly_stage(int s, u64& x, u64& y, const ulonglong2 w, u64 q) {
-  if (s % 2 == 0) ct_bfly<true>(x, y, w, q);
-  else ct_bfly<false>(x, y, w, q);
+__device__ __forceinline__ bool fwd_small(u64 q) { return q >= (3ull << 31) && q < (1ull << 57); }
+__device__ __forceinline__ bool inv_small(u64 q) { return q >= (3ull << 31) && q < (1ull << 55); }
+// what the first load of a forward transform adds to every word
+template <int LOGN>
+__device__ __forceinline__ u64 fwd_bias(u64 q) { return fwd_small(q) ? q * (3 * LOGN) : 0; }
+// canonical residue of a forward transform's lazy output (112q or 12q, see above)
+template <bool SMALL>
+__device__ __forceinline__ u64 fwd_canonical(u64 x, u64 q, uint32_t rc) {
+  if constexpr (SMALL) {
+    x = reduce_lazy(x, q, rc);
+  } else {
+    if (x >= q * 8) x -= q * 8;
+    if (x >= q * 4) x -= q * 4;
+    if (x >= q * 2) x -= q * 2;
+  }
+  return x >= q ? x - q : x;
 }
-__device__ __forceinline__ void gs_bfly(u64& x, u64& y, const ulonglong2 w, u64 q) {
-  const u64 q2 = q << 1;
-  u64 s = x + y;
-  if (s >= q2) s -= q2;
-  const u64 d = x + q2 - y;
-  y = shoup_mul_lazy(d, w.x, w.y, q);
-  x = s;
+// c - v for a lazy forward output v and a canonical c, as a non-negative 64-bit word
+template <bool SMALL>
+__device__ __forceinline__ u64 fwd_minus(u64 c, u64 v, u64 q) { return c + q * (SMALL ? 112 : 13) - v; }
+
+// K forward stages in registers on G columns of 2^K words: stage S + u (S the global index of the
+// first) pairs words 2^(K-1-u) apart; tw(u, mm) is the twiddle of sub-block mm of stage u
+template <bool SMALL, int S, int K, int G, class TW>
+__device__ __forceinline__ void fwd_pass(u64 (&v)[G][1 << K], u64 q, uint32_t nqi, TW tw) {
+#pragma unroll
+  for (int u = 0; u < K; ++u) {
+#pragma unroll
+    for (int mm = 0; mm < (1 << u); ++mm) {
+      const ulonglong2 w = tw(u, mm);
+#pragma unroll
+      for (int k = 0; k < (1 << (K - 1 - u)); ++k) {
+        const int m = (mm << (K - u)) + k, h = 1 << (K - 1 - u);
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          if ((S + u) % 2 == 0) ct_bfly<SMALL, true>(v[g][m], v[g][m + h], w, q, nqi);
+          else ct_bfly<SMALL, false>(v[g][m], v[g][m + h], w, q, nqi);
+        }
+      }
+    }
+  }
 }
-__device__ __forceinline__ u64 reduce8q(u64 x, u64 q) {
-  const u64 q4 = q << 2, q2 = q << 1;
-  if (x >= q4) x -= q4;
-  if (x >= q2) x -= q2;
-  if (x >= q) x -= q;
-  return x;
+// K inverse (Gentleman-Sande) stages in registers, the mirror image: stage u pairs words 2^u apart, its
+// sub-block mm spans 2^(u+1) words, tw(u', mm) with u' = K - 1 - u as in the forward pass.  SMALL: the
+// bound 2^E q doubles at every stage; otherwise sums are kept below 3q + 2^32 (differences are taken from 4q).
+template <bool SMALL, int E, int K, int G, class TW>
+__device__ __forceinline__ void inv_pass(u64 (&v)[G][1 << K], u64 q, uint32_t nqi, TW tw) {
+#pragma unroll
+  for (int u = 0; u < K; ++u) {
+#pragma unroll
+    for (int mm = 0; mm < (1 << (K - 1 - u)); ++mm) {
+      const ulonglong2 w = tw(K - 1 - u, mm);
+#pragma unroll
+      for (int k = 0; k < (1 << u); ++k) {
+        const int m = (mm << (u + 1)) + k, h = 1 << u;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          u64 &x = v[g][m], &y = v[g][m + h];
+          const u64 off = SMALL ? q << (E + u) : q * 4;
+          u64 s = x + y;
+          const u64 d = x + off - y;
+          if constexpr (!SMALL) s = sub_if_above(s, q * 3);
+          y = mont_mul_lazy(d, w.x, w.y, q, nqi);
+          x = s;
+        }
+      }
+    }
+  }
 }
+
+// ---------------------------------------------------------------- geometry
 // asynchronous global -> shared copies (cp.async): every copy of a tile is in flight at once, with
-// no register round trip; one wait_group 0 and a barrier make them visible to the CTA
+// no register round trip
 __device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(sdst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
-__device__ __forceinline__ void cp_async8(void* sdst, const void* gsrc) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(sdst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+__device__ __forceinline__ ulonglong2 ldg2(const u64* p) { return *reinterpret_cast<const ulonglong2*>(p); }
+__device__ __forceinline__ void stg2(u64* p, ulonglong2 v) { *reinterpret_cast<ulonglong2*>(p) = v; }
 
-// RL: stages per register pass (radix 2^RL), a template parameter of every kernel
+// A phase of L stages on 2^L words: pass 0 of K0 stages, thread `low` (of 2^K1) holding words
+// m 2^K1 + low; pass 1 of K1 stages, a thread holding the 2^K1 consecutive words of GP = 2^(K0-K1) groups.
+template <int L>
+struct Phase {
+  static constexpr int K0 = (L + 1) / 2, K1 = L / 2;
+  static constexpr int M0 = 1 << K0, M1 = 1 << K1;  // words of a group in pass 0 / pass 1
+  static constexpr int GP = 1 << (K0 - K1);         // pass-1 groups a thread owns
+  static constexpr int PER = 32 >> K1;              // blocks a warp holds
+};
+// column phase, a CTA of TH threads, one column a thread: word c of column cg at (c + (c >> K1)) COLS + cg (a row of
+// padding every 2^K1 rows, so that pass 1's reads are free of bank conflicts)
+template <int L1, int TH>
+struct ColGeo : Phase<L1> {
+  using P = Phase<L1>;
+  static constexpr int COLS = TH >> P::K1;
+  static constexpr int XWORDS = ((1 << L1) + P::M0) * COLS;  // exchange
+  static constexpr int TILE = (1 << L1) * COLS;              // one staged tile
+};
+// row phase, per warp: PER blocks, two words of padding every 2^K1 words (LDS.128 of consecutive words is free
+// of bank conflicts) and 2^K1 after each block when several blocks share a half-warp
+template <int L2>
+struct RowGeo : Phase<L2> {
+  using P = Phase<L2>;
+  static constexpr int GS = P::M1 + 2;                                           // stride of a group
+  static constexpr int BS = P::M0 * GS + (P::K1 < 4 ? P::M1 : 0);                // stride of a block
+  static constexpr int XWORDS = P::PER * BS;
+};
 
+// ---------------------------------------------------------------- fused loads
 // true when limb li of `part` is one of its digit's own limbs (skipped, see NttAux)
 __device__ __forceinline__ bool own_limb(const NttAux& A, int part, int li) {
   if (!A.own_alpha) return false;
   const int lo = (part % A.own_dn) * A.own_alpha;
   return li >= lo && li < min(lo + A.own_alpha, A.own_limit);
 }
-// source of limb li of `part` for the first phase (in place unless A.src)
-__device__ __forceinline__ const u64* first_src(const NttAux& A, const LimbSet& S, int part, int li, size_t N) {
-  return A.src ? A.src + part * A.src_stride + (size_t)li * N : S.limb(part, li, N);
-}
-
-// shared-memory index of element x of a row block: one pad word every 16
-__device__ __forceinline__ uint32_t padx(uint32_t x) { return x + (x >> 4); }
-// Row layout (rows of 2^L2 words, R = 2^L2 + 2^(L2-4) apart).  For the words idx = t + i TPB of an unrolled
-// loop (t = threadIdx.x; TPB and 2^L2 powers of two, TPB a multiple of 16) the offset is a per-thread part
-// row_off(t) plus a compile-time part row_step(i): no index arithmetic per word.
-template <int L2>
-__device__ __forceinline__ uint32_t row_off(uint32_t t) {
-  return (t >> L2) * ((1u << L2) + (1u << (L2 - 4))) + padx(t & ((1u << L2) - 1));
-}
-template <int L2, int TPB>
-__host__ __device__ constexpr uint32_t row_step(int i) {
-  constexpr uint32_t P2 = 1u << L2, R = P2 + (P2 >> 4);
-  return (uint32_t)TPB >= P2 ? (uint32_t)i * ((uint32_t)TPB >> L2) * R
-                             : (uint32_t)(i / (int)(P2 / TPB)) * R + (uint32_t)(i % (int)(P2 / TPB)) * TPB +
-                                   (((uint32_t)(i % (int)(P2 / TPB)) * TPB) >> 4);
-}
+// A first phase's input words of one limb, from the words z(t) of `ns` tiles: the digit's
+// coefficient-domain limbs (ModUp), the special limbs (ModDown; the last limb's coefficients as z(ns) when a
+// rescale is fused) or the last limb (rescale), at most three products.  They share one Montgomery
+// step.  ModUp: a term folded into the key is z itself, below the bound the key's construction checked (8q
+// in all).  ModDown: q - floor(P/2) mod q plus the products (below 4.2q).  The rescale's centred last
+// limb: x, plus -q_l mod q when x > q_l / 2, below 3q.  In all below 9.2q.
+enum LoadKind { LOAD_PLAIN = 0, LOAD_MODUP = 1, LOAD_MODDOWN = 2, LOAD_SPREAD = 3 };
+enum LastLimb { LAST_NONE = 0, LAST_RAW = 1, LAST_MONT = 2 };  // how a fused rescale's last limb enters the sum
+template <int KIND>
+struct FusedLoad {
+  static constexpr int MAXT = 3;
+  u64 f[MAXT], fb[MAXT], c[MAXT], pk[MAXT];  // products: factor pairs, and the ModDown's rounding constants
+  int tile[MAXT];                            // tile of product t
+  u64 off, half, sub;
+  PrimeDev P;
+  int nm, raw, last;  // products, the tile added as it is (-1: none), LastLimb
+  int ns;
+  // bias: added to every word (fwd_bias)
+  __device__ __forceinline__ void init(const NttAux& A, const Tables& T, const PrimeDev& p, u64 bias, int j, int li,
+                                       int n_tiles) {
+    P = p;
+    ns = n_tiles;
+    off = bias;
+    half = sub = 0;
+    raw = -1;
+    last = LAST_NONE;
+    nm = KIND == LOAD_SPREAD ? 0 : ns;
+    if (KIND == LOAD_MODUP) {
+      const u64* bc = A.bconv + (size_t)j * A.own_alpha * A.ext + li;
+#pragma unroll
+      for (int t = 0; t < MAXT; ++t)
+        if (t < ns && !bc[A.bconv_b_offset + (size_t)t * A.ext]) raw = t;  // at most one
+      nm = ns - (raw >= 0);
+#pragma unroll
+      for (int t = 0; t < MAXT; ++t) {
+        tile[t] = raw >= 0 && t >= raw ? t + 1 : t;
+        f[t] = t < nm ? bc[(size_t)tile[t] * A.ext] : 0;
+        fb[t] = t < nm ? bc[A.bconv_b_offset + (size_t)tile[t] * A.ext] : 0;
+      }
+    } else if (KIND == LOAD_MODDOWN) {
+#pragma unroll
+      for (int t = 0; t < MAXT; ++t) {
+        const bool on = t < ns;
+        tile[t] = t;
+        c[t] = on ? A.pconv_c[t] : 0;
+        pk[t] = on ? A.pconv_q[t] : 0;
+        f[t] = on ? A.pconv_phat[(size_t)t * A.pconv_ld + li] : 0;
+        fb[t] = on ? A.pconv_phat_b[(size_t)t * A.pconv_ld + li] : 0;
+      }
+      off += p.q - A.pconv_half[li];
+    }
+    if (KIND == LOAD_SPREAD || (KIND == LOAD_MODDOWN && A.spread)) {
+      const u64 ql = T.pr[A.spread_prime].q;
+      half = ql >> 1;
+      sub = p.q - A.spread_sub[li];
+      last = ql < 2 * p.q ? LAST_RAW : LAST_MONT;
+    }
+  }
+  template <int NM, bool RAW, int LAST, class Z>
+  __device__ __forceinline__ u64 word(Z z) const {
+    const u64 q = P.q;
+    u64 v = off;
+    MontAcc s{0, 0};
+#pragma unroll
+    for (int t = 0; t < NM; ++t) {
+      u64 x = z(tile[t]);
+      if (KIND == LOAD_MODDOWN) x = add_mod(x, c[t], pk[t]);
+      mont_mac(s, x, f[t], fb[t]);
+    }
+    if (RAW) v += z(raw);
+    if (LAST != LAST_NONE) {
+      const u64 x = z(KIND == LOAD_SPREAD ? 0 : ns);
+      if (LAST == LAST_RAW) v += x;
+      else mont_add(s, x, P.r64);
+      if (x > half) v += sub;
+    }
+    if (NM > 0 || LAST == LAST_MONT) v += mont_finish(s, q, P.nqi);
+    return v;
+  }
+  // calls body with a function word(z) for this limb's terms: no branch per word
+  template <class F>
+  __device__ __forceinline__ void apply(F body) const {
+#define HEDAP_WORDS(NM, RAW, LAST) body([&](auto z) { return word<NM, RAW, LAST>(z); })
+    if constexpr (KIND == LOAD_SPREAD) {
+      if (last == LAST_RAW) HEDAP_WORDS(0, false, LAST_RAW);
+      else HEDAP_WORDS(0, false, LAST_MONT);
+    } else if constexpr (KIND == LOAD_MODUP) {
+      if (raw >= 0) {
+        if (nm == 1) HEDAP_WORDS(1, true, LAST_NONE);
+        else if (nm == 2) HEDAP_WORDS(2, true, LAST_NONE);
+        else HEDAP_WORDS(0, true, LAST_NONE);
+      } else {
+        if (nm == 1) HEDAP_WORDS(1, false, LAST_NONE);
+        else if (nm == 2) HEDAP_WORDS(2, false, LAST_NONE);
+        else HEDAP_WORDS(3, false, LAST_NONE);
+      }
+    } else {
+      if (last == LAST_NONE) {
+        if (nm == 1) HEDAP_WORDS(1, false, LAST_NONE);
+        else if (nm == 2) HEDAP_WORDS(2, false, LAST_NONE);
+        else HEDAP_WORDS(3, false, LAST_NONE);
+      } else if (last == LAST_RAW) {
+        if (nm == 1) HEDAP_WORDS(1, false, LAST_RAW);
+        else if (nm == 2) HEDAP_WORDS(2, false, LAST_RAW);
+        else HEDAP_WORDS(3, false, LAST_RAW);
+      } else {
+        if (nm == 1) HEDAP_WORDS(1, false, LAST_MONT);
+        else if (nm == 2) HEDAP_WORDS(2, false, LAST_MONT);
+        else HEDAP_WORDS(3, false, LAST_MONT);
+      }
+    }
+#undef HEDAP_WORDS
+  }
+};
 
 // ---------------------------------------------------------------- forward, column phase
-// element (c, col) at sm[c * C + col]; global index j = r0 + col + c * 2^L2;
-// stage s couples c and c + 2^(L1-s-1); twiddle index 2^s + (c >> (L1 - s)).
-template <int L1, int C, int RL, int S0>
-__device__ __forceinline__ void fwd_cols_passes(u64* sm, const ulonglong2* tw, u64 q) {
-  if constexpr (S0 < L1) {
-    constexpr int K = (L1 - S0) < RL ? (L1 - S0) : RL;
-    constexpr int TL = 1 << (L1 - S0 - K);
-    constexpr int GROUPS = C << (L1 - K);
-    constexpr int TPB = (C << L1) >> RL;  // threads per CTA
+// both passes of one limb's columns: v holds pass 0's input (row m 2^K1 + low), out the limb's words at (row 0,
+// this thread's column); tw: global memory (L1) or shared memory
+template <bool SMALL, int L1, int L2, int TH>
+__device__ __forceinline__ void fwd_cols_body(u64 (&v)[1][1 << Phase<L1>::K0], u64* xs, const ulonglong2* tw, u64 q,
+                                              uint32_t nqi, int low, int cg, u64* out) {
+  using G = ColGeo<L1, TH>;
+  fwd_pass<SMALL, 0, G::K0, 1>(v, q, nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
+  __syncthreads();  // the last limb's exchange has been read
 #pragma unroll
-    for (int g = threadIdx.x; g < GROUPS; g += TPB) {
-      const uint32_t col = g % C, gg = g / C;
-      const uint32_t low = gg & (TL - 1), high = gg >> (L1 - S0 - K);
-      const uint32_t base = (high << (L1 - S0)) | low;
-      u64 v[1 << K];
+  for (int m = 0; m < G::M0; ++m) xs[(m * (G::M1 + 1) + low) * G::COLS + cg] = v[0][m];
+  __syncthreads();
 #pragma unroll
-      for (int m = 0; m < (1 << K); ++m) v[m] = sm[(base + m * TL) * C + col];
+  for (int i = 0; i < G::GP; ++i) {
+    const int hi = i * G::M1 + low;  // rows hi 2^K1 + m
+    u64 w[1][G::M1];
 #pragma unroll
-      for (int u = 0; u < K; ++u) {
-        const int half = 1 << (K - 1 - u);
+    for (int m = 0; m < G::M1; ++m) w[0][m] = xs[(hi * (G::M1 + 1) + m) * G::COLS + cg];
+    fwd_pass<SMALL, G::K0, G::K1, 1>(w, q, nqi, [&](int u, int mm) {
+      return tw[G::M0 + ((1 << u) - 1 + mm) * G::M0 + hi];
+    });
 #pragma unroll
-        for (int m1 = 0; m1 < (1 << K); ++m1) {
-          if (m1 & half) continue;
-          const uint32_t wi = (1u << (S0 + u)) + (high << u) + (m1 >> (K - u));
-          ct_bfly_stage(S0 + u, v[m1], v[m1 + half], tw[wi], q);
-        }
-      }
-#pragma unroll
-      for (int m = 0; m < (1 << K); ++m) sm[(base + m * TL) * C + col] = v[m];
-    }
-    __syncthreads();
-    fwd_cols_passes<L1, C, RL, S0 + K>(sm, tw, q);
+    for (int m = 0; m < G::M1; ++m) out[(size_t)(hi * G::M1 + m) << L2] = w[0][m];
   }
 }
-
-template <int L1, int L2, int C, int TPB, int MINB, int RL>
-__global__ void __launch_bounds__(TPB, MINB) k_ntt_fwd_cols(Tables T, LimbSet S, NttAux A) {
-  extern __shared__ u64 sm[];
+template <int N, int TH>  // N twiddles into shared memory
+__device__ __forceinline__ void stage_twiddles(ulonglong2* dst, const ulonglong2* src, int t) {
+#pragma unroll
+  for (int i = 0; i < (N + TH - 1) / TH; ++i)
+    if (N % TH == 0 || i * TH + t < N) cp_async16(dst + i * TH + t, src + i * TH + t);
+}
+template <int L1, int L2, int TH, int MINB>
+__global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols(Tables T, LimbSet S, NttAux A) {
+  using G = ColGeo<L1, TH>;
+  extern __shared__ __align__(16) u64 sm[];
   constexpr size_t N = (size_t)1 << (L1 + L2);
-  ulonglong2* tw = reinterpret_cast<ulonglong2*>(sm + (C << L1));
+  const int cg = threadIdx.x % G::COLS, low = threadIdx.x / G::COLS;
   const int y = blockIdx.y, part = y / S.n_limbs, li = S.limb_begin + y % S.n_limbs;
   if (own_limb(A, part, li)) return;
   const int pi = S.prime(li);
-  const u64 q = T.pr[pi].q;
-  u64* a = S.limb(part, li, N);
-  const ulonglong2* W = T.psi2 + (size_t)pi * N;
-#pragma unroll
-  for (int i = threadIdx.x; i < (1 << L1); i += TPB) cp_async16(tw + i, W + i);
-  const int r0 = blockIdx.x * C;
-  if (A.z) {  // fused ModUp: fast basis conversion of digit j into this limb's prime
-    // sum of na <= 8 Shoup products, each in [0, 2q), brought into [0, 4q): the
-    // first butterflies accept any input below 4q (a term folded into the key is z itself, below the
-    // bound the key's construction checked)
-    const int j = part % A.own_dn, lo = j * A.own_alpha, na = min(A.own_alpha, A.own_limit - lo);
-    const u64* zk = A.z + (size_t)(part / A.own_dn) * A.z_stride + (size_t)lo * N;
-    const u64* bc = A.bconv + (size_t)j * A.own_alpha * A.ext + li;
-    const u64* bcs = bc + A.bconv_sh_offset;
-    u64 f[8], fs[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      f[t] = t < na ? bc[(size_t)t * A.ext] : 0;
-      fs[t] = t < na ? bcs[(size_t)t * A.ext] : 0;
-    }
-    const u64 q4 = q << 2, q8 = q << 3;
-#pragma unroll
-    for (int idx = threadIdx.x; idx < (C << L1); idx += TPB) {
-      const int c = idx / C, col = idx % C;
-      const size_t n = ((size_t)c << L2) + r0 + col;
-      u64 v = 0;
-#pragma unroll
-      for (int t = 0; t < 8; ++t)
-        if (t < na) v += fs[t] ? shoup_mul_lazy(zk[(size_t)t * N + n], f[t], fs[t], q) : zk[(size_t)t * N + n];
-      if (v >= q8) v -= q8;
-      if (v >= q4) v -= q4;
-      sm[idx] = v;
-    }
-  } else if (A.pconv) {  // fused ModDown conversion of the special-prime limbs into this prime
-    const u64* zp = A.pconv + (size_t)part * A.pconv_stride;
-    u64 c[8], pk[8], f[8], fs[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const bool on = k < A.pconv_K;
-      c[k] = on ? A.pconv_c[k] : 0;
-      pk[k] = on ? A.pconv_q[k] : 0;
-      f[k] = on ? A.pconv_phat[(size_t)k * A.pconv_ld + li] : 0;
-      fs[k] = on ? A.pconv_phat_sh[(size_t)k * A.pconv_ld + li] : 0;
-    }
-    const u64 off = (q << 2) - A.pconv_half[li], q4 = q << 2, q8 = q << 3;
-    const bool lazy = A.pconv_K <= 5;
-#pragma unroll
-    for (int idx = threadIdx.x; idx < (C << L1); idx += TPB) {
-      const int cc = idx / C, col = idx % C;
-      const size_t n = ((size_t)cc << L2) + r0 + col;
-      // 4q - floor(S/2) mod q plus K products: lazy (< 2q each) for K <= 5, canonical (< q) for
-      // K <= 8, so the sum stays below 16q < 2^64
-      u64 v = off;
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (k < A.pconv_K) {
-          u64 term = shoup_mul_lazy(add_mod(zp[(size_t)k * N + n], c[k], pk[k]), f[k], fs[k], q);
-          if (!lazy && term >= q) term -= q;
-          v += term;
-        }
-      if (v >= q8) v -= q8;
-      if (v >= q4) v -= q4;
-      if (A.spread) {  // a ModDown fused with a rescale: plus the centred last limb, [0, 5q)
-        const u64 x = A.spread[(size_t)part * A.spread_stride + n];
-        const u64 half = T.pr[A.spread_prime].q >> 1;
-        u64 m = barrett_reduce(x, 0, T.pr[pi]);
-        if (x > half) m = sub_mod(m, A.spread_sub[li], q);
-        v += m;
-      }
-      sm[idx] = v;
-    }
-  } else if (A.spread) {  // fused rescale spread: centred residue of the last limb in this prime
-    const u64* x = A.spread + (size_t)part * A.spread_stride;
-    const u64 half = T.pr[A.spread_prime].q >> 1, sub = A.spread_sub[li];
-    const PrimeDev P = T.pr[pi];
-#pragma unroll
-    for (int idx = threadIdx.x; idx < (C << L1); idx += TPB) {
-      const int c = idx / C, col = idx % C;
-      const u64 v = x[((size_t)c << L2) + r0 + col];
-      u64 m = barrett_reduce(v, 0, P);
-      if (v > half) m = sub_mod(m, sub, q);
-      sm[idx] = m;
-    }
-  } else {
-    const u64* src = first_src(A, S, part, li, N);
-#pragma unroll
-    for (int idx = threadIdx.x; idx < (C << L1); idx += TPB) {
-      const int c = idx / C, col = idx % C;
-      cp_async8(sm + idx, src + ((size_t)c << L2) + r0 + col);
-    }
-  }
+  const PrimeDev P = T.pr[pi];
+  const size_t col = (size_t)blockIdx.x * G::COLS + cg;
+  const u64* src = (A.src ? A.src + part * A.src_stride + (size_t)li * N : S.limb(part, li, N)) + col;
+  ulonglong2* tw = reinterpret_cast<ulonglong2*>(sm + G::XWORDS);
+  stage_twiddles<1 << L1, TH>(tw, T.psi2 + (size_t)pi * tw_stride(L1, L2), threadIdx.x);
   cp_async_commit();
+  const u64 bias = fwd_bias<L1 + L2>(P.q);
+  u64 v[1][G::M0];
+#pragma unroll
+  for (int m = 0; m < G::M0; ++m) v[0][m] = src[(size_t)(m * G::M1 + low) << L2] + bias;
   cp_async_wait_all();
   __syncthreads();
-  fwd_cols_passes<L1, C, RL, 0>(sm, tw, q);
-#pragma unroll
-  for (int idx = threadIdx.x; idx < (C << L1); idx += TPB) {
-    const int c = idx / C, col = idx % C;
-    a[((size_t)c << L2) + r0 + col] = sm[idx];
-  }
+  u64* out = S.limb(part, li, N) + col;
+  if (fwd_small(P.q)) fwd_cols_body<true, L1, L2, TH>(v, sm, tw, P.q, P.nqi, low, cg, out);
+  else fwd_cols_body<false, L1, L2, TH>(v, sm, tw, P.q, P.nqi, low, cg, out);
 }
 
-// ---------------------------------------------------------------- forward, column phase from shared tiles, several limbs
-// Three fused first phases read the same few tiles for every output limb: the ModUp of one digit
-// (its na <= 3 coefficient-domain limbs z), the ModDown conversion (the K <= 3 special-prime limbs)
-// and the rescale spread (the last limb).  This kernel stages those tiles once (cp.async, straight
-// into shared memory) and runs the column phase of `lpc` consecutive output limbs of one part from
-// there, so the wait for global memory is paid once per lpc limbs; each limb's twiddles are
-// fetched with cp.async while the previous limb computes (two twiddle buffers).
-
-template <int L1, int L2, int C, int TPB, int MINB, int RL>
-__global__ void __launch_bounds__(TPB, MINB) k_ntt_fwd_cols_shared(Tables T, LimbSet S, NttAux A, int lpc) {
-  extern __shared__ u64 sm[];
+// The fused first phases read the same few tiles for every output limb: the ModUp of one digit its na <= 3
+// coefficient-domain limbs z, the ModDown conversion the K <= 3 special-prime limbs (plus the last limb when a
+// rescale is fused), the rescale spread the last limb.  A CTA stages the tiles of its TH / 2^K1 columns once
+// (cp.async, straight into shared memory) and runs the column phase of `lpc` consecutive output limbs of one
+// part from there.  One column a thread: with two, the tiles let only 8 warps fit an SM and the passes
+// waited on their own latency (1313 against 960 us, N = 2^16, 8 x 12 digits at level 23).
+template <int L1, int L2, int TH, int MINB, int KIND>
+__global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_shared(Tables T, LimbSet S, NttAux A, int lpc) {
+  using G = ColGeo<L1, TH>;
+  extern __shared__ __align__(16) u64 sm[];
   constexpr size_t N = (size_t)1 << (L1 + L2);
-  constexpr int E = C << L1;
-  ulonglong2* twb = reinterpret_cast<ulonglong2*>(sm + E);  // two buffers of 2^L1 pairs
-  u64* zt = sm + E + 4 * (1 << L1);                         // ns staged tiles of E words
+  const int cg = threadIdx.x % G::COLS, low = threadIdx.x / G::COLS;
   const int groups = (S.n_limbs + lpc - 1) / lpc;
   const int part = blockIdx.y / groups, g = blockIdx.y % groups;
   const int l0 = S.limb_begin + g * lpc, l1 = min(l0 + lpc, S.limb_begin + S.n_limbs);
-  // the shared tiles: ns limbs at src + t N (and, for a ModDown fused with a rescale, the last limb's
-  // coefficients as tile ns)
-  int ns, j = 0;
-  const u64* src;
-  const u64* spread_src = A.spread ? A.spread + (size_t)part * A.spread_stride : nullptr;
-  if (A.z) {
-    j = part % A.own_dn;
-    const int lo = j * A.own_alpha;
-    ns = min(A.own_alpha, A.own_limit - lo);
-    src = A.z + (size_t)(part / A.own_dn) * A.z_stride + (size_t)lo * N;
-  } else if (A.pconv) {
-    ns = A.pconv_K;
-    src = A.pconv + (size_t)part * A.pconv_stride;
-  } else {
-    ns = 0;
-    src = nullptr;
+  const size_t col = (size_t)blockIdx.x * G::COLS;
+  u64* zt = sm + G::XWORDS;
+  const int j = KIND == LOAD_MODUP ? part % A.own_dn : 0, lo = j * A.own_alpha;
+  const int ns = KIND == LOAD_MODUP ? min(A.own_alpha, A.own_limit - lo) : KIND == LOAD_MODDOWN ? A.pconv_K : 0;
+  const u64* base = KIND == LOAD_MODUP     ? A.z + (size_t)(part / A.own_dn) * A.z_stride + (size_t)lo * N
+                    : KIND == LOAD_MODDOWN ? A.pconv + (size_t)part * A.pconv_stride
+                                           : nullptr;
+  const u64* last = KIND != LOAD_MODUP && A.spread ? A.spread + (size_t)part * A.spread_stride : nullptr;
+  const int tiles = ns + (last ? 1 : 0);
+  for (int i = threadIdx.x; i < tiles * (G::TILE / 2); i += TH) {
+    const int t = i / (G::TILE / 2), e = 2 * (i % (G::TILE / 2)), row = e / G::COLS;
+    const u64* src = t < ns ? base + (size_t)t * N : last;
+    cp_async16(zt + (size_t)t * G::TILE + e, src + ((size_t)row << L2) + col + e % G::COLS);
   }
-  const int nt = ns + (spread_src ? 1 : 0);
-  const int r0 = blockIdx.x * C;
-  // row c of tile t holds words r0 .. r0 + C - 1 of column c (16-byte copies)
-  for (int idx = threadIdx.x; idx < nt * (E / 2); idx += TPB) {
-    const int t = idx / (E / 2), e = 2 * (idx % (E / 2));
-    const int c = e / C, col = e % C;
-    const u64* base = t < ns ? src + (size_t)t * N : spread_src;
-    cp_async16(zt + (size_t)t * E + e, base + ((size_t)c << L2) + r0 + col);
-  }
-  auto fetch_tw = [&](int li, int buf) {
-    const ulonglong2* W = T.psi2 + (size_t)S.prime(li) * N;
-    for (int i = threadIdx.x; i < (1 << L1); i += TPB) cp_async16(twb + buf * (1 << L1) + i, W + i);
-  };
-  int li = l0;
-  while (li < l1 && own_limb(A, part, li)) ++li;
-  if (li < l1) fetch_tw(li, 0);
   cp_async_commit();
-  int buf = 0;
-  for (; li < l1; buf ^= 1) {
-    int next = li + 1;
-    while (next < l1 && own_limb(A, part, next)) ++next;
-    cp_async_wait_all();
-    __syncthreads();  // the tiles and this limb's twiddles have landed; the previous limb is done
-    if (next < l1) fetch_tw(next, buf ^ 1);
-    cp_async_commit();
-    const int pi = S.prime(li);
-    const u64 q = T.pr[pi].q, q4 = q << 2, q8 = q << 3;
-    if (A.z) {  // ModUp: sum of na Shoup products (each < 2q; a folded term is z) brought into [0, 4q)
-      const u64* bc = A.bconv + (size_t)j * A.own_alpha * A.ext + li;
-      const u64* bcs = bc + A.bconv_sh_offset;
-      u64 f[3], fs[3];
-#pragma unroll
-      for (int t = 0; t < 3; ++t) {
-        f[t] = t < ns ? bc[(size_t)t * A.ext] : 0;
-        fs[t] = t < ns ? bcs[(size_t)t * A.ext] : 0;
-      }
-#pragma unroll
-      for (int idx = threadIdx.x; idx < E; idx += TPB) {
-        u64 v = 0;
-#pragma unroll
-        for (int t = 0; t < 3; ++t)
-          if (t < ns) v += fs[t] ? shoup_mul_lazy(zt[(size_t)t * E + idx], f[t], fs[t], q) : zt[(size_t)t * E + idx];
-        if (v >= q4) v -= q4;
-        sm[idx] = v;
-      }
-    } else if (A.pconv) {  // ModDown conversion: 4q - floor(P/2) mod q plus K lazy products (< 10q)
-      u64 c[3], pk[3], f[3], fs[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const bool on = k < ns;
-        c[k] = on ? A.pconv_c[k] : 0;
-        pk[k] = on ? A.pconv_q[k] : 0;
-        f[k] = on ? A.pconv_phat[(size_t)k * A.pconv_ld + li] : 0;
-        fs[k] = on ? A.pconv_phat_sh[(size_t)k * A.pconv_ld + li] : 0;
-      }
-      const u64 off = q4 - A.pconv_half[li];
-      // a ModDown fused with a rescale adds the centred last limb (tile ns, below q): [0, 5q)
-      const u64 half = spread_src ? T.pr[A.spread_prime].q >> 1 : 0, sub = spread_src ? A.spread_sub[li] : 0;
-      const PrimeDev P = T.pr[pi];
-#pragma unroll
-      for (int idx = threadIdx.x; idx < E; idx += TPB) {
-        u64 v = off;
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-          if (k < ns) v += shoup_mul_lazy(add_mod(zt[(size_t)k * E + idx], c[k], pk[k]), f[k], fs[k], q);
-        if (v >= q8) v -= q8;
-        if (v >= q4) v -= q4;
-        if (spread_src) {
-          const u64 x = zt[(size_t)ns * E + idx];
-          u64 m = barrett_reduce(x, 0, P);
-          if (x > half) m = sub_mod(m, sub, q);
-          v += m;
-        }
-        sm[idx] = v;
-      }
-    } else {  // rescale spread: centred residue of the last limb in this prime
-      const u64 half = T.pr[A.spread_prime].q >> 1, sub = A.spread_sub[li];
-      const PrimeDev P = T.pr[pi];
-#pragma unroll
-      for (int idx = threadIdx.x; idx < E; idx += TPB) {
-        const u64 v = zt[idx];
-        u64 m = barrett_reduce(v, 0, P);
-        if (v > half) m = sub_mod(m, sub, q);
-        sm[idx] = m;
-      }
-    }
-    __syncthreads();
-    fwd_cols_passes<L1, C, RL, 0>(sm, twb + buf * (1 << L1), q);
-    u64* a = S.limb(part, li, N);
-#pragma unroll
-    for (int idx = threadIdx.x; idx < E; idx += TPB) {
-      const int c = idx / C, col = idx % C;
-      a[((size_t)c << L2) + r0 + col] = sm[idx];
-    }
-    li = next;
-  }
-  cp_async_wait_all();
-}
-
-// ---------------------------------------------------------------- forward, block phase
-// block b, local x at sm[b * R + padx(x)]; j = (B0 + b) * 2^L2 + x; local stage s'
-// couples x and x + 2^(L2-s'-1); twiddle index 2^(L1+s') + ((B0+b) << s') + (x >> (L2 - s')).
-// For the CTA's blocks B0 .. B0+BPC-1 the twiddles of stage s' are the contiguous
-// range starting at 2^(L1+s') + (B0 << s') of BPC 2^s' entries; they are staged in
-// shared memory one stage after another (stage s' at offset BPC (2^s' - 1)), so
-// twiddle (b, s', r) sits at tw[BPC (2^s' - 1) + (b << s') + r].
-template <int L1, int L2, int BPC, int TPB>
-__device__ __forceinline__ void fwd_rows_stage_twiddles(ulonglong2* tw, const ulonglong2* W, uint32_t B0) {
-#pragma unroll
-  for (int sl = 0; sl < L2; ++sl) {
-    const ulonglong2* src = W + (1u << (L1 + sl)) + (B0 << sl);
-    ulonglong2* dst = tw + BPC * ((1 << sl) - 1);
-    for (int i = threadIdx.x; i < (BPC << sl); i += TPB) cp_async16(dst + i, src + i);
-  }
-}
-template <int L1, int L2, int BPC, int RL, int S0>
-__device__ __forceinline__ void fwd_rows_passes(u64* sm, const ulonglong2* tw, u64 q) {
-  if constexpr (S0 < L2) {
-    constexpr int K = (L2 - S0) < RL ? (L2 - S0) : RL;
-    constexpr int TL = 1 << (L2 - S0 - K);
-    constexpr int GPB = 1 << (L2 - K);
-    constexpr int R = (1 << L2) + (1 << (L2 - 4));
-    constexpr int TPB = (BPC << L2) >> RL;
-#pragma unroll
-    for (int g = threadIdx.x; g < BPC * GPB; g += TPB) {
-      const uint32_t b = g / GPB, gg = g % GPB;
-      const uint32_t low = gg & (TL - 1), high = gg >> (L2 - S0 - K);
-      const uint32_t base = (high << (L2 - S0)) | low;
-      // padx(base + m TL) = padx(base) + m TL + (m TL >> 4): base is aligned to the group's span except for
-      // low < TL, so the pad words between the group's elements depend on m only
-      u64* blk = sm + b * R + padx(base);
-      u64 v[1 << K];
-#pragma unroll
-      for (int m = 0; m < (1 << K); ++m) v[m] = blk[m * TL + ((m * TL) >> 4)];
-#pragma unroll
-      for (int u = 0; u < K; ++u) {
-        const int sl = S0 + u, half = 1 << (K - 1 - u);
-#pragma unroll
-        for (int m1 = 0; m1 < (1 << K); ++m1) {
-          if (m1 & half) continue;
-          const uint32_t wi = BPC * ((1u << sl) - 1) + (b << sl) + (high << u) + (m1 >> (K - u));
-          ct_bfly_stage(L1 + sl, v[m1], v[m1 + half], tw[wi], q);
-        }
-      }
-#pragma unroll
-      for (int m = 0; m < (1 << K); ++m) blk[m * TL + ((m * TL) >> 4)] = v[m];
-    }
-    __syncthreads();
-    fwd_rows_passes<L1, L2, BPC, RL, S0 + K>(sm, tw, q);
-  }
-}
-
-template <int L1, int L2, int BPC, int TPB, int MINB, int RL>
-__global__ void __launch_bounds__(TPB, MINB) k_ntt_fwd_rows(Tables T, LimbSet S, NttAux A) {
-  extern __shared__ u64 sm[];
-  constexpr size_t N = (size_t)1 << (L1 + L2);
-  constexpr int E = BPC << L2, R = (1 << L2) + (1 << (L2 - 4));
-  const int y = blockIdx.y, part = y / S.n_limbs, li = S.limb_begin + y % S.n_limbs;
-  if (own_limb(A, part, li)) return;
-  const int pi = S.prime(li);
-  const u64 q = T.pr[pi].q;
-  u64* a = S.limb(part, li, N);
-  ulonglong2* tw = reinterpret_cast<ulonglong2*>(sm + BPC * R);
-  const size_t j0 = (size_t)blockIdx.x * E;
-  u64* smt = sm + row_off<L2>(threadIdx.x);  // this thread's words: smt[row_step(i)] holds word t + i TPB
-#pragma unroll
-  for (int i = 0; i < E / TPB; ++i) cp_async8(smt + row_step<L2, TPB>(i), a + j0 + threadIdx.x + i * TPB);
-  fwd_rows_stage_twiddles<L1, L2, BPC, TPB>(tw, T.psi2 + (size_t)pi * N, (uint32_t)(blockIdx.x * BPC));
-  cp_async_commit();
-  if (A.fin_dst) {  // the epilogue's operands: fetched into L2 while the passes run (128-byte lines)
-    const u64* cp = A.fin_c + (size_t)part * A.fin_c_stride + (size_t)li * N + j0;
-    const u64* dp = A.fin_e ? A.fin_e + (size_t)part * A.fin_e_stride + (size_t)li * N + j0
-                            : A.fin_dst + (size_t)part * A.fin_dst_stride + (size_t)li * N + j0;
-    const bool acc = A.fin_e || ((part & 1) ? A.fin_acc_odd : A.fin_acc_even);
-    for (int idx = 16 * threadIdx.x; idx < E; idx += 16 * TPB) {
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(cp + idx));
-      if (acc) asm volatile("prefetch.global.L2 [%0];" ::"l"(dp + idx));
-    }
-  }
   cp_async_wait_all();
   __syncthreads();
-  fwd_rows_passes<L1, L2, BPC, RL, 0>(sm, tw, q);
-  if (A.fin_e) {  // ModDown fused with the rescale: c (P q_l)^-1 + (e - v) q_l^-1
-    const u64* cp = A.fin_c + (size_t)part * A.fin_c_stride + (size_t)li * N + j0;
-    const u64* ep = A.fin_e + (size_t)part * A.fin_e_stride + (size_t)li * N + j0;
-    u64* dp = A.fin_dst + (size_t)part * A.fin_dst_stride + (size_t)li * N + j0;
-    const u64 w = A.fin_w[li], wp = A.fin_wsh[li], w2 = A.fin_w2[li], w2p = A.fin_w2sh[li];
+  FusedLoad<KIND> F;
+  for (int li = l0; li < l1; ++li) {
+    if (own_limb(A, part, li)) continue;
+    const int pi = S.prime(li);
+    const PrimeDev P = T.pr[pi];
+    F.init(A, T, P, fwd_bias<L1 + L2>(P.q), j, li, ns);
+    u64 v[1][G::M0];
+    const u64* zl = zt + low * G::COLS + cg;
+    F.apply([&](auto word) {
 #pragma unroll
-    for (int i = 0; i < E / TPB; ++i) {
-      const int idx = threadIdx.x + i * TPB;
-      const u64 v = reduce8q(smt[row_step<L2, TPB>(i)], q);
-      const u64 z = add_mod(shoup_mul(cp[idx], w, wp, q), shoup_mul(sub_mod(ep[idx], v, q), w2, w2p, q), q);
-      dp[idx] = A.fin_neg ? sub_mod(0, z, q) : z;
-    }
-    return;
+      for (int m = 0; m < G::M0; ++m) v[0][m] = word([&](int t) { return zl[t * G::TILE + m * G::M1 * G::COLS]; });
+    });
+    const ulonglong2* tw = T.psi2 + (size_t)pi * tw_stride(L1, L2);
+    u64* out = S.limb(part, li, N) + col + cg;
+    if (fwd_small(P.q)) fwd_cols_body<true, L1, L2, TH>(v, sm, tw, P.q, P.nqi, low, cg, out);
+    else fwd_cols_body<false, L1, L2, TH>(v, sm, tw, P.q, P.nqi, low, cg, out);
   }
-  if (A.fin_dst) {  // fused epilogue of a rescale / ModDown: (c - v) * w (+ dst)
-    const u64* cp = A.fin_c + (size_t)part * A.fin_c_stride + (size_t)li * N + j0;
-    u64* dp = A.fin_dst + (size_t)part * A.fin_dst_stride + (size_t)li * N + j0;
-    const u64 w = A.fin_w[li], wp = A.fin_wsh[li];
+}
+
+// The same first phases with more than three products a word (digits of 4 to 8 primes, 4 to 8 special primes):
+// the tiles would fill the shared memory, so they are read from L2 term by term, all of a thread's words of
+// one term in flight, into open sums (MontAcc) in registers.
+template <int L1, int L2, int TH, int MINB, int KIND>
+__global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_wide(Tables T, LimbSet S, NttAux A) {
+  using G = ColGeo<L1, TH>;
+  extern __shared__ __align__(16) u64 sm[];
+  constexpr size_t N = (size_t)1 << (L1 + L2);
+  const int cg = threadIdx.x % G::COLS, low = threadIdx.x / G::COLS;
+  const int part = blockIdx.y / S.n_limbs, li = S.limb_begin + blockIdx.y % S.n_limbs;
+  if (own_limb(A, part, li)) return;
+  const int pi = S.prime(li);
+  const PrimeDev P = T.pr[pi];
+  const u64 q = P.q;
+  const size_t col = (size_t)blockIdx.x * G::COLS + cg;
+  const int j = KIND == LOAD_MODUP ? part % A.own_dn : 0, lo = j * A.own_alpha;
+  const int ns = KIND == LOAD_MODUP ? min(A.own_alpha, A.own_limit - lo) : A.pconv_K;
+  const u64* base = (KIND == LOAD_MODUP ? A.z + (size_t)(part / A.own_dn) * A.z_stride + (size_t)lo * N
+                                        : A.pconv + (size_t)part * A.pconv_stride) + ((size_t)low << L2) + col;
+  u64 off = fwd_bias<L1 + L2>(q);
+  if (KIND == LOAD_MODDOWN) off += q - A.pconv_half[li];
+  u64 v[1][G::M0];
+  MontAcc s[G::M0];
+#pragma unroll
+  for (int m = 0; m < G::M0; ++m) {
+    v[0][m] = 0;
+    s[m] = MontAcc{0, 0};
+  }
+  auto close = [&] {  // one Montgomery step: the column sums stay below 2^64 for four products
+#pragma unroll
+    for (int m = 0; m < G::M0; ++m) {
+      v[0][m] += mont_finish(s[m], q, P.nqi);
+      s[m] = MontAcc{0, 0};
+    }
+  };
+  for (int t = 0; t < ns; ++t) {
+    const u64* z = base + (size_t)t * N;
+    u64 f, fb, c = 0, pk = 0;
+    if (KIND == LOAD_MODUP) {
+      const u64* bc = A.bconv + ((size_t)j * A.own_alpha + t) * A.ext + li;
+      f = bc[0];
+      fb = bc[A.bconv_b_offset];
+    } else {
+      c = A.pconv_c[t];
+      pk = A.pconv_q[t];
+      f = A.pconv_phat[(size_t)t * A.pconv_ld + li];
+      fb = A.pconv_phat_b[(size_t)t * A.pconv_ld + li];
+    }
+    if (t == 4) close();
+    if (KIND == LOAD_MODUP && !fb) {  // folded into the key
+#pragma unroll
+      for (int m = 0; m < G::M0; ++m) v[0][m] += z[(size_t)(m * G::M1) << L2];
+    } else {
+#pragma unroll
+      for (int m = 0; m < G::M0; ++m) {
+        u64 x = z[(size_t)(m * G::M1) << L2];
+        if (KIND == LOAD_MODDOWN) x = add_mod(x, c, pk);
+        mont_mac(s[m], x, f, fb);
+      }
+    }
+  }
+  close();
+  // at most eight products (below 1.1q each, and 2q of the two steps) or a folded limb and seven: below 16q by the
+  // key's construction; brought below 10q, with the bias, the ModDown's constant and the last limb below 12q
+#pragma unroll
+  for (int m = 0; m < G::M0; ++m) v[0][m] = off + (v[0][m] >= q * 6 ? v[0][m] - q * 6 : v[0][m]);
+  if (KIND == LOAD_MODDOWN && A.spread) {
+    const u64* last = A.spread + (size_t)part * A.spread_stride + ((size_t)low << L2) + col;
+    const u64 ql = T.pr[A.spread_prime].q, half = ql >> 1, sub = q - A.spread_sub[li];
+#pragma unroll
+    for (int m = 0; m < G::M0; ++m) {
+      const u64 x = last[(size_t)(m * G::M1) << L2];
+      MontAcc a{0, 0};
+      mont_add(a, x, P.r64);
+      v[0][m] += mont_finish(a, q, P.nqi) + (x > half ? sub : 0);
+    }
+  }
+  const ulonglong2* tw = T.psi2 + (size_t)pi * tw_stride(L1, L2);
+  u64* out = S.limb(part, li, N) + col;
+  if (fwd_small(q)) fwd_cols_body<true, L1, L2, TH>(v, sm, tw, q, P.nqi, low, cg, out);
+  else fwd_cols_body<false, L1, L2, TH>(v, sm, tw, q, P.nqi, low, cg, out);
+}
+
+// ---------------------------------------------------------------- forward, row phase
+// A warp owns PER blocks of 2^L2 consecutive words of one limb; 2^K1 lanes per block.
+template <bool SMALL, int L1, int L2>
+__device__ __forceinline__ void fwd_rows_body(u64 (&v)[1][1 << Phase<L2>::K0], u64* xs, const ulonglong2* tw,
+                                              const PrimeDev& P, int low) {
+  using G = RowGeo<L2>;
+  const u64 q = P.q;
+  fwd_pass<SMALL, L1, G::K0, 1>(v, q, P.nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
+#pragma unroll
+  for (int m = 0; m < G::M0; ++m) xs[m * G::GS + low] = v[0][m];
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < G::GP; ++i) {
+    const int hi = i * G::M1 + low;
+    u64 w[1][G::M1];
+#pragma unroll
+    for (int m = 0; m < G::M1; m += 2) {
+      const ulonglong2 x = ldg2(xs + hi * G::GS + m);
+      w[0][m] = x.x;
+      w[0][m + 1] = x.y;
+    }
+    fwd_pass<SMALL, L1 + G::K0, G::K1, 1>(w, q, P.nqi, [&](int u, int mm) {
+      return tw[G::M0 + ((1 << u) - 1 + mm) * G::M0 + hi];
+    });
+#pragma unroll
+    for (int m = 0; m < G::M1; m += 2) stg2(xs + hi * G::GS + m, ulonglong2{w[0][m], w[0][m + 1]});
+  }
+  __syncwarp();
+}
+// word pair e (words 2 e, 2 e + 1) of a block in the exchange buffer
+template <int L2>
+__device__ __forceinline__ ulonglong2 row_pair(const u64* xs, int e) {
+  using G = RowGeo<L2>;
+  return ldg2(xs + (e >> (G::K1 - 1)) * G::GS + (e & (G::M1 / 2 - 1)) * 2);
+}
+template <bool SMALL, int L2>
+__device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u64* a, size_t at, int part, int li,
+                                               const PrimeDev& P, int low) {
+  using G = RowGeo<L2>;
+  const u64 q = P.q;
+  constexpr int PAIRS = G::M0 / 2;  // word pairs of a lane
+  if (A.fin_e) {  // ModDown fused with the rescale: c (P q_l)^-1 + (e - v) q_l^-1
+    const u64* cp = A.fin_c + (size_t)part * A.fin_c_stride + at;
+    const u64* ep = A.fin_e + (size_t)part * A.fin_e_stride + at;
+    u64* dp = A.fin_dst + (size_t)part * A.fin_dst_stride + at;
+    const u64 w = A.fin_w[li], wb = A.fin_wb[li], w2 = A.fin_w2[li], w2b = A.fin_w2b[li];
+    auto fin = [&](u64 c, u64 e, u64 v) {  // both products in one Montgomery step: below 4q
+      MontAcc s{0, 0};
+      mont_mac(s, c, w, wb);
+      mont_mac(s, fwd_minus<SMALL>(e, v, q), w2, w2b);
+      u64 z = mont_finish(s, q, P.nqi);
+      if (z >= q * 2) z -= q * 2;
+      return z >= q ? z - q : z;
+    };
+#pragma unroll
+    for (int k = 0; k < PAIRS; ++k) {
+      const int e = k * G::M1 + low;
+      const ulonglong2 v = row_pair<L2>(xs, e), c = ldg2(cp + 2 * e), ee = ldg2(ep + 2 * e);
+      ulonglong2 z;
+      z.x = fin(c.x, ee.x, v.x);
+      z.y = fin(c.y, ee.y, v.y);
+      if (A.fin_neg) {
+        z.x = sub_mod(0, z.x, q);
+        z.y = sub_mod(0, z.y, q);
+      }
+      stg2(dp + 2 * e, z);
+    }
+  } else if (A.fin_dst) {  // fused epilogue of a rescale / ModDown: (c - v) * w (+ dst)
+    const u64* cp = A.fin_c + (size_t)part * A.fin_c_stride + at;
+    u64* dp = A.fin_dst + (size_t)part * A.fin_dst_stride + at;
+    const u64 w = A.fin_w[li], wb = A.fin_wb[li];
+    auto fin = [&](u64 c, u64 v) {  // below 3q
+      u64 z = mont_mul_lazy(fwd_minus<SMALL>(c, v, q), w, wb, q, P.nqi);
+      if (z >= q * 2) z -= q * 2;
+      return z >= q ? z - q : z;
+    };
     const bool acc = (part & 1) ? A.fin_acc_odd : A.fin_acc_even;
 #pragma unroll
-    for (int i = 0; i < E / TPB; ++i) {
-      const int idx = threadIdx.x + i * TPB;
-      const u64 v = reduce8q(smt[row_step<L2, TPB>(i)], q);
-      u64 z = shoup_mul(sub_mod(cp[idx], v, q), w, wp, q);
-      if (acc) z = add_mod(z, dp[idx], q);
-      dp[idx] = z;
+    for (int k = 0; k < PAIRS; ++k) {
+      const int e = k * G::M1 + low;
+      const ulonglong2 v = row_pair<L2>(xs, e), c = ldg2(cp + 2 * e);
+      ulonglong2 z;
+      z.x = fin(c.x, v.x);
+      z.y = fin(c.y, v.y);
+      if (acc) {
+        const ulonglong2 d = ldg2(dp + 2 * e);
+        z.x = add_mod(z.x, d.x, q);
+        z.y = add_mod(z.y, d.y, q);
+      }
+      stg2(dp + 2 * e, z);
     }
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int i = 0; i < E / TPB; ++i) a[j0 + threadIdx.x + i * TPB] = reduce8q(smt[row_step<L2, TPB>(i)], q);
+    for (int k = 0; k < PAIRS; ++k) {
+      const int e = k * G::M1 + low;
+      const ulonglong2 v = row_pair<L2>(xs, e);
+      stg2(a + 2 * e, ulonglong2{fwd_canonical<SMALL>(v.x, q, P.rc), fwd_canonical<SMALL>(v.y, q, P.rc)});
+    }
+  }
 }
 
-// ---------------------------------------------------------------- forward, block phase fused with the key inner product
-// The extended digits of a key switch are transformed and immediately consumed by the inner product
-// with the switching key, so the transformed digits are never written.  A CTA owns one ciphertext k,
-// one extended limb t (prime pt) and one run of BPC row blocks; it stages the twiddles of prime pt
-// once and walks the dn digits: the column-phase output of digit j (or, for the digit that owns limb
-// t, the NTT-domain input d itself) is copied into shared memory with cp.async (the next digit's
-// copy in flight while this one computes), the row passes run, and every thread multiplies its
-// words by the two key words of digit j, limb t and adds the products into 128-bit accumulators.
-// One reduction per word at the end; acc[k][0/1][t] are the only stores.  Modular sums do not
-// depend on order, so the result equals the separate transform and inner product bit for bit.
-// Residues entering the products are canonical (< q < 2^61), so the sum of up to 64 products stays
-// below 2^128.
-template <int L1, int L2, int BPC, int TPB, int MINB, int RL>
-__global__ void __launch_bounds__(TPB, MINB) k_ntt_fwd_rows_ksk(Tables T, LimbSet S, NttAux A, KskFuse F) {
-  extern __shared__ u64 sm[];
+// `ppc` parts of one limb per warp, one after the other: they share the blocks' twiddles, staged once
+template <int L1, int L2, int W, int MINB>
+__global__ void __launch_bounds__(32 * W, MINB) k_ntt_fwd_rows(Tables T, LimbSet S, NttAux A, int ppc) {
+  using G = RowGeo<L2>;
+  extern __shared__ __align__(16) u64 sm[];
   constexpr size_t N = (size_t)1 << (L1 + L2);
-  constexpr int E = BPC << L2, R = (1 << L2) + (1 << (L2 - 4)), PER = E / TPB;
-  u64* buf[2] = {sm, sm + BPC * R};
-  ulonglong2* tw = reinterpret_cast<ulonglong2*>(sm + 2 * BPC * R);
-  const int k = blockIdx.x % F.batch, blk = blockIdx.x / F.batch;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, low = lane % G::M1, b = lane / G::M1;
+  const int pg = blockIdx.y / S.n_limbs, li = S.limb_begin + blockIdx.y % S.n_limbs;
+  const int pi = S.prime(li);
+  const PrimeDev P = T.pr[pi];
+  const int blk = (blockIdx.x * W + warp) * G::PER + b;
+  u64* xs = sm + warp * G::XWORDS + b * G::BS;
+  ulonglong2* tw = reinterpret_cast<ulonglong2*>(sm + W * G::XWORDS) + (warp * G::PER << L2);  // the warp's blocks
+  stage_twiddles<(G::PER << L2), 32>(tw, T.psi2 + (size_t)pi * tw_stride(L1, L2) + (1 << L1) + ((size_t)(blk - b) << L2),
+                                     lane);
+  cp_async_commit();
+  tw += b << L2;
+  const size_t j0 = (size_t)blk << L2, at = (size_t)li * N + j0;
+  bool staged = false;
+  for (int part = pg * ppc; part < min((pg + 1) * ppc, S.n_parts); ++part) {
+    if (own_limb(A, part, li)) continue;
+    u64* a = S.limb(part, li, N) + j0;
+    if (A.fin_dst) {  // the epilogue's operands: fetched into L2 while the passes run (128-byte lines)
+      const u64* cp = A.fin_c + (size_t)part * A.fin_c_stride + at;
+      const u64* dp = A.fin_e ? A.fin_e + (size_t)part * A.fin_e_stride + at
+                              : A.fin_dst + (size_t)part * A.fin_dst_stride + at;
+      const bool acc = A.fin_e || ((part & 1) ? A.fin_acc_odd : A.fin_acc_even);
+      for (int idx = 16 * low; idx < (1 << L2); idx += 16 * G::M1) {
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(cp + idx));
+        if (acc) asm volatile("prefetch.global.L2 [%0];" ::"l"(dp + idx));
+      }
+    }
+    u64 v[1][G::M0];
+#pragma unroll
+    for (int m = 0; m < G::M0; ++m) v[0][m] = a[m * G::M1 + low];
+    if (!staged) {
+      cp_async_wait_all();
+      __syncwarp();
+      staged = true;
+    }
+    if (fwd_small(P.q)) {
+      fwd_rows_body<true, L1, L2>(v, xs, tw, P, low);
+      fwd_rows_store<true, L2>(xs, A, a, at, part, li, P, low);
+    } else {
+      fwd_rows_body<false, L1, L2>(v, xs, tw, P, low);
+      fwd_rows_store<false, L2>(xs, A, a, at, part, li, P, low);
+    }
+    __syncwarp();
+  }
+  cp_async_wait_all();
+}
+
+// ---------------------------------------------------------------- forward, row phase fused with the key inner product
+// The extended digits of a key switch are transformed and immediately consumed by the inner product
+// with the switching key, so the transformed digits are never written.  A warp owns one ciphertext k, one
+// extended limb t (prime pt) and KB blocks of 2^L2 words (256 words in all, 8 a lane, so that the lane's
+// 16 sums of 128 bits stay in registers) and walks the dn digits: the column-phase output of digit j is copied
+// into the warp's shared memory with cp.async while the previous digit computes, the passes run between
+// warp barriers, and each word is multiplied by the two key words of digit j, limb t (loaded before the
+// passes).  The digit owning t comes last: there the NTT-domain input d itself.  One reduction per word at the end; acc[k][0/1][t]
+// are the only stores.  Modular sums do not depend on order, so the result equals the separate
+// transform and inner product bit for bit.  Consecutive warps hold the batch members of one block,
+// so each key word comes from L2 once per CTA and the block's twiddles, staged in shared memory once,
+// serve all of them.  Words entering the products are below 112q < 2^64 with q < 2^57, or below 3.1q with
+// q < 2^60.1: the sum of up to 64 products stays below 2^128.
+template <int L2>
+struct KskGeo {
+  static constexpr int PER = L2 > 8 ? (1 << (L2 - 5)) : 8;  // words a lane
+  static constexpr int LPB = (1 << L2) / PER;               // lanes a block
+  static constexpr int KB = 32 / LPB;                       // blocks a warp
+  // passes: a first one of F stages, then passes of 3
+  static constexpr int F = L2 % 3 ? L2 % 3 : 3, NP = (L2 + 2) / 3;
+  static constexpr int word(int x) { return x + 2 * (x >> 3) + 8 * (x >> 6); }  // padded index inside a block
+  static constexpr int BS = (1 << L2) + 2 * (1 << L2 >> 3) + 8 * ((1 << L2) >> 6) + (L2 < 6 ? 8 : 0);
+  static constexpr int XWORDS = KB * BS;
+};
+// twiddles of a block as staged for KskGeo's passes: those of a pass of K stages from local stage s0
+// at 2^s0: entry e = (1 << u) - 1 + mm of group `high` at 2^s0 + (e << s0) + high
+template <bool SMALL, int L1, int L2, int S0>
+__device__ __forceinline__ void ksk_passes(u64* xs, const ulonglong2* tw, u64 q, uint32_t nqi, int ll,
+                                           u64 (&out)[KskGeo<L2>::PER]) {
+  using G = KskGeo<L2>;
+  constexpr int K = S0 == 0 ? G::F : 3;
+  constexpr int TL = 1 << (L2 - S0 - K), GPT = G::PER >> K;
+  u64 v[GPT][1][1 << K];
+#pragma unroll
+  for (int i = 0; i < GPT; ++i) {
+    const int g = TL == 1 ? ll * GPT + i : i * G::LPB + ll, low = g & (TL - 1), high = g / TL;
+    const int base = high * (TL << K) + low;
+    if constexpr (TL == 1 && K == 3) {
+#pragma unroll
+      for (int m = 0; m < 8; m += 2) {
+        const ulonglong2 x = ldg2(xs + G::word(base) + m);
+        v[i][0][m] = x.x;
+        v[i][0][m + 1] = x.y;
+      }
+    } else {
+#pragma unroll
+      for (int m = 0; m < (1 << K); ++m) v[i][0][m] = xs[G::word(base + m * TL)];
+    }
+    fwd_pass<SMALL, L1 + S0, K, 1>(v[i], q, nqi, [&](int u, int mm) {
+      return tw[(1 << S0) + (((1 << u) - 1 + mm) << S0) + high];
+    });
+    if constexpr (TL > 1) {
+#pragma unroll
+      for (int m = 0; m < (1 << K); ++m) xs[G::word(base + m * TL)] = v[i][0][m];
+    } else {
+#pragma unroll
+      for (int m = 0; m < (1 << K); ++m) out[i * (1 << K) + m] = v[i][0][m];
+    }
+  }
+  if constexpr (TL > 1) {
+    __syncwarp();
+    ksk_passes<SMALL, L1, L2, S0 + K>(xs, tw, q, nqi, ll, out);
+  }
+}
+
+template <int L1, int L2, int W, int MINB>
+__global__ void __launch_bounds__(32 * W, MINB) k_ntt_fwd_rows_ksk(Tables T, LimbSet S, NttAux A, KskFuse F, int nstage) {
+  using G = KskGeo<L2>;
+  extern __shared__ __align__(16) u64 sm[];
+  constexpr size_t N = (size_t)1 << (L1 + L2);
+  constexpr int GROUPS = (1 << L1) / G::KB;  // block groups of a limb
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ll = lane % G::LPB, b = lane / G::LPB;
   const int t = S.limb_begin + blockIdx.y, pt = S.prime(t);
-  const u64 q = T.pr[pt].q;
-  const size_t j0 = (size_t)blk * E;
+  const PrimeDev P = T.pr[pt];
+  const u64 q = P.q;
+  // warp tasks: (block group, ciphertext), ciphertext fastest; the last CTA may have idle warps
+  const int task0 = blockIdx.x * W, task = task0 + warp;
+  const int g0 = task0 / F.batch, gw = min(task / F.batch, GROUPS - 1);
+  const bool live = task < GROUPS * F.batch;
+  // the twiddles of block groups g0 .. g0 + nstage - 1, re-ordered for KskGeo's passes
+  ulonglong2* tws = reinterpret_cast<ulonglong2*>(sm + W * 2 * G::XWORDS);
+  {
+    using R = Phase<L2>;
+    const ulonglong2* src = T.psi2 + (size_t)pt * tw_stride(L1, L2) + (1 << L1);
+    const int nblk = min(nstage, GROUPS - g0) * G::KB;
+    for (int i = threadIdx.x; i < nblk << L2; i += 32 * W) {
+      const int e = i & ((1 << L2) - 1);
+      if (e == 0) continue;
+      // slot e belongs to the pass from s0; its entry and group give the tree index 2^s (...) + ...
+      int s0 = 0;
+#pragma unroll
+      for (int s = G::F; s < L2; s += 3)
+        if (e >= 1 << s) s0 = s;
+      const int r = e - (1 << s0), ent = (r >> s0) + 1, high = r & ((1 << s0) - 1);
+      const int u = 31 - __clz(ent), mm = ent - (1 << u);
+      const int tree = (((1 << s0) + high) << u) + mm;
+      int slot = tree;
+      if (tree >= R::M0) {
+        const int s = 31 - __clz(tree), uu = s - R::K0, r2 = tree - (1 << s);
+        slot = R::M0 + ((1 << uu) - 1 + (r2 & ((1 << uu) - 1))) * R::M0 + (r2 >> uu);
+      }
+      cp_async16(tws + i, src + ((size_t)(g0 * G::KB + (i >> L2)) << L2) + slot);
+    }
+  }
+  const int k = task % F.batch;
+  const size_t j0 = (size_t)(gw * G::KB) << L2;
   const int dn = A.own_dn;
   const int own = (A.own_alpha && t < A.own_limit) ? t / A.own_alpha : -1;
-  const uint32_t toff = row_off<L2>(threadIdx.x);  // word t + i TPB of a buffer at toff + row_step(i)
+  const u64* src0 = S.limb(k * dn, t, N) + j0;  // digit j's run at + j part_stride
+  const int j_first = own == 0 ? 1 : 0;
+  u64* bufs = sm + warp * 2 * G::XWORDS;
   auto fetch = [&](int j, u64* dst) {
-    const u64* src = (j == own ? F.d + (size_t)k * F.d_stride + (size_t)t * N + j0
-                               : S.limb(k * dn + j, t, N) + j0) + threadIdx.x;
+    const u64* src = src0 + (size_t)j * S.part_stride + 2 * lane;
 #pragma unroll
-    for (int i = 0; i < E / TPB; ++i) cp_async8(dst + toff + row_step<L2, TPB>(i), src + i * TPB);
+    for (int i = 0; i < G::PER / 2; ++i) {
+      const int x = 2 * (i * 32 + lane), blk = x >> L2, in = x & ((1 << L2) - 1);
+      cp_async16(dst + blk * G::BS + G::word(in), src + i * 64);
+    }
   };
-  fwd_rows_stage_twiddles<L1, L2, BPC, TPB>(tw, T.psi2 + (size_t)pt * N, (uint32_t)(blk * BPC));
-  fetch(0, buf[0]);
+  if (live && j_first < dn) fetch(j_first, bufs);
   cp_async_commit();
-  Acc128 ab[PER], aa[PER];
+  Acc128 ab[G::PER], aa[G::PER];
 #pragma unroll
-  for (int i = 0; i < PER; ++i) ab[i] = aa[i] = Acc128{0, 0};
+  for (int i = 0; i < G::PER; ++i) ab[i] = aa[i] = Acc128{0, 0};
+  const ulonglong2* tw = tws + ((size_t)((gw - g0) * G::KB + b) << L2);
   const u64* kb = F.key + (size_t)pt * N + j0;
-  for (int j = 0; j < dn; ++j) {
-    u64* cur = buf[j & 1];
-    if (j + 1 < dn) {
-      fetch(j + 1, buf[(j + 1) & 1]);
-      cp_async_commit();
-      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-    } else {
-      cp_async_wait_all();
+  // word pair i of the lane (words 2 i, 2 i + 1 of its PER consecutive ones) of digit j's key run (key_pair: the
+  // lanes' pairs are consecutive)
+  auto key_words = [&](int j, size_t part, ulonglong2 (&w)[G::PER / 2]) {
+    const u64* at = kb + (size_t)j * F.key_digit_stride + part;
+#pragma unroll
+    for (int i = 0; i < G::PER / 2; ++i) w[i] = __ldg(reinterpret_cast<const ulonglong2*>(at + 2 * key_pair(lane * (G::PER / 2) + i)));
+  };
+  auto mac_words = [&](const u64 (&v)[G::PER], const ulonglong2 (&w)[G::PER / 2], Acc128 (&acc)[G::PER]) {
+#pragma unroll
+    for (int i = 0; i < G::PER / 2; ++i) {
+      mac128(acc[2 * i], v[2 * i], w[i].x);
+      mac128(acc[2 * i + 1], v[2 * i + 1], w[i].y);
     }
-    __syncthreads();
-    if (j != own) fwd_rows_passes<L1, L2, BPC, RL, 0>(cur, tw, q);
-    const u64* kbj = kb + (size_t)j * F.key_digit_stride;
-    const u64* kaj = kbj + F.key_a_offset;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      const int idx = threadIdx.x + i * TPB;  // consecutive threads, consecutive words
-      const u64 v = reduce8q(cur[toff + row_step<L2, TPB>(i)], q);
-      mac128(ab[i], v, __ldg(kbj + idx));
-      mac128(aa[i], v, __ldg(kaj + idx));
-    }
-    __syncthreads();  // every thread is done with `cur` before the copy of digit j + 2 lands there
-  }
-  const PrimeDev P = T.pr[pt];
-  const u64 r64 = F.r64[2 * pt], r64p = F.r64[2 * pt + 1];
-  u64* o0 = F.acc + (size_t)(2 * k) * F.acc_part_stride + (size_t)t * N + j0;
-  u64* o1 = o0 + F.acc_part_stride;
-#pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    const int idx = threadIdx.x + i * TPB;
-    o0[idx] = reduce128(ab[i], P, r64, r64p);
-    o1[idx] = reduce128(aa[i], P, r64, r64p);
-  }
-}
-
-// ---------------------------------------------------------------- inverse, block phase
-// GS stage with pair distance 2^lt (lt < L2): twiddle index 2^(LOGN-lt-1) + (j >> (lt+1)),
-// j >> (lt+1) = ((B0+b) << (L2-lt-1)) + (x >> (lt+1)); groups x = high*2^(LT0+K) + m*2^LT0 + low.
-// Staged like the forward phase: stage lt's range starts at 2^(LOGN-lt-1) + (B0 << (L2-lt-1))
-// with BPC 2^(L2-lt-1) entries, at offset BPC (2^L2 - 2^(L2-lt)) in shared memory.
-template <int L1, int L2, int BPC, int TPB>
-__device__ __forceinline__ void inv_rows_stage_twiddles(ulonglong2* tw, const ulonglong2* W, uint32_t B0) {
-#pragma unroll
-  for (int lt = 0; lt < L2; ++lt) {
-    const ulonglong2* src = W + (1u << (L1 + L2 - lt - 1)) + (B0 << (L2 - lt - 1));
-    ulonglong2* dst = tw + BPC * ((1 << L2) - (1 << (L2 - lt)));
-    for (int i = threadIdx.x; i < (BPC << (L2 - lt - 1)); i += TPB) cp_async16(dst + i, src + i);
-  }
-}
-template <int L1, int L2, int BPC, int RL, int LT0>
-__device__ __forceinline__ void inv_rows_passes(u64* sm, const ulonglong2* tw, u64 q) {
-  if constexpr (LT0 < L2) {
-    constexpr int K = (L2 - LT0) < RL ? (L2 - LT0) : RL;
-    constexpr int GPB = 1 << (L2 - K);
-    constexpr int R = (1 << L2) + (1 << (L2 - 4));
-    constexpr int TPB = (BPC << L2) >> RL;
-#pragma unroll
-    for (int g = threadIdx.x; g < BPC * GPB; g += TPB) {
-      const uint32_t b = g / GPB, gg = g % GPB;
-      const uint32_t low = gg & ((1u << LT0) - 1), high = gg >> LT0;
-      const uint32_t base = (high << (LT0 + K)) | low;
-      u64* blk = sm + b * R + padx(base);  // as in the forward passes: the pads depend on m only
-      u64 v[1 << K];
-#pragma unroll
-      for (int m = 0; m < (1 << K); ++m) v[m] = blk[(m << LT0) + ((m << LT0) >> 4)];
-#pragma unroll
-      for (int u = 0; u < K; ++u) {
-        const int lt = LT0 + u, half = 1 << u;
-#pragma unroll
-        for (int m1 = 0; m1 < (1 << K); ++m1) {
-          if (m1 & half) continue;
-          const uint32_t wi = BPC * ((1u << L2) - (1u << (L2 - lt))) + (b << (L2 - lt - 1)) + (high << (K - u - 1)) +
-                              (m1 >> (u + 1));
-          gs_bfly(v[m1], v[m1 + half], tw[wi], q);
-        }
-      }
-#pragma unroll
-      for (int m = 0; m < (1 << K); ++m) blk[(m << LT0) + ((m << LT0) >> 4)] = v[m];
-    }
-    __syncthreads();
-    inv_rows_passes<L1, L2, BPC, RL, LT0 + K>(sm, tw, q);
-  }
-}
-
-template <int L1, int L2, int BPC, int TPB, int MINB, int RL>
-__global__ void __launch_bounds__(TPB, MINB) k_ntt_inv_rows(Tables T, LimbSet S, NttAux A) {
-  extern __shared__ u64 sm[];
-  constexpr size_t N = (size_t)1 << (L1 + L2);
-  constexpr int E = BPC << L2, R = (1 << L2) + (1 << (L2 - 4));
-  const int y = blockIdx.y, part = y / S.n_limbs, li = S.limb_begin + y % S.n_limbs;
-  if (own_limb(A, part, li)) return;
-  const int pi = S.prime(li);
-  const u64 q = T.pr[pi].q;
-  u64* a = S.limb(part, li, N);
-  const u64* src = first_src(A, S, part, li, N);
-  ulonglong2* tw = reinterpret_cast<ulonglong2*>(sm + BPC * R);
-  const size_t j0 = (size_t)blockIdx.x * E;
-  u64* smt = sm + row_off<L2>(threadIdx.x);  // this thread's words: smt[row_step(i)] holds word t + i TPB
-#pragma unroll
-  for (int i = 0; i < E / TPB; ++i) cp_async8(smt + row_step<L2, TPB>(i), src + j0 + threadIdx.x + i * TPB);
-  inv_rows_stage_twiddles<L1, L2, BPC, TPB>(tw, T.ipsi2 + (size_t)pi * N, (uint32_t)(blockIdx.x * BPC));
-  cp_async_commit();
+  };
   cp_async_wait_all();
   __syncthreads();
-  inv_rows_passes<L1, L2, BPC, RL, 0>(sm, tw, q);
+  if (!live) return;
+  auto digits = [&](auto is_small) {
+    constexpr bool SMALL = decltype(is_small)::value;
+    for (int j = j_first, it = 0; j < dn; ++it) {
+      const int next = j + 1 == own ? j + 2 : j + 1;
+      u64* cur = bufs + (it & 1) * G::XWORDS;
+      if (it) {
+        cp_async_wait_all();
+        __syncwarp();
+      }
+      if (next < dn) fetch(next, bufs + ((it + 1) & 1) * G::XWORDS);
+      cp_async_commit();
+      ulonglong2 wb[G::PER / 2], wa[G::PER / 2];
+      key_words(j, 0, wb);
+      key_words(j, F.key_a_offset, wa);
+      u64 v[G::PER];
+      ksk_passes<SMALL, L1, L2, 0>(cur + b * G::BS, tw, q, P.nqi, ll, v);
+      if constexpr (!SMALL) {
 #pragma unroll
-  for (int i = 0; i < E / TPB; ++i) a[j0 + threadIdx.x + i * TPB] = smt[row_step<L2, TPB>(i)];  // [0, 2q)
+        for (int i = 0; i < G::PER; ++i) v[i] = sub_if_above(sub_if_above(v[i], q * 6), q * 3);
+      }
+      mac_words(v, wb, ab);
+      mac_words(v, wa, aa);
+      j = next;
+    }
+  };
+  if (fwd_small(q)) digits(std::true_type{});
+  else digits(std::false_type{});
+  const size_t wat = (size_t)lane * G::PER;  // this lane's words of the warp's run
+  if (own >= 0) {  // the digit that owns limb t: the NTT-domain input itself
+    const u64* src = F.d + (size_t)k * F.d_stride + (size_t)t * N + j0 + wat;
+    u64 v[G::PER];
+#pragma unroll
+    for (int i = 0; i < G::PER; i += 2) {
+      const ulonglong2 x = ldg2(src + i);
+      v[i] = x.x;
+      v[i + 1] = x.y;
+    }
+    ulonglong2 w[G::PER / 2];
+    key_words(own, 0, w);
+    mac_words(v, w, ab);
+    key_words(own, F.key_a_offset, w);
+    mac_words(v, w, aa);
+  }
+  u64* o0 = F.acc + (size_t)(2 * k) * F.acc_part_stride + (size_t)t * N + j0 + wat;
+  u64* o1 = o0 + F.acc_part_stride;
+#pragma unroll
+  for (int i = 0; i < G::PER; i += 2) {
+    stg2(o0 + i, ulonglong2{reduce128(ab[i], P), reduce128(ab[i + 1], P)});
+    stg2(o1 + i, ulonglong2{reduce128(aa[i], P), reduce128(aa[i + 1], P)});
+  }
+}
+
+// ---------------------------------------------------------------- inverse, row phase
+// The forward row phase mirrored: the 2^K1 consecutive words of a lane's groups first, then the words
+// 2^K1 apart.  Output left lazy (below 2^(L2+1) q for small primes, 3q otherwise).
+template <bool SMALL, int L1, int L2>
+__device__ __forceinline__ void inv_rows_body(u64* a, u64* xs, const ulonglong2* tw, const PrimeDev& P, int low) {
+  using G = RowGeo<L2>;
+  const u64 q = P.q;
+#pragma unroll
+  for (int i = 0; i < G::GP; ++i) {
+    const int hi = i * G::M1 + low;
+    u64 w[1][G::M1];
+#pragma unroll
+    for (int m = 0; m < G::M1; m += 2) {
+      const ulonglong2 x = ldg2(xs + hi * G::GS + m);
+      w[0][m] = x.x;
+      w[0][m + 1] = x.y;
+    }
+    inv_pass<SMALL, 1, G::K1, 1>(w, q, P.nqi, [&](int u, int mm) {
+      return tw[G::M0 + ((1 << u) - 1 + mm) * G::M0 + hi];
+    });
+#pragma unroll
+    for (int m = 0; m < G::M1; m += 2) stg2(xs + hi * G::GS + m, ulonglong2{w[0][m], w[0][m + 1]});
+  }
+  __syncwarp();
+  u64 v[1][G::M0];
+#pragma unroll
+  for (int m = 0; m < G::M0; ++m) v[0][m] = xs[m * G::GS + low];
+  constexpr bool MID = SMALL && 1 + L2 > 9;  // 2^(L2+1) q would pass 2^64: reduce between the passes
+  if constexpr (MID) {
+#pragma unroll
+    for (int m = 0; m < G::M0; ++m) v[0][m] = reduce_lazy(v[0][m], q, P.rc);
+  }
+  inv_pass<SMALL, MID ? 1 : 1 + G::K1, G::K0, 1>(v, q, P.nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
+#pragma unroll
+  for (int m = 0; m < G::M0; ++m) a[m * G::M1 + low] = v[0][m];
+}
+template <int L1, int L2, int W, int MINB>
+__global__ void __launch_bounds__(32 * W, MINB) k_ntt_inv_rows(Tables T, LimbSet S, NttAux A, int ppc) {
+  using G = RowGeo<L2>;
+  extern __shared__ __align__(16) u64 sm[];
+  constexpr size_t N = (size_t)1 << (L1 + L2);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, low = lane % G::M1, b = lane / G::M1;
+  const int pg = blockIdx.y / S.n_limbs, li = S.limb_begin + blockIdx.y % S.n_limbs;
+  const int pi = S.prime(li);
+  const PrimeDev P = T.pr[pi];
+  const int blk = (blockIdx.x * W + warp) * G::PER + b;
+  u64* xs = sm + warp * G::XWORDS + b * G::BS;
+  ulonglong2* tw = reinterpret_cast<ulonglong2*>(sm + W * G::XWORDS) + (warp * G::PER << L2);  // the warp's blocks
+  stage_twiddles<(G::PER << L2), 32>(tw, T.ipsi2 + (size_t)pi * tw_stride(L1, L2) + (1 << L1) + ((size_t)(blk - b) << L2),
+                                     lane);
+  tw += b << L2;
+  const size_t j0 = (size_t)blk << L2;
+  for (int part = pg * ppc; part < min((pg + 1) * ppc, S.n_parts); ++part) {
+    if (own_limb(A, part, li)) continue;
+    u64* a = S.limb(part, li, N) + j0;
+    const u64* src = A.src ? A.src + part * A.src_stride + (size_t)li * N + j0 : a;
+#pragma unroll
+    for (int k = 0; k < G::M0 / 2; ++k) {
+      const int e = k * G::M1 + low;
+      cp_async16(xs + (e >> (G::K1 - 1)) * G::GS + (e & (G::M1 / 2 - 1)) * 2, src + 2 * e);
+    }
+    cp_async_commit();
+    cp_async_wait_all();
+    __syncwarp();
+    if (inv_small(P.q)) inv_rows_body<true, L1, L2>(a, xs, tw, P, low);
+    else inv_rows_body<false, L1, L2>(a, xs, tw, P, low);
+    __syncwarp();
+  }
+  cp_async_wait_all();
 }
 
 // ---------------------------------------------------------------- inverse, column phase (+ N^-1)
-// column distance 2^lc (lt = L2 + lc): twiddle index 2^(L1-lc-1) + (c >> (lc+1)) < 2^L1
-template <int L1, int C, int RL, int LC0>
-__device__ __forceinline__ void inv_cols_passes(u64* sm, const ulonglong2* tw, u64 q) {
-  if constexpr (LC0 < L1) {
-    constexpr int K = (L1 - LC0) < RL ? (L1 - LC0) : RL;
-    constexpr int GROUPS = C << (L1 - K);
-    constexpr int TPB = (C << L1) >> RL;
+template <bool SMALL, int L1, int L2, int TH>
+__device__ __forceinline__ void inv_cols_body(u64 (&w)[Phase<L1>::GP][1][1 << Phase<L1>::K1], u64* a, u64* xs,
+                                              const ulonglong2* tw, const PrimeDev& P, int low, int cg, u64 ni, u64 nip) {
+  using G = ColGeo<L1, TH>;
+  const u64 q = P.q;
 #pragma unroll
-    for (int g = threadIdx.x; g < GROUPS; g += TPB) {
-      const uint32_t col = g % C, gg = g / C;
-      const uint32_t low = gg & ((1u << LC0) - 1), high = gg >> LC0;
-      const uint32_t base = (high << (LC0 + K)) | low;
-      u64 v[1 << K];
+  for (int i = 0; i < G::GP; ++i) {
+    const int hi = i * G::M1 + low;
+    if constexpr (SMALL) {
 #pragma unroll
-      for (int m = 0; m < (1 << K); ++m) v[m] = sm[(base + (m << LC0)) * C + col];
-#pragma unroll
-      for (int u = 0; u < K; ++u) {
-        const int lc = LC0 + u, half = 1 << u;
-#pragma unroll
-        for (int m1 = 0; m1 < (1 << K); ++m1) {
-          if (m1 & half) continue;
-          const uint32_t wi = (1u << (L1 - lc - 1)) + (high << (K - u - 1)) + (m1 >> (u + 1));
-          gs_bfly(v[m1], v[m1 + half], tw[wi], q);
-        }
-      }
-#pragma unroll
-      for (int m = 0; m < (1 << K); ++m) sm[(base + (m << LC0)) * C + col] = v[m];
+      for (int m = 0; m < G::M1; ++m) w[i][0][m] = reduce_lazy(w[i][0][m], q, P.rc);
     }
-    __syncthreads();
-    inv_cols_passes<L1, C, RL, LC0 + K>(sm, tw, q);
+    inv_pass<SMALL, 1, G::K1, 1>(w[i], q, P.nqi, [&](int u, int mm) {
+      return tw[G::M0 + ((1 << u) - 1 + mm) * G::M0 + hi];
+    });
+#pragma unroll
+    for (int m = 0; m < G::M1; ++m) xs[(hi * (G::M1 + 1) + m) * G::COLS + cg] = w[i][0][m];
   }
+  __syncthreads();
+  u64 v[1][G::M0];
+#pragma unroll
+  for (int m = 0; m < G::M0; ++m) v[0][m] = xs[(m * (G::M1 + 1) + low) * G::COLS + cg];
+  inv_pass<SMALL, 1 + G::K1, G::K0, 1>(v, q, P.nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
+#pragma unroll
+  for (int m = 0; m < G::M0; ++m) a[(size_t)(m * G::M1 + low) << L2] = shoup_mul(v[0][m], ni, nip, q);
 }
-
-template <int L1, int L2, int C, int TPB, int MINB, int RL>
-__global__ void __launch_bounds__(TPB, MINB) k_ntt_inv_cols(Tables T, LimbSet S, NttAux A) {
-  extern __shared__ u64 sm[];
+template <int L1, int L2, int TH, int MINB>
+__global__ void __launch_bounds__(TH, MINB) k_ntt_inv_cols(Tables T, LimbSet S, NttAux A) {
+  using G = ColGeo<L1, TH>;
+  extern __shared__ __align__(16) u64 sm[];
   constexpr size_t N = (size_t)1 << (L1 + L2);
-  ulonglong2* tw = reinterpret_cast<ulonglong2*>(sm + (C << L1));
+  const int cg = threadIdx.x % G::COLS, low = threadIdx.x / G::COLS;
   const int y = blockIdx.y, part = y / S.n_limbs, li = S.limb_begin + y % S.n_limbs;
   if (own_limb(A, part, li)) return;
   const int pi = S.prime(li);
-  const u64 q = T.pr[pi].q;
-  u64* a = S.limb(part, li, N);
-  const ulonglong2* W = T.ipsi2 + (size_t)pi * N;
-#pragma unroll
-  for (int i = threadIdx.x; i < (1 << L1); i += TPB) cp_async16(tw + i, W + i);
-  const int r0 = blockIdx.x * C;
-#pragma unroll
-  for (int idx = threadIdx.x; idx < (C << L1); idx += TPB) {
-    const int c = idx / C, col = idx % C;
-    cp_async8(sm + idx, a + ((size_t)c << L2) + r0 + col);
-  }
+  const PrimeDev P = T.pr[pi];
+  u64* a = S.limb(part, li, N) + (size_t)blockIdx.x * G::COLS + cg;
+  ulonglong2* tw = reinterpret_cast<ulonglong2*>(sm + G::XWORDS);
+  stage_twiddles<1 << L1, TH>(tw, T.ipsi2 + (size_t)pi * tw_stride(L1, L2), threadIdx.x);
   cp_async_commit();
+  u64 w[G::GP][1][G::M1];
+#pragma unroll
+  for (int i = 0; i < G::GP; ++i)
+#pragma unroll
+    for (int m = 0; m < G::M1; ++m) w[i][0][m] = a[(size_t)((i * G::M1 + low) * G::M1 + m) << L2];
+  const int r = li - S.limb_begin;
+  const u64 ni = A.post ? A.post[2 * r] : T.ninv[pi], nip = A.post ? A.post[2 * r + 1] : T.ninv_sh[pi];
   cp_async_wait_all();
   __syncthreads();
-  inv_cols_passes<L1, C, RL, 0>(sm, tw, q);
-  const int pr_ = li - S.limb_begin;
-  const u64 ni = A.post ? A.post[2 * pr_] : T.ninv[pi], nip = A.post ? A.post[2 * pr_ + 1] : T.ninv_sh[pi];
-#pragma unroll
-  for (int idx = threadIdx.x; idx < (C << L1); idx += TPB) {
-    const int c = idx / C, col = idx % C;
-    a[((size_t)c << L2) + r0 + col] = shoup_mul(sm[idx], ni, nip, q);
-  }
+  if (inv_small(P.q)) inv_cols_body<true, L1, L2, TH>(w, a, sm, tw, P, low, cg, ni, nip);
+  else inv_cols_body<false, L1, L2, TH>(w, a, sm, tw, P, low, cg, ni, nip);
 }
 
 // ---------------------------------------------------------------- dispatch
-// A variant fixes the words staged per CTA (E), the CTAs per SM the register
-// allocation must allow (MINB) and the stages per register pass (RL: radix 16 or
-// radix 8, the latter with half the registers per thread); threads per CTA = E / 2^RL.  The autotuner in
-// ntt_tune() times every variant and keeps the fastest per direction.
-// launch shape of the second phase fused with the key inner product (k_ntt_fwd_rows_ksk): 1024 words
-// per CTA, radix-8 passes (128 threads, 8 words and 32 accumulator registers each), registers left
-// uncapped (168 a thread, 3 CTAs per SM).  A batched HMult at the top level (N = 2^16, batch 8) took
-// 3.72 ms, against 3.95 ms with 2048 words and 2 CTAs per SM (128 registers, spilling), 3.82 ms with
-// 1024 words and 4 CTAs per SM (128 registers) and 3.78 ms with 512 words in radix-4 passes.
-constexpr int kKskWords = 1024, kKskMinBlocks = 2, kKskRL = 3;
+// A variant fixes the warps of a CTA and how many of them the register allocation must leave room for on an SM.
+// The autotuner in ntt_tune() times every shape and keeps the fastest per role.
+template <class Kernel>
+static void allow_smem(Kernel kern, size_t bytes) {
+  if (bytes > 48 * 1024)
+    HEDAP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+}
+// fused row phase: 4 warps a CTA and 168 registers (3 CTAs an SM): 908 us for 8 x 12 digits at level 23, against
+// 1195 us of the 128-thread CTAs with three barriers a digit
+constexpr int kKskWarps = 4, kKskMinBlocks = 3;
 
-template <int L1, int L2, int E, int MINB, int RL>
+template <int L1, int L2, int WW, int WPS>
 static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse, const NttAux& A,
                         const KskFuse* F) {
-  constexpr int LOGN = L1 + L2;
-  constexpr int EE = E <= (1 << LOGN) ? E : (1 << LOGN);
-  constexpr int C = EE >> L1, BPC = EE >> L2, TPB = EE >> RL;
-  const dim3 grid((unsigned)(((size_t)1 << LOGN) / EE), (unsigned)(S.n_parts * S.n_limbs));
-  const size_t smem_cols = (size_t)EE * sizeof(u64) + ((size_t)1 << L1) * sizeof(ulonglong2);
-  const size_t smem_rows =
-      (size_t)BPC * ((1 << L2) + (1 << (L2 - 4))) * sizeof(u64) + (size_t)BPC * (1 << L2) * sizeof(ulonglong2);
-  if (grid.y == 0) return;
-  static const bool attrs = [&] {  // opt in to more than 48 KB of dynamic shared memory, once per shape
-    if (smem_cols > 48 * 1024) {
-      HEDAP_CUDA(cudaFuncSetAttribute(k_ntt_fwd_cols<L1, L2, C, TPB, MINB, RL>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols));
-      HEDAP_CUDA(cudaFuncSetAttribute(k_ntt_inv_cols<L1, L2, C, TPB, MINB, RL>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols));
-    }
-    if (smem_rows > 48 * 1024) {
-      HEDAP_CUDA(cudaFuncSetAttribute(k_ntt_fwd_rows<L1, L2, BPC, TPB, MINB, RL>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows));
-      HEDAP_CUDA(cudaFuncSetAttribute(k_ntt_inv_rows<L1, L2, BPC, TPB, MINB, RL>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows));
-    }
-    return true;
-  }();
-  (void)attrs;
+  using RG = RowGeo<L2>;
+  constexpr int TH = std::min(32 * WW, (1 << L2) << Phase<L1>::K1);  // column phase: threads per CTA
+  using CG = ColGeo<L1, TH>;
+  constexpr int RW = std::min(WW, (1 << L1) / RG::PER);              // row phase: warps per CTA
+  constexpr int CB = std::max(1, WPS * 32 / TH), RB = std::max(1, WPS / RW);
+  const dim3 gc((unsigned)((1 << L2) / CG::COLS), (unsigned)(S.n_parts * S.n_limbs));
+  const unsigned rx = (unsigned)((1 << L1) / RG::PER / RW);
+  constexpr size_t smem_x = (size_t)CG::XWORDS * 8, smem_c = smem_x + ((size_t)16 << L1);
+  constexpr size_t smem_r = (size_t)RW * (RG::XWORDS * 8 + (RG::PER * (size_t)16 << L2));
+  if (gc.y == 0) return;
+  // parts of one limb that a warp takes in turn: as many as leave about four waves of warps
+  const size_t warps1 = (size_t)rx * RW * S.n_limbs * S.n_parts;
+  const int ppc = (int)std::max<size_t>(1, std::min<size_t>(std::min(S.n_parts, 8), warps1 / ((size_t)152 * WPS * 4)));
+  const dim3 gr(rx, (unsigned)(((S.n_parts + ppc - 1) / ppc) * S.n_limbs));
   // the first phase applies src / z / spread; the second runs in place on S (or into fin_dst)
   NttAux A2 = A;
   A2.src = nullptr;
@@ -770,48 +991,65 @@ static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool
   if (!inverse) {
     // staged tiles: the digit's limbs (ModUp), the special limbs (ModDown, plus the last limb when a
     // rescale is fused) or the last limb (rescale); at most 3 products per word in the load
-    const int ns_max = A.z ? std::min(A.own_alpha, A.own_limit)
-                           : A.pconv ? A.pconv_K + (A.spread ? 1 : 0) : A.spread ? 1 : 0;
-    const int n_prod = A.z ? ns_max : A.pconv ? A.pconv_K : 0;
-    if (ns_max >= 1 && ns_max <= 4 && n_prod <= 3 && !A.src) {
+    const int n_prod = A.z ? std::min(A.own_alpha, A.own_limit) : A.pconv ? A.pconv_K : 0;
+    const int nt = n_prod + (!A.z && A.spread ? 1 : 0);
+    if (nt >= 1 && n_prod <= 3 && !A.src) {
       // several output limbs per CTA, sharing the staged tiles: enough limb groups for about
-      // four waves of 4 CTAs on 152 SMs, at most all the limbs in one group
-      const size_t per_group = (size_t)grid.x * S.n_parts;
-      const int groups = (int)std::min<size_t>(S.n_limbs, std::max<size_t>(1, (2432 + per_group - 1) / per_group));
+      // four waves of 16 warps on 152 SMs, at most all the limbs in one group
+      const size_t per_group = (size_t)gc.x * TH / 32 * S.n_parts;
+      const size_t want = (size_t)152 * 16 * 4;
+      const int groups = (int)std::min<size_t>(S.n_limbs, std::max<size_t>(1, (want + per_group - 1) / per_group));
       const int lpc = (S.n_limbs + groups - 1) / groups;
-      const dim3 g2(grid.x, (unsigned)(S.n_parts * ((S.n_limbs + lpc - 1) / lpc)));
-      const size_t smem_m = (size_t)EE * sizeof(u64) + 2 * ((size_t)1 << L1) * sizeof(ulonglong2) +
-                            (size_t)ns_max * EE * sizeof(u64);
-      static const bool attr_m = [&] {
-        HEDAP_CUDA(cudaFuncSetAttribute(k_ntt_fwd_cols_shared<L1, L2, C, TPB, MINB, RL>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)((size_t)EE * 8 + 2 * ((size_t)1 << L1) * 16 + 4 * (size_t)EE * 8)));
+      const dim3 g2(gc.x, (unsigned)(S.n_parts * ((S.n_limbs + lpc - 1) / lpc)));
+      const size_t smem = smem_x + (size_t)nt * CG::TILE * 8;
+      constexpr size_t smem_max = smem_x + (size_t)4 * CG::TILE * 8;
+      static const bool attrs = [&] {
+        allow_smem(k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_MODUP>, smem_max);
+        allow_smem(k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_MODDOWN>, smem_max);
+        allow_smem(k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_SPREAD>, smem_max);
         return true;
       }();
-      (void)attr_m;
-      k_ntt_fwd_cols_shared<L1, L2, C, TPB, MINB, RL><<<g2, TPB, smem_m, st>>>(T, S, A, lpc);
+      (void)attrs;
+      if (A.z) k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_MODUP><<<g2, TH, smem, st>>>(T, S, A, lpc);
+      else if (A.pconv) k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_MODDOWN><<<g2, TH, smem, st>>>(T, S, A, lpc);
+      else k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_SPREAD><<<g2, TH, smem, st>>>(T, S, A, lpc);
+    } else if (n_prod > 3) {
+      constexpr int WB = std::max(1, 12 * 32 / TH);
+      if (A.z) k_ntt_fwd_cols_wide<L1, L2, TH, WB, LOAD_MODUP><<<gc, TH, smem_x, st>>>(T, S, A);
+      else k_ntt_fwd_cols_wide<L1, L2, TH, WB, LOAD_MODDOWN><<<gc, TH, smem_x, st>>>(T, S, A);
     } else {
-      k_ntt_fwd_cols<L1, L2, C, TPB, MINB, RL><<<grid, TPB, smem_cols, st>>>(T, S, A);
+      k_ntt_fwd_cols<L1, L2, TH, CB><<<gc, TH, smem_c, st>>>(T, S, A);
     }
     if (F) {
-      constexpr int EK = kKskWords <= (1 << LOGN) ? kKskWords : (1 << LOGN);
-      constexpr int BPCK = EK >> L2, TPBK = EK >> kKskRL;
-      const size_t smem_k = 2 * (size_t)BPCK * ((1 << L2) + (1 << (L2 - 4))) * sizeof(u64) +
-                            (size_t)BPCK * (1 << L2) * sizeof(ulonglong2);
+      using KG = KskGeo<L2>;
+      constexpr int GROUPS = (1 << L1) / KG::KB;
+      const int tasks = GROUPS * F->batch;
+      const int nstage = std::min(kKskWarps, (kKskWarps - 2 + F->batch) / F->batch + 1);  // block groups a CTA may touch
+      const size_t smem = (size_t)kKskWarps * 2 * KG::XWORDS * 8 + ((size_t)nstage * KG::KB << L2) * 16;
       static const bool attr_k = [&] {
-        HEDAP_CUDA(cudaFuncSetAttribute(k_ntt_fwd_rows_ksk<L1, L2, BPCK, TPBK, kKskMinBlocks, kKskRL>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_k));
+        allow_smem(k_ntt_fwd_rows_ksk<L1, L2, kKskWarps, kKskMinBlocks>,
+                   (size_t)kKskWarps * 2 * KG::XWORDS * 8 + ((size_t)kKskWarps * KG::KB << L2) * 16);
         return true;
       }();
       (void)attr_k;
-      const dim3 gk((unsigned)(F->batch * (((size_t)1 << LOGN) / EK)), (unsigned)S.n_limbs);
-      k_ntt_fwd_rows_ksk<L1, L2, BPCK, TPBK, kKskMinBlocks, kKskRL><<<gk, TPBK, smem_k, st>>>(T, S, A2, *F);
+      const dim3 gk((unsigned)((tasks + kKskWarps - 1) / kKskWarps), (unsigned)S.n_limbs);
+      k_ntt_fwd_rows_ksk<L1, L2, kKskWarps, kKskMinBlocks><<<gk, 32 * kKskWarps, smem, st>>>(T, S, A2, *F, nstage);
     } else {
-      k_ntt_fwd_rows<L1, L2, BPC, TPB, MINB, RL><<<grid, TPB, smem_rows, st>>>(T, S, A2);
+      static const bool attrs = [&] {
+        allow_smem(k_ntt_fwd_rows<L1, L2, RW, RB>, smem_r);
+        return true;
+      }();
+      (void)attrs;
+      k_ntt_fwd_rows<L1, L2, RW, RB><<<gr, 32 * RW, smem_r, st>>>(T, S, A2, ppc);
     }
   } else {
-    k_ntt_inv_rows<L1, L2, BPC, TPB, MINB, RL><<<grid, TPB, smem_rows, st>>>(T, S, A);
-    k_ntt_inv_cols<L1, L2, C, TPB, MINB, RL><<<grid, TPB, smem_cols, st>>>(T, S, A2);
+    static const bool attrs = [&] {
+      allow_smem(k_ntt_inv_rows<L1, L2, RW, RB>, smem_r);
+      return true;
+    }();
+    (void)attrs;
+    k_ntt_inv_rows<L1, L2, RW, RB><<<gr, 32 * RW, smem_r, st>>>(T, S, A, ppc);
+    k_ntt_inv_cols<L1, L2, TH, CB><<<gc, TH, smem_c, st>>>(T, S, A2);
   }
   HEDAP_LAUNCH_CHECK();
 }
@@ -819,19 +1057,11 @@ static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool
 template <int L1, int L2>
 static void launch_variant(int v, const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse,
                            const NttAux& A, const KskFuse* F) {
-  switch (v) {
-    case 0: launch_pair<L1, L2, 2048, 5, 3>(S, T, st, inverse, A, F); break;
-    case 1: launch_pair<L1, L2, 4096, 3, 4>(S, T, st, inverse, A, F); break;
-    case 2: launch_pair<L1, L2, 2048, 4, 4>(S, T, st, inverse, A, F); break;
-    case 3: launch_pair<L1, L2, 2048, 6, 4>(S, T, st, inverse, A, F); break;
-    case 4: launch_pair<L1, L2, 2048, 6, 3>(S, T, st, inverse, A, F); break;
-    case 5: launch_pair<L1, L2, 1024, 12, 3>(S, T, st, inverse, A, F); break;
-    case 6: launch_pair<L1, L2, 2048, 4, 3>(S, T, st, inverse, A, F); break;
-    default: launch_pair<L1, L2, 1024, 8, 3>(S, T, st, inverse, A, F); break;
-  }
+  if (v % kNttShapes == 0) launch_pair<L1, L2, 4, 16>(S, T, st, inverse, A, F);
+  else launch_pair<L1, L2, 4, 20>(S, T, st, inverse, A, F);
 }
 
-// one launch pair of the transform at N = 2^log_n (log_n 10 .. 16) with launch shape v; the
+// one launch pair of the transform at N = 2^log_n (log_n 10 .. 17) with launch shape v; the
 // instantiations are spread over the ntt_inst_*.cu translation units so that they compile in parallel
 void ntt_launch(int log_n, int v, const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse,
                 const NttAux& A, const KskFuse* F);

@@ -1,0 +1,11 @@
+// Instantiations of the transform kernels for N = 2^13 (see ntt_impl.cuh).
+#include "ntt_impl.cuh"
+
+namespace hedap {
+
+void ntt_launch_13(int v, const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse, const NttAux& A,
+                   const KskFuse* F) {
+  launch_variant<6, 7>(v, S, T, st, inverse, A, F);
+}
+
+}  // namespace hedap

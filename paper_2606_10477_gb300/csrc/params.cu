@@ -1,4 +1,5 @@
 // Host-side number theory, randomness and device buffers.
+#include <algorithm>
 #include <cmath>
 
 #include "internal.cuh"
@@ -76,6 +77,7 @@ u64 h_find_psi(u64 q, int log_n) {
   }
 }
 
+u64 h_mont(u64 w, u64 q) { return (u64)(((u128)w << 32) % q); }
 u64 h_shoup(u64 w, u64 q) { return (u64)(((u128)w << 64) / q); }
 
 PrimeDev h_prime_dev(u64 q) {
@@ -83,7 +85,14 @@ PrimeDev h_prime_dev(u64 q) {
   p.q = q;
   p.b = 64 - __builtin_clzll(q);
   p.mu = (u64)(((u128)1 << (2 * p.b)) / q);
+  uint32_t inv = 1;  // q^-1 mod 2^32 by Newton's iteration (doubling the correct low bits)
+  for (int i = 0; i < 5; ++i) inv *= 2u - (uint32_t)q * inv;
+  p.nqi = 0u - inv;
+  p.rc = (uint32_t)std::min<u128>((u128)0xffffffffu, ((u128)1 << 64) / q);
   p.pad = 0;
+  p.r64 = (u64)(((u128)1 << 64) % q);
+  p.r96 = h_mont(p.r64, q);
+  p.r128 = h_mont(p.r96, q);
   return p;
 }
 
