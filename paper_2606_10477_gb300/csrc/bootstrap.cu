@@ -231,25 +231,39 @@ __global__ void k_coeffs_to_limbs_kernel(const PrimeDev* __restrict__ pr, const 
     out[e] = (v < 0 && a) ? P.q - a : a;
   }
 }
-// acc[p][i][k] = sum_b ct_b[p][i][k] * pt_b[i][k]  (plaintext-ciphertext products of one giant step);
-// limb i < q_count has prime i, the others prime p_first + (i - q_count)
+// out_g[p][i][k] = sum_b ct_b[p][i][k] * pt_g,b[i][k]: the plaintext-ciphertext products of up to kPtGiants giant steps g
+// over their baby steps b (pt null where a diagonal is absent); limb i < q_count has prime i, the others prime
+// p_first + (i - q_count).  Bound by HBM.  The grid runs through the giant steps of a limb before it goes on to the
+// next limb: the limb's words of all baby steps (2 B babies limbs) then stay in L2 for the later giant
+// steps instead of coming from DRAM for each.
+constexpr int kPtBabies = 16, kPtGiants = 16;
 struct PtMacArgs {
-  const u64* ct[16];
-  size_t cs[16];
-  const u64* pt[16];
-  int count;
+  const u64* ct[kPtBabies];
+  const u64* pt[kPtGiants][kPtBabies];
+  u64* out[kPtGiants];
+  int babies, giants;
 };
-__global__ void k_pt_mac_kernel(const PrimeDev* __restrict__ pr, PtMacArgs A, u64* __restrict__ out, size_t os, int n_parts, int limbs, int log_n, int q_count,
-                                int p_first) {
-  const size_t per = (size_t)limbs << log_n, total = n_parts * per;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int p = (int)(e / per);
-    const size_t r = e - p * per;
-    const int li = (int)(r >> log_n), i = li < q_count ? li : p_first + (li - q_count);
-    Acc128 s{0, 0};
-    for (int b = 0; b < A.count; ++b) mac128(s, A.ct[b][p * A.cs[b] + r], A.pt[b][r]);
-    out[p * os + r] = reduce128(s, pr[i]);
+__global__ void __launch_bounds__(256) k_pt_mac_kernel(const PrimeDev* __restrict__ pr, const __grid_constant__ PtMacArgs A,
+                                                       size_t stride, int n_parts, int log_n, int q_count, int p_first) {
+  const size_t N = (size_t)1 << log_n;
+  const int li = blockIdx.y / A.giants, g = blockIdx.y % A.giants;
+  const int i = li < q_count ? li : p_first + (li - q_count);
+  const PrimeDev P = pr[i];
+  // blockIdx.x: (coefficient pairs, part), the part fastest, so that the parts share each diagonal word through L2
+  const int p = blockIdx.x % n_parts;
+  const size_t n = 2 * ((size_t)(blockIdx.x / n_parts) * blockDim.x + threadIdx.x), r = (size_t)li * N + n;
+  if (n >= N) return;
+  Acc128 s0{0, 0}, s1{0, 0};
+#pragma unroll 4
+  for (int b = 0; b < A.babies; ++b) {
+    const u64* pt = A.pt[g][b];
+    if (!pt) continue;
+    const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(pt + r);
+    const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(A.ct[b] + p * stride + r);
+    mac128(s0, c.x, w.x);
+    mac128(s1, c.y, w.y);
   }
+  *reinterpret_cast<ulonglong2*>(A.out[g] + p * stride + r) = ulonglong2{reduce128(s0, P), reduce128(s1, P)};
 }
 
 // ------------------------------------------------------------------ operations
@@ -375,36 +389,49 @@ static std::unique_ptr<Ct> lt_apply(Ctx& C, const Ct& v, const LTGroup& G, Plain
         break;
       }
   }
+  // sum_b diag o baby_b over Q_l u P for every giant step, then one ModDown for each
   std::unique_ptr<Ct> acc;
   const long n = (long)slots;
-  for (long g = 0; g < G.giants; ++g) {
-    PtMacArgs A;
-    A.count = 0;
-    for (long b = 0; b < G.n1; ++b) {
-      auto it = P.pt.find({g, b});
-      if (it == P.pt.end()) continue;
-      if (A.count == 16) throw Error(HEDAP_ERR_ARG, "more than 16 baby steps");
-      A.ct[A.count] = baby[b].p;
-      A.cs[A.count] = qp_stride;
-      A.pt[A.count] = it->second.p;
-      ++A.count;
+  if (G.n1 > kPtBabies) throw Error(HEDAP_ERR_ARG, "more than 16 baby steps");
+  for (long first = 0; first < G.giants; first += kPtGiants) {
+    PtMacArgs A{};
+    A.babies = (int)G.n1;
+    for (long b = 0; b < G.n1; ++b) A.ct[b] = baby[b].p;
+    std::vector<long> steps;
+    std::vector<DevBuf> sums;
+    double terms = 0;
+    for (long g = first; g < std::min(first + kPtGiants, G.giants); ++g) {
+      bool any = false;
+      for (long b = 0; b < G.n1; ++b) {
+        auto it = P.pt.find({g, b});
+        A.pt[steps.size()][b] = it == P.pt.end() ? nullptr : it->second.p;
+        any |= it != P.pt.end();
+        terms += it != P.pt.end();
+      }
+      if (!any) continue;
+      sums.emplace_back((size_t)v.parts() * qp_stride, C.stream);
+      A.out[steps.size()] = sums.back().p;
+      steps.push_back(g);
     }
-    if (!A.count) continue;
-    // sum_b diag o baby_b over Q_l u P, then one ModDown for the giant step
-    DevBuf sum((size_t)v.parts() * qp_stride, C.stream);
+    A.giants = (int)steps.size();
+    if (!A.giants) continue;
     {
-      ProfScope prof_(PROF_ELEMENTWISE, C.stream, (1.5 * A.count + 1.0) * v.parts() * ext * C.N * 8);
+      ProfScope prof_(PROF_ELEMENTWISE, C.stream,
+                      (terms + ((double)A.babies + A.giants) * v.parts()) * ext * C.N * 8);
       prof_count_launches(1);
-      k_pt_mac_kernel<<<grid_for((size_t)v.parts() * ext * C.N, 256), 256, 0, C.stream>>>(
-          C.tab.pr, A, sum.p, qp_stride, v.parts(), ext, C.log_n, l + 1, C.n_q);
+      const dim3 grid((unsigned)(((C.N / 2 + 255) / 256) * v.parts()), (unsigned)(ext * A.giants));
+      k_pt_mac_kernel<<<grid, 256, 0, C.stream>>>(C.tab.pr, A, qp_stride, v.parts(), C.log_n, l + 1, C.n_q);
       HEDAP_LAUNCH_CHECK();
     }
-    auto inner = ct_alloc(C, l, v.batch);
-    inner->scale = v.scale * sp;
-    ev_moddown_into(C, sum, v.batch, l, *inner);
-    const long Gs = G.h0 * (G.kmin + g * G.n1);
-    std::unique_ptr<Ct> r = (((Gs % n) + n) % n) ? ev_galois(C, *inner, galois_for_rotation(C, Gs)) : std::move(inner);
-    acc = acc ? ev_add(C, *acc, *r, false) : std::move(r);
+    for (size_t i = 0; i < steps.size(); ++i) {
+      auto inner = ct_alloc(C, l, v.batch);
+      inner->scale = v.scale * sp;
+      ev_moddown_into(C, sums[i], v.batch, l, *inner);
+      sums[i] = DevBuf();
+      const long Gs = G.h0 * (G.kmin + steps[i] * G.n1);
+      std::unique_ptr<Ct> r = (((Gs % n) + n) % n) ? ev_galois(C, *inner, galois_for_rotation(C, Gs)) : std::move(inner);
+      acc = acc ? ev_add(C, *acc, *r, false) : std::move(r);
+    }
   }
   auto out = ev_rescale(C, *acc);
   out->scale = target;

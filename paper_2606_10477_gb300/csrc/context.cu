@@ -155,6 +155,7 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
     md2.push_back(w);
     md2.push_back(h_shoup(w, pk));
   }
+  C->mdr_post = md2;
   for (int k = 0; k < K; ++k) md2.push_back(h_mulmod(halfP_mod(p_of(k)), phinv[k], p_of(k)));
   for (int k = 0; k < K; ++k) md2.push_back(p_of(k));
   for (int word = 0; word < 2; ++word)

@@ -211,6 +211,15 @@ const LevelConsts& level_consts(Ctx& C, int l) {
     M.off = (ql - h_mulmod(halfq, pinv, ql)) % ql;
     M.pinv = pinv;
     M.pinv_sh = h_shoup(pinv, ql);
+    std::vector<u64> mp(2 + 2 * (size_t)M.K);
+    mp[0] = h_invmod(C.N % ql, ql);
+    mp[1] = h_shoup(mp[0], ql);
+    for (int k = 0; k < M.K; ++k) {
+      mp[2 + 2 * k] = C.mdr_post[2 * k];
+      mp[3 + 2 * k] = C.mdr_post[2 * k + 1];
+    }
+    L->mdr_post = DevBuf(mp.size(), C.stream);
+    HEDAP_CUDA(cudaMemcpyAsync(L->mdr_post.p, mp.data(), mp.size() * 8, cudaMemcpyHostToDevice, C.stream));
     HEDAP_CUDA(cudaStreamSynchronize(C.stream));
   }
   auto& ref = *L;
@@ -299,16 +308,6 @@ static void ks_moddown(Ctx& C, const DevBuf& acc, int batch, int l, u64* out, si
   ntt_forward(C.tab, qset(v.p, nl * N, 2 * batch, 0, l + 1), C.stream, &fw);
 }
 
-// inner product of the transformed extended digits y (permuted by X -> X^perm when perm != 0) with
-// the key for `galois`, then ModDown into out
-static void ks_finish(Ctx& C, const DevBuf& y, const u64* d, size_t d_stride, int batch, int l, u64 galois, u64 perm,
-                      u64* out, size_t out_stride, bool acc0, bool acc1) {
-  const DevBuf& key = key_for(C, galois);
-  DevBuf acc((size_t)batch * 2 * (l + 1 + C.n_p) * C.N, C.stream);
-  k_ksk_inner(C, y.p, d, d_stride, key.p, acc.p, batch, l, perm);
-  ks_moddown(C, acc, batch, l, out, out_stride, acc0, acc1);
-}
-
 // The key switch up to the inner product: iNTT of d, the extended digits' forward transform with the
 // key inner product fused into its second phase (the transformed digits are never stored).  Returns the
 // sums acc [batch][2][ext][N] (NTT domain).
@@ -350,14 +349,17 @@ static void ks_moddown_rescale(Ctx& C, const DevBuf& acc, int batch, int l, cons
   const size_t N = C.N;
   const int K = C.n_p, ext = l + 1 + K, nq = C.n_q;
   const LevelConsts& LC = level_consts(C, l);
+  // limb l of the sums enters as e_l + acc_l P^-1 and the special limbs, which follow it, end with
+  // N^-1 phinv_k: one inverse transform of K + 1 limbs a part
   NttAux inv{};
-  inv.post = C.d_moddown2.p;  // the special limbs end with N^-1 phinv_k
-  ntt_inverse(C.tab, LimbSet{acc.p, (size_t)ext * N, 2 * batch, l + 1, K, l + 1, 0, C.n_q}, C.stream, &inv);
-  DevBuf t((size_t)2 * batch * N, C.stream), x((size_t)2 * batch * N, C.stream);
-  k_mdr_last_eval(C, e + (size_t)l * N, e_stride, acc.p + (size_t)l * N, (size_t)ext * N, t.p, 2 * batch, l,
-                  LC.mdr_last);
-  ntt_inverse(C.tab, qset(t.p, N, 2 * batch, 0, 1, l), C.stream);
-  k_mdr_last_coef(C, t.p, acc.p + (size_t)(l + 1) * N, (size_t)ext * N, x.p, 2 * batch, l, LC.mdr_last);
+  inv.post = LC.mdr_post.p;
+  inv.pre_e = e + (size_t)l * N;
+  inv.pre_e_stride = e_stride;
+  inv.pre_w = LC.mdr_last.pinv;
+  inv.pre_wsh = LC.mdr_last.pinv_sh;
+  ntt_inverse(C.tab, LimbSet{acc.p, (size_t)ext * N, 2 * batch, l, K + 1, l + 1, 0, C.n_q}, C.stream, &inv);
+  DevBuf x((size_t)2 * batch * N, C.stream);
+  k_mdr_last_coef(C, acc.p + (size_t)l * N, (size_t)ext * N, x.p, 2 * batch, l, LC.mdr_last);
   DevBuf v((size_t)2 * batch * l * N, C.stream);
   NttAux fw{};
   fw.pconv = acc.p + (size_t)(l + 1) * N;
@@ -392,35 +394,49 @@ static void ks_moddown_rescale(Ctx& C, const DevBuf& acc, int batch, int l, cons
 // automorphism to them inside the inner product.  The result differs from ev_galois (which
 // converts the rotated c1) by multiples of the digit moduli in the extended basis, within the
 // same noise bound.
+// The inner products of several rotations with the digits y, as many to a launch as the sums' memory allows:
+// about 1 GiB of them at a time (kKskRotations at most), handed to `done(i, acc)` in order.
+template <class F>
+static void hoisted_inner(Ctx& C, const Ct& a, const DevBuf& y, const std::vector<u64>& gs, const u64* c0, size_t chunk,
+                          F done) {
+  const int l = a.level;
+  const size_t words = (size_t)a.batch * 2 * (l + 1 + C.n_p) * C.N, ds = 2 * a.part_stride();
+  for (size_t first = 0; first < gs.size(); first += chunk) {
+    KskInnerArgs A;
+    A.count = (int)std::min(chunk, gs.size() - first);
+    std::vector<DevBuf> acc;
+    for (int r = 0; r < A.count; ++r) {
+      acc.emplace_back(words, C.stream);
+      A.key[r] = key_for(C, gs[first + r]).p;
+      A.acc[r] = acc.back().p;
+      A.g[r] = gs[first + r];
+    }
+    k_ksk_inner(C, y.p, a.part(1), ds, A, a.batch, l, c0, ds);
+    for (int r = 0; r < A.count; ++r) done(first + r, std::move(acc[r]));
+  }
+}
 std::vector<std::unique_ptr<Ct>> ev_galois_hoisted(Ctx& C, const Ct& a, const std::vector<u64>& gs) {
   const int l = a.level;
   for (u64 g : gs) key_for(C, g);
-  const u64* d = a.part(1);
-  const size_t ds = 2 * a.part_stride();
-  DevBuf y = ks_modup(C, d, ds, a.batch, l);
+  DevBuf y = ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, l);
   std::vector<std::unique_ptr<Ct>> out;
-  for (u64 g : gs) {
+  const size_t bytes = (size_t)a.batch * 2 * (l + 1 + C.n_p) * C.N * 8;
+  const size_t chunk = std::max<size_t>(1, std::min<size_t>(kKskRotations, ((size_t)1 << 30) / bytes));
+  hoisted_inner(C, a, y, gs, nullptr, chunk, [&](size_t i, DevBuf acc) {
     auto o = ct_alloc(C, l, a.batch);
     o->scale = a.scale;
-    k_automorph(C, a.part(0), 2 * a.part_stride(), o->part(0), 2 * o->part_stride(), a.batch, l + 1, g);
-    ks_finish(C, y, d, ds, a.batch, l, g, g, o->part(0), o->part_stride(), true, false);
+    k_automorph(C, a.part(0), 2 * a.part_stride(), o->part(0), 2 * o->part_stride(), a.batch, l + 1, gs[i]);
+    ks_moddown(C, acc, a.batch, l, o->part(0), o->part_stride(), true, false);
     out.push_back(std::move(o));
-  }
+  });
   return out;
 }
 
 std::vector<DevBuf> ev_galois_hoisted_qp(Ctx& C, const Ct& a, const std::vector<u64>& gs) {
-  const int l = a.level;
   for (u64 g : gs) key_for(C, g);
-  const u64* d = a.part(1);
-  const size_t ds = 2 * a.part_stride();
-  DevBuf y = ks_modup(C, d, ds, a.batch, l);
-  std::vector<DevBuf> out;
-  for (u64 g : gs) {
-    DevBuf acc((size_t)a.batch * 2 * (l + 1 + C.n_p) * C.N, C.stream);
-    k_ksk_inner(C, y.p, d, ds, key_for(C, g).p, acc.p, a.batch, l, g, a.part(0), ds);
-    out.push_back(std::move(acc));
-  }
+  DevBuf y = ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, a.level);
+  std::vector<DevBuf> out(gs.size());  // every sum is kept: one launch for all of them
+  hoisted_inner(C, a, y, gs, a.part(0), kKskRotations, [&](size_t i, DevBuf acc) { out[i] = std::move(acc); });
   return out;
 }
 void ev_moddown_into(Ctx& C, DevBuf& acc, int batch, int level, Ct& out) {

@@ -141,6 +141,11 @@ struct NttAux {
   // inverse only: the final factor of limb li is the pair post[2 r], post[2 r + 1] (value, Shoup
   // companion), r = li - limb_begin, instead of N^-1
   const u64* post = nullptr;
+  // inverse only: the first limb (limb_begin) of part p enters as pre_e[p * pre_e_stride + n] + x pre_w mod its prime,
+  // x the limb itself (canonical residues; pre_w with its Shoup companion pre_wsh)
+  const u64* pre_e = nullptr;
+  size_t pre_e_stride = 0;
+  u64 pre_w = 0, pre_wsh = 0;
   // skip the limbs li of digit j = part % own_dn, li in [j own_alpha, min((j + 1) own_alpha, own_limit))
   int own_alpha = 0;
   int own_dn = 1;
@@ -254,6 +259,15 @@ struct LinCombArgs {
   u64 c0[kLcLimbs];  // added to the even (c0) parts when add_c0
   int count, add_c0, accumulate;
 };
+// one launch of the inner products of hoisted rotations (k_ksk_inner): rotation r by the Galois element g[r] with
+// the key key[r], into acc[r]
+constexpr int kKskRotations = 16;
+struct KskInnerArgs {
+  const u64* key[kKskRotations];
+  u64* acc[kKskRotations];
+  u64 g[kKskRotations];
+  int count;
+};
 // rescale by q_l: per i < l, q_l mod q_i and q_l^-1 mod q_i (+ Shoup)
 struct RescaleConsts {
   u64 ql_mod[kMaxLimbs];
@@ -277,7 +291,9 @@ struct LevelConsts {  // device constants for one level (evaluator.cu)
   DevBuf d_rescale;   // [q_l mod q_i] and mont_mul_lazy's pair of q_l^-1 mod q_i, [first words][second words], i < l
   RescaleConsts rescale;
   DevBuf d_mdr;       // ModDown fused with the rescale: mont_mul_lazy's pair of (P q_l)^-1 mod q_i, i < l
-  MdrLast mdr_last;   // ... and the constants of its last limb (prime q_l)
+  MdrLast mdr_last;   // ... the constants of its last limb (prime q_l)
+  DevBuf mdr_post;    // ... and the final factors of its inverse transform, pairs (value, Shoup companion): N^-1 for
+                      // the last limb, N^-1 phinv_k for the special limbs after it
 };
 
 struct BtsState;  // bootstrapping state (bootstrap.cu)
@@ -311,6 +327,7 @@ struct Ctx {
                       // phat_q, [K][n_q] first words and [K][n_q] second words, and of P^-1 mod q_i, [n_q] and [n_q]
   DevBuf d_mdr;       // ModDown scaled by P^-1 (fused with a rescale): mont_mul_lazy's pairs of p_k^-1 mod q_i, [K][n_q]
                       // first and [K][n_q] second words, then floor(P/2) P^-1 mod q_i [n_q]
+  std::vector<u64> mdr_post;  // [N^-1 phinv_k, Shoup][K] pairs (host copy of d_moddown2's first)
   DevBuf d_pmod;      // per prime: P mod q_t (key generation)
   Tables tab{};
   std::vector<i64> sk;

@@ -218,46 +218,27 @@ void k_rescale_spread(const Ctx& C, const u64* last, size_t ls, u64* tmp, size_t
   HEDAP_LAUNCH_CHECK();
 }
 // ---------------------------------------------------------------- ModDown fused with a rescale: the last limb
-__global__ void k_mdr_last_eval_kernel(const u64* __restrict__ e, size_t es, const u64* __restrict__ acc, size_t as,
-                                       u64* __restrict__ t, int n_parts, int log_n, u64 q, u64 w, u64 wsh) {
-  const size_t N = (size_t)1 << log_n;
-  GRID_LOOP(i, (size_t)n_parts * N) {
-    const size_t p = i >> log_n, n = i & (N - 1);
-    t[i] = add_mod(e[p * es + n], shoup_mul(acc[p * as + n], w, wsh, q), q);
-  }
-}
-void k_mdr_last_eval(const Ctx& C, const u64* e, size_t es, const u64* acc, size_t as, u64* t, int n_parts, int l,
-                     const MdrLast& M) {
-  ProfScope prof_(PROF_RESCALE, C.stream, 3.0 * n_parts * C.N * 8);
-  prof_count_launches(1);
-  const size_t work = (size_t)n_parts * C.N;
-  k_mdr_last_eval_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(e, es, acc, as, t, n_parts, C.log_n,
-                                                                    C.primes[l], M.pinv, M.pinv_sh);
-  HEDAP_LAUNCH_CHECK();
-}
-// x = t - (off + sum_k [z_k + c_k]_{p_k} f_k) mod q_l: the K canonical products and off sum below
-// (K + 1) q_l <= 9 q_l < 2^64, reduced once
-__global__ void k_mdr_last_coef_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ t,
-                                       const u64* __restrict__ z, size_t zs, u64* __restrict__ x, int n_parts,
-                                       int log_n, int l, MdrLast M) {
+// x = t - (off + sum_k [z_k + c_k]_{p_k} f_k) mod q_l, t limb l of part p (coefficient domain, part stride zs) and z_k
+// the K limbs after it: the K canonical products and off sum below (K + 1) q_l <= 9 q_l < 2^64, reduced once
+__global__ void k_mdr_last_coef_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ t, size_t zs,
+                                       u64* __restrict__ x, int n_parts, int log_n, int l, MdrLast M) {
   const size_t N = (size_t)1 << log_n;
   const PrimeDev P = pr[l];
   GRID_LOOP(i, (size_t)n_parts * N) {
     const size_t p = i >> log_n, n = i & (N - 1);
-    const u64* zp = z + p * zs + n;
+    const u64* tp = t + p * zs + n;
     u64 v = M.off;
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-      if (k < M.K) v += shoup_mul(add_mod(zp[(size_t)k * N], M.c[k], M.p[k]), M.f[k], M.fs[k], P.q);
-    x[i] = sub_mod(t[i], barrett_reduce(v, 0, P), P.q);
+      if (k < M.K) v += shoup_mul(add_mod(tp[(size_t)(k + 1) * N], M.c[k], M.p[k]), M.f[k], M.fs[k], P.q);
+    x[i] = sub_mod(tp[0], barrett_reduce(v, 0, P), P.q);
   }
 }
-void k_mdr_last_coef(const Ctx& C, const u64* t, const u64* z, size_t zs, u64* x, int n_parts, int l,
-                     const MdrLast& M) {
+void k_mdr_last_coef(const Ctx& C, const u64* t, size_t zs, u64* x, int n_parts, int l, const MdrLast& M) {
   ProfScope prof_(PROF_RESCALE, C.stream, (2.0 + M.K) * n_parts * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * C.N;
-  k_mdr_last_coef_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(C.tab.pr, t, z, zs, x, n_parts, C.log_n, l, M);
+  k_mdr_last_coef_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(C.tab.pr, t, zs, x, n_parts, C.log_n, l, M);
   HEDAP_LAUNCH_CHECK();
 }
 
@@ -364,90 +345,73 @@ void k_modup(const Ctx& C, const u64* dcoef, u64* y, int batch, int level, const
   HEDAP_LAUNCH_CHECK();
 }
 
-// inner product with the switching key:
-//   acc[k][0|1][t] = sum_j y[k][j][t] * key_j[b|a][t]
-// key layout: [dnum_max][2][n_q + n_p][N]; y: [B][dn][ext][N]; acc: [B][2][ext][N].
+// inner products of hoisted rotations (the digits were converted once, before their automorphisms):
+//   acc_r[k][0|1][t] = sum_j sigma_r(y[k][j])[t] * key_r,j[b|a][t],  r < A.count
+// key layout: [dnum_max][2][n_q + n_p][N], pairs permuted (key_pair); y: [B][dn][ext][N]; acc: [B][2][ext][N].
 // A digit's own limbs (t in digit j) are not in y: there the extended digit equals
 // the NTT-domain input itself, read from d ([B] members of stride ds, limbs of N).
-// One thread per (k, t, pair of coefficients): a CTA holds the batch members of the same coefficients
-// (threadIdx.y = k), so each key word comes from DRAM once and from L1 for the
-// other members; few registers per thread keep many loads in flight.
-// With g != 0 the extended digits enter permuted by the automorphism X -> X^g (a
-// hoisted rotation: the digits were converted once, before the automorphism): the
-// NTT-domain value at n is read at the index whose evaluation point is the g-th
-// power of n's; within 32 consecutive indices the permutation stays inside one
-// aligned group of 32, so the gather is coalesced.
+// The extended digits enter permuted by the automorphism X -> X^g: the NTT-domain value at n is read at the
+// index whose evaluation point is the g-th power of n's; within 32 consecutive indices the permutation
+// stays inside one aligned group of 32, so the gather is coalesced.
+// One thread per (r, k, t, pair of coefficients): a CTA holds the batch members of the same coefficients
+// (threadIdx.y = k), so each key word comes from DRAM once and from L1 for the other members.
+// Bound by HBM: every rotation reads a key of its own (2 dn (l+1+K) limbs), and all of them the same digits. The grid runs
+// through the rotations of a limb before it goes on to the next limb, so that the limb's digits (B dn
+// limbs) stay in L2 for all of them instead of coming from DRAM for each.
 __device__ __forceinline__ uint32_t galois_index(uint32_t n, u64 g, int log_n) {
   const u64 e = 2 * (u64)(__brev(n) >> (32 - log_n)) + 1;
   const u64 eg = (g * e) & ((2ull << log_n) - 1);
   return __brev((uint32_t)((eg - 1) >> 1)) >> (32 - log_n);
 }
-// registers capped at 64 (512 threads, 2 CTAs): the kernel waits on memory, and 84 left 24 warps an SM instead of 32
+__device__ __forceinline__ ulonglong2 ld2_stream(const u64* p) { return __ldcs(reinterpret_cast<const ulonglong2*>(p)); }
 __global__ void __launch_bounds__(512, 2) k_ksk_inner_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ y,
-                                   const u64* __restrict__ d, size_t ds, const u64* __restrict__ key, u64* __restrict__ acc, int l, int dn, int alpha,
-                                   int n_q, int K, int log_n, u64 g, const u64* __restrict__ c0, size_t c0s,
-                                   const u64* __restrict__ pmod) {
-  // two consecutive coefficients per thread (16-byte loads: longer runs per DRAM page
-  // across the dn x B digit streams); a permuted source is read word by word
+                                                             const u64* __restrict__ d, size_t ds, KskInnerArgs A,
+                                                             int l, int dn, int alpha, int n_q, int K, int log_n,
+                                                             const u64* __restrict__ c0, size_t c0s,
+                                                             const u64* __restrict__ pmod) {
   const size_t N = (size_t)1 << log_n;
   const int ext = l + 1 + K, total_primes = n_q + K;
-  const int t = blockIdx.y, k = threadIdx.y;
+  const int t = blockIdx.y / A.count, rot = blockIdx.y % A.count, k = threadIdx.y;
   const size_t n = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
   const int pt = t <= l ? t : n_q + (t - l - 1);
   const int own = t <= l ? t / alpha : -1;
-  const size_t kn = 2 * key_pair(n / 2);
-  const u64* kb = key + (size_t)pt * N + kn;
-  const u64* ka = key + ((size_t)total_primes + pt) * N + kn;
-  const size_t key_step = (size_t)2 * total_primes * N, y_step = (size_t)ext * N;
+  const u64* kb = A.key[rot] + (size_t)pt * N + 2 * key_pair(n / 2);
+  const size_t key_a = (size_t)total_primes * N, key_step = 2 * key_a, y_step = (size_t)ext * N;
   const u64* yk = y + ((size_t)k * dn * ext + t) * N;
   const u64* dk = d + k * ds + (size_t)t * N;
+  const size_t s0 = galois_index((uint32_t)n, A.g[rot], log_n), s1 = galois_index((uint32_t)n + 1, A.g[rot], log_n);
   Acc128 a0{0, 0}, a1{0, 0}, b0{0, 0}, b1{0, 0};  // (coefficient n, n+1) x (key b, key a)
-  if (!g) {
-#pragma unroll 8
-    for (int j = 0; j < dn; ++j) {
-      const ulonglong2 v = j == own ? ld2(dk + n) : ld2(yk + j * y_step + n);
-      const ulonglong2 wb = ld2(kb + j * key_step), wa = ld2(ka + j * key_step);
-      mac128(a0, v.x, wb.x);
-      mac128(a1, v.x, wa.x);
-      mac128(b0, v.y, wb.y);
-      mac128(b1, v.y, wa.y);
-    }
-  } else {
-    const size_t s0 = galois_index((uint32_t)n, g, log_n), s1 = galois_index((uint32_t)n + 1, g, log_n);
-#pragma unroll 8
-    for (int j = 0; j < dn; ++j) {
-      const u64* src = j == own ? dk : yk + j * y_step;
-      const u64 v0 = src[s0], v1 = src[s1];
-      const ulonglong2 wb = ld2(kb + j * key_step), wa = ld2(ka + j * key_step);
-      mac128(a0, v0, wb.x);
-      mac128(a1, v0, wa.x);
-      mac128(b0, v1, wb.y);
-      mac128(b1, v1, wa.y);
-    }
+#pragma unroll 4
+  for (int j = 0; j < dn; ++j) {
+    const u64* src = j == own ? dk : yk + j * y_step;
+    const u64 v0 = src[s0], v1 = src[s1];
+    const ulonglong2 wb = ld2_stream(kb + j * key_step), wa = ld2_stream(kb + j * key_step + key_a);
+    mac128(a0, v0, wb.x);
+    mac128(a1, v0, wa.x);
+    mac128(b0, v1, wb.y);
+    mac128(b1, v1, wa.y);
   }
   if (c0 && t <= l) {  // the rotation kept over Q_l u P: part 0 gains P sigma_g(c0) on the Q limbs
     const u64* ck = c0 + k * c0s + (size_t)t * N;
-    const size_t s0 = g ? galois_index((uint32_t)n, g, log_n) : n;
-    const size_t s1 = g ? galois_index((uint32_t)n + 1, g, log_n) : n + 1;
     mac128(a0, ck[s0], pmod[pt]);
     mac128(b0, ck[s1], pmod[pt]);
   }
   const PrimeDev P = pr[pt];
-  st2(acc + (((size_t)k * 2) * ext + t) * N + n,
-      ulonglong2{reduce128(a0, P), reduce128(b0, P)});
-  st2(acc + (((size_t)k * 2 + 1) * ext + t) * N + n,
-      ulonglong2{reduce128(a1, P), reduce128(b1, P)});
+  u64* out = A.acc[rot] + (((size_t)k * 2) * ext + t) * N + n;
+  st2(out, ulonglong2{reduce128(a0, P), reduce128(b0, P)});
+  st2(out + (size_t)ext * N, ulonglong2{reduce128(a1, P), reduce128(b1, P)});
 }
-void k_ksk_inner(const Ctx& C, const u64* y, const u64* d, size_t d_stride, const u64* key, u64* acc, int batch,
-                 int level, u64 galois_perm, const u64* c0, size_t c0_stride) {
+void k_ksk_inner(const Ctx& C, const u64* y, const u64* d, size_t d_stride, const KskInnerArgs& A, int batch, int level,
+                 const u64* c0, size_t c0_stride) {
   if (batch < 1 || batch > kMaxBatch) throw Error(HEDAP_ERR_ARG, "batch must lie in [1, 16]");
   const int dn = C.dnum(level), ext = level + 1 + C.n_p;
-  ProfScope prof_(PROF_KSK_INNER, C.stream, ((double)batch * dn + 2.0 * dn + 2.0 * batch) * ext * C.N * 8);
+  ProfScope prof_(PROF_KSK_INNER, C.stream,
+                  ((double)batch * dn + A.count * (2.0 * dn + 2.0 * batch)) * ext * C.N * 8);
   prof_count_launches(1);
   const unsigned tx = 32u * (unsigned)std::max(1, 8 / batch);  // about 256 threads per CTA
-  const dim3 block(tx, (unsigned)batch), grid((unsigned)(C.N / 2 / tx), (unsigned)ext);
-  k_ksk_inner_kernel<<<grid, block, 0, C.stream>>>(C.tab.pr, y, d, d_stride, key, acc, level, dn, C.alpha,
-                                                   C.n_q, C.n_p, C.log_n, galois_perm, c0, c0_stride, C.d_pmod.p);
+  const dim3 block(tx, (unsigned)batch), grid((unsigned)(C.N / 2 / tx), (unsigned)(ext * A.count));
+  k_ksk_inner_kernel<<<grid, block, 0, C.stream>>>(C.tab.pr, y, d, d_stride, A, level, dn, C.alpha, C.n_q, C.n_p,
+                                                   C.log_n, c0, c0_stride, C.d_pmod.p);
   HEDAP_LAUNCH_CHECK();
 }
 

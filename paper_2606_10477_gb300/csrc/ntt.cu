@@ -42,6 +42,7 @@ static void dispatch(const Tables& T, const LimbSet& S, cudaStream_t st, bool in
   if (A.own_alpha && (A.own_dn < 1 || A.own_alpha > 8)) throw Error(HEDAP_ERR_ARG, "NTT: bad digit layout");
   if (A.z && (inverse || !A.own_alpha || !A.bconv || !A.bconv_b_offset)) throw Error(HEDAP_ERR_ARG, "NTT: bad ModUp fusion");
   if (A.post && !inverse) throw Error(HEDAP_ERR_ARG, "NTT: post factors apply to the inverse only");
+  if (A.pre_e && !inverse) throw Error(HEDAP_ERR_ARG, "NTT: a fused sum on load applies to the inverse only");
   if ((A.spread || A.fin_dst || A.pconv) && inverse)
     throw Error(HEDAP_ERR_ARG, "NTT: fused rescale / ModDown applies to the forward only");
   if (A.pconv && (A.pconv_K < 1 || A.pconv_K > 8 || A.z || A.src || (A.spread && !A.fin_e)))

@@ -884,10 +884,22 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_inv_rows(Tables T, LimbSet
     if (own_limb(A, part, li)) continue;
     u64* a = S.limb(part, li, N) + j0;
     const u64* src = A.src ? A.src + part * A.src_stride + (size_t)li * N + j0 : a;
+    if (A.pre_e && li == S.limb_begin) {  // the first limb enters as e + x w
+      const u64* ep = A.pre_e + part * A.pre_e_stride + j0;
 #pragma unroll
-    for (int k = 0; k < G::M0 / 2; ++k) {
-      const int e = k * G::M1 + low;
-      cp_async16(xs + (e >> (G::K1 - 1)) * G::GS + (e & (G::M1 / 2 - 1)) * 2, src + 2 * e);
+      for (int k = 0; k < G::M0 / 2; ++k) {
+        const int e = k * G::M1 + low;
+        const ulonglong2 x = ldg2(src + 2 * e), c = ldg2(ep + 2 * e);
+        stg2(xs + (e >> (G::K1 - 1)) * G::GS + (e & (G::M1 / 2 - 1)) * 2,
+             ulonglong2{add_mod(c.x, shoup_mul(x.x, A.pre_w, A.pre_wsh, P.q), P.q),
+                        add_mod(c.y, shoup_mul(x.y, A.pre_w, A.pre_wsh, P.q), P.q)});
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < G::M0 / 2; ++k) {
+        const int e = k * G::M1 + low;
+        cp_async16(xs + (e >> (G::K1 - 1)) * G::GS + (e & (G::M1 / 2 - 1)) * 2, src + 2 * e);
+      }
     }
     cp_async_commit();
     cp_async_wait_all();
