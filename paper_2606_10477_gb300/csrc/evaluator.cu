@@ -36,8 +36,7 @@ std::unique_ptr<Ct> ct_copy(Ctx& C, const Ct& a, int level) {
   if (level > a.level) throw Error(HEDAP_ERR_LEVEL, "cannot raise the level by copying");
   auto c = ct_alloc(C, level, a.batch);
   c->scale = a.scale;
-  HEDAP_CUDA(cudaMemcpy2DAsync(c->part(0), c->part_stride() * 8, a.part(0), a.part_stride() * 8,
-                               (size_t)(level + 1) * C.N * 8, a.parts(), cudaMemcpyDeviceToDevice, C.stream));
+  k_copy_parts(C, a.part(0), a.part_stride(), c->part(0), c->part_stride(), a.parts(), (size_t)(level + 1) * C.N);
   return c;
 }
 std::unique_ptr<Ct> ev_drop(Ctx& C, const Ct& a, int level) {
@@ -57,8 +56,8 @@ std::unique_ptr<Ct> batch_pack(Ctx& C, const std::vector<const Ct*>& cts) {
   b->scale = f.scale;
   int at = 0;
   for (const Ct* c : cts) {
-    HEDAP_CUDA(cudaMemcpy2DAsync(b->part(2 * at), b->part_stride() * 8, c->part(0), c->part_stride() * 8,
-                                 (size_t)(f.level + 1) * C.N * 8, c->parts(), cudaMemcpyDeviceToDevice, C.stream));
+    k_copy_parts(C, c->part(0), c->part_stride(), b->part(2 * at), b->part_stride(), c->parts(),
+                 (size_t)(f.level + 1) * C.N);
     at += c->batch;
   }
   return b;
@@ -67,16 +66,15 @@ std::unique_ptr<Ct> batch_slice(Ctx& C, const Ct& b, int first, int count) {
   if (first < 0 || count < 1 || first + count > b.batch) throw Error(HEDAP_ERR_ARG, "batch slice out of range");
   auto c = ct_alloc(C, b.level, count);
   c->scale = b.scale;
-  HEDAP_CUDA(cudaMemcpy2DAsync(c->part(0), c->part_stride() * 8, b.part(2 * first), b.part_stride() * 8,
-                               (size_t)(b.level + 1) * C.N * 8, 2 * count, cudaMemcpyDeviceToDevice, C.stream));
+  k_copy_parts(C, b.part(2 * first), b.part_stride(), c->part(0), c->part_stride(), 2 * count,
+               (size_t)(b.level + 1) * C.N);
   return c;
 }
 std::unique_ptr<Ct> batch_unpack(Ctx& C, const Ct& b, int k) {
   if (k < 0 || k >= b.batch) throw Error(HEDAP_ERR_ARG, "batch index out of range");
   auto c = ct_alloc(C, b.level, 1);
   c->scale = b.scale;
-  HEDAP_CUDA(cudaMemcpy2DAsync(c->part(0), c->part_stride() * 8, b.part(2 * k), b.part_stride() * 8,
-                               (size_t)(b.level + 1) * C.N * 8, 2, cudaMemcpyDeviceToDevice, C.stream));
+  k_copy_parts(C, b.part(2 * k), b.part_stride(), c->part(0), c->part_stride(), 2, (size_t)(b.level + 1) * C.N);
   return c;
 }
 
@@ -353,6 +351,7 @@ static void ks_moddown_rescale(Ctx& C, const DevBuf& acc, int batch, int l, cons
   // N^-1 phinv_k: one inverse transform of K + 1 limbs a part
   NttAux inv{};
   inv.post = LC.mdr_post.p;
+  inv.pre_scale = 1;
   inv.pre_e = e + (size_t)l * N;
   inv.pre_e_stride = e_stride;
   inv.pre_w = LC.mdr_last.pinv;
@@ -456,8 +455,11 @@ std::unique_ptr<Ct> ev_mul_relin(Ctx& C, const Ct& a, const Ct& b) {
   return o;
 }
 
-// rescale by q_l: c_i <- (c_i - [c_l]_centred) * q_l^-1 mod q_i, i < l
-std::unique_ptr<Ct> ev_rescale(Ctx& C, const Ct& a) {
+// rescale by q_l: c_i <- (c_i - [c_l]_centred) * q_l^-1 mod q_i, i < l.  With K (w the per-limb constants): of the
+// product c w, in the same two transforms: the last limb enters its inverse transform as c_l w_l, and the
+// finish computes c_i (w_i q_l^-1) - v q_l^-1, so the product is never formed apart (one pass over the
+// ciphertext less; Mul_P by a constant of 8 ciphertexts at level 23).
+static std::unique_ptr<Ct> rescale_scaled(Ctx& C, const Ct& a, const LimbConsts* K) {
   const int l = a.level;
   if (l < 1) throw Error(HEDAP_ERR_LEVEL, "rescale needs level >= 1");
   const size_t N = C.N;
@@ -467,13 +469,31 @@ std::unique_ptr<Ct> ev_rescale(Ctx& C, const Ct& a) {
   o->scale = a.scale / (double)C.primes[l];
   // the last limb to the coefficient domain (read in place), then one forward transform whose
   // load spreads its centred residue into every other prime and whose store finishes the rescale
-  DevBuf last(P * N, C.stream);
+  DevBuf last(P * N, C.stream), factors;
   NttAux inv{};
   inv.src = a.part(0) + (size_t)l * N;
   inv.src_stride = a.part_stride();
+  NttAux fw{};
+  fw.fin_w = LC.d_rescale.p + l;
+  fw.fin_wb = LC.d_rescale.p + 2 * l;
+  if (K) {
+    inv.pre_scale = 1;
+    inv.pre_w = K->w[l];
+    inv.pre_wsh = h_shoup(K->w[l], C.primes[l]);
+    LimbConsts F;  // mont_mul_lazy's pairs of w_i q_l^-1
+    for (int i = 0; i < l; ++i) {
+      F.w[i] = h_mont(h_mulmod(K->w[i], LC.rescale.inv[i], C.primes[i]), C.primes[i]);
+      F.wsh[i] = h_mont(F.w[i], C.primes[i]);
+    }
+    factors = DevBuf(2 * (size_t)l, C.stream);
+    k_put_limbconst(C, factors.p, l, F);
+    fw.fin_w2 = fw.fin_w;
+    fw.fin_w2b = fw.fin_wb;
+    fw.fin_w = factors.p;
+    fw.fin_wb = factors.p + l;
+  }
   ntt_inverse(C.tab, qset(last.p, N, P, 0, 1, l), C.stream, &inv);
   DevBuf tmp((size_t)P * l * N, C.stream);
-  NttAux fw{};
   fw.spread = last.p;
   fw.spread_stride = N;
   fw.spread_sub = LC.d_rescale.p;
@@ -482,11 +502,10 @@ std::unique_ptr<Ct> ev_rescale(Ctx& C, const Ct& a) {
   fw.fin_dst_stride = o->part_stride();
   fw.fin_c = a.part(0);
   fw.fin_c_stride = a.part_stride();
-  fw.fin_w = LC.d_rescale.p + l;
-  fw.fin_wb = LC.d_rescale.p + 2 * l;
   ntt_forward(C.tab, qset(tmp.p, (size_t)l * N, P, 0, l), C.stream, &fw);
   return o;
 }
+std::unique_ptr<Ct> ev_rescale(Ctx& C, const Ct& a) { return rescale_scaled(C, a, nullptr); }
 
 // A relinearised product entering a linear combination that is rescaled next, as one fused
 // operation: rescale(m (d01 + ModDown(acc)) + sum_j c_j t_j + c0), m the product's integer constant.
@@ -636,7 +655,12 @@ std::unique_ptr<Ct> ev_lincomb_raw(Ctx& C, const std::vector<std::pair<const Ct*
 }
 
 std::unique_ptr<Ct> ev_mul_const(Ctx& C, const Ct& a, double c, double target) {
-  auto o = ev_rescale(C, *ev_mul_const_raw(C, a, c, target));
+  const int l = a.level;
+  if (l < 1) throw Error(HEDAP_ERR_LEVEL, "constant multiplication needs level >= 1");
+  const double v = std::round(c * (target * (double)C.primes[l] / a.scale));  // as in ev_mul_const_raw
+  LimbConsts K;
+  for (int i = 0; i <= l; ++i) K.w[i] = h_double_to_mod(v, C.primes[i]);
+  auto o = rescale_scaled(C, a, &K);
   o->scale = target;
   return o;
 }
@@ -645,8 +669,9 @@ std::unique_ptr<Ct> ev_add_const(Ctx& C, const Ct& a, double c) {
   const double v = std::round(c * a.scale);
   LimbConsts K;
   for (int i = 0; i <= a.level; ++i) K.w[i] = h_double_to_mod(v, C.primes[i]);
-  auto o = ct_copy(C, a, a.level);
-  k_add_limbconst(C, o->part(0), 2 * o->part_stride(), a.batch, a.level + 1, K);
+  auto o = ct_alloc(C, a.level, a.batch);
+  o->scale = a.scale;
+  k_add_limbconst(C, a.part(0), a.part_stride(), o->part(0), o->part_stride(), a.parts(), a.level + 1, K);
   return o;
 }
 

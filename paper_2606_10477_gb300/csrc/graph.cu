@@ -7,6 +7,7 @@
 // intermediates are allocated and freed inside the graph (stream-ordered memory
 // nodes), the result is copied into a buffer the graph object owns.
 #include "internal.cuh"
+#include "kernels.cuh"
 #include "profiler.cuh"
 
 struct hedap_graph {
@@ -27,8 +28,8 @@ namespace {
 using namespace hedap;
 
 void copy_ct(Ctx& C, const Ct& src, Ct& dst) {
-  HEDAP_CUDA(cudaMemcpy2DAsync(dst.part(0), dst.part_stride() * 8, src.part(0), src.part_stride() * 8,
-                               (size_t)(src.level + 1) * C.N * 8, src.parts(), cudaMemcpyDeviceToDevice, C.stream));
+  k_copy_parts(C, src.part(0), src.part_stride(), dst.part(0), dst.part_stride(), src.parts(),
+               (size_t)(src.level + 1) * C.N);
 }
 
 template <class F>

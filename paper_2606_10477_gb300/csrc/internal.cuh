@@ -141,8 +141,9 @@ struct NttAux {
   // inverse only: the final factor of limb li is the pair post[2 r], post[2 r + 1] (value, Shoup
   // companion), r = li - limb_begin, instead of N^-1
   const u64* post = nullptr;
-  // inverse only: the first limb (limb_begin) of part p enters as pre_e[p * pre_e_stride + n] + x pre_w mod its prime,
-  // x the limb itself (canonical residues; pre_w with its Shoup companion pre_wsh)
+  // inverse only, with pre_scale: the first limb (limb_begin) of part p enters as pre_e[p * pre_e_stride + n] + x pre_w
+  // mod its prime, x the limb itself (canonical residues; pre_w with its Shoup companion pre_wsh), pre_e null for 0
+  int pre_scale = 0;
   const u64* pre_e = nullptr;
   size_t pre_e_stride = 0;
   u64 pre_w = 0, pre_wsh = 0;
@@ -196,6 +197,7 @@ struct NttAux {
   size_t fin_e_stride = 0;
   const u64* fin_w2 = nullptr;
   const u64* fin_w2b = nullptr;
+  // with fin_w2 and no fin_e: the same with 0 in its place (a rescale of c times a constant)
   int fin_neg = 0;  // with fin_e: store the negated residues
 };
 // Forward only: the second phase of the ModUp transform of a key switch fused with the key inner

@@ -44,6 +44,29 @@ void k_add_sub(const Ctx& C, const u64* a, size_t as, const u64* b, size_t bs, u
   HEDAP_LAUNCH_CHECK();
 }
 
+// ---------------------------------------------------------------- part copies
+// `words` words of each of n_parts parts of a ciphertext (part strides ss, ds; whole limbs)
+__global__ void k_copy_parts_kernel(const u64* __restrict__ src, size_t ss, u64* __restrict__ dst, size_t ds,
+                                    int n_parts, size_t words) {
+  const size_t pairs = words / 2;
+  GRID_LOOP(t, n_parts * pairs) {
+    const size_t p = t / pairs, r = 2 * (t - p * pairs);
+    st2(dst + p * ds + r, ld2(src + p * ss + r));
+  }
+}
+// Bound by HBM.  Flat ranges go to the copy engine's kernel; strided ones here, which cudaMemcpy2DAsync moves at less
+// than half the rate.
+void k_copy_parts(const Ctx& C, const u64* src, size_t ss, u64* dst, size_t ds, int n_parts, size_t words) {
+  if (n_parts == 1 || (ss == words && ds == words)) {
+    HEDAP_CUDA(cudaMemcpyAsync(dst, src, n_parts * words * 8, cudaMemcpyDeviceToDevice, C.stream));
+    return;
+  }
+  prof_count_launches(1);
+  const size_t work = n_parts * words / 2;
+  k_copy_parts_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(src, ss, dst, ds, n_parts, words);
+  HEDAP_LAUNCH_CHECK();
+}
+
 // ---------------------------------------------------------------- residue range check
 // flag[0] |= 1 when some word of the n_parts x limbs limbs at a (part stride as) is not below its prime
 __global__ void k_check_residues_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ a, size_t as,
@@ -164,28 +187,44 @@ void k_lincomb(const Ctx& C, u64* out, size_t os, int n_parts, int limbs, const 
   HEDAP_LAUNCH_CHECK();
 }
 
-// add a per-limb constant to n_parts parts spaced `stride` apart (the c0 parts of a batch)
-__global__ void k_add_limbconst_kernel(const PrimeDev* __restrict__ pr, u64* __restrict__ io, size_t stride,
-                                       int n_parts, int limbs, int log_n, LimbConsts K) {
+// out = in, plus a per-limb constant on the even parts (the c0 of each batch member)
+__global__ void k_add_limbconst_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ in, size_t is,
+                                       u64* __restrict__ out, size_t os, int n_parts, int limbs, int log_n,
+                                       LimbConsts K) {
   const size_t per_part = (size_t)limbs << log_n;
   GRID_LOOP(t, n_parts * per_part / 2) {
     const size_t e = 2 * t;
     const size_t p = e / per_part, r = e - p * per_part;
-    const int i = (int)(r >> log_n);
-    const u64 q = pr[i].q, w = K.w[i];
-    u64* at = io + p * stride + r;
-    ulonglong2 x = ld2(at);
-    x.x = add_mod(x.x, w, q);
-    x.y = add_mod(x.y, w, q);
-    st2(at, x);
+    ulonglong2 x = ld2(in + p * is + r);
+    if (!(p & 1)) {
+      const int i = (int)(r >> log_n);
+      const u64 q = pr[i].q, w = K.w[i];
+      x.x = add_mod(x.x, w, q);
+      x.y = add_mod(x.y, w, q);
+    }
+    st2(out + p * os + r, x);
   }
 }
-void k_add_limbconst(const Ctx& C, u64* io, size_t stride, int n_parts, int limbs, const LimbConsts& K) {
+void k_add_limbconst(const Ctx& C, const u64* in, size_t is, u64* out, size_t os, int n_parts, int limbs,
+                     const LimbConsts& K) {
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, 2.0 * n_parts * limbs * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * limbs * C.N / 2;
-  k_add_limbconst_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(C.tab.pr, io, stride, n_parts, limbs, C.log_n,
+  k_add_limbconst_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(C.tab.pr, in, is, out, os, n_parts, limbs, C.log_n,
                                                                    K);
+  HEDAP_LAUNCH_CHECK();
+}
+// K's words to device memory: w [n], then wsh [n]
+__global__ void k_put_limbconst_kernel(u64* __restrict__ out, int n, const __grid_constant__ LimbConsts K) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    out[i] = K.w[i];
+    out[n + i] = K.wsh[i];
+  }
+}
+void k_put_limbconst(const Ctx& C, u64* out, int n, const LimbConsts& K) {
+  ProfScope prof_(PROF_ELEMENTWISE, C.stream, 16.0 * n);
+  prof_count_launches(1);
+  k_put_limbconst_kernel<<<1, 64, 0, C.stream>>>(out, n, K);
   HEDAP_LAUNCH_CHECK();
 }
 
@@ -419,7 +458,7 @@ void k_ksk_inner(const Ctx& C, const u64* y, const u64* d, size_t d_stride, cons
 __global__ void k_lift_qp_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ pmod,
                                  const u64* __restrict__ in, size_t is, u64* __restrict__ out, int n_parts, int l,
                                  int ext, int log_n) {
-  const size_t N = (size_t)1 << log_n, per = (size_t)ext << log_n;
+  const size_t per = (size_t)ext << log_n;
   GRID_LOOP(e, (size_t)n_parts * per) {
     const size_t p = e / per, r = e - p * per;
     const int t = (int)(r >> log_n);

@@ -16,7 +16,11 @@ void k_tensor(const Ctx& C, const u64* a, size_t as, const u64* b, size_t bs, u6
               int limbs);
 void k_mul_limbconst(const Ctx& C, const u64* in, size_t is, u64* out, size_t os, int n_parts, int limbs,
                      const LimbConsts& K);
-void k_add_limbconst(const Ctx& C, u64* io, size_t stride, int n_parts, int limbs, const LimbConsts& K);
+void k_add_limbconst(const Ctx& C, const u64* in, size_t is, u64* out, size_t os, int n_parts, int limbs,
+                     const LimbConsts& K);
+void k_put_limbconst(const Ctx& C, u64* out, int n, const LimbConsts& K);
+// device-to-device copy of `words` words of each of n_parts parts
+void k_copy_parts(const Ctx& C, const u64* src, size_t ss, u64* dst, size_t ds, int n_parts, size_t words);
 void k_rescale_spread(const Ctx& C, const u64* last, size_t ls, u64* tmp, size_t ts, int n_parts, int l,
                       const RescaleConsts& R);
 void k_rescale_finish(const Ctx& C, const u64* in, size_t is, const u64* tmp, size_t ts, u64* out, size_t os,

@@ -42,7 +42,7 @@ static void dispatch(const Tables& T, const LimbSet& S, cudaStream_t st, bool in
   if (A.own_alpha && (A.own_dn < 1 || A.own_alpha > 8)) throw Error(HEDAP_ERR_ARG, "NTT: bad digit layout");
   if (A.z && (inverse || !A.own_alpha || !A.bconv || !A.bconv_b_offset)) throw Error(HEDAP_ERR_ARG, "NTT: bad ModUp fusion");
   if (A.post && !inverse) throw Error(HEDAP_ERR_ARG, "NTT: post factors apply to the inverse only");
-  if (A.pre_e && !inverse) throw Error(HEDAP_ERR_ARG, "NTT: a fused sum on load applies to the inverse only");
+  if ((A.pre_scale || A.pre_e) && (!inverse || !A.pre_scale)) throw Error(HEDAP_ERR_ARG, "NTT: a fused sum on load applies to the inverse only");
   if ((A.spread || A.fin_dst || A.pconv) && inverse)
     throw Error(HEDAP_ERR_ARG, "NTT: fused rescale / ModDown applies to the forward only");
   if (A.pconv && (A.pconv_K < 1 || A.pconv_K > 8 || A.z || A.src || (A.spread && !A.fin_e)))
@@ -50,6 +50,8 @@ static void dispatch(const Tables& T, const LimbSet& S, cudaStream_t st, bool in
   if (A.fin_e && (!A.fin_dst || !A.fin_w2 || !A.fin_w2b || !A.pconv || !A.spread))
     throw Error(HEDAP_ERR_ARG, "NTT: bad ModDown-rescale fusion");
   if (A.spread && (A.z || A.src || !A.spread_sub)) throw Error(HEDAP_ERR_ARG, "NTT: bad spread fusion");
+  if (A.fin_w2 && (!A.fin_dst || !A.fin_w2b || (!A.fin_e && (A.fin_acc_even || A.fin_acc_odd || A.fin_neg))))
+    throw Error(HEDAP_ERR_ARG, "NTT: bad scaled epilogue fusion");
   if (A.fin_dst && (!A.fin_c || !A.fin_w || !A.fin_wb)) throw Error(HEDAP_ERR_ARG, "NTT: bad epilogue fusion");
   const int v = inverse ? T.ntt_inv_variant
                         : A.z ? T.ntt_modup_variant

@@ -521,9 +521,9 @@ __device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u
   using G = RowGeo<L2>;
   const u64 q = P.q;
   constexpr int PAIRS = G::M0 / 2;  // word pairs of a lane
-  if (A.fin_e) {  // ModDown fused with the rescale: c (P q_l)^-1 + (e - v) q_l^-1
+  if (A.fin_w2) {  // ModDown fused with the rescale: c (P q_l)^-1 + (e - v) q_l^-1; or a rescale of c times a constant
     const u64* cp = A.fin_c + (size_t)part * A.fin_c_stride + at;
-    const u64* ep = A.fin_e + (size_t)part * A.fin_e_stride + at;
+    const u64* ep = A.fin_e ? A.fin_e + (size_t)part * A.fin_e_stride + at : nullptr;
     u64* dp = A.fin_dst + (size_t)part * A.fin_dst_stride + at;
     const u64 w = A.fin_w[li], wb = A.fin_wb[li], w2 = A.fin_w2[li], w2b = A.fin_w2b[li];
     auto fin = [&](u64 c, u64 e, u64 v) {  // both products in one Montgomery step: below 4q
@@ -537,7 +537,8 @@ __device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u
 #pragma unroll
     for (int k = 0; k < PAIRS; ++k) {
       const int e = k * G::M1 + low;
-      const ulonglong2 v = row_pair<L2>(xs, e), c = ldg2(cp + 2 * e), ee = ldg2(ep + 2 * e);
+      const ulonglong2 v = row_pair<L2>(xs, e), c = ldg2(cp + 2 * e);
+      const ulonglong2 ee = ep ? ldg2(ep + 2 * e) : ulonglong2{0, 0};
       ulonglong2 z;
       z.x = fin(c.x, ee.x, v.x);
       z.y = fin(c.y, ee.y, v.y);
@@ -884,12 +885,12 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_inv_rows(Tables T, LimbSet
     if (own_limb(A, part, li)) continue;
     u64* a = S.limb(part, li, N) + j0;
     const u64* src = A.src ? A.src + part * A.src_stride + (size_t)li * N + j0 : a;
-    if (A.pre_e && li == S.limb_begin) {  // the first limb enters as e + x w
-      const u64* ep = A.pre_e + part * A.pre_e_stride + j0;
+    if (A.pre_scale && li == S.limb_begin) {  // the first limb enters as e + x w
+      const u64* ep = A.pre_e ? A.pre_e + part * A.pre_e_stride + j0 : nullptr;
 #pragma unroll
       for (int k = 0; k < G::M0 / 2; ++k) {
         const int e = k * G::M1 + low;
-        const ulonglong2 x = ldg2(src + 2 * e), c = ldg2(ep + 2 * e);
+        const ulonglong2 x = ldg2(src + 2 * e), c = ep ? ldg2(ep + 2 * e) : ulonglong2{0, 0};
         stg2(xs + (e >> (G::K1 - 1)) * G::GS + (e & (G::M1 / 2 - 1)) * 2,
              ulonglong2{add_mod(c.x, shoup_mul(x.x, A.pre_w, A.pre_wsh, P.q), P.q),
                         add_mod(c.y, shoup_mul(x.y, A.pre_w, A.pre_wsh, P.q), P.q)});
