@@ -165,6 +165,8 @@ struct RowGeo : Phase<L2> {
   static constexpr int GS = P::M1 + 2;                                           // stride of a group
   static constexpr int BS = P::M0 * GS + (P::K1 < 4 ? P::M1 : 0);                // stride of a block
   static constexpr int XWORDS = P::PER * BS;
+  // place of word pair e (words 2 e, 2 e + 1) of a block; additive over numbers without a common bit
+  static constexpr int pair(int e) { return (e >> (P::K1 - 1)) * GS + (e & (P::M1 / 2 - 1)) * 2; }
 };
 
 // ---------------------------------------------------------------- fused loads
@@ -509,11 +511,11 @@ __device__ __forceinline__ void fwd_rows_body(u64 (&v)[1][1 << Phase<L2>::K0], u
   }
   __syncwarp();
 }
-// word pair e (words 2 e, 2 e + 1) of a block in the exchange buffer
+// word pair e = k 2^K1 + low (words 2 e, 2 e + 1) of a block in the exchange buffer
 template <int L2>
-__device__ __forceinline__ ulonglong2 row_pair(const u64* xs, int e) {
+__device__ __forceinline__ ulonglong2 row_pair(const u64* xs, int k, int low) {
   using G = RowGeo<L2>;
-  return ldg2(xs + (e >> (G::K1 - 1)) * G::GS + (e & (G::M1 / 2 - 1)) * 2);
+  return ldg2(xs + G::pair(low) + G::pair(k * G::M1));
 }
 template <bool SMALL, int L2>
 __device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u64* a, size_t at, int part, int li,
@@ -537,7 +539,7 @@ __device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u
 #pragma unroll
     for (int k = 0; k < PAIRS; ++k) {
       const int e = k * G::M1 + low;
-      const ulonglong2 v = row_pair<L2>(xs, e), c = ldg2(cp + 2 * e);
+      const ulonglong2 v = row_pair<L2>(xs, k, low), c = ldg2(cp + 2 * e);
       const ulonglong2 ee = ep ? ldg2(ep + 2 * e) : ulonglong2{0, 0};
       ulonglong2 z;
       z.x = fin(c.x, ee.x, v.x);
@@ -561,7 +563,7 @@ __device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u
 #pragma unroll
     for (int k = 0; k < PAIRS; ++k) {
       const int e = k * G::M1 + low;
-      const ulonglong2 v = row_pair<L2>(xs, e), c = ldg2(cp + 2 * e);
+      const ulonglong2 v = row_pair<L2>(xs, k, low), c = ldg2(cp + 2 * e);
       ulonglong2 z;
       z.x = fin(c.x, v.x);
       z.y = fin(c.y, v.y);
@@ -576,7 +578,7 @@ __device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u
 #pragma unroll
     for (int k = 0; k < PAIRS; ++k) {
       const int e = k * G::M1 + low;
-      const ulonglong2 v = row_pair<L2>(xs, e);
+      const ulonglong2 v = row_pair<L2>(xs, k, low);
       stg2(a + 2 * e, ulonglong2{fwd_canonical<SMALL>(v.x, q, P.rc), fwd_canonical<SMALL>(v.y, q, P.rc)});
     }
   }
@@ -654,8 +656,11 @@ struct KskGeo {
   static constexpr int KB = 32 / LPB;                       // blocks a warp
   // passes: a first one of F stages, then passes of 3
   static constexpr int F = L2 % 3 ? L2 % 3 : 3, NP = (L2 + 2) / 3;
-  static constexpr int word(int x) { return x + 2 * (x >> 3) + 8 * (x >> 6); }  // padded index inside a block
   static constexpr int BS = (1 << L2) + 2 * (1 << L2 >> 3) + 8 * ((1 << L2) >> 6) + (L2 < 6 ? 8 : 0);
+  // padded index inside a block, and of a word of the warp's run; both are additive over numbers without a common
+  // bit, which keeps the lane's part out of the unrolled loops
+  static constexpr int word(int x) { return x + 2 * (x >> 3) + 8 * (x >> 6); }
+  static constexpr int run_word(int x) { return (x >> L2) * BS + word(x & ((1 << L2) - 1)); }
   static constexpr int XWORDS = KB * BS;
 };
 // twiddles of a block as staged for KskGeo's passes: those of a pass of K stages from local stage s0
@@ -680,14 +685,14 @@ __device__ __forceinline__ void ksk_passes(u64* xs, const ulonglong2* tw, u64 q,
       }
     } else {
 #pragma unroll
-      for (int m = 0; m < (1 << K); ++m) v[i][0][m] = xs[G::word(base + m * TL)];
+      for (int m = 0; m < (1 << K); ++m) v[i][0][m] = xs[G::word(base) + G::word(m * TL)];
     }
     fwd_pass<SMALL, L1 + S0, K, 1>(v[i], q, nqi, [&](int u, int mm) {
       return tw[(1 << S0) + (((1 << u) - 1 + mm) << S0) + high];
     });
     if constexpr (TL > 1) {
 #pragma unroll
-      for (int m = 0; m < (1 << K); ++m) xs[G::word(base + m * TL)] = v[i][0][m];
+      for (int m = 0; m < (1 << K); ++m) xs[G::word(base) + G::word(m * TL)] = v[i][0][m];
     } else {
 #pragma unroll
       for (int m = 0; m < (1 << K); ++m) out[i * (1 << K) + m] = v[i][0][m];
@@ -747,11 +752,9 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_fwd_rows_ksk(Tables T, Lim
   u64* bufs = sm + warp * 2 * G::XWORDS;
   auto fetch = [&](int j, u64* dst) {
     const u64* src = src0 + (size_t)j * S.part_stride + 2 * lane;
+    dst += G::run_word(2 * lane);
 #pragma unroll
-    for (int i = 0; i < G::PER / 2; ++i) {
-      const int x = 2 * (i * 32 + lane), blk = x >> L2, in = x & ((1 << L2) - 1);
-      cp_async16(dst + blk * G::BS + G::word(in), src + i * 64);
-    }
+    for (int i = 0; i < G::PER / 2; ++i) cp_async16(dst + G::run_word(64 * i), src + i * 64);
   };
   if (live && j_first < dn) fetch(j_first, bufs);
   cp_async_commit();
@@ -763,9 +766,9 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_fwd_rows_ksk(Tables T, Lim
   // word pair i of the lane (words 2 i, 2 i + 1 of its PER consecutive ones) of digit j's key run (key_pair: the
   // lanes' pairs are consecutive)
   auto key_words = [&](int j, size_t part, ulonglong2 (&w)[G::PER / 2]) {
-    const u64* at = kb + (size_t)j * F.key_digit_stride + part;
+    const u64* at = kb + (size_t)j * F.key_digit_stride + part + 2 * key_pair(lane * (G::PER / 2));
 #pragma unroll
-    for (int i = 0; i < G::PER / 2; ++i) w[i] = __ldg(reinterpret_cast<const ulonglong2*>(at + 2 * key_pair(lane * (G::PER / 2) + i)));
+    for (int i = 0; i < G::PER / 2; ++i) w[i] = __ldg(reinterpret_cast<const ulonglong2*>(at + 2 * key_pair(i)));
   };
   auto mac_words = [&](const u64 (&v)[G::PER], const ulonglong2 (&w)[G::PER / 2], Acc128 (&acc)[G::PER]) {
 #pragma unroll
@@ -891,7 +894,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_inv_rows(Tables T, LimbSet
       for (int k = 0; k < G::M0 / 2; ++k) {
         const int e = k * G::M1 + low;
         const ulonglong2 x = ldg2(src + 2 * e), c = ep ? ldg2(ep + 2 * e) : ulonglong2{0, 0};
-        stg2(xs + (e >> (G::K1 - 1)) * G::GS + (e & (G::M1 / 2 - 1)) * 2,
+        stg2(xs + G::pair(low) + G::pair(k * G::M1),
              ulonglong2{add_mod(c.x, shoup_mul(x.x, A.pre_w, A.pre_wsh, P.q), P.q),
                         add_mod(c.y, shoup_mul(x.y, A.pre_w, A.pre_wsh, P.q), P.q)});
       }
@@ -899,7 +902,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_inv_rows(Tables T, LimbSet
 #pragma unroll
       for (int k = 0; k < G::M0 / 2; ++k) {
         const int e = k * G::M1 + low;
-        cp_async16(xs + (e >> (G::K1 - 1)) * G::GS + (e & (G::M1 / 2 - 1)) * 2, src + 2 * e);
+        cp_async16(xs + G::pair(low) + G::pair(k * G::M1), src + 2 * e);
       }
     }
     cp_async_commit();
