@@ -224,6 +224,12 @@ struct KskFuse {
 void ntt_forward(const Tables& T, const LimbSet& S, cudaStream_t st, const NttAux* aux = nullptr,
                  const KskFuse* fuse = nullptr);
 void ntt_inverse(const Tables& T, const LimbSet& S, cudaStream_t st, const NttAux* aux = nullptr);
+// whether a transform of `limbs` limbs at N = 2^log_n with n_prod products a word in its load runs with a whole limb
+// per cluster (ntt_impl.cuh): up to 2^21 words in all (a rescale of 8 ciphertexts of 21 limbs at N = 2^12, 1.4 M words,
+// 25.7 us against 29.1 us); beyond, the two-launch kernels carry more at a time
+inline bool ntt_whole_limb(int log_n, size_t limbs, int n_prod) {
+  return log_n <= 13 && n_prod <= 3 && (limbs << log_n) <= (size_t)1 << 21;
+}
 struct Ctx;
 void ntt_tune(Ctx& C, int limbs, int reps, std::vector<float>* fwd_ms, std::vector<float>* inv_ms);
 double butterfly_rate(Ctx& C);  // butterflies per second of a register-only loop

@@ -292,11 +292,12 @@ struct FusedLoad {
 };
 
 // ---------------------------------------------------------------- forward, column phase
-// both passes of one limb's columns: v holds pass 0's input (row m 2^K1 + low), out the limb's words at (row 0,
-// this thread's column); tw: global memory (L1) or shared memory
-template <bool SMALL, int L1, int L2, int TH>
-__device__ __forceinline__ void fwd_cols_body(u64 (&v)[1][1 << Phase<L1>::K0], u64* xs, const ulonglong2* tw, u64 q,
-                                              uint32_t nqi, int low, int cg, u64* out) {
+// both passes of one limb's columns: v holds pass 0's input (row m 2^K1 + low), o pass 1's output (row
+// (i 2^K1 + low) 2^K1 + m of this thread's column); tw: global memory (L1) or shared memory
+template <bool SMALL, int L1, int TH>
+__device__ __forceinline__ void fwd_cols_passes(u64 (&v)[1][1 << Phase<L1>::K0], u64* xs, const ulonglong2* tw, u64 q,
+                                                uint32_t nqi, int low, int cg,
+                                                u64 (&o)[Phase<L1>::GP][1][1 << Phase<L1>::K1]) {
   using G = ColGeo<L1, TH>;
   fwd_pass<SMALL, 0, G::K0, 1>(v, q, nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
   __syncthreads();  // the last limb's exchange has been read
@@ -306,15 +307,24 @@ __device__ __forceinline__ void fwd_cols_body(u64 (&v)[1][1 << Phase<L1>::K0], u
 #pragma unroll
   for (int i = 0; i < G::GP; ++i) {
     const int hi = i * G::M1 + low;  // rows hi 2^K1 + m
-    u64 w[1][G::M1];
 #pragma unroll
-    for (int m = 0; m < G::M1; ++m) w[0][m] = xs[(hi * (G::M1 + 1) + m) * G::COLS + cg];
-    fwd_pass<SMALL, G::K0, G::K1, 1>(w, q, nqi, [&](int u, int mm) {
+    for (int m = 0; m < G::M1; ++m) o[i][0][m] = xs[(hi * (G::M1 + 1) + m) * G::COLS + cg];
+    fwd_pass<SMALL, G::K0, G::K1, 1>(o[i], q, nqi, [&](int u, int mm) {
       return tw[G::M0 + ((1 << u) - 1 + mm) * G::M0 + hi];
     });
-#pragma unroll
-    for (int m = 0; m < G::M1; ++m) out[(size_t)(hi * G::M1 + m) << L2] = w[0][m];
   }
+}
+// the same, the output stored to global memory: out at (row 0, this thread's column)
+template <bool SMALL, int L1, int L2, int TH>
+__device__ __forceinline__ void fwd_cols_body(u64 (&v)[1][1 << Phase<L1>::K0], u64* xs, const ulonglong2* tw, u64 q,
+                                              uint32_t nqi, int low, int cg, u64* out) {
+  using G = ColGeo<L1, TH>;
+  u64 o[G::GP][1][G::M1];
+  fwd_cols_passes<SMALL, L1, TH>(v, xs, tw, q, nqi, low, cg, o);
+#pragma unroll
+  for (int i = 0; i < G::GP; ++i)
+#pragma unroll
+    for (int m = 0; m < G::M1; ++m) out[(size_t)((i * G::M1 + low) * G::M1 + m) << L2] = o[i][0][m];
 }
 template <int N, int TH>  // N twiddles into shared memory
 __device__ __forceinline__ void stage_twiddles(ulonglong2* dst, const ulonglong2* src, int t) {
@@ -835,8 +845,9 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_fwd_rows_ksk(Tables T, Lim
 // ---------------------------------------------------------------- inverse, row phase
 // The forward row phase mirrored: the 2^K1 consecutive words of a lane's groups first, then the words
 // 2^K1 apart.  Output left lazy (below 2^(L2+1) q for small primes, 3q otherwise).
-template <bool SMALL, int L1, int L2>
-__device__ __forceinline__ void inv_rows_body(u64* a, u64* xs, const ulonglong2* tw, const PrimeDev& P, int low) {
+template <bool SMALL, int L2>
+__device__ __forceinline__ void inv_rows_passes(u64 (&v)[1][1 << Phase<L2>::K0], u64* xs, const ulonglong2* tw,
+                                                const PrimeDev& P, int low) {
   using G = RowGeo<L2>;
   const u64 q = P.q;
 #pragma unroll
@@ -856,7 +867,6 @@ __device__ __forceinline__ void inv_rows_body(u64* a, u64* xs, const ulonglong2*
     for (int m = 0; m < G::M1; m += 2) stg2(xs + hi * G::GS + m, ulonglong2{w[0][m], w[0][m + 1]});
   }
   __syncwarp();
-  u64 v[1][G::M0];
 #pragma unroll
   for (int m = 0; m < G::M0; ++m) v[0][m] = xs[m * G::GS + low];
   constexpr bool MID = SMALL && 1 + L2 > 9;  // 2^(L2+1) q would pass 2^64: reduce between the passes
@@ -865,8 +875,29 @@ __device__ __forceinline__ void inv_rows_body(u64* a, u64* xs, const ulonglong2*
     for (int m = 0; m < G::M0; ++m) v[0][m] = reduce_lazy(v[0][m], q, P.rc);
   }
   inv_pass<SMALL, MID ? 1 : 1 + G::K1, G::K0, 1>(v, q, P.nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
+}
+// a block's words from global memory into the exchange buffer: j0 the block's first word of the limb
+template <int L2>
+__device__ __forceinline__ void inv_rows_load(const NttAux& A, const LimbSet& S, int part, int li, const u64* src, u64* xs,
+                                              size_t j0, const PrimeDev& P, int low) {
+  using G = RowGeo<L2>;
+  if (A.pre_scale && li == S.limb_begin) {  // the first limb enters as e + x w
+    const u64* ep = A.pre_e ? A.pre_e + part * A.pre_e_stride + j0 : nullptr;
 #pragma unroll
-  for (int m = 0; m < G::M0; ++m) a[m * G::M1 + low] = v[0][m];
+    for (int k = 0; k < G::M0 / 2; ++k) {
+      const int e = k * G::M1 + low;
+      const ulonglong2 x = ldg2(src + 2 * e), c = ep ? ldg2(ep + 2 * e) : ulonglong2{0, 0};
+      stg2(xs + G::pair(low) + G::pair(k * G::M1),
+           ulonglong2{add_mod(c.x, shoup_mul(x.x, A.pre_w, A.pre_wsh, P.q), P.q),
+                      add_mod(c.y, shoup_mul(x.y, A.pre_w, A.pre_wsh, P.q), P.q)});
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < G::M0 / 2; ++k) {
+      const int e = k * G::M1 + low;
+      cp_async16(xs + G::pair(low) + G::pair(k * G::M1), src + 2 * e);
+    }
+  }
 }
 template <int L1, int L2, int W, int MINB>
 __global__ void __launch_bounds__(32 * W, MINB) k_ntt_inv_rows(Tables T, LimbSet S, NttAux A, int ppc) {
@@ -888,28 +919,15 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_inv_rows(Tables T, LimbSet
     if (own_limb(A, part, li)) continue;
     u64* a = S.limb(part, li, N) + j0;
     const u64* src = A.src ? A.src + part * A.src_stride + (size_t)li * N + j0 : a;
-    if (A.pre_scale && li == S.limb_begin) {  // the first limb enters as e + x w
-      const u64* ep = A.pre_e ? A.pre_e + part * A.pre_e_stride + j0 : nullptr;
-#pragma unroll
-      for (int k = 0; k < G::M0 / 2; ++k) {
-        const int e = k * G::M1 + low;
-        const ulonglong2 x = ldg2(src + 2 * e), c = ep ? ldg2(ep + 2 * e) : ulonglong2{0, 0};
-        stg2(xs + G::pair(low) + G::pair(k * G::M1),
-             ulonglong2{add_mod(c.x, shoup_mul(x.x, A.pre_w, A.pre_wsh, P.q), P.q),
-                        add_mod(c.y, shoup_mul(x.y, A.pre_w, A.pre_wsh, P.q), P.q)});
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < G::M0 / 2; ++k) {
-        const int e = k * G::M1 + low;
-        cp_async16(xs + G::pair(low) + G::pair(k * G::M1), src + 2 * e);
-      }
-    }
+    inv_rows_load<L2>(A, S, part, li, src, xs, j0, P, low);
     cp_async_commit();
     cp_async_wait_all();
     __syncwarp();
-    if (inv_small(P.q)) inv_rows_body<true, L1, L2>(a, xs, tw, P, low);
-    else inv_rows_body<false, L1, L2>(a, xs, tw, P, low);
+    u64 v[1][G::M0];
+    if (inv_small(P.q)) inv_rows_passes<true, L2>(v, xs, tw, P, low);
+    else inv_rows_passes<false, L2>(v, xs, tw, P, low);
+#pragma unroll
+    for (int m = 0; m < G::M0; ++m) a[m * G::M1 + low] = v[0][m];
     __syncwarp();
   }
   cp_async_wait_all();
@@ -967,6 +985,205 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_inv_cols(Tables T, LimbSet S, 
   __syncthreads();
   if (inv_small(P.q)) inv_cols_body<true, L1, L2, TH>(w, a, sm, tw, P, low, cg, ni, nip);
   else inv_cols_body<false, L1, L2, TH>(w, a, sm, tw, P, low, cg, ni, nip);
+}
+
+// ---------------------------------------------------------------- small rings: a whole limb per cluster
+// N <= 2^13: a cluster of CTAs (1024 words and 128 threads each, 2048 and 256 at 2^13) holds a whole limb in shared memory
+// and hands it from one phase to the other through distributed shared memory, so that one launch does both.  For a
+// few limbs a launch costs its latency (5 us), not its work; a limb on one SM alone (N = 2^12: 10 us) loses
+// what the launch saves.  8 words a thread (16 in the row phase at 2^13, where half of the threads work); the
+// twiddles of the CTA's columns and blocks are staged with the first load.
+template <int L1, int L2>
+struct WholeGeo {
+  static constexpr int CW = L1 + L2 == 13 ? 2048 : 1024;     // words of a CTA
+  static constexpr int CS = (1 << (L1 + L2)) / CW;           // CTAs of a cluster
+  static constexpr int TH = CW / 8, BLK = (1 << L1) / CS;    // threads, row blocks of a CTA
+  using C = ColGeo<L1, TH>;
+  using R = RowGeo<L2>;
+  static_assert(C::COLS * CS == 1 << L2 && C::M0 == 8 && BLK * R::M1 <= TH, "8 words a thread in the column phase");
+  static constexpr int YWORDS = BLK * R::BS;                 // words of the row layout, block after block
+  static constexpr int XWORDS = (C::XWORDS + 1) & ~1;
+  static constexpr int TW = (1 << L1) + (BLK << L2);
+  static constexpr size_t SMEM = (size_t)(XWORDS + YWORDS) * 8 + (size_t)TW * 16;
+};
+template <int CS>
+__device__ __forceinline__ void cluster_arrive() {
+  if constexpr (CS > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+template <int CS>
+__device__ __forceinline__ void cluster_wait() {
+  if constexpr (CS > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  else __syncthreads();
+}
+// the address of shared-memory word p in CTA `rank` of the cluster, and a store there
+__device__ __forceinline__ uint32_t cluster_addr(const u64* p, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_store(uint32_t addr, u64 v) {
+  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+template <int L1, int L2>
+__global__ void __cluster_dims__(WholeGeo<L1, L2>::CS, 1, 1) __launch_bounds__(WholeGeo<L1, L2>::TH)
+    k_ntt_inv_whole(Tables T, LimbSet S, NttAux A) {
+  using W = WholeGeo<L1, L2>;
+  using G = typename W::C;
+  using R = typename W::R;
+  extern __shared__ __align__(16) u64 sm[];
+  constexpr size_t N = (size_t)1 << (L1 + L2);
+  const int li = S.limb_begin + blockIdx.x / W::CS, rank = blockIdx.x % W::CS, part = blockIdx.y;
+  if (own_limb(A, part, li)) return;
+  cluster_arrive<W::CS>();  // the others run before their shared memory is written
+  const int pi = S.prime(li);
+  const PrimeDev P = T.pr[pi];
+  u64 *X = sm, *Y = sm + W::XWORDS;
+  ulonglong2* tw = reinterpret_cast<ulonglong2*>(Y + W::YWORDS);
+  const ulonglong2* src_tw = T.ipsi2 + (size_t)pi * tw_stride(L1, L2);
+  stage_twiddles<1 << L1, W::TH>(tw, src_tw, threadIdx.x);
+  stage_twiddles<(W::BLK << L2), W::TH>(tw + (1 << L1), src_tw + (1 << L1) + ((size_t)rank * W::BLK << L2), threadIdx.x);
+  u64* a = S.limb(part, li, N);
+  const u64* src = A.src ? A.src + part * A.src_stride + (size_t)li * N : a;
+  const int low = threadIdx.x % R::M1, b = threadIdx.x / R::M1, blk = rank * W::BLK + b;  // row phase: block blk
+  const int cg = threadIdx.x % G::COLS, clow = threadIdx.x / G::COLS;
+  const bool row = b < W::BLK;
+  u64* ys = Y + b * R::BS;
+  if (row) inv_rows_load<L2>(A, S, part, li, src + ((size_t)blk << L2), ys, (size_t)blk << L2, P, low);
+  cp_async_commit();
+  const int r = li - S.limb_begin;
+  const u64 ni = A.post ? A.post[2 * r] : T.ninv[pi], nip = A.post ? A.post[2 * r + 1] : T.ninv_sh[pi];
+  cp_async_wait_all();
+  __syncthreads();
+  auto body = [&](auto is_small) {
+    constexpr bool SMALL = decltype(is_small)::value;
+    u64 v[1][R::M0];
+    if (row) inv_rows_passes<SMALL, L2>(v, ys, tw + (1 << L1) + (b << L2), P, low);
+    cluster_wait<W::CS>();
+    if (row) {
+#pragma unroll
+      for (int m = 0; m < R::M0; ++m) {  // row blk, column m 2^K1 + low
+        const int col = m * R::M1 + low;
+        u64* at = X + (blk + (blk >> G::K1)) * G::COLS + col % G::COLS;
+        if constexpr (W::CS > 1) cluster_store(cluster_addr(at, col / G::COLS), v[0][m]);
+        else *at = v[0][m];
+      }
+    }
+    cluster_arrive<W::CS>();
+    cluster_wait<W::CS>();
+    u64 w[G::GP][1][G::M1];
+#pragma unroll
+    for (int i = 0; i < G::GP; ++i)
+#pragma unroll
+      for (int m = 0; m < G::M1; ++m) w[i][0][m] = X[((i * G::M1 + clow) * (G::M1 + 1) + m) * G::COLS + cg];
+    // every thread writes back the words that it read: no barrier before inv_cols_body's exchange
+    inv_cols_body<SMALL, L1, L2, W::TH>(w, a + rank * G::COLS + cg, X, tw, P, clow, cg, ni, nip);
+  };
+  if (inv_small(P.q)) body(std::true_type{});
+  else body(std::false_type{});
+}
+template <int L1, int L2, int KIND>
+__global__ void __cluster_dims__(WholeGeo<L1, L2>::CS, 1, 1) __launch_bounds__(WholeGeo<L1, L2>::TH)
+    k_ntt_fwd_whole(Tables T, LimbSet S, NttAux A) {
+  using W = WholeGeo<L1, L2>;
+  using G = typename W::C;
+  using R = typename W::R;
+  extern __shared__ __align__(16) u64 sm[];
+  constexpr size_t N = (size_t)1 << (L1 + L2);
+  const int li = S.limb_begin + blockIdx.x / W::CS, rank = blockIdx.x % W::CS, part = blockIdx.y;
+  if (own_limb(A, part, li)) return;
+  cluster_arrive<W::CS>();  // the others run before their shared memory is written
+  const int pi = S.prime(li);
+  const PrimeDev P = T.pr[pi];
+  u64 *X = sm, *Y = sm + W::XWORDS;
+  ulonglong2* tw = reinterpret_cast<ulonglong2*>(Y + W::YWORDS);
+  const ulonglong2* src_tw = T.psi2 + (size_t)pi * tw_stride(L1, L2);
+  stage_twiddles<1 << L1, W::TH>(tw, src_tw, threadIdx.x);
+  stage_twiddles<(W::BLK << L2), W::TH>(tw + (1 << L1), src_tw + (1 << L1) + ((size_t)rank * W::BLK << L2), threadIdx.x);
+  cp_async_commit();
+  const int cg = threadIdx.x % G::COLS, clow = threadIdx.x / G::COLS;
+  const int low = threadIdx.x % R::M1, b = threadIdx.x / R::M1, blk = rank * W::BLK + b;  // row phase: block blk
+  const u64 bias = fwd_bias<L1 + L2>(P.q);
+  u64* a = S.limb(part, li, N);
+  // this thread's word of row clow; row m 2^K1 + clow is m N / M0 further
+  const size_t c0 = ((size_t)clow << L2) + rank * G::COLS + cg;
+  u64 v[1][G::M0];
+  if constexpr (KIND == LOAD_PLAIN) {
+    const u64* src = (A.src ? A.src + part * A.src_stride + (size_t)li * N : a) + c0;
+#pragma unroll
+    for (int m = 0; m < G::M0; ++m) v[0][m] = src[m * (N / G::M0)] + bias;
+  } else {
+    const int j = KIND == LOAD_MODUP ? part % A.own_dn : 0, lo = j * A.own_alpha;
+    const int ns = KIND == LOAD_MODUP ? min(A.own_alpha, A.own_limit - lo) : KIND == LOAD_MODDOWN ? A.pconv_K : 0;
+    const u64* base = (KIND == LOAD_MODUP     ? A.z + (size_t)(part / A.own_dn) * A.z_stride + (size_t)lo * N
+                       : KIND == LOAD_MODDOWN ? A.pconv + (size_t)part * A.pconv_stride
+                                              : A.spread) + c0;
+    const u64* last = KIND != LOAD_MODUP && A.spread ? A.spread + (size_t)part * A.spread_stride + c0 : nullptr;
+    FusedLoad<KIND> F;
+    F.init(A, T, P, bias, j, li, ns);
+    F.apply([&](auto word) {
+#pragma unroll
+      for (int m = 0; m < G::M0; ++m)
+        v[0][m] = word([&](int t) { return t < ns ? base[(size_t)t * N + m * (N / G::M0)] : last[m * (N / G::M0)]; });
+    });
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  auto body = [&](auto is_small) {
+    constexpr bool SMALL = decltype(is_small)::value;
+    u64 o[G::GP][1][G::M1];
+    fwd_cols_passes<SMALL, L1, W::TH>(v, X, tw, P.q, P.nqi, clow, cg, o);
+    cluster_wait<W::CS>();
+    const int col = rank * G::COLS + cg;
+#pragma unroll
+    for (int i = 0; i < G::GP; ++i)
+#pragma unroll
+      for (int m = 0; m < G::M1; ++m) {  // row c, this thread's column
+        const int c = (i * G::M1 + clow) * G::M1 + m;
+        u64* at = Y + (c % W::BLK) * R::BS + (col / R::M1) * R::GS + col % R::M1;
+        if constexpr (W::CS > 1) cluster_store(cluster_addr(at, c / W::BLK), o[i][0][m]);
+        else *at = o[i][0][m];
+      }
+    cluster_arrive<W::CS>();
+    cluster_wait<W::CS>();
+    if (b < W::BLK) {
+      u64* ys = Y + b * R::BS;
+      u64 w[1][R::M0];
+#pragma unroll
+      for (int m = 0; m < R::M0; ++m) w[0][m] = ys[m * R::GS + low];
+      __syncwarp();
+      fwd_rows_body<SMALL, L1, L2>(w, ys, tw + (1 << L1) + (b << L2), P, low);
+      fwd_rows_store<SMALL, L2>(ys, A, a + ((size_t)blk << L2), (size_t)li * N + ((size_t)blk << L2), part, li, P, low);
+    }
+  };
+  if (fwd_small(P.q)) body(std::true_type{});
+  else body(std::false_type{});
+}
+template <int L1, int L2>
+static bool launch_whole(const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse, const NttAux& A,
+                         const KskFuse* F) {
+  if constexpr (L1 + L2 <= 13) {
+    using W = WholeGeo<L1, L2>;
+    const int n_prod = A.z ? std::min(A.own_alpha, A.own_limit) : A.pconv ? A.pconv_K : 0;
+    if (F || !ntt_whole_limb(L1 + L2, (size_t)S.n_limbs * S.n_parts, n_prod)) return false;
+    static const bool attrs = [&] {
+      allow_smem(k_ntt_inv_whole<L1, L2>, W::SMEM);
+      allow_smem(k_ntt_fwd_whole<L1, L2, LOAD_PLAIN>, W::SMEM);
+      allow_smem(k_ntt_fwd_whole<L1, L2, LOAD_MODUP>, W::SMEM);
+      allow_smem(k_ntt_fwd_whole<L1, L2, LOAD_MODDOWN>, W::SMEM);
+      allow_smem(k_ntt_fwd_whole<L1, L2, LOAD_SPREAD>, W::SMEM);
+      return true;
+    }();
+    (void)attrs;
+    const dim3 g((unsigned)(S.n_limbs * W::CS), (unsigned)S.n_parts);
+    if (inverse) k_ntt_inv_whole<L1, L2><<<g, W::TH, W::SMEM, st>>>(T, S, A);
+    else if (A.z) k_ntt_fwd_whole<L1, L2, LOAD_MODUP><<<g, W::TH, W::SMEM, st>>>(T, S, A);
+    else if (A.pconv) k_ntt_fwd_whole<L1, L2, LOAD_MODDOWN><<<g, W::TH, W::SMEM, st>>>(T, S, A);
+    else if (A.spread) k_ntt_fwd_whole<L1, L2, LOAD_SPREAD><<<g, W::TH, W::SMEM, st>>>(T, S, A);
+    else k_ntt_fwd_whole<L1, L2, LOAD_PLAIN><<<g, W::TH, W::SMEM, st>>>(T, S, A);
+    HEDAP_LAUNCH_CHECK();
+    return true;
+  }
+  return false;
 }
 
 // ---------------------------------------------------------------- dispatch
@@ -1073,6 +1290,7 @@ static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool
 template <int L1, int L2>
 static void launch_variant(int v, const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse,
                            const NttAux& A, const KskFuse* F) {
+  if (launch_whole<L1, L2>(S, T, st, inverse, A, F)) return;
   if (v % kNttShapes == 0) launch_pair<L1, L2, 4, 16>(S, T, st, inverse, A, F);
   else launch_pair<L1, L2, 4, 20>(S, T, st, inverse, A, F);
 }
