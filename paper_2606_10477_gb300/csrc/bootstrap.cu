@@ -187,8 +187,9 @@ void BtsStateDeleter::operator()(BtsState* p) const { delete p; }
 // ------------------------------------------------------------------ kernels
 // ModRaise: from limb 0 in the coefficient domain (both parts, stride N) to every
 // limb 0..L of out: the centred representative of x mod q_0, reduced mod q_i.
-__global__ void k_mod_raise_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ x, u64* __restrict__ out,
+__global__ void k_mod_raise_kernel(const PrimeDev* __restrict__ pr, const u64* x, u64* out,
                                    size_t os, int n_parts, int limbs, int log_n) {
+  grid_wait();
   const size_t N = (size_t)1 << log_n, per = (size_t)limbs << log_n, total = n_parts * per;
   const u64 q0 = pr[0].q, h = q0 >> 1;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
@@ -205,8 +206,9 @@ __global__ void k_mod_raise_kernel(const PrimeDev* __restrict__ pr, const u64* _
 // multiply by X^(N/2) (factor iota_i) or X^(3N/2) (factor -iota_i), iota_i = psi_i^(N/2):
 // the evaluation at psi^(2 bitrev(j) + 1) picks up iota^(2 bitrev(j)+1) = iota (-1)^bitrev(j),
 // and bitrev(j) is odd exactly when j >= N/2.
-__global__ void k_monomial_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ in, size_t is,
-                                  u64* __restrict__ out, size_t os, int n_parts, int limbs, int log_n, LimbConsts F) {
+__global__ void k_monomial_kernel(const PrimeDev* __restrict__ pr, const u64* in, size_t is,
+                                  u64* out, size_t os, int n_parts, int limbs, int log_n, LimbConsts F) {
+  grid_wait();
   const size_t N = (size_t)1 << log_n, per = (size_t)limbs << log_n, total = n_parts * per;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     const int p = (int)(e / per);
@@ -245,6 +247,7 @@ struct PtMacArgs {
 };
 __global__ void __launch_bounds__(256) k_pt_mac_kernel(const PrimeDev* __restrict__ pr, const __grid_constant__ PtMacArgs A,
                                                        size_t stride, int n_parts, int log_n, int q_count, int p_first) {
+  grid_wait();
   const size_t N = (size_t)1 << log_n;
   const int li = blockIdx.y / A.giants, g = blockIdx.y % A.giants;
   const int i = li < q_count ? li : p_first + (li - q_count);
@@ -280,7 +283,7 @@ std::unique_ptr<Ct> mod_raise(Ctx& C, const Ct& a) {
   {
     ProfScope prof_(PROF_ELEMENTWISE, C.stream, (1.0 + (L + 1.0)) * P * N * 8);
     prof_count_launches(1);
-    k_mod_raise_kernel<<<grid_for((size_t)P * (L + 1) * N, 256), 256, 0, C.stream>>>(C.tab.pr, x.p, o->part(0),
+    launch(k_mod_raise_kernel, dim3(grid_for((size_t)P * (L + 1) * N, 256)), dim3(256), 0, C.stream, C.tab.pr, x.p, o->part(0),
                                                                                       o->part_stride(), P, L + 1,
                                                                                       C.log_n);
     HEDAP_LAUNCH_CHECK();
@@ -303,8 +306,7 @@ std::unique_ptr<Ct> mul_monomial(Ctx& C, const Ct& a, u64 e) {
   o->scale = a.scale;
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, 2.0 * a.parts() * (a.level + 1) * C.N * 8);
   prof_count_launches(1);
-  k_monomial_kernel<<<grid_for((size_t)a.parts() * (a.level + 1) * C.N, 256), 256, 0, C.stream>>>(
-      C.tab.pr, a.part(0), a.part_stride(), o->part(0), o->part_stride(), a.parts(), a.level + 1, C.log_n, F);
+  launch(k_monomial_kernel, dim3(grid_for((size_t)a.parts() * (a.level + 1) * C.N, 256)), dim3(256), 0, C.stream, C.tab.pr, a.part(0), a.part_stride(), o->part(0), o->part_stride(), a.parts(), a.level + 1, C.log_n, F);
   HEDAP_LAUNCH_CHECK();
   return o;
 }
@@ -420,7 +422,7 @@ static std::unique_ptr<Ct> lt_apply(Ctx& C, const Ct& v, const LTGroup& G, Plain
                       (terms + ((double)A.babies + A.giants) * v.parts()) * ext * C.N * 8);
       prof_count_launches(1);
       const dim3 grid((unsigned)(((C.N / 2 + 255) / 256) * v.parts()), (unsigned)(ext * A.giants));
-      k_pt_mac_kernel<<<grid, 256, 0, C.stream>>>(C.tab.pr, A, qp_stride, v.parts(), C.log_n, l + 1, C.n_q);
+      launch(k_pt_mac_kernel, dim3(grid), dim3(256), 0, C.stream, C.tab.pr, A, qp_stride, v.parts(), C.log_n, l + 1, C.n_q);
       HEDAP_LAUNCH_CHECK();
     }
     for (size_t i = 0; i < steps.size(); ++i) {

@@ -11,6 +11,7 @@
 #include <memory>
 #include <stdexcept>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "hedap.h"
@@ -470,6 +471,32 @@ hedap_status run_on_ctx(const hedap_ctx* ctx, const std::function<void()>& f);
 u64* noalloc_scratch_address(int device);
 
 // ------------------------------------------------------------------ launch helpers
+// Programmatic dependent launch: a kernel launched with launch() is set up while the kernel before it on the stream
+// still runs and starts as its last CTAs end, so that launch latencies drop out of a chain of kernels.  Such
+// a kernel calls grid_wait() before it touches anything that earlier work on the stream wrote or still reads: the
+// wait returns when all of that has finished and its writes are visible.  Only constants (prime tables,
+// twiddles) are read before it.  Data of earlier kernels is read with plain loads (no const __restrict__, no
+// __ldg): non-coherent loads could be taken before the wait.  No kernel lets its successor start earlier
+// (griddepcontrol.launch_dependents): waiting CTAs in the slots cost more than they hid.  HMult on the device,
+// with plain launches / early starts / this: N = 2^10 44 / 28 / 25 us, N = 2^12 (3 ciphertexts, 12 digits) 66 / 56 /
+// 45 us, N = 2^16 (one ciphertext, level 23) 383 / 363 / 357 us; forward of 384 limbs at N = 2^16 221 / 234 / 216 us.
+template <class... P, class... A>
+inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  HEDAP_CUDA(cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...));
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
 inline int grid_for(size_t work, int threads) {
   size_t g = (work + threads - 1) / threads;
   if (g > 152 * 32) g = 152 * 32;

@@ -20,9 +20,10 @@ __device__ __forceinline__ void st2(u64* p, ulonglong2 v) { *reinterpret_cast<ul
   for (size_t var = blockIdx.x * (size_t)blockDim.x + threadIdx.x; var < (total); var += (size_t)gridDim.x * blockDim.x)
 
 // ---------------------------------------------------------------- add / sub
-__global__ void k_add_sub_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ a, size_t as,
-                                 const u64* __restrict__ b, size_t bs, u64* __restrict__ o, size_t os, int n_parts,
+__global__ void k_add_sub_kernel(const PrimeDev* __restrict__ pr, const u64* a, size_t as,
+                                 const u64* b, size_t bs, u64* o, size_t os, int n_parts,
                                  int limbs, int log_n, int sub) {
+  grid_wait();
   const size_t per_part = (size_t)limbs << log_n;
   GRID_LOOP(t, n_parts * per_part / 2) {
     const size_t e = 2 * t;
@@ -39,15 +40,16 @@ void k_add_sub(const Ctx& C, const u64* a, size_t as, const u64* b, size_t bs, u
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, 3.0 * n_parts * limbs * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * limbs * C.N / 2;
-  k_add_sub_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(C.tab.pr, a, as, b, bs, o, os, n_parts, limbs,
+  launch(k_add_sub_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, a, as, b, bs, o, os, n_parts, limbs,
                                                               C.log_n, sub);
   HEDAP_LAUNCH_CHECK();
 }
 
 // ---------------------------------------------------------------- part copies
 // `words` words of each of n_parts parts of a ciphertext (part strides ss, ds; whole limbs)
-__global__ void k_copy_parts_kernel(const u64* __restrict__ src, size_t ss, u64* __restrict__ dst, size_t ds,
+__global__ void k_copy_parts_kernel(const u64* src, size_t ss, u64* dst, size_t ds,
                                     int n_parts, size_t words) {
+  grid_wait();
   const size_t pairs = words / 2;
   GRID_LOOP(t, n_parts * pairs) {
     const size_t p = t / pairs, r = 2 * (t - p * pairs);
@@ -63,7 +65,7 @@ void k_copy_parts(const Ctx& C, const u64* src, size_t ss, u64* dst, size_t ds, 
   }
   prof_count_launches(1);
   const size_t work = n_parts * words / 2;
-  k_copy_parts_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(src, ss, dst, ds, n_parts, words);
+  launch(k_copy_parts_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, src, ss, dst, ds, n_parts, words);
   HEDAP_LAUNCH_CHECK();
 }
 
@@ -93,9 +95,10 @@ void k_check_residues(const Ctx& C, const u64* a, size_t as, int n_parts, int li
 // ---------------------------------------------------------------- tensor product
 // ciphertext k: (a_2k, a_2k+1) x (b_2k, b_2k+1) -> d0 = o_2k, d1 = o_2k+1, d2 at d2 + k*limbs*N.  Three Montgomery
 // reductions a coefficient instead of four Barrett ones: 148 -> 118 us for 8 ciphertexts of 24 limbs, N = 2^16.
-__global__ void k_tensor_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ a, size_t as,
-                                const u64* __restrict__ b, size_t bs, u64* __restrict__ o, size_t os,
-                                u64* __restrict__ d2, int batch, int limbs, int log_n) {
+__global__ void k_tensor_kernel(const PrimeDev* __restrict__ pr, const u64* a, size_t as,
+                                const u64* b, size_t bs, u64* o, size_t os,
+                                u64* d2, int batch, int limbs, int log_n) {
+  grid_wait();
   const size_t per = (size_t)limbs << log_n;
   GRID_LOOP(t, batch * per / 2) {
     const size_t e = 2 * t;
@@ -124,15 +127,16 @@ void k_tensor(const Ctx& C, const u64* a, size_t as, const u64* b, size_t bs, u6
   ProfScope prof_(PROF_TENSOR, C.stream, 7.0 * batch * limbs * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)batch * limbs * C.N / 2;
-  k_tensor_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(C.tab.pr, a, as, b, bs, o, os, d2, batch, limbs,
+  launch(k_tensor_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, a, as, b, bs, o, os, d2, batch, limbs,
                                                              C.log_n);
   HEDAP_LAUNCH_CHECK();
 }
 
 // ---------------------------------------------------------------- per-limb constants
-__global__ void k_mul_limbconst_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ in, size_t is,
-                                       u64* __restrict__ out, size_t os, int n_parts, int limbs, int log_n,
+__global__ void k_mul_limbconst_kernel(const PrimeDev* __restrict__ pr, const u64* in, size_t is,
+                                       u64* out, size_t os, int n_parts, int limbs, int log_n,
                                        LimbConsts K) {
+  grid_wait();
   const size_t per_part = (size_t)limbs << log_n;
   GRID_LOOP(t, n_parts * per_part / 2) {
     const size_t e = 2 * t;
@@ -150,7 +154,7 @@ void k_mul_limbconst(const Ctx& C, const u64* in, size_t is, u64* out, size_t os
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, 2.0 * n_parts * limbs * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * limbs * C.N / 2;
-  k_mul_limbconst_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(C.tab.pr, in, is, out, os, n_parts, limbs,
+  launch(k_mul_limbconst_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, in, is, out, os, n_parts, limbs,
                                                                    C.log_n, K);
   HEDAP_LAUNCH_CHECK();
 }
@@ -158,8 +162,9 @@ void k_mul_limbconst(const Ctx& C, const u64* in, size_t is, u64* out, size_t os
 // out = sum_j in_j * w_j (+ c0 on the even parts, the c0 of each batch member) over limbs 0..limbs-1:
 // the leaf sum of a Chebyshev evaluation in one pass (inputs read at their own part strides, so
 // ciphertexts above the output level are read without a copy)
-__global__ void k_lincomb_kernel(const PrimeDev* __restrict__ pr, u64* __restrict__ out, size_t os, int n_parts,
+__global__ void k_lincomb_kernel(const PrimeDev* __restrict__ pr, u64* out, size_t os, int n_parts,
                                  int limbs, int log_n, LinCombArgs A) {
+  grid_wait();
   const size_t per_part = (size_t)limbs << log_n;
   GRID_LOOP(t, n_parts * per_part / 2) {
     const size_t e = 2 * t;
@@ -183,14 +188,15 @@ void k_lincomb(const Ctx& C, u64* out, size_t os, int n_parts, int limbs, const 
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, (A.count + 1.0 + A.accumulate) * n_parts * limbs * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * limbs * C.N / 2;
-  k_lincomb_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(C.tab.pr, out, os, n_parts, limbs, C.log_n, A);
+  launch(k_lincomb_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, out, os, n_parts, limbs, C.log_n, A);
   HEDAP_LAUNCH_CHECK();
 }
 
 // out = in, plus a per-limb constant on the even parts (the c0 of each batch member)
-__global__ void k_add_limbconst_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ in, size_t is,
-                                       u64* __restrict__ out, size_t os, int n_parts, int limbs, int log_n,
+__global__ void k_add_limbconst_kernel(const PrimeDev* __restrict__ pr, const u64* in, size_t is,
+                                       u64* out, size_t os, int n_parts, int limbs, int log_n,
                                        LimbConsts K) {
+  grid_wait();
   const size_t per_part = (size_t)limbs << log_n;
   GRID_LOOP(t, n_parts * per_part / 2) {
     const size_t e = 2 * t;
@@ -210,12 +216,13 @@ void k_add_limbconst(const Ctx& C, const u64* in, size_t is, u64* out, size_t os
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, 2.0 * n_parts * limbs * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * limbs * C.N / 2;
-  k_add_limbconst_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(C.tab.pr, in, is, out, os, n_parts, limbs, C.log_n,
+  launch(k_add_limbconst_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, in, is, out, os, n_parts, limbs, C.log_n,
                                                                    K);
   HEDAP_LAUNCH_CHECK();
 }
 // K's words to device memory: w [n], then wsh [n]
-__global__ void k_put_limbconst_kernel(u64* __restrict__ out, int n, const __grid_constant__ LimbConsts K) {
+__global__ void k_put_limbconst_kernel(u64* out, int n, const __grid_constant__ LimbConsts K) {
+  grid_wait();
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     out[i] = K.w[i];
     out[n + i] = K.wsh[i];
@@ -224,7 +231,7 @@ __global__ void k_put_limbconst_kernel(u64* __restrict__ out, int n, const __gri
 void k_put_limbconst(const Ctx& C, u64* out, int n, const LimbConsts& K) {
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, 16.0 * n);
   prof_count_launches(1);
-  k_put_limbconst_kernel<<<1, 64, 0, C.stream>>>(out, n, K);
+  launch(k_put_limbconst_kernel, dim3(1), dim3(64), 0, C.stream, out, n, K);
   HEDAP_LAUNCH_CHECK();
 }
 
@@ -259,8 +266,9 @@ void k_rescale_spread(const Ctx& C, const u64* last, size_t ls, u64* tmp, size_t
 // ---------------------------------------------------------------- ModDown fused with a rescale: the last limb
 // x = t - (off + sum_k [z_k + c_k]_{p_k} f_k) mod q_l, t limb l of part p (coefficient domain, part stride zs) and z_k
 // the K limbs after it: the K canonical products and off sum below (K + 1) q_l <= 9 q_l < 2^64, reduced once
-__global__ void k_mdr_last_coef_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ t, size_t zs,
-                                       u64* __restrict__ x, int n_parts, int log_n, int l, MdrLast M) {
+__global__ void k_mdr_last_coef_kernel(const PrimeDev* __restrict__ pr, const u64* t, size_t zs,
+                                       u64* x, int n_parts, int log_n, int l, MdrLast M) {
+  grid_wait();
   const size_t N = (size_t)1 << log_n;
   const PrimeDev P = pr[l];
   GRID_LOOP(i, (size_t)n_parts * N) {
@@ -277,7 +285,7 @@ void k_mdr_last_coef(const Ctx& C, const u64* t, size_t zs, u64* x, int n_parts,
   ProfScope prof_(PROF_RESCALE, C.stream, (2.0 + M.K) * n_parts * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * C.N;
-  k_mdr_last_coef_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(C.tab.pr, t, zs, x, n_parts, C.log_n, l, M);
+  launch(k_mdr_last_coef_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, t, zs, x, n_parts, C.log_n, l, M);
   HEDAP_LAUNCH_CHECK();
 }
 
@@ -309,8 +317,9 @@ void k_rescale_finish(const Ctx& C, const u64* in, size_t is, const u64* tmp, si
 // ---------------------------------------------------------------- automorphism (NTT domain)
 // evaluation j sits at psi^(2 bitrev(j) + 1); X -> X^g maps it to the evaluation at
 // psi^(g (2 bitrev(j) + 1)), i.e. input index bitrev(((g e_j mod 2N) - 1) / 2).
-__global__ void k_automorph_kernel(const u64* __restrict__ in, size_t is, u64* __restrict__ out, size_t os,
+__global__ void k_automorph_kernel(const u64* in, size_t is, u64* out, size_t os,
                                    int n_parts, int limbs, int log_n, u64 g) {
+  grid_wait();
   const size_t N = (size_t)1 << log_n, per_part = (size_t)limbs << log_n;
   const u64 mask2n = 2 * N - 1;
   GRID_LOOP(e, n_parts * per_part) {
@@ -327,7 +336,7 @@ void k_automorph(const Ctx& C, const u64* in, size_t is, u64* out, size_t os, in
   ProfScope prof_(PROF_AUTOMORPH, C.stream, 2.0 * n_parts * limbs * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * limbs * C.N;
-  k_automorph_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(in, is, out, os, n_parts, limbs, C.log_n, g);
+  launch(k_automorph_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, in, is, out, os, n_parts, limbs, C.log_n, g);
   HEDAP_LAUNCH_CHECK();
 }
 
@@ -403,11 +412,12 @@ __device__ __forceinline__ uint32_t galois_index(uint32_t n, u64 g, int log_n) {
   return __brev((uint32_t)((eg - 1) >> 1)) >> (32 - log_n);
 }
 __device__ __forceinline__ ulonglong2 ld2_stream(const u64* p) { return __ldcs(reinterpret_cast<const ulonglong2*>(p)); }
-__global__ void __launch_bounds__(512, 2) k_ksk_inner_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ y,
-                                                             const u64* __restrict__ d, size_t ds, KskInnerArgs A,
+__global__ void __launch_bounds__(512, 2) k_ksk_inner_kernel(const PrimeDev* __restrict__ pr, const u64* y,
+                                                             const u64* d, size_t ds, KskInnerArgs A,
                                                              int l, int dn, int alpha, int n_q, int K, int log_n,
-                                                             const u64* __restrict__ c0, size_t c0s,
+                                                             const u64* c0, size_t c0s,
                                                              const u64* __restrict__ pmod) {
+  grid_wait();
   const size_t N = (size_t)1 << log_n;
   const int ext = l + 1 + K, total_primes = n_q + K;
   const int t = blockIdx.y / A.count, rot = blockIdx.y % A.count, k = threadIdx.y;
@@ -449,15 +459,16 @@ void k_ksk_inner(const Ctx& C, const u64* y, const u64* d, size_t d_stride, cons
   prof_count_launches(1);
   const unsigned tx = 32u * (unsigned)std::max(1, 8 / batch);  // about 256 threads per CTA
   const dim3 block(tx, (unsigned)batch), grid((unsigned)(C.N / 2 / tx), (unsigned)(ext * A.count));
-  k_ksk_inner_kernel<<<grid, block, 0, C.stream>>>(C.tab.pr, y, d, d_stride, A, level, dn, C.alpha, C.n_q, C.n_p,
+  launch(k_ksk_inner_kernel, dim3(grid), dim3(block), 0, C.stream, C.tab.pr, y, d, d_stride, A, level, dn, C.alpha, C.n_q, C.n_p,
                                                    C.log_n, c0, c0_stride, C.d_pmod.p);
   HEDAP_LAUNCH_CHECK();
 }
 
 // a batch over Q_l u P: (P c0, P c1) on the Q limbs (P mod q_i by Barrett), 0 on the special limbs
 __global__ void k_lift_qp_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ pmod,
-                                 const u64* __restrict__ in, size_t is, u64* __restrict__ out, int n_parts, int l,
+                                 const u64* in, size_t is, u64* out, int n_parts, int l,
                                  int ext, int log_n) {
+  grid_wait();
   const size_t per = (size_t)ext << log_n;
   GRID_LOOP(e, (size_t)n_parts * per) {
     const size_t p = e / per, r = e - p * per;
@@ -470,7 +481,7 @@ void k_lift_qp(const Ctx& C, const u64* in, size_t is, u64* out, int n_parts, in
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, (double)n_parts * (level + 1 + ext) * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * ext * C.N;
-  k_lift_qp_kernel<<<grid_for(work, 256), 256, 0, C.stream>>>(C.tab.pr, C.d_pmod.p, in, is, out, n_parts, level,
+  launch(k_lift_qp_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, C.d_pmod.p, in, is, out, n_parts, level,
                                                                 ext, C.log_n);
   HEDAP_LAUNCH_CHECK();
 }

@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols(Tables T, LimbSet S, 
   constexpr size_t N = (size_t)1 << (L1 + L2);
   const int cg = threadIdx.x % G::COLS, low = threadIdx.x / G::COLS;
   const int y = blockIdx.y, part = y / S.n_limbs, li = S.limb_begin + y % S.n_limbs;
-  if (own_limb(A, part, li)) return;
+  if (own_limb(A, part, li)) return grid_wait();
   const int pi = S.prime(li);
   const PrimeDev P = T.pr[pi];
   const size_t col = (size_t)blockIdx.x * G::COLS + cg;
@@ -348,6 +348,7 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols(Tables T, LimbSet S, 
   stage_twiddles<1 << L1, TH>(tw, T.psi2 + (size_t)pi * tw_stride(L1, L2), threadIdx.x);
   cp_async_commit();
   const u64 bias = fwd_bias<L1 + L2>(P.q);
+  grid_wait();
   u64 v[1][G::M0];
 #pragma unroll
   for (int m = 0; m < G::M0; ++m) v[0][m] = src[(size_t)(m * G::M1 + low) << L2] + bias;
@@ -382,6 +383,7 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_shared(Tables T, Limb
                                            : nullptr;
   const u64* last = KIND != LOAD_MODUP && A.spread ? A.spread + (size_t)part * A.spread_stride : nullptr;
   const int tiles = ns + (last ? 1 : 0);
+  grid_wait();
   for (int i = threadIdx.x; i < tiles * (G::TILE / 2); i += TH) {
     const int t = i / (G::TILE / 2), e = 2 * (i % (G::TILE / 2)), row = e / G::COLS;
     const u64* src = t < ns ? base + (size_t)t * N : last;
@@ -419,6 +421,7 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_wide(Tables T, LimbSe
   constexpr size_t N = (size_t)1 << (L1 + L2);
   const int cg = threadIdx.x % G::COLS, low = threadIdx.x / G::COLS;
   const int part = blockIdx.y / S.n_limbs, li = S.limb_begin + blockIdx.y % S.n_limbs;
+  grid_wait();
   if (own_limb(A, part, li)) return;
   const int pi = S.prime(li);
   const PrimeDev P = T.pr[pi];
@@ -612,6 +615,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_fwd_rows(Tables T, LimbSet
   cp_async_commit();
   tw += b << L2;
   const size_t j0 = (size_t)blk << L2, at = (size_t)li * N + j0;
+  grid_wait();
   bool staged = false;
   for (int part = pg * ppc; part < min((pg + 1) * ppc, S.n_parts); ++part) {
     if (own_limb(A, part, li)) continue;
@@ -766,6 +770,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_fwd_rows_ksk(Tables T, Lim
 #pragma unroll
     for (int i = 0; i < G::PER / 2; ++i) cp_async16(dst + G::run_word(64 * i), src + i * 64);
   };
+  grid_wait();
   if (live && j_first < dn) fetch(j_first, bufs);
   cp_async_commit();
   Acc128 ab[G::PER], aa[G::PER];
@@ -915,6 +920,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_inv_rows(Tables T, LimbSet
                                      lane);
   tw += b << L2;
   const size_t j0 = (size_t)blk << L2;
+  grid_wait();
   for (int part = pg * ppc; part < min((pg + 1) * ppc, S.n_parts); ++part) {
     if (own_limb(A, part, li)) continue;
     u64* a = S.limb(part, li, N) + j0;
@@ -967,13 +973,14 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_inv_cols(Tables T, LimbSet S, 
   constexpr size_t N = (size_t)1 << (L1 + L2);
   const int cg = threadIdx.x % G::COLS, low = threadIdx.x / G::COLS;
   const int y = blockIdx.y, part = y / S.n_limbs, li = S.limb_begin + y % S.n_limbs;
-  if (own_limb(A, part, li)) return;
+  if (own_limb(A, part, li)) return grid_wait();
   const int pi = S.prime(li);
   const PrimeDev P = T.pr[pi];
   u64* a = S.limb(part, li, N) + (size_t)blockIdx.x * G::COLS + cg;
   ulonglong2* tw = reinterpret_cast<ulonglong2*>(sm + G::XWORDS);
   stage_twiddles<1 << L1, TH>(tw, T.ipsi2 + (size_t)pi * tw_stride(L1, L2), threadIdx.x);
   cp_async_commit();
+  grid_wait();
   u64 w[G::GP][1][G::M1];
 #pragma unroll
   for (int i = 0; i < G::GP; ++i)
@@ -1033,7 +1040,7 @@ __global__ void __cluster_dims__(WholeGeo<L1, L2>::CS, 1, 1) __launch_bounds__(W
   extern __shared__ __align__(16) u64 sm[];
   constexpr size_t N = (size_t)1 << (L1 + L2);
   const int li = S.limb_begin + blockIdx.x / W::CS, rank = blockIdx.x % W::CS, part = blockIdx.y;
-  if (own_limb(A, part, li)) return;
+  if (own_limb(A, part, li)) return grid_wait();
   cluster_arrive<W::CS>();  // the others run before their shared memory is written
   const int pi = S.prime(li);
   const PrimeDev P = T.pr[pi];
@@ -1048,6 +1055,7 @@ __global__ void __cluster_dims__(WholeGeo<L1, L2>::CS, 1, 1) __launch_bounds__(W
   const int cg = threadIdx.x % G::COLS, clow = threadIdx.x / G::COLS;
   const bool row = b < W::BLK;
   u64* ys = Y + b * R::BS;
+  grid_wait();
   if (row) inv_rows_load<L2>(A, S, part, li, src + ((size_t)blk << L2), ys, (size_t)blk << L2, P, low);
   cp_async_commit();
   const int r = li - S.limb_begin;
@@ -1090,7 +1098,7 @@ __global__ void __cluster_dims__(WholeGeo<L1, L2>::CS, 1, 1) __launch_bounds__(W
   extern __shared__ __align__(16) u64 sm[];
   constexpr size_t N = (size_t)1 << (L1 + L2);
   const int li = S.limb_begin + blockIdx.x / W::CS, rank = blockIdx.x % W::CS, part = blockIdx.y;
-  if (own_limb(A, part, li)) return;
+  if (own_limb(A, part, li)) return grid_wait();
   cluster_arrive<W::CS>();  // the others run before their shared memory is written
   const int pi = S.prime(li);
   const PrimeDev P = T.pr[pi];
@@ -1106,6 +1114,7 @@ __global__ void __cluster_dims__(WholeGeo<L1, L2>::CS, 1, 1) __launch_bounds__(W
   u64* a = S.limb(part, li, N);
   // this thread's word of row clow; row m 2^K1 + clow is m N / M0 further
   const size_t c0 = ((size_t)clow << L2) + rank * G::COLS + cg;
+  grid_wait();
   u64 v[1][G::M0];
   if constexpr (KIND == LOAD_PLAIN) {
     const u64* src = (A.src ? A.src + part * A.src_stride + (size_t)li * N : a) + c0;
@@ -1175,11 +1184,11 @@ static bool launch_whole(const LimbSet& S, const Tables& T, cudaStream_t st, boo
     }();
     (void)attrs;
     const dim3 g((unsigned)(S.n_limbs * W::CS), (unsigned)S.n_parts);
-    if (inverse) k_ntt_inv_whole<L1, L2><<<g, W::TH, W::SMEM, st>>>(T, S, A);
-    else if (A.z) k_ntt_fwd_whole<L1, L2, LOAD_MODUP><<<g, W::TH, W::SMEM, st>>>(T, S, A);
-    else if (A.pconv) k_ntt_fwd_whole<L1, L2, LOAD_MODDOWN><<<g, W::TH, W::SMEM, st>>>(T, S, A);
-    else if (A.spread) k_ntt_fwd_whole<L1, L2, LOAD_SPREAD><<<g, W::TH, W::SMEM, st>>>(T, S, A);
-    else k_ntt_fwd_whole<L1, L2, LOAD_PLAIN><<<g, W::TH, W::SMEM, st>>>(T, S, A);
+    if (inverse) launch(k_ntt_inv_whole<L1, L2>, g, dim3(W::TH), W::SMEM, st, T, S, A);
+    else if (A.z) launch(k_ntt_fwd_whole<L1, L2, LOAD_MODUP>, g, dim3(W::TH), W::SMEM, st, T, S, A);
+    else if (A.pconv) launch(k_ntt_fwd_whole<L1, L2, LOAD_MODDOWN>, g, dim3(W::TH), W::SMEM, st, T, S, A);
+    else if (A.spread) launch(k_ntt_fwd_whole<L1, L2, LOAD_SPREAD>, g, dim3(W::TH), W::SMEM, st, T, S, A);
+    else launch(k_ntt_fwd_whole<L1, L2, LOAD_PLAIN>, g, dim3(W::TH), W::SMEM, st, T, S, A);
     HEDAP_LAUNCH_CHECK();
     return true;
   }
@@ -1198,6 +1207,22 @@ static void allow_smem(Kernel kern, size_t bytes) {
 // 1195 us of the 128-thread CTAs with three barriers a digit
 constexpr int kKskWarps = 4, kKskMinBlocks = 3;
 
+// Output limbs per CTA of the shared-tile column phase: the number that minimises waves x (limbs + 0.3), the 0.3 limb
+// being the staging of the tiles; `ctas` CTAs per group of limbs, `slots` resident at a time.  One ciphertext at
+// level 23 (N = 2^16): 9 limbs a CTA, 1.9 waves, where a fixed target of four waves gave 4 limbs and 4.4 waves.
+inline int limbs_per_cta(size_t ctas, int limbs, size_t slots) {
+  int best = 1;
+  double best_cost = 1e300;
+  for (int n = 1; n <= limbs; ++n) {
+    const size_t all = ctas * (size_t)((limbs + n - 1) / n);
+    const double cost = (double)((all + slots - 1) / slots) * (n + 0.3);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = n;
+    }
+  }
+  return best;
+}
 template <int L1, int L2, int WW, int WPS>
 static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse, const NttAux& A,
                         const KskFuse* F) {
@@ -1227,14 +1252,9 @@ static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool
     const int n_prod = A.z ? std::min(A.own_alpha, A.own_limit) : A.pconv ? A.pconv_K : 0;
     const int nt = n_prod + (!A.z && A.spread ? 1 : 0);
     if (nt >= 1 && n_prod <= 3 && !A.src) {
-      // several output limbs per CTA, sharing the staged tiles: enough limb groups for about
-      // four waves of 16 warps on 152 SMs, at most all the limbs in one group
-      const size_t per_group = (size_t)gc.x * TH / 32 * S.n_parts;
-      const size_t want = (size_t)152 * 16 * 4;
-      const int groups = (int)std::min<size_t>(S.n_limbs, std::max<size_t>(1, (want + per_group - 1) / per_group));
-      const int lpc = (S.n_limbs + groups - 1) / groups;
-      const dim3 g2(gc.x, (unsigned)(S.n_parts * ((S.n_limbs + lpc - 1) / lpc)));
       const size_t smem = smem_x + (size_t)nt * CG::TILE * 8;
+      const int lpc = limbs_per_cta((size_t)gc.x * S.n_parts, S.n_limbs, 152 * std::min<size_t>(CB, 232448 / (smem + 1024)));
+      const dim3 g2(gc.x, (unsigned)(S.n_parts * ((S.n_limbs + lpc - 1) / lpc)));
       constexpr size_t smem_max = smem_x + (size_t)4 * CG::TILE * 8;
       static const bool attrs = [&] {
         allow_smem(k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_MODUP>, smem_max);
@@ -1243,15 +1263,15 @@ static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool
         return true;
       }();
       (void)attrs;
-      if (A.z) k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_MODUP><<<g2, TH, smem, st>>>(T, S, A, lpc);
-      else if (A.pconv) k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_MODDOWN><<<g2, TH, smem, st>>>(T, S, A, lpc);
-      else k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_SPREAD><<<g2, TH, smem, st>>>(T, S, A, lpc);
+      if (A.z) launch(k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_MODUP>, g2, dim3(TH), smem, st, T, S, A, lpc);
+      else if (A.pconv) launch(k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_MODDOWN>, g2, dim3(TH), smem, st, T, S, A, lpc);
+      else launch(k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_SPREAD>, g2, dim3(TH), smem, st, T, S, A, lpc);
     } else if (n_prod > 3) {
       constexpr int WB = std::max(1, 12 * 32 / TH);
-      if (A.z) k_ntt_fwd_cols_wide<L1, L2, TH, WB, LOAD_MODUP><<<gc, TH, smem_x, st>>>(T, S, A);
-      else k_ntt_fwd_cols_wide<L1, L2, TH, WB, LOAD_MODDOWN><<<gc, TH, smem_x, st>>>(T, S, A);
+      if (A.z) launch(k_ntt_fwd_cols_wide<L1, L2, TH, WB, LOAD_MODUP>, gc, dim3(TH), smem_x, st, T, S, A);
+      else launch(k_ntt_fwd_cols_wide<L1, L2, TH, WB, LOAD_MODDOWN>, gc, dim3(TH), smem_x, st, T, S, A);
     } else {
-      k_ntt_fwd_cols<L1, L2, TH, CB><<<gc, TH, smem_c, st>>>(T, S, A);
+      launch(k_ntt_fwd_cols<L1, L2, TH, CB>, gc, dim3(TH), smem_c, st, T, S, A);
     }
     if (F) {
       using KG = KskGeo<L2>;
@@ -1266,14 +1286,14 @@ static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool
       }();
       (void)attr_k;
       const dim3 gk((unsigned)((tasks + kKskWarps - 1) / kKskWarps), (unsigned)S.n_limbs);
-      k_ntt_fwd_rows_ksk<L1, L2, kKskWarps, kKskMinBlocks><<<gk, 32 * kKskWarps, smem, st>>>(T, S, A2, *F, nstage);
+      launch(k_ntt_fwd_rows_ksk<L1, L2, kKskWarps, kKskMinBlocks>, gk, dim3(32 * kKskWarps), smem, st, T, S, A2, *F, nstage);
     } else {
       static const bool attrs = [&] {
         allow_smem(k_ntt_fwd_rows<L1, L2, RW, RB>, smem_r);
         return true;
       }();
       (void)attrs;
-      k_ntt_fwd_rows<L1, L2, RW, RB><<<gr, 32 * RW, smem_r, st>>>(T, S, A2, ppc);
+      launch(k_ntt_fwd_rows<L1, L2, RW, RB>, gr, dim3(32 * RW), smem_r, st, T, S, A2, ppc);
     }
   } else {
     static const bool attrs = [&] {
@@ -1281,8 +1301,8 @@ static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool
       return true;
     }();
     (void)attrs;
-    k_ntt_inv_rows<L1, L2, RW, RB><<<gr, 32 * RW, smem_r, st>>>(T, S, A, ppc);
-    k_ntt_inv_cols<L1, L2, TH, CB><<<gc, TH, smem_c, st>>>(T, S, A2);
+    launch(k_ntt_inv_rows<L1, L2, RW, RB>, gr, dim3(32 * RW), smem_r, st, T, S, A, ppc);
+    launch(k_ntt_inv_cols<L1, L2, TH, CB>, gc, dim3(TH), smem_c, st, T, S, A2);
   }
   HEDAP_LAUNCH_CHECK();
 }
