@@ -97,11 +97,10 @@ def measured_peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}, "fallback"
 
 
-# The NTT is bound by the integer multiply-add pipe (there is no 64-bit multiplier): a lazy Shoup
-# butterfly needs the exact high half of x * w' (seven 32 x 32 half products: the low half of x0 w'0 is
-# never needed) and the low halves of x * w and qh * q (two 32 x 32 -> 64 products, two slots each, and
-# four low products) = 15 multiply-pipe slots per butterfly, against 64 multiply-add lanes per SM.
-NTT_MUL_SLOTS_PER_BUTTERFLY = 15
+# The NTT is bound by the integer multiply-add pipe (there is no 64-bit multiplier): a butterfly's product by a
+# constant is four 32 x 32 -> 64 products (two slots each) and one Montgomery step by 2^32, a low product and
+# two wide ones = 13 multiply-pipe slots per butterfly, against 64 multiply-add lanes per SM.
+NTT_MUL_SLOTS_PER_BUTTERFLY = 13
 IMAD_LANES_PER_SM = 64
 # DRAM bytes per transformed limb: dram__bytes_read.sum + dram__bytes_write.sum of the transform launches of one
 # batched HMult with rescale at the top level (`--only hmult --batch 8 --profile-region` under ncu: 4553.6 MB for
@@ -112,10 +111,9 @@ NTT_DRAM_BYTES_PER_LIMB = 1.564e6
 
 def ntt_alu_roofline(n, alg_bytes, ms, groups, peaks, slots):
     """The transform class against the multiply pipe.  Work = the library's algorithmic count of 32-bit
-    multiply-pipe slots of the class (15 per Shoup product by a constant: every butterfly and every product of
-    a fused basis conversion; 8 per 64 x 64 -> 128-bit product of the fused key inner product); peak = SMs x 64
-    multiply-add lanes x clock.  The butterfly-only view (the transforms' butterflies against 15 slots each) is
-    kept beside it."""
+    multiply-pipe slots of the class (13 per butterfly; 8 per product and 5 per word of a fused basis conversion; 8
+    per 64 x 64 -> 128-bit product of the fused key inner product); peak = SMs x 64 multiply-add lanes x clock.
+    The butterfly-only view (the transforms' butterflies against 13 slots each) is kept beside it."""
     log_n = int(n).bit_length() - 1
     limbs = alg_bytes / (16.0 * n)
     bfly = limbs * (n // 2) * log_n
@@ -139,7 +137,7 @@ def ntt_alu_roofline(n, alg_bytes, ms, groups, peaks, slots):
             "butterfly_view": {"achieved_gbutterfly_s": bfly / sec / 1e9, "peak_gbutterfly_s": bfly_peak,
                                "frac": bfly / sec / 1e9 / bfly_peak,
                                "butterflies_per_group": bfly / max(1, groups),
-                               "peak_source": f"{NTT_MUL_SLOTS_PER_BUTTERFLY} multiply slots per Shoup butterfly"}}
+                               "peak_source": f"{NTT_MUL_SLOTS_PER_BUTTERFLY} multiply slots per butterfly"}}
 
 
 class ClockSampler:

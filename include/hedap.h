@@ -504,8 +504,8 @@ hedap_status hedap_graph_run_many(hedap_graph* g, const hedap_ct* const* in, siz
 hedap_status hedap_graph_kernels(const hedap_graph* g, uint64_t* n);
 void hedap_graph_destroy(hedap_graph* g);
 
-/* NTT autotuner: times every NTT launch shape (words staged per CTA, CTAs per
- * SM, radix 16 or 8 register passes) on `limbs` limbs of scratch, forward and inverse separately (best of
+/* NTT autotuner: times every NTT launch shape (warps an SM must have registers
+ * for; variants of equal parity are one shape) on `limbs` limbs of scratch, forward and inverse separately (best of
  * `reps`), and makes the fastest the context's shape.  Per-variant times go
  * to fwd_ms / inv_ms (capacity cap, may be NULL); the chosen variant indices
  * to *fwd_variant / *inv_variant.  The forward transforms with a fused key-switch
@@ -549,9 +549,9 @@ hedap_status hedap_ntt_get_role_variant(const hedap_ctx* ctx, int role, int* var
 hedap_status hedap_profile_enable(int on);
 hedap_status hedap_profile_read(const char* kernel_class, uint64_t* groups, double* ms, double* bytes);
 /* The class's algorithmic multiply work over the same groups, in 32-bit
- * multiply-pipe slots (kept for "ntt": 16 per Shoup product by a constant --
- * every butterfly and every term of a fused basis conversion -- and 8 per
- * 64 x 64 -> 128-bit product of the fused key inner product). */
+ * multiply-pipe slots (kept for "ntt": 13 per butterfly; 8 per product and 5 per
+ * word of a fused basis conversion; 8 per 64 x 64 -> 128-bit product of the fused
+ * key inner product). */
 hedap_status hedap_profile_read_slots(const char* kernel_class, double* slots);
 hedap_status hedap_launch_count(uint64_t* out);
 

@@ -156,8 +156,8 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
     md2.push_back(h_shoup(w, pk));
   }
   C->mdr_post = md2;
+  md2.push_back(0);  // the rounding constants of limb l and the special limbs of a fused rescale start here
   for (int k = 0; k < K; ++k) md2.push_back(h_mulmod(halfP_mod(p_of(k)), phinv[k], p_of(k)));
-  for (int k = 0; k < K; ++k) md2.push_back(p_of(k));
   for (int word = 0; word < 2; ++word)
     for (int k = 0; k < K; ++k)
       for (int i = 0; i < nq; ++i) {

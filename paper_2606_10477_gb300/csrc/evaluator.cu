@@ -195,13 +195,6 @@ const LevelConsts& level_consts(Ctx& C, int l) {
     const u64 pinv = h_invmod(P_mod(ql), ql);
     for (int k = 0; k < M.K; ++k) {
       const u64 pk = q[C.n_q + k];
-      u64 h = 1;  // phinv_k = (P / p_k)^-1 mod p_k
-      for (int m = 0; m < K; ++m)
-        if (m != k) h = h_mulmod(h, q[C.n_q + m] % pk, pk);
-      const u64 phinv = h_invmod(h, pk);
-      const u64 halfp = h_mulmod((P_mod(pk) + pk - 1) % pk, h_invmod(2, pk), pk);  // floor(P/2) mod p_k
-      M.p[k] = pk;
-      M.c[k] = h_mulmod(halfp, phinv, pk);
       M.f[k] = h_invmod(pk % ql, ql);
       M.fs[k] = h_shoup(M.f[k], ql);
     }
@@ -269,8 +262,9 @@ static const DevBuf& key_for(Ctx& C, u64 galois) {
 }
 // iNTT of the P limbs of the key-switch sums acc [batch][2][ext][N], ModDown, NTT, written to / added
 // into out
-static void ks_moddown(Ctx& C, const DevBuf& acc, int batch, int l, u64* out, size_t out_stride, bool acc0,
-                       bool acc1) {
+// with c0 (part stride c0_stride): the even parts gain sigma_g(c0), gathered by the finishing store
+static void ks_moddown(Ctx& C, const DevBuf& acc, int batch, int l, u64* out, size_t out_stride, bool acc0, bool acc1,
+                       const u64* c0 = nullptr, size_t c0_stride = 0, u64 g = 0) {
   const size_t N = C.N, nl = (size_t)l + 1;
   const int K = C.n_p, ext = l + 1 + K;
   // ModDown: the special-prime limbs to the coefficient domain (ending with N^-1 phinv_k when the
@@ -278,21 +272,22 @@ static void ks_moddown(Ctx& C, const DevBuf& acc, int batch, int l, u64* out, si
   // (acc - v) P^-1 (+ out) fused into its store
   const bool fuse = K <= 8;
   NttAux inv{};
-  if (fuse) inv.post = C.d_moddown2.p;
+  if (fuse) {
+    inv.post = C.d_moddown2.p;
+    inv.post_add = C.d_moddown2.p + 2 * K + 1;
+  }
   ntt_inverse(C.tab, LimbSet{acc.p, (size_t)ext * N, 2 * batch, l + 1, K, l + 1, 0, C.n_q}, C.stream, &inv);
   DevBuf v((size_t)batch * 2 * nl * N, C.stream);
   if (!fuse) k_moddown_spread(C, acc.p, v.p, 2 * batch, l);
-  const u64* Pinv = C.d_moddown2.p + 4 * K + 2 * (size_t)K * C.n_q;
+  const u64* Pinv = C.d_moddown2.p + 3 * K + 1 + 2 * (size_t)K * C.n_q;
   NttAux fw{};
   if (fuse) {
     fw.pconv = acc.p + nl * N;
     fw.pconv_stride = (size_t)ext * N;
     fw.pconv_K = K;
     fw.pconv_ld = C.n_q;
-    fw.pconv_q = C.d_moddown2.p + 3 * K;
-    fw.pconv_c = C.d_moddown2.p + 2 * K;
-    fw.pconv_phat = C.d_moddown2.p + 4 * K;
-    fw.pconv_phat_b = C.d_moddown2.p + 4 * K + (size_t)K * C.n_q;
+    fw.pconv_phat = C.d_moddown2.p + 3 * K + 1;
+    fw.pconv_phat_b = C.d_moddown2.p + 3 * K + 1 + (size_t)K * C.n_q;
     fw.pconv_half = C.d_moddown.p + 3 * K + (size_t)K * C.n_q + 2 * (size_t)C.n_q;
   }
   fw.fin_dst = out;
@@ -303,6 +298,9 @@ static void ks_moddown(Ctx& C, const DevBuf& acc, int batch, int l, u64* out, si
   fw.fin_wb = Pinv + C.n_q;
   fw.fin_acc_even = acc0 ? 1 : 0;
   fw.fin_acc_odd = acc1 ? 1 : 0;
+  fw.fin_d = c0;
+  fw.fin_d_stride = c0_stride;
+  fw.fin_g = g;
   ntt_forward(C.tab, qset(v.p, nl * N, 2 * batch, 0, l + 1), C.stream, &fw);
 }
 
@@ -365,6 +363,7 @@ static void ks_moddown_rescale(Ctx& C, const DevBuf& acc, int batch, int l, cons
   // N^-1 phinv_k: one inverse transform of K + 1 limbs a part
   NttAux inv{};
   inv.post = LC.mdr_post.p;
+  inv.post_add = C.d_moddown2.p + 2 * K;  // 0 for limb l, c_k for the special limbs
   inv.pre_scale = 1;
   inv.pre_e = e + (size_t)l * N;
   inv.pre_e_stride = e_stride;
@@ -379,8 +378,6 @@ static void ks_moddown_rescale(Ctx& C, const DevBuf& acc, int batch, int l, cons
   fw.pconv_stride = (size_t)ext * N;
   fw.pconv_K = K;
   fw.pconv_ld = nq;
-  fw.pconv_q = C.d_moddown2.p + 3 * K;
-  fw.pconv_c = C.d_moddown2.p + 2 * K;
   fw.pconv_phat = C.d_mdr.p;
   fw.pconv_phat_b = C.d_mdr.p + (size_t)K * nq;
   fw.pconv_half = C.d_mdr.p + 2 * (size_t)K * nq;
@@ -438,8 +435,7 @@ std::vector<std::unique_ptr<Ct>> ev_galois_hoisted(Ctx& C, const Ct& a, const st
   hoisted_inner(C, a, y, gs, nullptr, chunk, [&](size_t i, DevBuf acc) {
     auto o = ct_alloc(C, l, a.batch);
     o->scale = a.scale;
-    k_automorph(C, a.part(0), 2 * a.part_stride(), o->part(0), 2 * o->part_stride(), a.batch, l + 1, gs[i]);
-    ks_moddown(C, acc, a.batch, l, o->part(0), o->part_stride(), true, false);
+    ks_moddown(C, acc, a.batch, l, o->part(0), o->part_stride(), true, false, a.part(0), a.part_stride(), gs[i]);
     out.push_back(std::move(o));
   });
   return out;
@@ -588,8 +584,12 @@ std::unique_ptr<Ct> ev_galois(Ctx& C, const Ct& a, u64 g) {
   const int l = a.level;
   auto o = ct_alloc(C, l, a.batch);
   o->scale = a.scale;
-  k_automorph(C, a.part(0), a.part_stride(), o->part(0), o->part_stride(), a.parts(), l + 1, g);
-  key_switch(C, o->part(1), 2 * o->part_stride(), a.batch, l, g, o->part(0), o->part_stride(), true, false);
+  // sigma_g(c1) is switched; sigma_g(c0) is gathered by the ModDown's finishing store
+  const size_t per = (size_t)(l + 1) * C.N;
+  DevBuf d(a.batch * per, C.stream);
+  k_automorph(C, a.part(1), 2 * a.part_stride(), d.p, per, a.batch, l + 1, g);
+  DevBuf acc = ks_inner(C, d.p, per, a.batch, l, g);
+  ks_moddown(C, acc, a.batch, l, o->part(0), o->part_stride(), true, false, a.part(0), a.part_stride(), g);
   return o;
 }
 

@@ -142,6 +142,8 @@ struct NttAux {
   // inverse only: the final factor of limb li is the pair post[2 r], post[2 r + 1] (value, Shoup
   // companion), r = li - limb_begin, instead of N^-1
   const u64* post = nullptr;
+  // inverse only, with post: the constants post_add[r] (canonical) are added after the final factor
+  const u64* post_add = nullptr;
   // inverse only, with pre_scale: the first limb (limb_begin) of part p enters as pre_e[p * pre_e_stride + n] + x pre_w
   // mod its prime, x the limb itself (canonical residues; pre_w with its Shoup companion pre_wsh), pre_e null for 0
   int pre_scale = 0;
@@ -168,15 +170,13 @@ struct NttAux {
   size_t spread_stride = 0;
   const u64* spread_sub = nullptr;
   int spread_prime = 0;
-  // forward only: the first phase loads the ModDown conversion of K special limbs (coefficient
-  // domain, z_k = x_k shat_k^-1 at pconv + part * pconv_stride + k * N, moduli s_k = pconv_q[k],
-  // S = prod s_k) into the prime of limb li: sum_k [z_k + c_k]_{s_k} shat_k mod q_li - floor(S/2)
+  // forward only: the first phase loads the ModDown conversion of K special limbs (coefficient domain,
+  // z_k = x_k shat_k^-1 + floor(S/2) shat_k^-1 mod s_k at pconv + part * pconv_stride + k * N, S = prod s_k) into the
+  // prime of limb li: sum_k z_k shat_k mod q_li - floor(S/2)
   const u64* pconv = nullptr;
   size_t pconv_stride = 0;
   int pconv_K = 0;
   int pconv_ld = 0;                   // row length of the per-target tables
-  const u64* pconv_q = nullptr;       // [K] the special moduli s_k
-  const u64* pconv_c = nullptr;       // [K] floor(S/2) shat_k^-1 mod s_k
   const u64* pconv_phat = nullptr;    // [K][ld] (S / s_k) 2^32 mod q_i
   const u64* pconv_phat_b = nullptr;  // [K][ld] (S / s_k) 2^64 mod q_i
   const u64* pconv_half = nullptr;    // [ld] floor(S/2) mod q_i
@@ -190,6 +190,10 @@ struct NttAux {
   const u64* fin_w = nullptr;
   const u64* fin_wb = nullptr;
   int fin_acc_even = 0, fin_acc_odd = 0;
+  // with fin_d: what is added is not fin_dst but fin_d[part][li] permuted by the automorphism X -> X^fin_g
+  const u64* fin_d = nullptr;
+  size_t fin_d_stride = 0;
+  u64 fin_g = 0;
   // with fin_e: a key switch's ModDown fused with the rescale that follows it (see ks_moddown_rescale):
   //   fin_dst[part][li] = fin_c[part][li] * fin_w[li] + (fin_e[part][li] - v) * fin_w2[li]
   // (fin_w = (P q_l)^-1, fin_w2 = q_l^-1), and the first phase loads the ModDown conversion with its
@@ -212,6 +216,21 @@ struct NttAux {
 __host__ __device__ constexpr size_t key_pair(size_t p) {
   return (p & ~(size_t)127) + (p & 3) * 32 + ((p >> 2) & 31);
 }
+// NTT-domain index whose value the automorphism X -> X^g brings to index n: evaluation j sits at
+// psi^(2 bitrev(j) + 1).  Within 32 consecutive indices it stays inside one aligned group of 32: gathers are coalesced.
+// For an even n the index of n + 1 is that of n with its lowest bit flipped (bitrev(n + 1) = bitrev(n) + N/2, and g N = N
+// mod 2N for an odd g), so that a pair of words is one aligned pair, perhaps swapped (galois_pair).
+#ifdef __CUDACC__
+__device__ __forceinline__ uint32_t galois_index(uint32_t n, u64 g, int log_n) {
+  const u64 e = 2 * (u64)(__brev(n) >> (32 - log_n)) + 1;
+  const u64 eg = (g * e) & ((2ull << log_n) - 1);
+  return __brev((uint32_t)((eg - 1) >> 1)) >> (32 - log_n);
+}
+__device__ __forceinline__ ulonglong2 galois_pair(const u64* limb, uint32_t s) {  // s = galois_index of an even index
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(limb + (s & ~1u));
+  return s & 1 ? ulonglong2{v.y, v.x} : v;
+}
+#endif
 struct KskFuse {
   const u64* d = nullptr;        // NTT-domain inputs: ciphertext k's limb t at d + k d_stride + t N
   size_t d_stride = 0;
@@ -284,9 +303,9 @@ struct RescaleConsts {
   u64 inv_sh[kMaxLimbs];
 };
 
-// ModDown of limb l (prime q_l) scaled by P^-1: x - (sum_k [z_k + c_k]_{p_k} p_k^-1 + off) mod q_l
+// ModDown of limb l (prime q_l) scaled by P^-1: x - (sum_k z_k p_k^-1 + off) mod q_l
 struct MdrLast {
-  u64 p[8], c[8], f[8], fs[8];  // p_k, floor(P/2) phinv_k mod p_k, p_k^-1 mod q_l and its Shoup companion
+  u64 f[8], fs[8];              // p_k^-1 mod q_l and its Shoup companion
   u64 off;                      // -floor(P/2) P^-1 mod q_l
   u64 pinv, pinv_sh;            // P^-1 mod q_l and its Shoup companion
   int K;
@@ -332,8 +351,8 @@ struct Ctx {
   std::vector<PrimeDev> pdev;
   DevBuf d_primes, d_psi2, d_ipsi2, d_ninv, d_ninv_sh;
   DevBuf d_moddown;   // level-independent ModDown constants
-  DevBuf d_moddown2;  // fused ModDown: [N^-1 phinv_k, Shoup][K] pairs, c_k [K], p_k [K], then mont_mul_lazy's pairs of
-                      // phat_q, [K][n_q] first words and [K][n_q] second words, and of P^-1 mod q_i, [n_q] and [n_q]
+  DevBuf d_moddown2;  // fused ModDown: [N^-1 phinv_k, Shoup][K] pairs, 0, c_k [K], then mont_mul_lazy's pairs of phat_q,
+                      // [K][n_q] first words and [K][n_q] second words, and of P^-1 mod q_i, [n_q] and [n_q]
   DevBuf d_mdr;       // ModDown scaled by P^-1 (fused with a rescale): mont_mul_lazy's pairs of p_k^-1 mod q_i, [K][n_q]
                       // first and [K][n_q] second words, then floor(P/2) P^-1 mod q_i [n_q]
   std::vector<u64> mdr_post;  // [N^-1 phinv_k, Shoup][K] pairs (host copy of d_moddown2's first)

@@ -264,8 +264,8 @@ void k_rescale_spread(const Ctx& C, const u64* last, size_t ls, u64* tmp, size_t
   HEDAP_LAUNCH_CHECK();
 }
 // ---------------------------------------------------------------- ModDown fused with a rescale: the last limb
-// x = t - (off + sum_k [z_k + c_k]_{p_k} f_k) mod q_l, t limb l of part p (coefficient domain, part stride zs) and z_k
-// the K limbs after it: the K canonical products and off sum below (K + 1) q_l <= 9 q_l < 2^64, reduced once
+// x = t - (off + sum_k z_k f_k) mod q_l, t limb l of part p (coefficient domain, part stride zs) and z_k the K limbs
+// after it: the K canonical products and off sum below (K + 1) q_l <= 9 q_l < 2^64, reduced once
 __global__ void k_mdr_last_coef_kernel(const PrimeDev* __restrict__ pr, const u64* t, size_t zs,
                                        u64* x, int n_parts, int log_n, int l, MdrLast M) {
   grid_wait();
@@ -277,7 +277,7 @@ __global__ void k_mdr_last_coef_kernel(const PrimeDev* __restrict__ pr, const u6
     u64 v = M.off;
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-      if (k < M.K) v += shoup_mul(add_mod(tp[(size_t)(k + 1) * N], M.c[k], M.p[k]), M.f[k], M.fs[k], P.q);
+      if (k < M.K) v += shoup_mul(tp[(size_t)(k + 1) * N], M.f[k], M.fs[k], P.q);
     x[i] = sub_mod(tp[0], barrett_reduce(v, 0, P), P.q);
   }
 }
@@ -321,21 +321,17 @@ __global__ void k_automorph_kernel(const u64* in, size_t is, u64* out, size_t os
                                    int n_parts, int limbs, int log_n, u64 g) {
   grid_wait();
   const size_t N = (size_t)1 << log_n, per_part = (size_t)limbs << log_n;
-  const u64 mask2n = 2 * N - 1;
-  GRID_LOOP(e, n_parts * per_part) {
+  GRID_LOOP(t, n_parts * per_part / 2) {
+    const size_t e = 2 * t;
     const size_t p = e / per_part, r = e - p * per_part;
     const size_t base = r & ~(N - 1);
-    const uint32_t j = (uint32_t)(r & (N - 1));
-    const u64 ej = 2 * (u64)(__brev(j) >> (32 - log_n)) + 1;
-    const u64 ek = (g * ej) & mask2n;
-    const uint32_t k = __brev((uint32_t)((ek - 1) >> 1)) >> (32 - log_n);
-    out[p * os + r] = in[p * is + base + k];
+    st2(out + p * os + r, galois_pair(in + p * is + base, galois_index((uint32_t)(r & (N - 1)), g, log_n)));
   }
 }
 void k_automorph(const Ctx& C, const u64* in, size_t is, u64* out, size_t os, int n_parts, int limbs, u64 g) {
   ProfScope prof_(PROF_AUTOMORPH, C.stream, 2.0 * n_parts * limbs * C.N * 8);
   prof_count_launches(1);
-  const size_t work = (size_t)n_parts * limbs * C.N;
+  const size_t work = (size_t)n_parts * limbs * C.N / 2;
   launch(k_automorph_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, in, is, out, os, n_parts, limbs, C.log_n, g);
   HEDAP_LAUNCH_CHECK();
 }
@@ -406,11 +402,6 @@ void k_modup(const Ctx& C, const u64* dcoef, u64* y, int batch, int level, const
 // Bound by HBM: every rotation reads a key of its own (2 dn (l+1+K) limbs), and all of them the same digits. The grid runs
 // through the rotations of a limb before it goes on to the next limb, so that the limb's digits (B dn
 // limbs) stay in L2 for all of them instead of coming from DRAM for each.
-__device__ __forceinline__ uint32_t galois_index(uint32_t n, u64 g, int log_n) {
-  const u64 e = 2 * (u64)(__brev(n) >> (32 - log_n)) + 1;
-  const u64 eg = (g * e) & ((2ull << log_n) - 1);
-  return __brev((uint32_t)((eg - 1) >> 1)) >> (32 - log_n);
-}
 __device__ __forceinline__ ulonglong2 ld2_stream(const u64* p) { return __ldcs(reinterpret_cast<const ulonglong2*>(p)); }
 __global__ void __launch_bounds__(512, 2) k_ksk_inner_kernel(const PrimeDev* __restrict__ pr, const u64* y,
                                                              const u64* d, size_t ds, KskInnerArgs A,
@@ -428,22 +419,23 @@ __global__ void __launch_bounds__(512, 2) k_ksk_inner_kernel(const PrimeDev* __r
   const size_t key_a = (size_t)total_primes * N, key_step = 2 * key_a, y_step = (size_t)ext * N;
   const u64* yk = y + ((size_t)k * dn * ext + t) * N;
   const u64* dk = d + k * ds + (size_t)t * N;
-  const size_t s0 = galois_index((uint32_t)n, A.g[rot], log_n), s1 = galois_index((uint32_t)n + 1, A.g[rot], log_n);
+  const uint32_t s0 = galois_index((uint32_t)n, A.g[rot], log_n);
   Acc128 a0{0, 0}, a1{0, 0}, b0{0, 0}, b1{0, 0};  // (coefficient n, n+1) x (key b, key a)
 #pragma unroll 4
   for (int j = 0; j < dn; ++j) {
     const u64* src = j == own ? dk : yk + j * y_step;
-    const u64 v0 = src[s0], v1 = src[s1];
+    const ulonglong2 v = galois_pair(src, s0);
     const ulonglong2 wb = ld2_stream(kb + j * key_step), wa = ld2_stream(kb + j * key_step + key_a);
-    mac128(a0, v0, wb.x);
-    mac128(a1, v0, wa.x);
-    mac128(b0, v1, wb.y);
-    mac128(b1, v1, wa.y);
+    mac128(a0, v.x, wb.x);
+    mac128(a1, v.x, wa.x);
+    mac128(b0, v.y, wb.y);
+    mac128(b1, v.y, wa.y);
   }
   if (c0 && t <= l) {  // the rotation kept over Q_l u P: part 0 gains P sigma_g(c0) on the Q limbs
     const u64* ck = c0 + k * c0s + (size_t)t * N;
-    mac128(a0, ck[s0], pmod[pt]);
-    mac128(b0, ck[s1], pmod[pt]);
+    const ulonglong2 v = galois_pair(ck, s0);
+    mac128(a0, v.x, pmod[pt]);
+    mac128(b0, v.y, pmod[pt]);
   }
   const PrimeDev P = pr[pt];
   u64* out = A.acc[rot] + (((size_t)k * 2) * ext + t) * N + n;

@@ -41,6 +41,8 @@ static void dispatch(const Tables& T, const LimbSet& S, cudaStream_t st, bool in
     throw Error(HEDAP_ERR_ARG, "NTT: bad key inner product fusion");
   if (A.own_alpha && (A.own_dn < 1 || A.own_alpha > 8)) throw Error(HEDAP_ERR_ARG, "NTT: bad digit layout");
   if (A.z && (inverse || !A.own_alpha || !A.bconv || !A.bconv_b_offset)) throw Error(HEDAP_ERR_ARG, "NTT: bad ModUp fusion");
+  if (A.fin_d && (!A.fin_dst || A.fin_w2 || !A.fin_g)) throw Error(HEDAP_ERR_ARG, "NTT: bad gathered epilogue fusion");
+  if (A.post_add && !A.post) throw Error(HEDAP_ERR_ARG, "NTT: constants after the final factors need these");
   if (A.post && !inverse) throw Error(HEDAP_ERR_ARG, "NTT: post factors apply to the inverse only");
   if ((A.pre_scale || A.pre_e) && (!inverse || !A.pre_scale)) throw Error(HEDAP_ERR_ARG, "NTT: a fused sum on load applies to the inverse only");
   if ((A.spread || A.fin_dst || A.pconv) && inverse)
@@ -60,16 +62,15 @@ static void dispatch(const Tables& T, const LimbSet& S, cudaStream_t st, bool in
   const double limbs = (double)S.n_parts * S.n_limbs - (A.own_alpha ? (double)S.n_parts / A.own_dn * A.own_limit : 0.0);
   const double n = (double)((size_t)1 << T.log_n);
   ProfScope prof_(PROF_NTT, st, 16.0 * limbs * n);
-  // algorithmic multiply work in 32-bit multiply-pipe slots (one 32 x 32 -> 32 product, low or high half):
-  // a Shoup product by a constant is 7 half products for the exact high half of x w' and 2 wide (2 slots each)
-  // plus 4 low products for x w - qh q = 15 slots; every butterfly has one, and so does every product of a
-  // fused basis conversion (ModUp: one per digit limb, less a factor folded into the key; ModDown: K per word);
-  // the fused key inner product multiplies every word of every digit by two key words, a full 64 x 64 ->
-  // 128-bit product of 8 half products = 8 slots each
-  double shoup = limbs * n / 2 * T.log_n;
-  if (A.z) shoup += A.z_products >= 0 ? A.z_products : limbs * n * std::min(A.own_alpha, A.own_limit);
-  if (A.pconv) shoup += limbs * n * A.pconv_K;
-  prof_.slots = 15.0 * shoup;
+  // algorithmic multiply work in 32-bit multiply-pipe slots (one 32 x 32 -> 32 product; a 32 x 32 -> 64 product takes
+  // two): a butterfly's product by a constant is four wide products and a Montgomery step of a low and two wide
+  // ones = 13 slots; a fused basis conversion has four wide products a term (ModUp: one term per digit limb,
+  // less a factor folded into the key; ModDown: K) and one Montgomery step a word = 5 slots; the fused key inner
+  // product multiplies every word of every digit by two key words, four wide products = 8 slots each
+  double slots = 13.0 * limbs * n / 2 * T.log_n;
+  if (A.z) slots += 8.0 * (A.z_products >= 0 ? A.z_products : limbs * n * std::min(A.own_alpha, A.own_limit)) + 5.0 * limbs * n;
+  if (A.pconv) slots += limbs * n * (8.0 * A.pconv_K + 5.0);
+  prof_.slots = slots;
   if (F) prof_.slots += 8.0 * 2.0 * F->batch * (double)S.n_limbs * A.own_dn * n;
   prof_count_launches(2);
   ntt_launch(T.log_n, v, S, T, st, inverse, A, F);

@@ -187,8 +187,8 @@ enum LastLimb { LAST_NONE = 0, LAST_RAW = 1, LAST_MONT = 2 };  // how a fused re
 template <int KIND>
 struct FusedLoad {
   static constexpr int MAXT = 3;
-  u64 f[MAXT], fb[MAXT], c[MAXT], pk[MAXT];  // products: factor pairs, and the ModDown's rounding constants
-  int tile[MAXT];                            // tile of product t
+  u64 f[MAXT], fb[MAXT];  // products: factor pairs
+  int tile[MAXT];         // tile of product t
   u64 off, half, sub;
   PrimeDev P;
   int nm, raw, last;  // products, the tile added as it is (-1: none), LastLimb
@@ -220,8 +220,6 @@ struct FusedLoad {
       for (int t = 0; t < MAXT; ++t) {
         const bool on = t < ns;
         tile[t] = t;
-        c[t] = on ? A.pconv_c[t] : 0;
-        pk[t] = on ? A.pconv_q[t] : 0;
         f[t] = on ? A.pconv_phat[(size_t)t * A.pconv_ld + li] : 0;
         fb[t] = on ? A.pconv_phat_b[(size_t)t * A.pconv_ld + li] : 0;
       }
@@ -240,11 +238,7 @@ struct FusedLoad {
     u64 v = off;
     MontAcc s{0, 0};
 #pragma unroll
-    for (int t = 0; t < NM; ++t) {
-      u64 x = z(tile[t]);
-      if (KIND == LOAD_MODDOWN) x = add_mod(x, c[t], pk[t]);
-      mont_mac(s, x, f[t], fb[t]);
-    }
+    for (int t = 0; t < NM; ++t) mont_mac(s, z(tile[t]), f[t], fb[t]);
     if (RAW) v += z(raw);
     if (LAST != LAST_NONE) {
       const u64 x = z(KIND == LOAD_SPREAD ? 0 : ns);
@@ -449,14 +443,12 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_wide(Tables T, LimbSe
   };
   for (int t = 0; t < ns; ++t) {
     const u64* z = base + (size_t)t * N;
-    u64 f, fb, c = 0, pk = 0;
+    u64 f, fb;
     if (KIND == LOAD_MODUP) {
       const u64* bc = A.bconv + ((size_t)j * A.own_alpha + t) * A.ext + li;
       f = bc[0];
       fb = bc[A.bconv_b_offset];
     } else {
-      c = A.pconv_c[t];
-      pk = A.pconv_q[t];
       f = A.pconv_phat[(size_t)t * A.pconv_ld + li];
       fb = A.pconv_phat_b[(size_t)t * A.pconv_ld + li];
     }
@@ -466,11 +458,7 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_wide(Tables T, LimbSe
       for (int m = 0; m < G::M0; ++m) v[0][m] += z[(size_t)(m * G::M1) << L2];
     } else {
 #pragma unroll
-      for (int m = 0; m < G::M0; ++m) {
-        u64 x = z[(size_t)(m * G::M1) << L2];
-        if (KIND == LOAD_MODDOWN) x = add_mod(x, c, pk);
-        mont_mac(s[m], x, f, fb);
-      }
+      for (int m = 0; m < G::M0; ++m) mont_mac(s[m], z[(size_t)(m * G::M1) << L2], f, fb);
     }
   }
   close();
@@ -530,9 +518,11 @@ __device__ __forceinline__ ulonglong2 row_pair(const u64* xs, int k, int low) {
   using G = RowGeo<L2>;
   return ldg2(xs + G::pair(low) + G::pair(k * G::M1));
 }
-template <bool SMALL, int L2>
-__device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u64* a, size_t at, int part, int li,
-                                               const PrimeDev& P, int low) {
+// n0: the block's first word of the limb, at: of the part
+template <bool SMALL, int L1, int L2>
+__device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u64* a, uint32_t n0, size_t at, int part,
+                                               int li, const PrimeDev& P, int low) {
+  constexpr int LOGN = L1 + L2;
   using G = RowGeo<L2>;
   const u64 q = P.q;
   constexpr int PAIRS = G::M0 / 2;  // word pairs of a lane
@@ -581,7 +571,13 @@ __device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u
       z.x = fin(c.x, v.x);
       z.y = fin(c.y, v.y);
       if (acc) {
-        const ulonglong2 d = ldg2(dp + 2 * e);
+        ulonglong2 d;
+        if (A.fin_d) {
+          const u64* limb = A.fin_d + (size_t)part * A.fin_d_stride + (at - n0);
+          d = galois_pair(limb, galois_index(n0 + 2 * e, A.fin_g, LOGN));
+        } else {
+          d = ldg2(dp + 2 * e);
+        }
         z.x = add_mod(z.x, d.x, q);
         z.y = add_mod(z.y, d.y, q);
       }
@@ -624,7 +620,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_fwd_rows(Tables T, LimbSet
       const u64* cp = A.fin_c + (size_t)part * A.fin_c_stride + at;
       const u64* dp = A.fin_e ? A.fin_e + (size_t)part * A.fin_e_stride + at
                               : A.fin_dst + (size_t)part * A.fin_dst_stride + at;
-      const bool acc = A.fin_e || ((part & 1) ? A.fin_acc_odd : A.fin_acc_even);
+      const bool acc = A.fin_e || (!A.fin_d && ((part & 1) ? A.fin_acc_odd : A.fin_acc_even));
       for (int idx = 16 * low; idx < (1 << L2); idx += 16 * G::M1) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(cp + idx));
         if (acc) asm volatile("prefetch.global.L2 [%0];" ::"l"(dp + idx));
@@ -640,10 +636,10 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_fwd_rows(Tables T, LimbSet
     }
     if (fwd_small(P.q)) {
       fwd_rows_body<true, L1, L2>(v, xs, tw, P, low);
-      fwd_rows_store<true, L2>(xs, A, a, at, part, li, P, low);
+      fwd_rows_store<true, L1, L2>(xs, A, a, (uint32_t)j0, at, part, li, P, low);
     } else {
       fwd_rows_body<false, L1, L2>(v, xs, tw, P, low);
-      fwd_rows_store<false, L2>(xs, A, a, at, part, li, P, low);
+      fwd_rows_store<false, L1, L2>(xs, A, a, (uint32_t)j0, at, part, li, P, low);
     }
     __syncwarp();
   }
@@ -942,7 +938,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_inv_rows(Tables T, LimbSet
 // ---------------------------------------------------------------- inverse, column phase (+ N^-1)
 template <bool SMALL, int L1, int L2, int TH>
 __device__ __forceinline__ void inv_cols_body(u64 (&w)[Phase<L1>::GP][1][1 << Phase<L1>::K1], u64* a, u64* xs,
-                                              const ulonglong2* tw, const PrimeDev& P, int low, int cg, u64 ni, u64 nip) {
+                                              const ulonglong2* tw, const PrimeDev& P, int low, int cg, u64 ni, u64 nip, u64 add) {
   using G = ColGeo<L1, TH>;
   const u64 q = P.q;
 #pragma unroll
@@ -964,7 +960,7 @@ __device__ __forceinline__ void inv_cols_body(u64 (&w)[Phase<L1>::GP][1][1 << Ph
   for (int m = 0; m < G::M0; ++m) v[0][m] = xs[(m * (G::M1 + 1) + low) * G::COLS + cg];
   inv_pass<SMALL, 1 + G::K1, G::K0, 1>(v, q, P.nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
 #pragma unroll
-  for (int m = 0; m < G::M0; ++m) a[(size_t)(m * G::M1 + low) << L2] = shoup_mul(v[0][m], ni, nip, q);
+  for (int m = 0; m < G::M0; ++m) a[(size_t)(m * G::M1 + low) << L2] = add_mod(shoup_mul(v[0][m], ni, nip, q), add, q);
 }
 template <int L1, int L2, int TH, int MINB>
 __global__ void __launch_bounds__(TH, MINB) k_ntt_inv_cols(Tables T, LimbSet S, NttAux A) {
@@ -988,10 +984,11 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_inv_cols(Tables T, LimbSet S, 
     for (int m = 0; m < G::M1; ++m) w[i][0][m] = a[(size_t)((i * G::M1 + low) * G::M1 + m) << L2];
   const int r = li - S.limb_begin;
   const u64 ni = A.post ? A.post[2 * r] : T.ninv[pi], nip = A.post ? A.post[2 * r + 1] : T.ninv_sh[pi];
+  const u64 add = A.post_add ? A.post_add[r] : 0;
   cp_async_wait_all();
   __syncthreads();
-  if (inv_small(P.q)) inv_cols_body<true, L1, L2, TH>(w, a, sm, tw, P, low, cg, ni, nip);
-  else inv_cols_body<false, L1, L2, TH>(w, a, sm, tw, P, low, cg, ni, nip);
+  if (inv_small(P.q)) inv_cols_body<true, L1, L2, TH>(w, a, sm, tw, P, low, cg, ni, nip, add);
+  else inv_cols_body<false, L1, L2, TH>(w, a, sm, tw, P, low, cg, ni, nip, add);
 }
 
 // ---------------------------------------------------------------- small rings: a whole limb per cluster
@@ -1060,6 +1057,7 @@ __global__ void __cluster_dims__(WholeGeo<L1, L2>::CS, 1, 1) __launch_bounds__(W
   cp_async_commit();
   const int r = li - S.limb_begin;
   const u64 ni = A.post ? A.post[2 * r] : T.ninv[pi], nip = A.post ? A.post[2 * r + 1] : T.ninv_sh[pi];
+  const u64 add = A.post_add ? A.post_add[r] : 0;
   cp_async_wait_all();
   __syncthreads();
   auto body = [&](auto is_small) {
@@ -1084,7 +1082,7 @@ __global__ void __cluster_dims__(WholeGeo<L1, L2>::CS, 1, 1) __launch_bounds__(W
 #pragma unroll
       for (int m = 0; m < G::M1; ++m) w[i][0][m] = X[((i * G::M1 + clow) * (G::M1 + 1) + m) * G::COLS + cg];
     // every thread writes back the words that it read: no barrier before inv_cols_body's exchange
-    inv_cols_body<SMALL, L1, L2, W::TH>(w, a + rank * G::COLS + cg, X, tw, P, clow, cg, ni, nip);
+    inv_cols_body<SMALL, L1, L2, W::TH>(w, a + rank * G::COLS + cg, X, tw, P, clow, cg, ni, nip, add);
   };
   if (inv_small(P.q)) body(std::true_type{});
   else body(std::false_type{});
@@ -1161,7 +1159,8 @@ __global__ void __cluster_dims__(WholeGeo<L1, L2>::CS, 1, 1) __launch_bounds__(W
       for (int m = 0; m < R::M0; ++m) w[0][m] = ys[m * R::GS + low];
       __syncwarp();
       fwd_rows_body<SMALL, L1, L2>(w, ys, tw + (1 << L1) + (b << L2), P, low);
-      fwd_rows_store<SMALL, L2>(ys, A, a + ((size_t)blk << L2), (size_t)li * N + ((size_t)blk << L2), part, li, P, low);
+      fwd_rows_store<SMALL, L1, L2>(ys, A, a + ((size_t)blk << L2), (uint32_t)blk << L2, (size_t)li * N + ((size_t)blk << L2),
+                                    part, li, P, low);
     }
   };
   if (fwd_small(P.q)) body(std::true_type{});
