@@ -226,30 +226,50 @@ const LevelConsts& level_consts(Ctx& C, int l) {
 // the inverse NTT reads d out of place and ends with N^-1 qhat_i^-1, the forward
 // NTT of each extended limb loads the basis conversion directly, and a digit's
 // own limbs (whose NTT is d itself) are neither converted nor transformed.
+//
+// An operation's temporaries come from one allocation, in which what ends with the inner product gives its place
+// to ModDown's workspace: on a small ring each allocation with its release costs the host a good part of a launch.
+struct Scratch {
+  DevBuf buf;
+  size_t at = 0;  // set back by the caller once what lies above has been used
+  Scratch(Ctx& C, size_t words) : buf(words, C.stream) {}
+  u64* take(size_t words) {
+    if (at + words > buf.words) throw Error(HEDAP_ERR_ARG, "scratch exhausted");
+    u64* p = buf.p + at;
+    at += words;
+    return p;
+  }
+};
+// words of ks_modup's workspace: the coefficient-domain limbs and the extended digits
+static size_t modup_words(const Ctx& C, int batch, int l) {
+  return (size_t)batch * C.N * ((l + 1) + (size_t)C.dnum(l) * (l + 1 + C.n_p));
+}
+static size_t acc_words(const Ctx& C, int batch, int l) { return (size_t)batch * 2 * (l + 1 + C.n_p) * C.N; }
 // ModUp of a batch of NTT-domain polynomials d (member stride d_stride) into NTT-domain extended
-// digits [B][dn][ext][N] (a digit's own limbs are left out: they are d itself)
-static DevBuf ks_modup(Ctx& C, const u64* d, size_t d_stride, int batch, int l, const KskFuse* fuse = nullptr) {
+// digits [B][dn][ext][N] (a digit's own limbs are left out: they are d itself), in ws (modup_words)
+static const u64* ks_modup(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64* ws,
+                           const KskFuse* fuse = nullptr) {
   const size_t N = C.N, nl = (size_t)l + 1;
   const int ext = l + 1 + C.n_p, dn = C.dnum(l);
   const LevelConsts& LC = level_consts(C, l);
-  DevBuf dc((size_t)batch * nl * N, C.stream);  // z_i = [x_i qhat_i^-1]_{q_i}, coefficient domain
+  u64* dc = ws;  // z_i = [x_i qhat_i^-1]_{q_i}, coefficient domain
+  u64* y = ws + (size_t)batch * nl * N;
   NttAux inv{};
   inv.src = d;
   inv.src_stride = d_stride;
   inv.post = LC.intt_post.p;
-  ntt_inverse(C.tab, qset(dc.p, nl * N, batch, 0, l + 1), C.stream, &inv);
-  DevBuf y((size_t)batch * dn * ext * N, C.stream);
+  ntt_inverse(C.tab, qset(dc, nl * N, batch, 0, l + 1), C.stream, &inv);
   NttAux up{};
   up.own_alpha = C.alpha;
   up.own_dn = dn;
   up.own_limit = l + 1;
-  up.z = dc.p;
+  up.z = dc;
   up.z_stride = nl * N;
   up.bconv = LC.modup_ks.p;  // factors divided by the key's folded ones
   up.bconv_b_offset = (size_t)dn * C.alpha * ext;
   up.ext = ext;
   up.z_products = LC.modup_products * batch * (double)N;
-  ntt_forward(C.tab, LimbSet{y.p, (size_t)ext * N, batch * dn, 0, ext, l + 1, 0, C.n_q}, C.stream, &up, fuse);
+  ntt_forward(C.tab, LimbSet{y, (size_t)ext * N, batch * dn, 0, ext, l + 1, 0, C.n_q}, C.stream, &up, fuse);
   return y;
 }
 static const DevBuf& key_for(Ctx& C, u64 galois) {
@@ -263,7 +283,9 @@ static const DevBuf& key_for(Ctx& C, u64 galois) {
 // iNTT of the P limbs of the key-switch sums acc [batch][2][ext][N], ModDown, NTT, written to / added
 // into out
 // with c0 (part stride c0_stride): the even parts gain sigma_g(c0), gathered by the finishing store
-static void ks_moddown(Ctx& C, const DevBuf& acc, int batch, int l, u64* out, size_t out_stride, bool acc0, bool acc1,
+// v: workspace of moddown_words
+static size_t moddown_words(const Ctx& C, int batch, int l) { return (size_t)batch * 2 * (l + 1) * C.N; }
+static void ks_moddown(Ctx& C, u64* acc, u64* v, int batch, int l, u64* out, size_t out_stride, bool acc0, bool acc1,
                        const u64* c0 = nullptr, size_t c0_stride = 0, u64 g = 0) {
   const size_t N = C.N, nl = (size_t)l + 1;
   const int K = C.n_p, ext = l + 1 + K;
@@ -276,13 +298,12 @@ static void ks_moddown(Ctx& C, const DevBuf& acc, int batch, int l, u64* out, si
     inv.post = C.d_moddown2.p;
     inv.post_add = C.d_moddown2.p + 2 * K + 1;
   }
-  ntt_inverse(C.tab, LimbSet{acc.p, (size_t)ext * N, 2 * batch, l + 1, K, l + 1, 0, C.n_q}, C.stream, &inv);
-  DevBuf v((size_t)batch * 2 * nl * N, C.stream);
-  if (!fuse) k_moddown_spread(C, acc.p, v.p, 2 * batch, l);
+  ntt_inverse(C.tab, LimbSet{acc, (size_t)ext * N, 2 * batch, l + 1, K, l + 1, 0, C.n_q}, C.stream, &inv);
+  if (!fuse) k_moddown_spread(C, acc, v, 2 * batch, l);
   const u64* Pinv = C.d_moddown2.p + 3 * K + 1 + 2 * (size_t)K * C.n_q;
   NttAux fw{};
   if (fuse) {
-    fw.pconv = acc.p + nl * N;
+    fw.pconv = acc + nl * N;
     fw.pconv_stride = (size_t)ext * N;
     fw.pconv_K = K;
     fw.pconv_ld = C.n_q;
@@ -292,7 +313,7 @@ static void ks_moddown(Ctx& C, const DevBuf& acc, int batch, int l, u64* out, si
   }
   fw.fin_dst = out;
   fw.fin_dst_stride = out_stride;
-  fw.fin_c = acc.p;
+  fw.fin_c = acc;
   fw.fin_c_stride = (size_t)ext * N;
   fw.fin_w = Pinv;
   fw.fin_wb = Pinv + C.n_q;
@@ -301,29 +322,28 @@ static void ks_moddown(Ctx& C, const DevBuf& acc, int batch, int l, u64* out, si
   fw.fin_d = c0;
   fw.fin_d_stride = c0_stride;
   fw.fin_g = g;
-  ntt_forward(C.tab, qset(v.p, nl * N, 2 * batch, 0, l + 1), C.stream, &fw);
+  ntt_forward(C.tab, qset(v, nl * N, 2 * batch, 0, l + 1), C.stream, &fw);
 }
 
 // The key switch up to the inner product: iNTT of d, the extended digits' forward transform with the
-// key inner product fused into its second phase (the transformed digits are never stored).  Returns the
-// sums acc [batch][2][ext][N] (NTT domain).
-static DevBuf ks_inner(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64 galois) {
+// key inner product fused into its second phase (the transformed digits are never stored).  The
+// sums acc [batch][2][ext][N] (NTT domain) go to acc; ws: workspace of modup_words.
+static void ks_inner(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64 galois, u64* acc, u64* ws) {
   const DevBuf& key = key_for(C, galois);
   const int T = C.total_primes();
-  DevBuf acc((size_t)batch * 2 * (l + 1 + C.n_p) * C.N, C.stream);
   if (C.log_n <= 13 && C.alpha <= 3 && ((size_t)batch * (l + 1 + C.n_p) << C.log_n) <= (size_t)1 << 18) {
     // a small ring's few limbs: the digits transformed in one launch, all of them at once, and the inner product in
     // a second; fused, one warp for 256 words would walk the digits one after the other with fewer than 1024
     // warps on the GPU (N = 2^12, HMult: 12 digits of 3 ciphertexts, 160 K words a digit, 65 against 71 us;
     // 7 digits of 295 K words 82 against 78 us)
-    DevBuf y = ks_modup(C, d, d_stride, batch, l);
+    const u64* y = ks_modup(C, d, d_stride, batch, l, ws);
     KskInnerArgs A;
     A.count = 1;
     A.key[0] = key.p;
-    A.acc[0] = acc.p;
+    A.acc[0] = acc;
     A.g[0] = 1;
-    k_ksk_inner(C, y.p, d, d_stride, A, batch, l);
-    return acc;
+    k_ksk_inner(C, y, d, d_stride, A, batch, l);
+    return;
   }
   KskFuse F;
   F.d = d;
@@ -331,18 +351,21 @@ static DevBuf ks_inner(Ctx& C, const u64* d, size_t d_stride, int batch, int l, 
   F.key = key.p;
   F.key_digit_stride = (size_t)2 * T * C.N;
   F.key_a_offset = (size_t)T * C.N;
-  F.acc = acc.p;
+  F.acc = acc;
   F.acc_part_stride = (size_t)(l + 1 + C.n_p) * C.N;
   F.batch = batch;
-  ks_modup(C, d, d_stride, batch, l, &F);  // its column-phase buffer is released stream-ordered
-  return acc;
+  ks_modup(C, d, d_stride, batch, l, ws, &F);
 }
 
 // One key switch: the inner product, then ModDown.
 void key_switch(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64 galois, u64* out, size_t out_stride,
                 bool acc0, bool acc1) {
-  DevBuf acc = ks_inner(C, d, d_stride, batch, l, galois);
-  ks_moddown(C, acc, batch, l, out, out_stride, acc0, acc1);
+  Scratch S(C, acc_words(C, batch, l) + std::max(modup_words(C, batch, l), moddown_words(C, batch, l)));
+  u64* acc = S.take(acc_words(C, batch, l));
+  const size_t mark = S.at;
+  ks_inner(C, d, d_stride, batch, l, galois, acc, S.take(modup_words(C, batch, l)));
+  S.at = mark;
+  ks_moddown(C, acc, S.take(moddown_words(C, batch, l)), batch, l, out, out_stride, acc0, acc1);
 }
 
 // ModDown of the key-switch sums acc added to e (NTT domain, level l, part stride e_stride), followed
@@ -354,7 +377,9 @@ void key_switch(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64 gal
 // constants scaled by P^-1).  The last limb's coefficients come first: INTT(e_l + acc_l P^-1) minus
 // the conversion of the special limbs into q_l scaled by P^-1.  Every residue equals that of ModDown
 // followed by the rescale.
-static void ks_moddown_rescale(Ctx& C, const DevBuf& acc, int batch, int l, const u64* e, size_t e_stride, u64* out,
+// ws: workspace of mdr_words.
+static size_t mdr_words(const Ctx& C, int batch, int l) { return (size_t)2 * batch * (l + 1) * C.N; }
+static void ks_moddown_rescale(Ctx& C, u64* acc, u64* ws, int batch, int l, const u64* e, size_t e_stride, u64* out,
                                size_t out_stride, bool negate = false) {
   const size_t N = C.N;
   const int K = C.n_p, ext = l + 1 + K, nq = C.n_q;
@@ -369,25 +394,24 @@ static void ks_moddown_rescale(Ctx& C, const DevBuf& acc, int batch, int l, cons
   inv.pre_e_stride = e_stride;
   inv.pre_w = LC.mdr_last.pinv;
   inv.pre_wsh = LC.mdr_last.pinv_sh;
-  ntt_inverse(C.tab, LimbSet{acc.p, (size_t)ext * N, 2 * batch, l, K + 1, l + 1, 0, C.n_q}, C.stream, &inv);
-  DevBuf x((size_t)2 * batch * N, C.stream);
-  k_mdr_last_coef(C, acc.p + (size_t)l * N, (size_t)ext * N, x.p, 2 * batch, l, LC.mdr_last);
-  DevBuf v((size_t)2 * batch * l * N, C.stream);
+  ntt_inverse(C.tab, LimbSet{acc, (size_t)ext * N, 2 * batch, l, K + 1, l + 1, 0, C.n_q}, C.stream, &inv);
+  u64 *x = ws, *v = ws + (size_t)2 * batch * N;
+  k_mdr_last_coef(C, acc + (size_t)l * N, (size_t)ext * N, x, 2 * batch, l, LC.mdr_last);
   NttAux fw{};
-  fw.pconv = acc.p + (size_t)(l + 1) * N;
+  fw.pconv = acc + (size_t)(l + 1) * N;
   fw.pconv_stride = (size_t)ext * N;
   fw.pconv_K = K;
   fw.pconv_ld = nq;
   fw.pconv_phat = C.d_mdr.p;
   fw.pconv_phat_b = C.d_mdr.p + (size_t)K * nq;
   fw.pconv_half = C.d_mdr.p + 2 * (size_t)K * nq;
-  fw.spread = x.p;
+  fw.spread = x;
   fw.spread_stride = N;
   fw.spread_sub = LC.d_rescale.p;
   fw.spread_prime = l;
   fw.fin_dst = out;
   fw.fin_dst_stride = out_stride;
-  fw.fin_c = acc.p;
+  fw.fin_c = acc;
   fw.fin_c_stride = (size_t)ext * N;
   fw.fin_w = LC.d_mdr.p;
   fw.fin_wb = LC.d_mdr.p + l;
@@ -396,7 +420,7 @@ static void ks_moddown_rescale(Ctx& C, const DevBuf& acc, int batch, int l, cons
   fw.fin_w2 = LC.d_rescale.p + l;
   fw.fin_w2b = LC.d_rescale.p + 2 * l;
   fw.fin_neg = negate ? 1 : 0;
-  ntt_forward(C.tab, qset(v.p, (size_t)l * N, 2 * batch, 0, l), C.stream, &fw);
+  ntt_forward(C.tab, qset(v, (size_t)l * N, 2 * batch, 0, l), C.stream, &fw);
 }
 
 // Rotations of one (batched) ciphertext by several Galois elements sharing one ModUp of its
@@ -407,7 +431,7 @@ static void ks_moddown_rescale(Ctx& C, const DevBuf& acc, int batch, int l, cons
 // The inner products of several rotations with the digits y, as many to a launch as the sums' memory allows:
 // about 1 GiB of them at a time (kKskRotations at most), handed to `done(i, acc)` in order.
 template <class F>
-static void hoisted_inner(Ctx& C, const Ct& a, const DevBuf& y, const std::vector<u64>& gs, const u64* c0, size_t chunk,
+static void hoisted_inner(Ctx& C, const Ct& a, const u64* y, const std::vector<u64>& gs, const u64* c0, size_t chunk,
                           F done) {
   const int l = a.level;
   const size_t words = (size_t)a.batch * 2 * (l + 1 + C.n_p) * C.N, ds = 2 * a.part_stride();
@@ -421,21 +445,23 @@ static void hoisted_inner(Ctx& C, const Ct& a, const DevBuf& y, const std::vecto
       A.acc[r] = acc.back().p;
       A.g[r] = gs[first + r];
     }
-    k_ksk_inner(C, y.p, a.part(1), ds, A, a.batch, l, c0, ds);
+    k_ksk_inner(C, y, a.part(1), ds, A, a.batch, l, c0, ds);
     for (int r = 0; r < A.count; ++r) done(first + r, std::move(acc[r]));
   }
 }
 std::vector<std::unique_ptr<Ct>> ev_galois_hoisted(Ctx& C, const Ct& a, const std::vector<u64>& gs) {
   const int l = a.level;
   for (u64 g : gs) key_for(C, g);
-  DevBuf y = ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, l);
+  Scratch S(C, modup_words(C, a.batch, l) + moddown_words(C, a.batch, l));
+  const u64* y = ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, l, S.take(modup_words(C, a.batch, l)));
+  u64* v = S.take(moddown_words(C, a.batch, l));
   std::vector<std::unique_ptr<Ct>> out;
   const size_t bytes = (size_t)a.batch * 2 * (l + 1 + C.n_p) * C.N * 8;
   const size_t chunk = std::max<size_t>(1, std::min<size_t>(kKskRotations, ((size_t)1 << 30) / bytes));
   hoisted_inner(C, a, y, gs, nullptr, chunk, [&](size_t i, DevBuf acc) {
     auto o = ct_alloc(C, l, a.batch);
     o->scale = a.scale;
-    ks_moddown(C, acc, a.batch, l, o->part(0), o->part_stride(), true, false, a.part(0), a.part_stride(), gs[i]);
+    ks_moddown(C, acc.p, v, a.batch, l, o->part(0), o->part_stride(), true, false, a.part(0), a.part_stride(), gs[i]);
     out.push_back(std::move(o));
   });
   return out;
@@ -443,13 +469,15 @@ std::vector<std::unique_ptr<Ct>> ev_galois_hoisted(Ctx& C, const Ct& a, const st
 
 std::vector<DevBuf> ev_galois_hoisted_qp(Ctx& C, const Ct& a, const std::vector<u64>& gs) {
   for (u64 g : gs) key_for(C, g);
-  DevBuf y = ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, a.level);
+  Scratch S(C, modup_words(C, a.batch, a.level));
+  const u64* y = ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, a.level, S.buf.p);
   std::vector<DevBuf> out(gs.size());  // every sum is kept: one launch for all of them
   hoisted_inner(C, a, y, gs, a.part(0), kKskRotations, [&](size_t i, DevBuf acc) { out[i] = std::move(acc); });
   return out;
 }
 void ev_moddown_into(Ctx& C, DevBuf& acc, int batch, int level, Ct& out) {
-  ks_moddown(C, acc, batch, level, out.part(0), out.part_stride(), false, false);
+  DevBuf v(moddown_words(C, batch, level), C.stream);
+  ks_moddown(C, acc.p, v.p, batch, level, out.part(0), out.part_stride(), false, false);
 }
 
 std::unique_ptr<Ct> ev_mul_relin(Ctx& C, const Ct& a, const Ct& b) {
@@ -479,7 +507,8 @@ static std::unique_ptr<Ct> rescale_scaled(Ctx& C, const Ct& a, const LimbConsts*
   o->scale = a.scale / (double)C.primes[l];
   // the last limb to the coefficient domain (read in place), then one forward transform whose
   // load spreads its centred residue into every other prime and whose store finishes the rescale
-  DevBuf last(P * N, C.stream), factors;
+  Scratch S(C, (size_t)P * (l + 1) * N + (K ? 2 * (size_t)l : 0));
+  u64 *last = S.take(P * N), *tmp = S.take((size_t)P * l * N);
   NttAux inv{};
   inv.src = a.part(0) + (size_t)l * N;
   inv.src_stride = a.part_stride();
@@ -495,16 +524,15 @@ static std::unique_ptr<Ct> rescale_scaled(Ctx& C, const Ct& a, const LimbConsts*
       F.w[i] = h_mont(h_mulmod(K->w[i], LC.rescale.inv[i], C.primes[i]), C.primes[i]);
       F.wsh[i] = h_mont(F.w[i], C.primes[i]);
     }
-    factors = DevBuf(2 * (size_t)l, C.stream);
-    k_put_limbconst(C, factors.p, l, F);
+    u64* factors = S.take(2 * (size_t)l);
+    k_put_limbconst(C, factors, l, F);
     fw.fin_w2 = fw.fin_w;
     fw.fin_w2b = fw.fin_wb;
-    fw.fin_w = factors.p;
-    fw.fin_wb = factors.p + l;
+    fw.fin_w = factors;
+    fw.fin_wb = factors + l;
   }
-  ntt_inverse(C.tab, qset(last.p, N, P, 0, 1, l), C.stream, &inv);
-  DevBuf tmp((size_t)P * l * N, C.stream);
-  fw.spread = last.p;
+  ntt_inverse(C.tab, qset(last, N, P, 0, 1, l), C.stream, &inv);
+  fw.spread = last;
   fw.spread_stride = N;
   fw.spread_sub = LC.d_rescale.p;
   fw.spread_prime = l;
@@ -512,7 +540,7 @@ static std::unique_ptr<Ct> rescale_scaled(Ctx& C, const Ct& a, const LimbConsts*
   fw.fin_dst_stride = o->part_stride();
   fw.fin_c = a.part(0);
   fw.fin_c_stride = a.part_stride();
-  ntt_forward(C.tab, qset(tmp.p, (size_t)l * N, P, 0, l), C.stream, &fw);
+  ntt_forward(C.tab, qset(tmp, (size_t)l * N, P, 0, l), C.stream, &fw);
   return o;
 }
 std::unique_ptr<Ct> ev_rescale(Ctx& C, const Ct& a) { return rescale_scaled(C, a, nullptr); }
@@ -541,16 +569,22 @@ std::unique_ptr<Ct> ev_mul_lincomb_rescale(Ctx& C, const Ct& a, const Ct& b, dou
   auto d01 = ct_alloc(C, l, a.batch);
   d01->scale = prod_scale;
   const size_t per = (size_t)(l + 1) * C.N;
-  DevBuf d2(a.batch * per, C.stream);
-  k_tensor(C, a.part(0), a.part_stride(), b.part(0), b.part_stride(), d01->part(0), d01->part_stride(), d2.p,
-           a.batch, l + 1);
-  DevBuf acc = ks_inner(C, d2.p, per, a.batch, l, 0);
+  Scratch S(C, acc_words(C, a.batch, l) +
+                   std::max(a.batch * per + modup_words(C, a.batch, l), mdr_words(C, a.batch, l)));
+  u64* acc = S.take(acc_words(C, a.batch, l));
+  const size_t mark = S.at;
+  u64* d2 = S.take(a.batch * per);
+  k_tensor(C, a.part(0), a.part_stride(), b.part(0), b.part_stride(), d01->part(0), d01->part_stride(), d2, a.batch,
+           l + 1);
+  ks_inner(C, d2, per, a.batch, l, 0, acc, S.take(modup_words(C, a.batch, l)));
+  S.at = mark;
   std::vector<std::pair<const Ct*, double>> all{{d01.get(), m * prod_coef}};
   for (const auto& t : terms) all.emplace_back(t.first, m * t.second);
   auto e = ev_lincomb_raw(C, all, l, target, m * c0);
   auto o = ct_alloc(C, l - 1, a.batch);
   o->scale = e->scale / (double)C.primes[l];
-  ks_moddown_rescale(C, acc, a.batch, l, e->part(0), e->part_stride(), o->part(0), o->part_stride(), m < 0);
+  ks_moddown_rescale(C, acc, S.take(mdr_words(C, a.batch, l)), a.batch, l, e->part(0), e->part_stride(), o->part(0),
+                     o->part_stride(), m < 0);
   return o;
 }
 
@@ -562,15 +596,18 @@ std::unique_ptr<Ct> ev_mul(Ctx& C, const Ct& a, const Ct& b) {
   if (l < 1) throw Error(HEDAP_ERR_LEVEL, "rescale needs level >= 1");
   if (C.n_p > 8) return ev_rescale(C, *ev_mul_relin(C, a, b));
   check_batches(a, b);
-  auto e = ct_alloc(C, l, a.batch);
   const size_t per = (size_t)(l + 1) * C.N;
-  DevBuf d2(a.batch * per, C.stream);
-  k_tensor(C, a.part(0), a.part_stride(), b.part(0), b.part_stride(), e->part(0), e->part_stride(), d2.p, a.batch,
-           l + 1);
-  DevBuf acc = ks_inner(C, d2.p, per, a.batch, l, 0);
+  Scratch S(C, 2 * a.batch * per + acc_words(C, a.batch, l) +
+                   std::max(a.batch * per + modup_words(C, a.batch, l), mdr_words(C, a.batch, l)));
+  u64 *e = S.take(2 * a.batch * per), *acc = S.take(acc_words(C, a.batch, l));  // e: the tensor's d0, d1
+  const size_t mark = S.at;
+  u64* d2 = S.take(a.batch * per);
+  k_tensor(C, a.part(0), a.part_stride(), b.part(0), b.part_stride(), e, per, d2, a.batch, l + 1);
+  ks_inner(C, d2, per, a.batch, l, 0, acc, S.take(modup_words(C, a.batch, l)));
+  S.at = mark;
   auto o = ct_alloc(C, l - 1, a.batch);
   o->scale = a.scale * b.scale / (double)C.primes[l];
-  ks_moddown_rescale(C, acc, a.batch, l, e->part(0), e->part_stride(), o->part(0), o->part_stride());
+  ks_moddown_rescale(C, acc, S.take(mdr_words(C, a.batch, l)), a.batch, l, e, per, o->part(0), o->part_stride());
   return o;
 }
 
@@ -586,10 +623,16 @@ std::unique_ptr<Ct> ev_galois(Ctx& C, const Ct& a, u64 g) {
   o->scale = a.scale;
   // sigma_g(c1) is switched; sigma_g(c0) is gathered by the ModDown's finishing store
   const size_t per = (size_t)(l + 1) * C.N;
-  DevBuf d(a.batch * per, C.stream);
-  k_automorph(C, a.part(1), 2 * a.part_stride(), d.p, per, a.batch, l + 1, g);
-  DevBuf acc = ks_inner(C, d.p, per, a.batch, l, g);
-  ks_moddown(C, acc, a.batch, l, o->part(0), o->part_stride(), true, false, a.part(0), a.part_stride(), g);
+  Scratch S(C, acc_words(C, a.batch, l) +
+                   std::max(a.batch * per + modup_words(C, a.batch, l), moddown_words(C, a.batch, l)));
+  u64* acc = S.take(acc_words(C, a.batch, l));
+  const size_t mark = S.at;
+  u64* d = S.take(a.batch * per);
+  k_automorph(C, a.part(1), 2 * a.part_stride(), d, per, a.batch, l + 1, g);
+  ks_inner(C, d, per, a.batch, l, g, acc, S.take(modup_words(C, a.batch, l)));
+  S.at = mark;
+  ks_moddown(C, acc, S.take(moddown_words(C, a.batch, l)), a.batch, l, o->part(0), o->part_stride(), true, false,
+             a.part(0), a.part_stride(), g);
   return o;
 }
 
