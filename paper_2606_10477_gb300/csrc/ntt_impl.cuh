@@ -406,8 +406,10 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_shared(Tables T, Limb
 }
 
 // The same first phases with more than three products a word (digits of 4 to 8 primes, 4 to 8 special primes):
-// the tiles would fill the shared memory, so they are read from L2 term by term, all of a thread's words of
-// one term in flight, into open sums (MontAcc) in registers.
+// the tiles would fill the shared memory, so they are read from L2 term by term into open sums (MontAcc) in registers.
+// Three warps a scheduler do not hide L2 by themselves: a thread's words go in two halves, the loads of one in flight
+// while the products of the other are formed (N = 2^16, 3 ciphertexts at level 18, eight primes a digit, seven
+// special ones: ModUp 136 -> 130 us, ModDown with the rescale 145 -> 87 us, as against a term's words at once).
 template <int L1, int L2, int TH, int MINB, int KIND>
 __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_wide(Tables T, LimbSet S, NttAux A) {
   using G = ColGeo<L1, TH>;
@@ -441,40 +443,60 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_wide(Tables T, LimbSe
       s[m] = MontAcc{0, 0};
     }
   };
+  constexpr int H = G::M0 / 2;
+  const u64* last =
+      KIND == LOAD_MODDOWN && A.spread ? A.spread + (size_t)part * A.spread_stride + ((size_t)low << L2) + col : nullptr;
+  u64 x[2][H];
+  auto load = [&](const u64* z, auto half) {
+#pragma unroll
+    for (int m = 0; m < H; ++m) x[half()][m] = z[(size_t)((half() * H + m) * G::M1) << L2];
+  };
+  const auto h0 = std::integral_constant<int, 0>{};
+  const auto h1 = std::integral_constant<int, 1>{};
+  const u64* fp = KIND == LOAD_MODUP ? A.bconv + (size_t)lo * A.ext + li : A.pconv_phat + li;
+  const u64* fbp = KIND == LOAD_MODUP ? fp + A.bconv_b_offset : A.pconv_phat_b + li;
+  const int fld = KIND == LOAD_MODUP ? A.ext : A.pconv_ld;
+  load(base, h0);
+  u64 f = *fp, fb = *fbp;
+#pragma unroll 1
   for (int t = 0; t < ns; ++t) {
-    const u64* z = base + (size_t)t * N;
-    u64 f, fb;
-    if (KIND == LOAD_MODUP) {
-      const u64* bc = A.bconv + ((size_t)j * A.own_alpha + t) * A.ext + li;
-      f = bc[0];
-      fb = bc[A.bconv_b_offset];
-    } else {
-      f = A.pconv_phat[(size_t)t * A.pconv_ld + li];
-      fb = A.pconv_phat_b[(size_t)t * A.pconv_ld + li];
+    const u64 *z = base + (size_t)t * N, *next = t + 1 < ns ? z + N : last;
+    load(z, h1);
+    u64 f_next = 0, fb_next = 0;
+    if (t + 1 < ns) {
+      f_next = fp[(size_t)(t + 1) * fld];
+      fb_next = fbp[(size_t)(t + 1) * fld];
     }
     if (t == 4) close();
-    if (KIND == LOAD_MODUP && !fb) {  // folded into the key
+    auto take = [&](auto half) {
+      if (KIND == LOAD_MODUP && !fb) {  // folded into the key
 #pragma unroll
-      for (int m = 0; m < G::M0; ++m) v[0][m] += z[(size_t)(m * G::M1) << L2];
-    } else {
+        for (int m = 0; m < H; ++m) v[0][half() * H + m] += x[half()][m];
+      } else {
 #pragma unroll
-      for (int m = 0; m < G::M0; ++m) mont_mac(s[m], z[(size_t)(m * G::M1) << L2], f, fb);
-    }
+        for (int m = 0; m < H; ++m) mont_mac(s[half() * H + m], x[half()][m], f, fb);
+      }
+    };
+    take(h0);
+    if (next) load(next, h0);
+    take(h1);
+    f = f_next;
+    fb = fb_next;
   }
+  if (KIND == LOAD_MODDOWN && last) load(last, h1);
   close();
   // at most eight products (below 1.1q each, and 2q of the two steps) or a folded limb and seven: below 16q by the
   // key's construction; brought below 10q, with the bias, the ModDown's constant and the last limb below 12q
 #pragma unroll
   for (int m = 0; m < G::M0; ++m) v[0][m] = off + (v[0][m] >= q * 6 ? v[0][m] - q * 6 : v[0][m]);
-  if (KIND == LOAD_MODDOWN && A.spread) {
-    const u64* last = A.spread + (size_t)part * A.spread_stride + ((size_t)low << L2) + col;
+  if (KIND == LOAD_MODDOWN && last) {
     const u64 ql = T.pr[A.spread_prime].q, half = ql >> 1, sub = q - A.spread_sub[li];
 #pragma unroll
     for (int m = 0; m < G::M0; ++m) {
-      const u64 x = last[(size_t)(m * G::M1) << L2];
+      const u64 y = x[m / H][m % H];
       MontAcc a{0, 0};
-      mont_add(a, x, P.r64);
-      v[0][m] += mont_finish(a, q, P.nqi) + (x > half ? sub : 0);
+      mont_add(a, y, P.r64);
+      v[0][m] += mont_finish(a, q, P.nqi) + (y > half ? sub : 0);
     }
   }
   const ulonglong2* tw = T.psi2 + (size_t)pi * tw_stride(L1, L2);
