@@ -281,12 +281,20 @@ static const DevBuf& key_for(Ctx& C, u64 galois) {
   return it->second;
 }
 // iNTT of the P limbs of the key-switch sums acc [batch][2][ext][N], ModDown, NTT, written to / added
-// into out
-// with c0 (part stride c0_stride): the even parts gain sigma_g(c0), gathered by the finishing store
-// v: workspace of moddown_words
+// into out; v: workspace of moddown_words
 static size_t moddown_words(const Ctx& C, int batch, int l) { return (size_t)batch * 2 * (l + 1) * C.N; }
+// several rotations of one ciphertext at once: sums acc [count][batch][2][ext][N], rotation r's ModDown to out[r] with
+// sigma_gs[r](c0) (part stride c0_stride) added to the even parts, gathered by the finishing store
+struct RotationOut {
+  const u64* c0;
+  size_t c0_stride;
+  int count;
+  u64* out[kKskRotations];
+  u64 gs[kKskRotations];
+};
 static void ks_moddown(Ctx& C, u64* acc, u64* v, int batch, int l, u64* out, size_t out_stride, bool acc0, bool acc1,
-                       const u64* c0 = nullptr, size_t c0_stride = 0, u64 g = 0) {
+                       const RotationOut* R = nullptr) {
+  const int parts = 2 * batch * (R ? R->count : 1);
   const size_t N = C.N, nl = (size_t)l + 1;
   const int K = C.n_p, ext = l + 1 + K;
   // ModDown: the special-prime limbs to the coefficient domain (ending with N^-1 phinv_k when the
@@ -298,8 +306,8 @@ static void ks_moddown(Ctx& C, u64* acc, u64* v, int batch, int l, u64* out, siz
     inv.post = C.d_moddown2.p;
     inv.post_add = C.d_moddown2.p + 2 * K + 1;
   }
-  ntt_inverse(C.tab, LimbSet{acc, (size_t)ext * N, 2 * batch, l + 1, K, l + 1, 0, C.n_q}, C.stream, &inv);
-  if (!fuse) k_moddown_spread(C, acc, v, 2 * batch, l);
+  ntt_inverse(C.tab, LimbSet{acc, (size_t)ext * N, parts, l + 1, K, l + 1, 0, C.n_q}, C.stream, &inv);
+  if (!fuse) k_moddown_spread(C, acc, v, parts, l);
   const u64* Pinv = C.d_moddown2.p + 3 * K + 1 + 2 * (size_t)K * C.n_q;
   NttAux fw{};
   if (fuse) {
@@ -319,10 +327,14 @@ static void ks_moddown(Ctx& C, u64* acc, u64* v, int batch, int l, u64* out, siz
   fw.fin_wb = Pinv + C.n_q;
   fw.fin_acc_even = acc0 ? 1 : 0;
   fw.fin_acc_odd = acc1 ? 1 : 0;
-  fw.fin_d = c0;
-  fw.fin_d_stride = c0_stride;
-  fw.fin_g = g;
-  ntt_forward(C.tab, qset(v, nl * N, 2 * batch, 0, l + 1), C.stream, &fw);
+  if (R) {
+    fw.fin_d = R->c0;
+    fw.fin_d_stride = R->c0_stride;
+    fw.fin_per = 2 * batch;
+    std::copy_n(R->out, R->count, fw.fin_dsts);
+    std::copy_n(R->gs, R->count, fw.fin_gs);
+  }
+  ntt_forward(C.tab, qset(v, nl * N, parts, 0, l + 1), C.stream, &fw);
 }
 
 // The key switch up to the inner product: iNTT of d, the extended digits' forward transform with the
@@ -428,42 +440,47 @@ static void ks_moddown_rescale(Ctx& C, u64* acc, u64* ws, int batch, int l, cons
 // automorphism to them inside the inner product.  The result differs from ev_galois (which
 // converts the rotated c1) by multiples of the digit moduli in the extended basis, within the
 // same noise bound.
-// The inner products of several rotations with the digits y, as many to a launch as the sums' memory allows:
-// about 1 GiB of them at a time (kKskRotations at most), handed to `done(i, acc)` in order.
-template <class F>
-static void hoisted_inner(Ctx& C, const Ct& a, const u64* y, const std::vector<u64>& gs, const u64* c0, size_t chunk,
-                          F done) {
-  const int l = a.level;
-  const size_t words = (size_t)a.batch * 2 * (l + 1 + C.n_p) * C.N, ds = 2 * a.part_stride();
-  for (size_t first = 0; first < gs.size(); first += chunk) {
-    KskInnerArgs A;
-    A.count = (int)std::min(chunk, gs.size() - first);
-    std::vector<DevBuf> acc;
-    for (int r = 0; r < A.count; ++r) {
-      acc.emplace_back(words, C.stream);
-      A.key[r] = key_for(C, gs[first + r]).p;
-      A.acc[r] = acc.back().p;
-      A.g[r] = gs[first + r];
-    }
-    k_ksk_inner(C, y, a.part(1), ds, A, a.batch, l, c0, ds);
-    for (int r = 0; r < A.count; ++r) done(first + r, std::move(acc[r]));
+// The inner products of the rotations gs with the digits y, in one launch: the sums of rotation r go to acc[r].
+// c0: P times its rotation is added to the even parts
+static void hoisted_inner(Ctx& C, const Ct& a, const u64* y, const u64* gs, int count, u64* const* acc, const u64* c0) {
+  KskInnerArgs A;
+  A.count = count;
+  for (int r = 0; r < count; ++r) {
+    A.key[r] = key_for(C, gs[r]).p;
+    A.acc[r] = acc[r];
+    A.g[r] = gs[r];
   }
+  k_ksk_inner(C, y, a.part(1), 2 * a.part_stride(), A, a.batch, a.level, c0, 2 * a.part_stride());
 }
 std::vector<std::unique_ptr<Ct>> ev_galois_hoisted(Ctx& C, const Ct& a, const std::vector<u64>& gs) {
   const int l = a.level;
   for (u64 g : gs) key_for(C, g);
-  Scratch S(C, modup_words(C, a.batch, l) + moddown_words(C, a.batch, l));
+  // as many rotations at a time as about 1 GiB of sums (and 32 K limbs a launch) allows, and one ModDown for all of
+  // them: a rotation's few special limbs alone fill a fraction of the GPU, and its last wave is nearly empty (five
+  // rotations of two ciphertexts, N = 2^16, level 14, 1 / 2 / 3 / 5 at a time: 1074 / 961 / 905 / 836 us)
+  const size_t per = acc_words(C, a.batch, l), limbs = (size_t)2 * a.batch * (l + 1 + C.n_p);
+  const size_t chunk =
+      std::max<size_t>(1, std::min({gs.size(), (size_t)kKskRotations, ((size_t)1 << 27) / per, 32768 / limbs}));
+  Scratch S(C, modup_words(C, a.batch, l) + chunk * (per + moddown_words(C, a.batch, l)));
   const u64* y = ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, l, S.take(modup_words(C, a.batch, l)));
-  u64* v = S.take(moddown_words(C, a.batch, l));
+  u64 *acc = S.take(chunk * per), *v = S.take(chunk * moddown_words(C, a.batch, l));
   std::vector<std::unique_ptr<Ct>> out;
-  const size_t bytes = (size_t)a.batch * 2 * (l + 1 + C.n_p) * C.N * 8;
-  const size_t chunk = std::max<size_t>(1, std::min<size_t>(kKskRotations, ((size_t)1 << 30) / bytes));
-  hoisted_inner(C, a, y, gs, nullptr, chunk, [&](size_t i, DevBuf acc) {
-    auto o = ct_alloc(C, l, a.batch);
-    o->scale = a.scale;
-    ks_moddown(C, acc.p, v, a.batch, l, o->part(0), o->part_stride(), true, false, a.part(0), a.part_stride(), gs[i]);
-    out.push_back(std::move(o));
-  });
+  for (size_t first = 0; first < gs.size(); first += chunk) {
+    RotationOut R{a.part(0), a.part_stride(), (int)std::min(chunk, gs.size() - first), {}, {}};
+    u64* accs[kKskRotations];
+    size_t out_stride = 0;
+    for (int r = 0; r < R.count; ++r) {
+      auto o = ct_alloc(C, l, a.batch);
+      o->scale = a.scale;
+      out_stride = o->part_stride();
+      R.out[r] = o->part(0);
+      R.gs[r] = gs[first + r];
+      accs[r] = acc + r * per;
+      out.push_back(std::move(o));
+    }
+    hoisted_inner(C, a, y, R.gs, R.count, accs, nullptr);
+    ks_moddown(C, acc, v, a.batch, l, R.out[0], out_stride, true, false, &R);
+  }
   return out;
 }
 
@@ -471,8 +488,16 @@ std::vector<DevBuf> ev_galois_hoisted_qp(Ctx& C, const Ct& a, const std::vector<
   for (u64 g : gs) key_for(C, g);
   Scratch S(C, modup_words(C, a.batch, a.level));
   const u64* y = ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, a.level, S.buf.p);
-  std::vector<DevBuf> out(gs.size());  // every sum is kept: one launch for all of them
-  hoisted_inner(C, a, y, gs, a.part(0), kKskRotations, [&](size_t i, DevBuf acc) { out[i] = std::move(acc); });
+  std::vector<DevBuf> out(gs.size());  // every sum is kept: as many rotations to a launch as it takes
+  for (size_t first = 0; first < gs.size(); first += kKskRotations) {
+    const int count = (int)std::min<size_t>(kKskRotations, gs.size() - first);
+    u64* accs[kKskRotations];
+    for (int r = 0; r < count; ++r) {
+      out[first + r] = DevBuf(acc_words(C, a.batch, a.level), C.stream);
+      accs[r] = out[first + r].p;
+    }
+    hoisted_inner(C, a, y, gs.data() + first, count, accs, a.part(0));
+  }
   return out;
 }
 void ev_moddown_into(Ctx& C, DevBuf& acc, int batch, int level, Ct& out) {
@@ -631,8 +656,8 @@ std::unique_ptr<Ct> ev_galois(Ctx& C, const Ct& a, u64 g) {
   k_automorph(C, a.part(1), 2 * a.part_stride(), d, per, a.batch, l + 1, g);
   ks_inner(C, d, per, a.batch, l, g, acc, S.take(modup_words(C, a.batch, l)));
   S.at = mark;
-  ks_moddown(C, acc, S.take(moddown_words(C, a.batch, l)), a.batch, l, o->part(0), o->part_stride(), true, false,
-             a.part(0), a.part_stride(), g);
+  const RotationOut R{a.part(0), a.part_stride(), 1, {o->part(0)}, {g}};
+  ks_moddown(C, acc, S.take(moddown_words(C, a.batch, l)), a.batch, l, o->part(0), o->part_stride(), true, false, &R);
   return o;
 }
 

@@ -134,6 +134,8 @@ struct LimbSet {
   }
 };
 
+constexpr int kKskRotations = 16;  // hoisted rotations of one launch
+
 // Optional fusions of one batched transform (value-initialised: a plain in-place transform).
 struct NttAux {
   // out of place: the first phase reads limb li of part p at src + p * src_stride + li * N
@@ -190,10 +192,13 @@ struct NttAux {
   const u64* fin_w = nullptr;
   const u64* fin_wb = nullptr;
   int fin_acc_even = 0, fin_acc_odd = 0;
-  // with fin_d: what is added is not fin_dst but fin_d[part][li] permuted by the automorphism X -> X^fin_g
+  // with fin_d: the parts are those of several rotations, fin_per each; rotation r's go to fin_dsts[r], and what is added
+  // to them is fin_d[part % fin_per][li] permuted by the automorphism X -> X^fin_gs[r]
   const u64* fin_d = nullptr;
   size_t fin_d_stride = 0;
-  u64 fin_g = 0;
+  int fin_per = 0;
+  u64* fin_dsts[kKskRotations];
+  u64 fin_gs[kKskRotations];
   // with fin_e: a key switch's ModDown fused with the rescale that follows it (see ks_moddown_rescale):
   //   fin_dst[part][li] = fin_c[part][li] * fin_w[li] + (fin_e[part][li] - v) * fin_w2[li]
   // (fin_w = (P q_l)^-1, fin_w2 = q_l^-1), and the first phase loads the ModDown conversion with its
@@ -289,7 +294,6 @@ struct LinCombArgs {
 };
 // one launch of the inner products of hoisted rotations (k_ksk_inner): rotation r by the Galois element g[r] with
 // the key key[r], into acc[r]
-constexpr int kKskRotations = 16;
 struct KskInnerArgs {
   const u64* key[kKskRotations];
   u64* acc[kKskRotations];

@@ -41,7 +41,8 @@ static void dispatch(const Tables& T, const LimbSet& S, cudaStream_t st, bool in
     throw Error(HEDAP_ERR_ARG, "NTT: bad key inner product fusion");
   if (A.own_alpha && (A.own_dn < 1 || A.own_alpha > 8)) throw Error(HEDAP_ERR_ARG, "NTT: bad digit layout");
   if (A.z && (inverse || !A.own_alpha || !A.bconv || !A.bconv_b_offset)) throw Error(HEDAP_ERR_ARG, "NTT: bad ModUp fusion");
-  if (A.fin_d && (!A.fin_dst || A.fin_w2 || !A.fin_g)) throw Error(HEDAP_ERR_ARG, "NTT: bad gathered epilogue fusion");
+  if (A.fin_d && (!A.fin_dst || A.fin_w2 || A.fin_per < 1 || S.n_parts > kKskRotations * A.fin_per || A.fin_acc_odd))
+    throw Error(HEDAP_ERR_ARG, "NTT: bad gathered epilogue fusion");
   if (A.post_add && !A.post) throw Error(HEDAP_ERR_ARG, "NTT: constants after the final factors need these");
   if (A.post && !inverse) throw Error(HEDAP_ERR_ARG, "NTT: post factors apply to the inverse only");
   if ((A.pre_scale || A.pre_e) && (!inverse || !A.pre_scale)) throw Error(HEDAP_ERR_ARG, "NTT: a fused sum on load applies to the inverse only");

@@ -577,7 +577,8 @@ __device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u
     }
   } else if (A.fin_dst) {  // fused epilogue of a rescale / ModDown: (c - v) * w (+ dst)
     const u64* cp = A.fin_c + (size_t)part * A.fin_c_stride + at;
-    u64* dp = A.fin_dst + (size_t)part * A.fin_dst_stride + at;
+    const int r = A.fin_d ? part / A.fin_per : 0, rp = part - r * A.fin_per;
+    u64* dp = (A.fin_d ? A.fin_dsts[r] : A.fin_dst) + (size_t)rp * A.fin_dst_stride + at;
     const u64 w = A.fin_w[li], wb = A.fin_wb[li];
     auto fin = [&](u64 c, u64 v) {  // below 3q
       u64 z = mont_mul_lazy(fwd_minus<SMALL>(c, v, q), w, wb, q, P.nqi);
@@ -595,8 +596,8 @@ __device__ __forceinline__ void fwd_rows_store(const u64* xs, const NttAux& A, u
       if (acc) {
         ulonglong2 d;
         if (A.fin_d) {
-          const u64* limb = A.fin_d + (size_t)part * A.fin_d_stride + (at - n0);
-          d = galois_pair(limb, galois_index(n0 + 2 * e, A.fin_g, LOGN));
+          const u64* limb = A.fin_d + (size_t)rp * A.fin_d_stride + (at - n0);
+          d = galois_pair(limb, galois_index(n0 + 2 * e, A.fin_gs[r], LOGN));
         } else {
           d = ldg2(dp + 2 * e);
         }

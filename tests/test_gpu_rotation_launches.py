@@ -35,6 +35,24 @@ def test_hoisted_rotations_of_a_batch():
             assert np.array_equal(g.unpack(a, k).limbs(), b.limbs()), k
 
 
+@pytest.mark.parametrize("log_n,n_q,n_p,alpha,batch,count", [
+    (13, 8, 2, 2, 3, 5),   # more than 2^21 words: column and row launches over the parts of all rotations
+    (13, 8, 2, 2, 1, 17),  # 16 rotations at once and one by itself
+    (10, 10, 8, 8, 2, 3),  # the most special primes a chain may have
+])
+def test_hoisted_moddown_of_several_rotations(log_n, n_q, n_p, alpha, batch, count):
+    """Every rotation of a batch against the oracle's rotations of its members."""
+    args = (log_n, [50] * n_q, [60] * n_p, alpha, 50, 64, 1)
+    g, o = hedap.Context(*args), oracle.Context(*args)
+    level = n_q - 1
+    x = [inputs.random_ciphertext_limbs(50 + k, o.primes(), level, o.N) for k in range(batch)]
+    steps = [k - 1 for k in range(count)]
+    rot = g.rotate_hoisted(g.pack([g.ct_import(v, level, o.scale) for v in x]), steps)
+    for k, v in enumerate(x):
+        for a, b in zip(rot, o.rotate_hoisted(o.ct_import(v, level, o.scale), steps)):
+            assert np.array_equal(g.unpack(a, k).limbs(), b.limbs()), k
+
+
 @pytest.mark.parametrize("inverse", [True, False])
 def test_diagonal_products_past_one_launch(inverse):
     """One grouped factor over all 512 slots: 64 giant steps of 16 baby steps."""
