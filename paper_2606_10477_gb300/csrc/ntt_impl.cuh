@@ -25,7 +25,7 @@
 //    other primes reduce the first operand at every other stage (below 12q).  Inverse: for 1.5 2^32 <= q < 2^55
 //    bounds double unreduced through a phase.
 // GB300, N = 2^16, against Shoup butterflies in radix-8 passes with a CTA barrier each: forward of 384 limbs
-// 304 -> 222 us, HMult with rescale of 8 ciphertexts at level 23 3.28 -> 2.37 ms.  The big kernels then issue
+// 304 -> 216 us, HMult with rescale of 8 ciphertexts at level 23 3.28 -> 2.30 ms.  The big kernels then issue
 // 0.45 - 0.47 instructions a cycle with the multiply pipe 68 - 78% busy, as the register loop of the
 // butterfly itself does (0.48 and 82%): what is left is their instruction count.
 // Optional fusions (NttAux): the first phase may read another buffer (out of place) or compute its
@@ -1225,7 +1225,7 @@ static void allow_smem(Kernel kern, size_t bytes) {
   if (bytes > 48 * 1024)
     HEDAP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
 }
-// fused row phase: 4 warps a CTA and 168 registers (3 CTAs an SM): 908 us for 8 x 12 digits at level 23, against
+// fused row phase: 4 warps a CTA and 168 registers (3 CTAs an SM): 859 us for 8 x 12 digits at level 23, against
 // 1195 us of the 128-thread CTAs with three barriers a digit
 constexpr int kKskWarps = 4, kKskMinBlocks = 3;
 
