@@ -60,7 +60,7 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
   const size_t N = C->N;
 
   // NTT tables: (w 2^32, w 2^64) mod q of w = psi^bitrev(i) and psi^-bitrev(i), in the transforms' order (Tables)
-  const int l1 = C->log_n / 2, l2 = C->log_n - l1;
+  const int l1 = ntt_l1(C->log_n), l2 = C->log_n - l1;
   const size_t TS = tw_stride(l1, l2);
   std::vector<u64> psi2(2 * T * TS), ipsi2(2 * T * TS), ninv(T), ninv_sh(T);
   std::vector<u64> pw(N), ipw(N);

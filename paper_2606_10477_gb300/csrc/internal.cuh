@@ -82,14 +82,17 @@ struct DevBuf {
 };
 
 // ------------------------------------------------------------------ tables and limb sets
-// Twiddles of one prime, N = 2^(L1+L2), L1 = floor(log2 N / 2): first the column phase's (stages 0 .. L1-1), then
+// A transform of N = 2^(L1+L2) words is a column phase of L1 stages and a row phase of L2 (ntt_impl.cuh): halves, the
+// odd stage in the row phase, except at 2^17, whose row phase stays that of 2^16.
+__host__ __device__ constexpr int ntt_l1(int log_n) { return log_n == 17 ? 9 : log_n / 2; }
+// Twiddles of one prime, N = 2^(L1+L2): first the column phase's (stages 0 .. L1-1), then
 // a run of 2^L2 for each of the 2^L1 blocks of the row phase.  Within a phase of L stages the twiddle of stage s,
 // sub-block r has tree index 2^s + r; tw_slot gives its place, so that the lanes of a warp, one group each,
-// read consecutive pairs: the first K0 = ceil(L/2) stages in tree order, then entry by entry (stage K0 + u, sub-block
-// mm of a group) over the 2^K0 groups.  Slot 0 of a run is unused.
+// read consecutive pairs: the K0 stages before the last pass (ceil(L/2); 6 for L = 9) in tree order, then entry by entry
+// (stage K0 + u, sub-block mm of a group) over the 2^K0 groups.  Slot 0 of a run is unused.
 __host__ __device__ constexpr size_t tw_stride(int l1, int l2) { return ((size_t)1 << (l1 + l2)) + ((size_t)1 << l1); }
 inline uint32_t tw_slot(int l, uint32_t tree) {
-  const int k0 = (l + 1) / 2;
+  const int k0 = l == 9 ? 6 : (l + 1) / 2;
   if (tree < (1u << k0)) return tree;
   const int s = 31 - __builtin_clz(tree), u = s - k0;
   const uint32_t r = tree - (1u << s);

@@ -13,7 +13,7 @@
 // butterfly as it can.
 //  * A phase of L stages is two register passes of K0 = ceil(L / 2) and K1 = floor(L / 2) stages
 //    (radix 16 twice for L = 8) with one exchange through shared memory between them, every thread
-//    holding 2^K0 words of a column or a block.  The 2^K1 threads of one block lie in one warp: the row phase
+//    holding 2^K0 words of a column or a block (2^17: L1 = 9 in three passes of 8 words, ColGeo; L2 stays 8).  The 2^K1 threads of one block lie in one warp: the row phase
 //    has no CTA barrier.
 //  * The first pass of the column phase and the last one read and write global memory from
 //    registers (8 adjacent columns a CTA: whole 32-byte sectors).
@@ -148,19 +148,31 @@ struct Phase {
   static constexpr int GP = 1 << (K0 - K1);         // pass-1 groups a thread owns
   static constexpr int PER = 32 >> K1;              // blocks a warp holds
 };
-// column phase, a CTA of TH threads, one column a thread: word c of column cg at (c + (c >> K1)) COLS + cg (a row of
-// padding every 2^K1 rows, so that pass 1's reads are free of bank conflicts)
+// column phase, a CTA of TH threads, one column a thread, TPC threads a column: the first pass holds words m TPC + low
+// (m < M0), the last one words (i TPC + low) M1 + m (i < GP, m < M1).  Word c of column cg at (c + (c >> K1)) COLS + cg (a
+// row of padding every 2^K1 rows, so that the last pass's reads are free of bank conflicts).
+// The 2^9 rows of N = 2^17 take three passes of three stages, 8 words a thread.  With 2^9 words in the row phase instead, a
+// thread held 32 words, or 16 with their 128-bit key sums, and both spilled (the key product's 912 bytes a thread): forward
+// of 160 limbs 312 -> 219 us (primes of 60 bits 363 -> 237 us), HMult of 8 ciphertexts at level 7 1263 -> 1006 us, of one
+// 273 -> 175 us, rescale of 8 at level 8 with 58-bit primes 465 -> 291 us.
 template <int L1, int TH>
-struct ColGeo : Phase<L1> {
-  using P = Phase<L1>;
-  static constexpr int COLS = TH >> P::K1;
-  static constexpr int XWORDS = ((1 << L1) + P::M0) * COLS;  // exchange
-  static constexpr int TILE = (1 << L1) * COLS;              // one staged tile
+struct ColGeo {
+  static constexpr bool THREE = L1 == 9;
+  static constexpr int K0 = THREE ? 3 : Phase<L1>::K0, K1 = THREE ? 3 : Phase<L1>::K1;
+  static constexpr int M0 = 1 << K0, M1 = 1 << K1, TPC = (1 << L1) / M0;
+  static constexpr int GP = M0 / M1;
+  static constexpr int COLS = TH / TPC;
+  static constexpr int XWORDS = ((1 << L1) + (1 << (L1 - K1))) * COLS;  // exchange
+  static constexpr int TILE = (1 << L1) * COLS;                         // one staged tile
+  // row of word c in the exchange, additive over numbers without a common bit; of a thread's offset low < TPC
+  static __device__ constexpr int row(int c) { return c + (c >> K1); }
+  static __device__ constexpr int low_row(int low) { return THREE ? row(low) : low; }
 };
 // row phase, per warp: PER blocks, two words of padding every 2^K1 words (LDS.128 of consecutive words is free
 // of bank conflicts) and 2^K1 after each block when several blocks share a half-warp
 template <int L2>
 struct RowGeo : Phase<L2> {
+  static_assert(L2 <= 8, "at most 16 words a thread; the inverse's 2^(L2+1) q stay below 2^64");
   using P = Phase<L2>;
   static constexpr int GS = P::M1 + 2;                                           // stride of a group
   static constexpr int BS = P::M0 * GS + (P::K1 < 4 ? P::M1 : 0);                // stride of a block
@@ -286,31 +298,42 @@ struct FusedLoad {
 };
 
 // ---------------------------------------------------------------- forward, column phase
-// both passes of one limb's columns: v holds pass 0's input (row m 2^K1 + low), o pass 1's output (row
-// (i 2^K1 + low) 2^K1 + m of this thread's column); tw: global memory (L1) or shared memory
+// all passes of one limb's columns: v holds the first pass's input (row m TPC + low), o the last one's output (row
+// (i TPC + low) M1 + m of this thread's column); tw: global memory (L1) or shared memory
 template <bool SMALL, int L1, int TH>
-__device__ __forceinline__ void fwd_cols_passes(u64 (&v)[1][1 << Phase<L1>::K0], u64* xs, const ulonglong2* tw, u64 q,
+__device__ __forceinline__ void fwd_cols_passes(u64 (&v)[1][ColGeo<L1, TH>::M0], u64* xs, const ulonglong2* tw, u64 q,
                                                 uint32_t nqi, int low, int cg,
-                                                u64 (&o)[Phase<L1>::GP][1][1 << Phase<L1>::K1]) {
+                                                u64 (&o)[ColGeo<L1, TH>::GP][1][ColGeo<L1, TH>::M1]) {
   using G = ColGeo<L1, TH>;
   fwd_pass<SMALL, 0, G::K0, 1>(v, q, nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
   __syncthreads();  // the last limb's exchange has been read
 #pragma unroll
-  for (int m = 0; m < G::M0; ++m) xs[(m * (G::M1 + 1) + low) * G::COLS + cg] = v[0][m];
+  for (int m = 0; m < G::M0; ++m) xs[(G::row(m * G::TPC) + G::low_row(low)) * G::COLS + cg] = v[0][m];
   __syncthreads();
+  if constexpr (G::THREE) {  // the middle pass: rows hi 64 + m 8 + low % 8
+    const int hi = low >> 3;
+    u64* x = xs + (hi * G::row(64) + (low & 7)) * G::COLS + cg;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) v[0][m] = x[G::row(m * 8) * G::COLS];
+    fwd_pass<SMALL, 3, 3, 1>(v, q, nqi, [&](int u, int mm) { return tw[(8 << u) + (hi << u) + mm]; });
+#pragma unroll
+    for (int m = 0; m < 8; ++m) x[G::row(m * 8) * G::COLS] = v[0][m];
+    __syncthreads();
+  }
 #pragma unroll
   for (int i = 0; i < G::GP; ++i) {
-    const int hi = i * G::M1 + low;  // rows hi 2^K1 + m
+    const int hi = i * G::TPC + low;  // rows hi 2^K1 + m
 #pragma unroll
     for (int m = 0; m < G::M1; ++m) o[i][0][m] = xs[(hi * (G::M1 + 1) + m) * G::COLS + cg];
-    fwd_pass<SMALL, G::K0, G::K1, 1>(o[i], q, nqi, [&](int u, int mm) {
-      return tw[G::M0 + ((1 << u) - 1 + mm) * G::M0 + hi];
+    constexpr int GROUPS = 1 << (L1 - G::K1);
+    fwd_pass<SMALL, L1 - G::K1, G::K1, 1>(o[i], q, nqi, [&](int u, int mm) {
+      return tw[GROUPS + ((1 << u) - 1 + mm) * GROUPS + hi];
     });
   }
 }
 // the same, the output stored to global memory: out at (row 0, this thread's column)
 template <bool SMALL, int L1, int L2, int TH>
-__device__ __forceinline__ void fwd_cols_body(u64 (&v)[1][1 << Phase<L1>::K0], u64* xs, const ulonglong2* tw, u64 q,
+__device__ __forceinline__ void fwd_cols_body(u64 (&v)[1][ColGeo<L1, TH>::M0], u64* xs, const ulonglong2* tw, u64 q,
                                               uint32_t nqi, int low, int cg, u64* out) {
   using G = ColGeo<L1, TH>;
   u64 o[G::GP][1][G::M1];
@@ -318,7 +341,7 @@ __device__ __forceinline__ void fwd_cols_body(u64 (&v)[1][1 << Phase<L1>::K0], u
 #pragma unroll
   for (int i = 0; i < G::GP; ++i)
 #pragma unroll
-    for (int m = 0; m < G::M1; ++m) out[(size_t)((i * G::M1 + low) * G::M1 + m) << L2] = o[i][0][m];
+    for (int m = 0; m < G::M1; ++m) out[(size_t)((i * G::TPC + low) * G::M1 + m) << L2] = o[i][0][m];
 }
 template <int N, int TH>  // N twiddles into shared memory
 __device__ __forceinline__ void stage_twiddles(ulonglong2* dst, const ulonglong2* src, int t) {
@@ -345,7 +368,7 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols(Tables T, LimbSet S, 
   grid_wait();
   u64 v[1][G::M0];
 #pragma unroll
-  for (int m = 0; m < G::M0; ++m) v[0][m] = src[(size_t)(m * G::M1 + low) << L2] + bias;
+  for (int m = 0; m < G::M0; ++m) v[0][m] = src[(size_t)(m * G::TPC + low) << L2] + bias;
   cp_async_wait_all();
   __syncthreads();
   u64* out = S.limb(part, li, N) + col;
@@ -396,7 +419,7 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_shared(Tables T, Limb
     const u64* zl = zt + low * G::COLS + cg;
     F.apply([&](auto word) {
 #pragma unroll
-      for (int m = 0; m < G::M0; ++m) v[0][m] = word([&](int t) { return zl[t * G::TILE + m * G::M1 * G::COLS]; });
+      for (int m = 0; m < G::M0; ++m) v[0][m] = word([&](int t) { return zl[t * G::TILE + m * G::TPC * G::COLS]; });
     });
     const ulonglong2* tw = T.psi2 + (size_t)pi * tw_stride(L1, L2);
     u64* out = S.limb(part, li, N) + col + cg;
@@ -449,7 +472,7 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_wide(Tables T, LimbSe
   u64 x[2][H];
   auto load = [&](const u64* z, auto half) {
 #pragma unroll
-    for (int m = 0; m < H; ++m) x[half()][m] = z[(size_t)((half() * H + m) * G::M1) << L2];
+    for (int m = 0; m < H; ++m) x[half()][m] = z[(size_t)((half() * H + m) * G::TPC) << L2];
   };
   const auto h0 = std::integral_constant<int, 0>{};
   const auto h1 = std::integral_constant<int, 1>{};
@@ -684,7 +707,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_fwd_rows(Tables T, LimbSet
 // q < 2^60.1: the sum of up to 64 products stays below 2^128.
 template <int L2>
 struct KskGeo {
-  static constexpr int PER = L2 > 8 ? (1 << (L2 - 5)) : 8;  // words a lane
+  static constexpr int PER = 8;                             // words a lane
   static constexpr int LPB = (1 << L2) / PER;               // lanes a block
   static constexpr int KB = 32 / LPB;                       // blocks a warp
   // passes: a first one of F stages, then passes of 3
@@ -893,12 +916,7 @@ __device__ __forceinline__ void inv_rows_passes(u64 (&v)[1][1 << Phase<L2>::K0],
   __syncwarp();
 #pragma unroll
   for (int m = 0; m < G::M0; ++m) v[0][m] = xs[m * G::GS + low];
-  constexpr bool MID = SMALL && 1 + L2 > 9;  // 2^(L2+1) q would pass 2^64: reduce between the passes
-  if constexpr (MID) {
-#pragma unroll
-    for (int m = 0; m < G::M0; ++m) v[0][m] = reduce_lazy(v[0][m], q, P.rc);
-  }
-  inv_pass<SMALL, MID ? 1 : 1 + G::K1, G::K0, 1>(v, q, P.nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
+  inv_pass<SMALL, 1 + G::K1, G::K0, 1>(v, q, P.nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
 }
 // a block's words from global memory into the exchange buffer: j0 the block's first word of the limb
 template <int L2>
@@ -960,30 +978,45 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_inv_rows(Tables T, LimbSet
 
 // ---------------------------------------------------------------- inverse, column phase (+ N^-1)
 template <bool SMALL, int L1, int L2, int TH>
-__device__ __forceinline__ void inv_cols_body(u64 (&w)[Phase<L1>::GP][1][1 << Phase<L1>::K1], u64* a, u64* xs,
+__device__ __forceinline__ void inv_cols_body(u64 (&w)[ColGeo<L1, TH>::GP][1][ColGeo<L1, TH>::M1], u64* a, u64* xs,
                                               const ulonglong2* tw, const PrimeDev& P, int low, int cg, u64 ni, u64 nip, u64 add) {
   using G = ColGeo<L1, TH>;
   const u64 q = P.q;
 #pragma unroll
   for (int i = 0; i < G::GP; ++i) {
-    const int hi = i * G::M1 + low;
+    const int hi = i * G::TPC + low;
     if constexpr (SMALL) {
 #pragma unroll
       for (int m = 0; m < G::M1; ++m) w[i][0][m] = reduce_lazy(w[i][0][m], q, P.rc);
     }
+    constexpr int GROUPS = 1 << (L1 - G::K1);
     inv_pass<SMALL, 1, G::K1, 1>(w[i], q, P.nqi, [&](int u, int mm) {
-      return tw[G::M0 + ((1 << u) - 1 + mm) * G::M0 + hi];
+      return tw[GROUPS + ((1 << u) - 1 + mm) * GROUPS + hi];
     });
 #pragma unroll
     for (int m = 0; m < G::M1; ++m) xs[(hi * (G::M1 + 1) + m) * G::COLS + cg] = w[i][0][m];
   }
   __syncthreads();
   u64 v[1][G::M0];
+  if constexpr (G::THREE) {  // the middle pass, as in fwd_cols_passes
+    const int hi = low >> 3;
+    u64* x = xs + (hi * G::row(64) + (low & 7)) * G::COLS + cg;
 #pragma unroll
-  for (int m = 0; m < G::M0; ++m) v[0][m] = xs[(m * (G::M1 + 1) + low) * G::COLS + cg];
-  inv_pass<SMALL, 1 + G::K1, G::K0, 1>(v, q, P.nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
+    for (int m = 0; m < 8; ++m) v[0][m] = x[G::row(m * 8) * G::COLS];
+    inv_pass<SMALL, 1 + G::K1, 3, 1>(v, q, P.nqi, [&](int u, int mm) { return tw[(8 << u) + (hi << u) + mm]; });
 #pragma unroll
-  for (int m = 0; m < G::M0; ++m) a[(size_t)(m * G::M1 + low) << L2] = add_mod(shoup_mul(v[0][m], ni, nip, q), add, q);
+    for (int m = 0; m < 8; ++m) x[G::row(m * 8) * G::COLS] = v[0][m];
+    __syncthreads();
+  }
+#pragma unroll
+  for (int m = 0; m < G::M0; ++m) v[0][m] = xs[(G::row(m * G::TPC) + G::low_row(low)) * G::COLS + cg];
+  if constexpr (SMALL && G::THREE) {  // nine doublings of 2q would pass 2^64
+#pragma unroll
+    for (int m = 0; m < G::M0; ++m) v[0][m] = reduce_lazy(v[0][m], q, P.rc);
+  }
+  inv_pass<SMALL, G::THREE ? 1 : 1 + G::K1, G::K0, 1>(v, q, P.nqi, [&](int u, int mm) { return tw[(1 << u) + mm]; });
+#pragma unroll
+  for (int m = 0; m < G::M0; ++m) a[(size_t)(m * G::TPC + low) << L2] = add_mod(shoup_mul(v[0][m], ni, nip, q), add, q);
 }
 template <int L1, int L2, int TH, int MINB>
 __global__ void __launch_bounds__(TH, MINB) k_ntt_inv_cols(Tables T, LimbSet S, NttAux A) {
@@ -1004,7 +1037,7 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_inv_cols(Tables T, LimbSet S, 
 #pragma unroll
   for (int i = 0; i < G::GP; ++i)
 #pragma unroll
-    for (int m = 0; m < G::M1; ++m) w[i][0][m] = a[(size_t)((i * G::M1 + low) * G::M1 + m) << L2];
+    for (int m = 0; m < G::M1; ++m) w[i][0][m] = a[(size_t)((i * G::TPC + low) * G::M1 + m) << L2];
   const int r = li - S.limb_begin;
   const u64 ni = A.post ? A.post[2 * r] : T.ninv[pi], nip = A.post ? A.post[2 * r + 1] : T.ninv_sh[pi];
   const u64 add = A.post_add ? A.post_add[r] : 0;
@@ -1249,10 +1282,10 @@ template <int L1, int L2, int WW, int WPS>
 static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool inverse, const NttAux& A,
                         const KskFuse* F) {
   using RG = RowGeo<L2>;
-  constexpr int TH = std::min(32 * WW, (1 << L2) << Phase<L1>::K1);  // column phase: threads per CTA
+  constexpr int TH = L1 == 9 ? 256 : std::min(32 * WW, (1 << L2) << Phase<L1>::K1);  // column phase: threads per CTA
   using CG = ColGeo<L1, TH>;
   constexpr int RW = std::min(WW, (1 << L1) / RG::PER);              // row phase: warps per CTA
-  constexpr int CB = std::max(1, WPS * 32 / TH), RB = std::max(1, WPS / RW);
+  constexpr int CB = std::max(1, (WPS * 32 + TH - 1) / TH), RB = std::max(1, WPS / RW);
   const dim3 gc((unsigned)((1 << L2) / CG::COLS), (unsigned)(S.n_parts * S.n_limbs));
   const unsigned rx = (unsigned)((1 << L1) / RG::PER / RW);
   constexpr size_t smem_x = (size_t)CG::XWORDS * 8, smem_c = smem_x + ((size_t)16 << L1);
@@ -1289,7 +1322,7 @@ static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool
       else if (A.pconv) launch(k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_MODDOWN>, g2, dim3(TH), smem, st, T, S, A, lpc);
       else launch(k_ntt_fwd_cols_shared<L1, L2, TH, CB, LOAD_SPREAD>, g2, dim3(TH), smem, st, T, S, A, lpc);
     } else if (n_prod > 3) {
-      constexpr int WB = std::max(1, 12 * 32 / TH);
+      constexpr int WB = std::max(1, (L1 == 9 ? 16 : 12) * 32 / TH);
       if (A.z) launch(k_ntt_fwd_cols_wide<L1, L2, TH, WB, LOAD_MODUP>, gc, dim3(TH), smem_x, st, T, S, A);
       else launch(k_ntt_fwd_cols_wide<L1, L2, TH, WB, LOAD_MODDOWN>, gc, dim3(TH), smem_x, st, T, S, A);
     } else {
