@@ -322,8 +322,8 @@ API hedap_status hedap_ntt(hedap_ctx* ctx, uint64_t* limbs, size_t n_limbs, uint
     const size_t words = n_limbs * C.N;
     hedap::DevBuf tmp;
     uint64_t* d = limbs;
-    // the transforms load and store 16 bytes: words at an 8-byte boundary go through a buffer
-    const bool staged = !on_device || ((uintptr_t)limbs & 15);
+    // the transforms take limbs at any 8-byte boundary; others go through a buffer
+    const bool staged = !on_device || ((uintptr_t)limbs & 7);
     if (staged) {
       tmp = hedap::DevBuf(words, C.stream);
       HEDAP_CUDA(cudaMemcpyAsync(tmp.p, limbs, words * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
@@ -596,8 +596,8 @@ API hedap_status hedap_ntt_batch(hedap_ctx* ctx, uint64_t* limbs, size_t n_limbs
     const size_t words = n_polys * n_limbs * C.N;
     hedap::DevBuf tmp;
     uint64_t* d = limbs;
-    // the transforms load and store 16 bytes: words at an 8-byte boundary go through a buffer
-    const bool staged = !on_device || ((uintptr_t)limbs & 15);
+    // the transforms take limbs at any 8-byte boundary; others go through a buffer
+    const bool staged = !on_device || ((uintptr_t)limbs & 7);
     if (staged) {
       tmp = hedap::DevBuf(words, C.stream);
       HEDAP_CUDA(cudaMemcpyAsync(tmp.p, limbs, words * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
