@@ -539,7 +539,8 @@ hedap_status hedap_ntt_get_role_variant(const hedap_ctx* ctx, int role, int* var
 /* Profiling (process-wide, not part of the paper's interface).
  * hedap_profile_enable(1) resets the counters and, until disabled, records a
  * CUDA event pair around every launch group of these kernel classes:
- * "ntt" (one forward or inverse transform of a limb batch: two launches),
+ * "ntt" (one forward or inverse transform of a limb batch: two launches, one
+ * where a whole limb fits a thread-block cluster),
  * "modup", "ksk_inner", "moddown", "tensor", "rescale", "automorph",
  * "elementwise".  hedap_profile_read synchronises and returns, for one class,
  * the number of timed groups, their summed event time in ms, and their summed

@@ -73,7 +73,6 @@ static void dispatch(const Tables& T, const LimbSet& S, cudaStream_t st, bool in
   if (A.pconv) slots += limbs * n * (8.0 * A.pconv_K + 5.0);
   prof_.slots = slots;
   if (F) prof_.slots += 8.0 * 2.0 * F->batch * (double)S.n_limbs * A.own_dn * n;
-  prof_count_launches(2);
   ntt_launch(T.log_n, v, S, T, st, inverse, A, F);
 }
 

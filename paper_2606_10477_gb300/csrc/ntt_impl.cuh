@@ -1260,6 +1260,7 @@ static bool launch_whole(const LimbSet& S, const Tables& T, cudaStream_t st, boo
     else if (A.spread) launch(k_ntt_fwd_whole<L1, L2, LOAD_SPREAD>, g, dim3(W::TH), W::SMEM, st, T, S, A);
     else launch(k_ntt_fwd_whole<L1, L2, LOAD_PLAIN>, g, dim3(W::TH), W::SMEM, st, T, S, A);
     HEDAP_LAUNCH_CHECK();
+    prof_count_launches(1);
     return true;
   }
   return false;
@@ -1375,6 +1376,7 @@ static void launch_pair(const LimbSet& S, const Tables& T, cudaStream_t st, bool
     launch(k_ntt_inv_cols<L1, L2, TH, CB>, gc, dim3(TH), smem_c, st, T, S, A2);
   }
   HEDAP_LAUNCH_CHECK();
+  prof_count_launches(2);
 }
 
 template <int L1, int L2>
