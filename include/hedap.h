@@ -512,7 +512,9 @@ void hedap_graph_destroy(hedap_graph* g);
  * conversion (HEDAP_NTT_ROLE_MODUP) or a fused ModDown / rescale
  * (HEDAP_NTT_ROLE_FINISH) are then tuned apart, each on an HMult with rescale of a
  * batch of 4 ciphertexts at the top level (when the relinearisation key exists);
- * hedap_ntt_get_role_variant reports their choices. */
+ * hedap_ntt_get_role_variant reports their choices.  Rings up to 2^13 use the
+ * shapes for transforms of more than 2^21 words (smaller ones run as thread-block
+ * clusters); the tuner times the shapes there too. */
 hedap_status hedap_ntt_tune(hedap_ctx* ctx, int limbs, int reps, float* fwd_ms, float* inv_ms, int cap,
                             int* fwd_variant, int* inv_variant);
 /* Butterflies per second of a register-only loop of the NTT's butterfly (no

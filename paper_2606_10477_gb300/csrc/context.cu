@@ -1,6 +1,7 @@
 // Context creation (prime chain, NTT tables, RNS constants), key generation,
 // encoding (CKKS canonical embedding over the 5^j orbit, FP64 on the host),
 // encryption and decryption.
+#include <algorithm>
 #include <cmath>
 #include <complex>
 
@@ -104,7 +105,7 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
   upload(*C, C->d_ninv, ninv);
   upload(*C, C->d_ninv_sh, ninv_sh);
   C->tab = Tables{(const PrimeDev*)C->d_primes.p, (const ulonglong2*)C->d_psi2.p, (const ulonglong2*)C->d_ipsi2.p,
-                  C->d_ninv.p, C->d_ninv_sh.p, C->log_n, 3, 3, 3, 3};
+                  C->d_ninv.p, C->d_ninv_sh.p, C->log_n, 3, 3, 3, 3, true};
 
   // P = prod p_k; ModDown constants and P mod q_t
   const int K = C->n_p, nq = C->n_q;
@@ -231,7 +232,8 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
   upload(*C, C->d_sk, skr);
   ntt_forward(C->tab, LimbSet{C->d_sk.p, 0, 1, 0, T, nq, 0, nq}, C->stream);
   gen_galois_key(*C, 0);
-  ntt_tune(*C, 8 * C->n_q, 2, nullptr, nullptr);  // pick the NTT launch shape for this ring
+  // pick the NTT launch shape for this ring, on as many limbs as a call has that runs in these shapes (ntt_whole_limb)
+  ntt_tune(*C, std::max(8 * C->n_q, C->log_n <= 13 ? (int)(kWholeLimbWords >> C->log_n) + C->n_q : 0), 2, nullptr, nullptr);
   HEDAP_CUDA(cudaStreamSynchronize(C->stream));
   return C.release();
 }

@@ -343,7 +343,7 @@ static void ks_moddown(Ctx& C, u64* acc, u64* v, int batch, int l, u64* out, siz
 static void ks_inner(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64 galois, u64* acc, u64* ws) {
   const DevBuf& key = key_for(C, galois);
   const int T = C.total_primes();
-  if (C.log_n <= 13 && C.alpha <= 3 && ((size_t)batch * (l + 1 + C.n_p) << C.log_n) <= (size_t)1 << 18) {
+  if (C.tab.small_routes && C.log_n <= 13 && C.alpha <= 3 && ((size_t)batch * (l + 1 + C.n_p) << C.log_n) <= (size_t)1 << 18) {
     // a small ring's few limbs: the digits transformed in one launch, all of them at once, and the inner product in
     // a second; fused, one warp for 256 words would walk the digits one after the other with fewer than 1024
     // warps on the GPU (N = 2^12, HMult: 12 digits of 3 ciphertexts, 160 K words a digit, 65 against 71 us;

@@ -112,6 +112,9 @@ struct Tables {
   int ntt_inv_variant;
   int ntt_modup_variant;
   int ntt_fin_variant;
+  // small rings take their routes for a few limbs (a whole limb per cluster, the separate key inner product); off while
+  // ntt_tune times the launch shapes, which those routes do not have
+  bool small_routes;
 };
 constexpr int kNttVariants = 8, kNttShapes = 2;  // variants v and v + kNttShapes are one launch shape
 enum NttRole { NTT_ROLE_FORWARD = 0, NTT_ROLE_INVERSE = 1, NTT_ROLE_MODUP = 2, NTT_ROLE_FINISH = 3 };
@@ -252,11 +255,13 @@ struct KskFuse {
 void ntt_forward(const Tables& T, const LimbSet& S, cudaStream_t st, const NttAux* aux = nullptr,
                  const KskFuse* fuse = nullptr);
 void ntt_inverse(const Tables& T, const LimbSet& S, cudaStream_t st, const NttAux* aux = nullptr);
-// whether a transform of `limbs` limbs at N = 2^log_n with n_prod products a word in its load runs with a whole limb
+// whether a transform of `limbs` limbs at N = 2^T.log_n with n_prod products a word in its load runs with a whole limb
 // per cluster (ntt_impl.cuh): up to 2^21 words in all (a rescale of 8 ciphertexts of 21 limbs at N = 2^12, 1.4 M words,
 // 25.7 us against 29.1 us); beyond, the two-launch kernels carry more at a time
-inline bool ntt_whole_limb(int log_n, size_t limbs, int n_prod) {
-  return log_n <= 13 && n_prod <= 3 && (limbs << log_n) <= (size_t)1 << 21;
+constexpr size_t kWholeLimbWords = (size_t)1 << 21;
+inline bool ntt_whole_limb(const Tables& T, size_t limbs, int n_prod) {
+  const int log_n = T.log_n;
+  return T.small_routes && log_n <= 13 && n_prod <= 3 && (limbs << log_n) <= kWholeLimbWords;
 }
 struct Ctx;
 void ntt_tune(Ctx& C, int limbs, int reps, std::vector<float>* fwd_ms, std::vector<float>* inv_ms);

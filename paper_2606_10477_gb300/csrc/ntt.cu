@@ -140,12 +140,13 @@ int& ntt_role_variant(Tables& T, int role) {
   }
 }
 
-// Time every variant on `limbs` limbs of scratch (forward and inverse separately, best of `reps` after
+// Time every launch shape on `limbs` limbs of scratch (forward and inverse separately, best of `reps` after
 // one warm-up) and keep the fastest in C.tab.  The fused roles run other code around the same passes
 // (the ModUp conversion, the ModDown / rescale finish), and the shape that suits the plain transform
 // need not suit them, so when the relinearisation key exists they are tuned on what they serve: an
 // HMult with rescale of a batch of 4 at the top level (tensor, key switch, ModDown fused with the
-// rescale), timed for every shape of one role with the other roles fixed.
+// rescale), timed for every shape of one role with the other roles fixed.  A small ring's routes for few limbs have no
+// launch shapes: they are off meanwhile, so that what is timed is what the shapes serve (large batches there).
 void ntt_tune(Ctx& C, int limbs, int reps, std::vector<float>* fwd_ms, std::vector<float>* inv_ms) {
   const int n = std::max(1, std::min(limbs / C.n_q, 65535 / std::max(1, C.n_q)));
   DevBuf buf((size_t)n * C.n_q * C.N, C.stream);
@@ -173,6 +174,7 @@ void ntt_tune(Ctx& C, int limbs, int reps, std::vector<float>* fwd_ms, std::vect
     float shape_ms[kNttShapes];
     for (int v = 0; v < kNttVariants; ++v) {
       Tables T = C.tab;
+      T.small_routes = false;
       T.ntt_fwd_variant = T.ntt_inv_variant = v;
       if (v < kNttShapes) shape_ms[v] = best_of([&] { dispatch(T, S, C.stream, dir == 1, nullptr); });
       const float ms = shape_ms[v % kNttShapes];
@@ -188,6 +190,11 @@ void ntt_tune(Ctx& C, int limbs, int reps, std::vector<float>* fwd_ms, std::vect
     const int l = C.L(), batch = 4;
     auto ct = ct_alloc(C, l, batch);
     HEDAP_CUDA(cudaMemsetAsync(ct->buf.p, 0, ct->buf.words * 8, C.stream));
+    struct Routes {  // back on when the timing ends or fails
+      bool& on;
+      explicit Routes(bool& r) : on(r) { on = false; }
+      ~Routes() { on = true; }
+    } off(C.tab.small_routes);
     for (int role : {NTT_ROLE_MODUP, NTT_ROLE_FINISH}) {
       int& slot = ntt_role_variant(C.tab, role);
       float best = 1e30f;

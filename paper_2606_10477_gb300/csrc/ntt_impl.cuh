@@ -1243,7 +1243,7 @@ static bool launch_whole(const LimbSet& S, const Tables& T, cudaStream_t st, boo
   if constexpr (L1 + L2 <= 13) {
     using W = WholeGeo<L1, L2>;
     const int n_prod = A.z ? std::min(A.own_alpha, A.own_limit) : A.pconv ? A.pconv_K : 0;
-    if (F || !ntt_whole_limb(L1 + L2, (size_t)S.n_limbs * S.n_parts, n_prod)) return false;
+    if (F || !ntt_whole_limb(T, (size_t)S.n_limbs * S.n_parts, n_prod)) return false;
     static const bool attrs = [&] {
       allow_smem(k_ntt_inv_whole<L1, L2>, W::SMEM);
       allow_smem(k_ntt_fwd_whole<L1, L2, LOAD_PLAIN>, W::SMEM);
