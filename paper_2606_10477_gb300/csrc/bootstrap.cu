@@ -395,28 +395,40 @@ static std::unique_ptr<Ct> lt_apply(Ctx& C, const Ct& v, const LTGroup& G, Plain
   std::unique_ptr<Ct> acc;
   const long n = (long)slots;
   if (G.n1 > kPtBabies) throw Error(HEDAP_ERR_ARG, "more than 16 baby steps");
-  for (long first = 0; first < G.giants; first += kPtGiants) {
+  std::vector<long> steps;  // giant steps that have diagonals
+  for (long g = 0; g < G.giants; ++g)
+    for (long b = 0; b < G.n1; ++b)
+      if (P.pt.count({g, b})) {
+        steps.push_back(g);
+        break;
+      }
+  // Giant steps to a launch, so that their sums take no more memory than one giant step at a time does, whose peak is the
+  // baby steps, a sum, its ModDown and the rotation of that: all of them, the baby steps released after the
+  // launch, when there are at most as many as baby steps and the sums but one fit where the rotation works;
+  // else two (a sum is released before its rotation).
+  const size_t sum_words = (size_t)v.parts() * qp_stride;
+  size_t babies = 0;
+  for (const DevBuf& b : baby) babies += b.p != nullptr;
+  const size_t room = (size_t)v.parts() * (l + 1) * C.N + galois_words(C, v.batch, l);
+  const bool at_once = steps.size() <= (size_t)kPtGiants && steps.size() <= babies + 1 &&
+                       steps.size() * sum_words <= sum_words + room;
+  const size_t width = at_once ? steps.size() : 2;
+  for (size_t first = 0; first < steps.size(); first += width) {
     PtMacArgs A{};
     A.babies = (int)G.n1;
     for (long b = 0; b < G.n1; ++b) A.ct[b] = baby[b].p;
-    std::vector<long> steps;
+    A.giants = (int)std::min(width, steps.size() - first);
     std::vector<DevBuf> sums;
     double terms = 0;
-    for (long g = first; g < std::min(first + kPtGiants, G.giants); ++g) {
-      bool any = false;
+    for (int i = 0; i < A.giants; ++i) {
       for (long b = 0; b < G.n1; ++b) {
-        auto it = P.pt.find({g, b});
-        A.pt[steps.size()][b] = it == P.pt.end() ? nullptr : it->second.p;
-        any |= it != P.pt.end();
+        auto it = P.pt.find({steps[first + i], b});
+        A.pt[i][b] = it == P.pt.end() ? nullptr : it->second.p;
         terms += it != P.pt.end();
       }
-      if (!any) continue;
-      sums.emplace_back((size_t)v.parts() * qp_stride, C.stream);
-      A.out[steps.size()] = sums.back().p;
-      steps.push_back(g);
+      sums.emplace_back(sum_words, C.stream);
+      A.out[i] = sums.back().p;
     }
-    A.giants = (int)steps.size();
-    if (!A.giants) continue;
     {
       ProfScope prof_(PROF_ELEMENTWISE, C.stream,
                       (terms + ((double)A.babies + A.giants) * v.parts()) * ext * C.N * 8);
@@ -425,12 +437,13 @@ static std::unique_ptr<Ct> lt_apply(Ctx& C, const Ct& v, const LTGroup& G, Plain
       launch(k_pt_mac_kernel, dim3(grid), dim3(256), 0, C.stream, C.tab.pr, A, qp_stride, v.parts(), C.log_n, l + 1, C.n_q);
       HEDAP_LAUNCH_CHECK();
     }
-    for (size_t i = 0; i < steps.size(); ++i) {
+    if (first + width >= steps.size()) baby.clear();
+    for (size_t i = 0; i < sums.size(); ++i) {
       auto inner = ct_alloc(C, l, v.batch);
       inner->scale = v.scale * sp;
       ev_moddown_into(C, sums[i], v.batch, l, *inner);
       sums[i] = DevBuf();
-      const long Gs = G.h0 * (G.kmin + steps[i] * G.n1);
+      const long Gs = G.h0 * (G.kmin + steps[first + i] * G.n1);
       std::unique_ptr<Ct> r = (((Gs % n) + n) % n) ? ev_galois(C, *inner, galois_for_rotation(C, Gs)) : std::move(inner);
       acc = acc ? ev_add(C, *acc, *r, false) : std::move(r);
     }

@@ -229,6 +229,9 @@ const LevelConsts& level_consts(Ctx& C, int l) {
 //
 // An operation's temporaries come from one allocation, in which what ends with the inner product gives its place
 // to ModDown's workspace: on a small ring each allocation with its release costs the host a good part of a launch.
+// What is written last is a workspace until then, so that an operation holds no more than with an allocation each: the
+// coefficient-domain limbs of the ModUp lie in the sums' place (read before the first sum is stored), the polynomial
+// that is switched, and ModDown's transform where the finishing store adds nothing to it, in the result's.
 struct Scratch {
   DevBuf buf;
   size_t at = 0;  // set back by the caller once what lies above has been used
@@ -240,24 +243,23 @@ struct Scratch {
     return p;
   }
 };
-// words of ks_modup's workspace: the coefficient-domain limbs and the extended digits
-static size_t modup_words(const Ctx& C, int batch, int l) {
-  return (size_t)batch * C.N * ((l + 1) + (size_t)C.dnum(l) * (l + 1 + C.n_p));
+// words of ks_modup's extended digits; its coefficient-domain limbs (batch (l + 1) N words) fit in the sums' place
+static size_t digit_words(const Ctx& C, int batch, int l) {
+  return (size_t)batch * C.N * C.dnum(l) * (l + 1 + C.n_p);
 }
 static size_t acc_words(const Ctx& C, int batch, int l) { return (size_t)batch * 2 * (l + 1 + C.n_p) * C.N; }
 // ModUp of a batch of NTT-domain polynomials d (member stride d_stride) into NTT-domain extended
-// digits [B][dn][ext][N] (a digit's own limbs are left out: they are d itself), in ws (modup_words)
-static const u64* ks_modup(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64* ws,
-                           const KskFuse* fuse = nullptr) {
+// digits y [B][dn][ext][N] (a digit's own limbs are left out: they are d itself; with fuse, y holds the column phase's
+// output).  dc: workspace of B (l + 1) N words, free again before the inner product.
+static void ks_modup(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64* dc, u64* y,
+                     const KskFuse* fuse = nullptr) {
   const size_t N = C.N, nl = (size_t)l + 1;
   const int ext = l + 1 + C.n_p, dn = C.dnum(l);
   const LevelConsts& LC = level_consts(C, l);
-  u64* dc = ws;  // z_i = [x_i qhat_i^-1]_{q_i}, coefficient domain
-  u64* y = ws + (size_t)batch * nl * N;
   NttAux inv{};
   inv.src = d;
   inv.src_stride = d_stride;
-  inv.post = LC.intt_post.p;
+  inv.post = LC.intt_post.p;  // dc: z_i = [x_i qhat_i^-1]_{q_i}, coefficient domain
   ntt_inverse(C.tab, qset(dc, nl * N, batch, 0, l + 1), C.stream, &inv);
   NttAux up{};
   up.own_alpha = C.alpha;
@@ -270,7 +272,6 @@ static const u64* ks_modup(Ctx& C, const u64* d, size_t d_stride, int batch, int
   up.ext = ext;
   up.z_products = LC.modup_products * batch * (double)N;
   ntt_forward(C.tab, LimbSet{y, (size_t)ext * N, batch * dn, 0, ext, l + 1, 0, C.n_q}, C.stream, &up, fuse);
-  return y;
 }
 static const DevBuf& key_for(Ctx& C, u64 galois) {
   auto it = C.keys.find(galois);
@@ -339,8 +340,8 @@ static void ks_moddown(Ctx& C, u64* acc, u64* v, int batch, int l, u64* out, siz
 
 // The key switch up to the inner product: iNTT of d, the extended digits' forward transform with the
 // key inner product fused into its second phase (the transformed digits are never stored).  The
-// sums acc [batch][2][ext][N] (NTT domain) go to acc; ws: workspace of modup_words.
-static void ks_inner(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64 galois, u64* acc, u64* ws) {
+// sums acc [batch][2][ext][N] (NTT domain) go to acc; y: workspace of digit_words.
+static void ks_inner(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64 galois, u64* acc, u64* y) {
   const DevBuf& key = key_for(C, galois);
   const int T = C.total_primes();
   if (C.tab.small_routes && C.log_n <= 13 && C.alpha <= 3 && ((size_t)batch * (l + 1 + C.n_p) << C.log_n) <= (size_t)1 << 18) {
@@ -348,7 +349,7 @@ static void ks_inner(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u6
     // a second; fused, one warp for 256 words would walk the digits one after the other with fewer than 1024
     // warps on the GPU (N = 2^12, HMult: 12 digits of 3 ciphertexts, 160 K words a digit, 65 against 71 us;
     // 7 digits of 295 K words 82 against 78 us)
-    const u64* y = ks_modup(C, d, d_stride, batch, l, ws);
+    ks_modup(C, d, d_stride, batch, l, acc, y);
     KskInnerArgs A;
     A.count = 1;
     A.key[0] = key.p;
@@ -366,16 +367,16 @@ static void ks_inner(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u6
   F.acc = acc;
   F.acc_part_stride = (size_t)(l + 1 + C.n_p) * C.N;
   F.batch = batch;
-  ks_modup(C, d, d_stride, batch, l, ws, &F);
+  ks_modup(C, d, d_stride, batch, l, acc, y, &F);
 }
 
 // One key switch: the inner product, then ModDown.
 void key_switch(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64 galois, u64* out, size_t out_stride,
                 bool acc0, bool acc1) {
-  Scratch S(C, acc_words(C, batch, l) + std::max(modup_words(C, batch, l), moddown_words(C, batch, l)));
+  Scratch S(C, acc_words(C, batch, l) + std::max(digit_words(C, batch, l), moddown_words(C, batch, l)));
   u64* acc = S.take(acc_words(C, batch, l));
   const size_t mark = S.at;
-  ks_inner(C, d, d_stride, batch, l, galois, acc, S.take(modup_words(C, batch, l)));
+  ks_inner(C, d, d_stride, batch, l, galois, acc, S.take(digit_words(C, batch, l)));
   S.at = mark;
   ks_moddown(C, acc, S.take(moddown_words(C, batch, l)), batch, l, out, out_stride, acc0, acc1);
 }
@@ -389,9 +390,9 @@ void key_switch(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u64 gal
 // constants scaled by P^-1).  The last limb's coefficients come first: INTT(e_l + acc_l P^-1) minus
 // the conversion of the special limbs into q_l scaled by P^-1.  Every residue equals that of ModDown
 // followed by the rescale.
-// ws: workspace of mdr_words.
-static size_t mdr_words(const Ctx& C, int batch, int l) { return (size_t)2 * batch * (l + 1) * C.N; }
-static void ks_moddown_rescale(Ctx& C, u64* acc, u64* ws, int batch, int l, const u64* e, size_t e_stride, u64* out,
+// x: workspace of mdr_words; the transform runs in out's place (2 batch parts of l limbs, out_stride >= l N apart).
+static size_t mdr_words(const Ctx& C, int batch) { return (size_t)2 * batch * C.N; }
+static void ks_moddown_rescale(Ctx& C, u64* acc, u64* x, int batch, int l, const u64* e, size_t e_stride, u64* out,
                                size_t out_stride, bool negate = false) {
   const size_t N = C.N;
   const int K = C.n_p, ext = l + 1 + K, nq = C.n_q;
@@ -407,7 +408,6 @@ static void ks_moddown_rescale(Ctx& C, u64* acc, u64* ws, int batch, int l, cons
   inv.pre_w = LC.mdr_last.pinv;
   inv.pre_wsh = LC.mdr_last.pinv_sh;
   ntt_inverse(C.tab, LimbSet{acc, (size_t)ext * N, 2 * batch, l, K + 1, l + 1, 0, C.n_q}, C.stream, &inv);
-  u64 *x = ws, *v = ws + (size_t)2 * batch * N;
   k_mdr_last_coef(C, acc + (size_t)l * N, (size_t)ext * N, x, 2 * batch, l, LC.mdr_last);
   NttAux fw{};
   fw.pconv = acc + (size_t)(l + 1) * N;
@@ -432,7 +432,7 @@ static void ks_moddown_rescale(Ctx& C, u64* acc, u64* ws, int batch, int l, cons
   fw.fin_w2 = LC.d_rescale.p + l;
   fw.fin_w2b = LC.d_rescale.p + 2 * l;
   fw.fin_neg = negate ? 1 : 0;
-  ntt_forward(C.tab, qset(v, (size_t)l * N, 2 * batch, 0, l), C.stream, &fw);
+  ntt_forward(C.tab, qset(out, out_stride, 2 * batch, 0, l), C.stream, &fw);
 }
 
 // Rotations of one (batched) ciphertext by several Galois elements sharing one ModUp of its
@@ -452,18 +452,13 @@ static void hoisted_inner(Ctx& C, const Ct& a, const u64* y, const u64* gs, int 
   }
   k_ksk_inner(C, y, a.part(1), 2 * a.part_stride(), A, a.batch, a.level, c0, 2 * a.part_stride());
 }
-std::vector<std::unique_ptr<Ct>> ev_galois_hoisted(Ctx& C, const Ct& a, const std::vector<u64>& gs) {
+// `chunk` rotations at a time
+static std::vector<std::unique_ptr<Ct>> hoisted_chunks(Ctx& C, const Ct& a, const std::vector<u64>& gs, size_t chunk) {
   const int l = a.level;
-  for (u64 g : gs) key_for(C, g);
-  // as many rotations at a time as about 1 GiB of sums (and 32 K limbs a launch) allows, and one ModDown for all of
-  // them: a rotation's few special limbs alone fill a fraction of the GPU, and its last wave is nearly empty (five
-  // rotations of two ciphertexts, N = 2^16, level 14, 1 / 2 / 3 / 5 at a time: 1074 / 961 / 905 / 836 us)
-  const size_t per = acc_words(C, a.batch, l), limbs = (size_t)2 * a.batch * (l + 1 + C.n_p);
-  const size_t chunk =
-      std::max<size_t>(1, std::min({gs.size(), (size_t)kKskRotations, ((size_t)1 << 27) / per, 32768 / limbs}));
-  Scratch S(C, modup_words(C, a.batch, l) + chunk * (per + moddown_words(C, a.batch, l)));
-  const u64* y = ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, l, S.take(modup_words(C, a.batch, l)));
-  u64 *acc = S.take(chunk * per), *v = S.take(chunk * moddown_words(C, a.batch, l));
+  const size_t per = acc_words(C, a.batch, l);
+  Scratch S(C, digit_words(C, a.batch, l) + chunk * (per + moddown_words(C, a.batch, l)));
+  u64 *acc = S.take(chunk * per), *y = S.take(digit_words(C, a.batch, l)), *v = S.take(chunk * moddown_words(C, a.batch, l));
+  ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, l, acc, y);
   std::vector<std::unique_ptr<Ct>> out;
   for (size_t first = 0; first < gs.size(); first += chunk) {
     RotationOut R{a.part(0), a.part_stride(), (int)std::min(chunk, gs.size() - first), {}, {}};
@@ -484,16 +479,38 @@ std::vector<std::unique_ptr<Ct>> ev_galois_hoisted(Ctx& C, const Ct& a, const st
   return out;
 }
 
+std::vector<std::unique_ptr<Ct>> ev_galois_hoisted(Ctx& C, const Ct& a, const std::vector<u64>& gs) {
+  for (u64 g : gs) key_for(C, g);
+  // as many rotations at a time as about 1 GiB of sums (and 32 K limbs a launch) allows, and one ModDown for all of
+  // them: a rotation's few special limbs alone fill a fraction of the GPU, and its last wave is nearly empty (five
+  // rotations of two ciphertexts, N = 2^16, level 14, 1 / 2 / 3 / 5 at a time: 1074 / 961 / 905 / 836 us).  Where the
+  // memory for that is not there, one at a time: the sums and the ModDown workspace of a single rotation.
+  const size_t per = acc_words(C, a.batch, a.level), limbs = (size_t)2 * a.batch * (a.level + 1 + C.n_p);
+  const size_t chunk =
+      std::max<size_t>(1, std::min({gs.size(), (size_t)kKskRotations, ((size_t)1 << 27) / per, 32768 / limbs}));
+  if (chunk > 1) {
+    try {
+      return hoisted_chunks(C, a, gs, chunk);
+    } catch (const Error& e) {
+      if (e.code != HEDAP_ERR_OOM) throw;
+    }
+  }
+  return hoisted_chunks(C, a, gs, 1);
+}
+
 std::vector<DevBuf> ev_galois_hoisted_qp(Ctx& C, const Ct& a, const std::vector<u64>& gs) {
   for (u64 g : gs) key_for(C, g);
-  Scratch S(C, modup_words(C, a.batch, a.level));
-  const u64* y = ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, a.level, S.buf.p);
   std::vector<DevBuf> out(gs.size());  // every sum is kept: as many rotations to a launch as it takes
+  if (gs.empty()) return out;
+  out[0] = DevBuf(acc_words(C, a.batch, a.level), C.stream);
+  DevBuf digits(digit_words(C, a.batch, a.level), C.stream);
+  u64* y = digits.p;
+  ks_modup(C, a.part(1), 2 * a.part_stride(), a.batch, a.level, out[0].p, y);
   for (size_t first = 0; first < gs.size(); first += kKskRotations) {
     const int count = (int)std::min<size_t>(kKskRotations, gs.size() - first);
     u64* accs[kKskRotations];
     for (int r = 0; r < count; ++r) {
-      out[first + r] = DevBuf(acc_words(C, a.batch, a.level), C.stream);
+      if (first + r) out[first + r] = DevBuf(acc_words(C, a.batch, a.level), C.stream);
       accs[r] = out[first + r].p;
     }
     hoisted_inner(C, a, y, gs.data() + first, count, accs, a.part(0));
@@ -570,6 +587,14 @@ static std::unique_ptr<Ct> rescale_scaled(Ctx& C, const Ct& a, const LimbConsts*
 }
 std::unique_ptr<Ct> ev_rescale(Ctx& C, const Ct& a) { return rescale_scaled(C, a, nullptr); }
 
+static void check_terms(const std::vector<std::pair<const Ct*, double>>& terms, int level) {
+  for (const auto& t : terms) {
+    if (t.first->level < level) throw Error(HEDAP_ERR_LEVEL, "linear combination operand below the output level");
+    if (t.first->batch != terms[0].first->batch) throw Error(HEDAP_ERR_ARG, "operands have different batch sizes");
+  }
+}
+static void lincomb_into(Ctx& C, const std::vector<std::pair<const Ct*, double>>& terms, int level, double target,
+                         double c0, Ct& o);
 // A relinearised product entering a linear combination that is rescaled next, as one fused
 // operation: rescale(m (d01 + ModDown(acc)) + sum_j c_j t_j + c0), m the product's integer constant.
 // With m = 1 the sum e = d01 + sum_j c_j t_j + c0 is formed first (one linear-combination pass) and
@@ -593,22 +618,23 @@ std::unique_ptr<Ct> ev_mul_lincomb_rescale(Ctx& C, const Ct& a, const Ct& b, dou
   }
   auto d01 = ct_alloc(C, l, a.batch);
   d01->scale = prod_scale;
+  auto o = ct_alloc(C, l - 1, a.batch);  // holds d2 first: batch (l + 1) N of its 2 batch l N words
   const size_t per = (size_t)(l + 1) * C.N;
-  Scratch S(C, acc_words(C, a.batch, l) +
-                   std::max(a.batch * per + modup_words(C, a.batch, l), mdr_words(C, a.batch, l)));
+  Scratch S(C, acc_words(C, a.batch, l) + std::max(digit_words(C, a.batch, l), mdr_words(C, a.batch)));
   u64* acc = S.take(acc_words(C, a.batch, l));
   const size_t mark = S.at;
-  u64* d2 = S.take(a.batch * per);
+  u64* d2 = o->part(0);
   k_tensor(C, a.part(0), a.part_stride(), b.part(0), b.part_stride(), d01->part(0), d01->part_stride(), d2, a.batch,
            l + 1);
-  ks_inner(C, d2, per, a.batch, l, 0, acc, S.take(modup_words(C, a.batch, l)));
+  ks_inner(C, d2, per, a.batch, l, 0, acc, S.take(digit_words(C, a.batch, l)));
   S.at = mark;
   std::vector<std::pair<const Ct*, double>> all{{d01.get(), m * prod_coef}};
   for (const auto& t : terms) all.emplace_back(t.first, m * t.second);
-  auto e = ev_lincomb_raw(C, all, l, target, m * c0);
-  auto o = ct_alloc(C, l - 1, a.batch);
-  o->scale = e->scale / (double)C.primes[l];
-  ks_moddown_rescale(C, acc, S.take(mdr_words(C, a.batch, l)), a.batch, l, e->part(0), e->part_stride(), o->part(0),
+  check_terms(all, l);
+  lincomb_into(C, all, l, target, m * c0, *d01);  // e, in d01's place
+  const double raw = target * (double)C.primes[l];
+  o->scale = raw / (double)C.primes[l];
+  ks_moddown_rescale(C, acc, S.take(mdr_words(C, a.batch)), a.batch, l, d01->part(0), d01->part_stride(), o->part(0),
                      o->part_stride(), m < 0);
   return o;
 }
@@ -622,17 +648,17 @@ std::unique_ptr<Ct> ev_mul(Ctx& C, const Ct& a, const Ct& b) {
   if (C.n_p > 8) return ev_rescale(C, *ev_mul_relin(C, a, b));
   check_batches(a, b);
   const size_t per = (size_t)(l + 1) * C.N;
+  auto o = ct_alloc(C, l - 1, a.batch);  // holds d2 first: batch (l + 1) N of its 2 batch l N words
+  o->scale = a.scale * b.scale / (double)C.primes[l];
   Scratch S(C, 2 * a.batch * per + acc_words(C, a.batch, l) +
-                   std::max(a.batch * per + modup_words(C, a.batch, l), mdr_words(C, a.batch, l)));
+                   std::max(digit_words(C, a.batch, l), mdr_words(C, a.batch)));
   u64 *e = S.take(2 * a.batch * per), *acc = S.take(acc_words(C, a.batch, l));  // e: the tensor's d0, d1
   const size_t mark = S.at;
-  u64* d2 = S.take(a.batch * per);
+  u64* d2 = o->part(0);
   k_tensor(C, a.part(0), a.part_stride(), b.part(0), b.part_stride(), e, per, d2, a.batch, l + 1);
-  ks_inner(C, d2, per, a.batch, l, 0, acc, S.take(modup_words(C, a.batch, l)));
+  ks_inner(C, d2, per, a.batch, l, 0, acc, S.take(digit_words(C, a.batch, l)));
   S.at = mark;
-  auto o = ct_alloc(C, l - 1, a.batch);
-  o->scale = a.scale * b.scale / (double)C.primes[l];
-  ks_moddown_rescale(C, acc, S.take(mdr_words(C, a.batch, l)), a.batch, l, e, per, o->part(0), o->part_stride());
+  ks_moddown_rescale(C, acc, S.take(mdr_words(C, a.batch)), a.batch, l, e, per, o->part(0), o->part_stride());
   return o;
 }
 
@@ -642,19 +668,20 @@ u64 galois_for_rotation(const Ctx& C, i64 steps) {
   return h_powmod(5, (u64)r, 2 * C.N);
 }
 
+size_t galois_words(const Ctx& C, int batch, int l) {
+  return moddown_words(C, batch, l) /* the result */ + acc_words(C, batch, l) +
+         std::max(digit_words(C, batch, l), moddown_words(C, batch, l));
+}
 std::unique_ptr<Ct> ev_galois(Ctx& C, const Ct& a, u64 g) {
   const int l = a.level;
   auto o = ct_alloc(C, l, a.batch);
   o->scale = a.scale;
-  // sigma_g(c1) is switched; sigma_g(c0) is gathered by the ModDown's finishing store
-  const size_t per = (size_t)(l + 1) * C.N;
-  Scratch S(C, acc_words(C, a.batch, l) +
-                   std::max(a.batch * per + modup_words(C, a.batch, l), moddown_words(C, a.batch, l)));
+  // sigma_g(c1) is switched, from the result's place; sigma_g(c0) is gathered by the ModDown's finishing store
+  Scratch S(C, acc_words(C, a.batch, l) + std::max(digit_words(C, a.batch, l), moddown_words(C, a.batch, l)));
   u64* acc = S.take(acc_words(C, a.batch, l));
   const size_t mark = S.at;
-  u64* d = S.take(a.batch * per);
-  k_automorph(C, a.part(1), 2 * a.part_stride(), d, per, a.batch, l + 1, g);
-  ks_inner(C, d, per, a.batch, l, g, acc, S.take(modup_words(C, a.batch, l)));
+  k_automorph(C, a.part(1), 2 * a.part_stride(), o->part(1), 2 * o->part_stride(), a.batch, l + 1, g);
+  ks_inner(C, o->part(1), 2 * o->part_stride(), a.batch, l, g, acc, S.take(digit_words(C, a.batch, l)));
   S.at = mark;
   const RotationOut R{a.part(0), a.part_stride(), 1, {o->part(0)}, {g}};
   ks_moddown(C, acc, S.take(moddown_words(C, a.batch, l)), a.batch, l, o->part(0), o->part_stride(), true, false, &R);
@@ -695,10 +722,7 @@ std::unique_ptr<Ct> ev_lincomb_raw(Ctx& C, const std::vector<std::pair<const Ct*
   if (level < 1) throw Error(HEDAP_ERR_LEVEL, "constant multiplication needs level >= 1");
   const double raw = target * (double)C.primes[level];
   const int batch = terms[0].first->batch;
-  for (const auto& t : terms) {
-    if (t.first->level < level) throw Error(HEDAP_ERR_LEVEL, "linear combination operand below the output level");
-    if (t.first->batch != batch) throw Error(HEDAP_ERR_ARG, "operands have different batch sizes");
-  }
+  check_terms(terms, level);
   auto o = ct_alloc(C, level, batch);
   o->scale = raw;
   if (level + 1 > kLcLimbs) {  // wide chains: one product and one addition at a time
@@ -711,6 +735,14 @@ std::unique_ptr<Ct> ev_lincomb_raw(Ctx& C, const std::vector<std::pair<const Ct*
     acc->scale = raw;
     return ev_add_const(C, *acc, c0);
   }
+  lincomb_into(C, terms, level, target, c0, *o);
+  return o;
+}
+// the sum itself, into o (at `level`, at most kLcLimbs limbs; it may be the first term: a thread reads the words that it
+// writes, and only in the first launch)
+static void lincomb_into(Ctx& C, const std::vector<std::pair<const Ct*, double>>& terms, int level, double target,
+                         double c0, Ct& o) {
+  const double raw = target * (double)C.primes[level];
   for (size_t first = 0; first < terms.size(); first += kLcTerms) {
     LinCombArgs A{};
     A.count = (int)std::min<size_t>(kLcTerms, terms.size() - first);
@@ -731,9 +763,8 @@ std::unique_ptr<Ct> ev_lincomb_raw(Ctx& C, const std::vector<std::pair<const Ct*
       const double v0 = std::round(c0 * raw);  // as in ev_add_const on the sum
       for (int i = 0; i <= level; ++i) A.c0[i] = h_double_to_mod(v0, C.primes[i]);
     }
-    k_lincomb(C, o->part(0), o->part_stride(), o->parts(), level + 1, A);
+    k_lincomb(C, o.part(0), o.part_stride(), o.parts(), level + 1, A);
   }
-  return o;
 }
 
 std::unique_ptr<Ct> ev_mul_const(Ctx& C, const Ct& a, double c, double target) {

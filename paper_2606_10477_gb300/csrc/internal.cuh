@@ -411,6 +411,7 @@ std::unique_ptr<Ct> ev_mul_lincomb_rescale(Ctx& C, const Ct& a, const Ct& b, dou
                                            const std::vector<std::pair<const Ct*, double>>& terms, double target,
                                            double c0);
 std::unique_ptr<Ct> ev_galois(Ctx& C, const Ct& a, u64 g);
+size_t galois_words(const Ctx& C, int batch, int l);  // device words that ev_galois takes: its result and its workspace
 std::vector<std::unique_ptr<Ct>> ev_galois_hoisted(Ctx& C, const Ct& a, const std::vector<u64>& gs);
 std::unique_ptr<Ct> ev_drop(Ctx& C, const Ct& a, int level);
 std::unique_ptr<Ct> ev_mul_const(Ctx& C, const Ct& a, double c, double target_scale);

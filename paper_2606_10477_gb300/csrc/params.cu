@@ -173,7 +173,12 @@ std::vector<i64> draw_ternary(SplitMix& s, int log_n, int hw) {
 
 // ------------------------------------------------------------------ device buffers
 DevBuf::DevBuf(size_t n, cudaStream_t st) : words(n), s(st) {
-  if (n) HEDAP_CUDA(cudaMallocAsync((void**)&p, n * sizeof(u64), st));
+  if (!n) return;
+  const cudaError_t e = cudaMallocAsync((void**)&p, n * sizeof(u64), st);
+  if (e == cudaSuccess) return;
+  cudaGetLastError();  // reported here: the next launch check must not find it
+  throw Error(e == cudaErrorMemoryAllocation ? HEDAP_ERR_OOM : HEDAP_ERR_CUDA,
+              std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
 }
 DevBuf::~DevBuf() {
   if (p) cudaFreeAsync(p, s);
