@@ -1,4 +1,4 @@
-// Device modular arithmetic on 64-bit words, primes 2^32 < q < 2^61.
+// Device modular arithmetic on 64-bit words, primes 1.5 2^32 <= q < 2^60.1 (33 to 60 bits, see h_prime_chain).
 //
 //  * Shoup multiplication by a fixed operand w with companion
 //    w' = floor(w * 2^64 / q): result in [0, 2q) for any 64-bit input
@@ -14,6 +14,7 @@
 namespace hedap {
 
 typedef uint64_t u64;
+constexpr u64 kMinPrime = 3ull << 31;  // reduce_lazy's estimate; h_prime_dev refuses smaller ones
 
 struct PrimeDev {  // per-prime constants used by the kernels
   u64 q;

@@ -13,17 +13,17 @@
 // butterfly as it can.
 //  * A phase of L stages is two register passes of K0 = ceil(L / 2) and K1 = floor(L / 2) stages
 //    (radix 16 twice for L = 8) with one exchange through shared memory between them, every thread
-//    holding 2^K0 words of a column or a block (2^17: L1 = 9 in three passes of 8 words, ColGeo; L2 stays 8).  The 2^K1 threads of one block lie in one warp: the row phase
-//    has no CTA barrier.
+//    holding 2^K0 words of a column or a block (2^17: L1 = 9 in three passes of 8 words, ColGeo; L2 stays 8).
+//    The 2^K1 threads of one block lie in one warp: the row phase has no CTA barrier.
 //  * The first pass of the column phase and the last one read and write global memory from
 //    registers (8 adjacent columns a CTA: whole 32-byte sectors).
 //  * Twiddles are (w 2^32, w 2^64) mod q pairs (mont_mul_lazy), stored per phase and block in the
 //    order in which the lanes of a warp read them (tw_slot): every load is coalesced and
 //    free of bank conflicts, and a block's twiddles are one run of 2^L2 pairs.
-//  * Residues stay lazy (Harvey 2014).  For 1.5 2^32 <= q < 2^57 the forward stages reduce nothing: the first load adds a
-//    multiple of q that keeps every difference non-negative, and the last store reduces (below 112q < 2^64);
-//    other primes reduce the first operand at every other stage (below 12q).  Inverse: for 1.5 2^32 <= q < 2^55
-//    bounds double unreduced through a phase.
+//  * Residues stay lazy (Harvey 2014).  For q < 2^57 (and at least kMinPrime, as every q) the forward stages
+//    reduce nothing: the first load adds a multiple of q that keeps every difference non-negative, and the last
+//    store reduces (below 112q < 2^64); larger primes reduce the first operand at every other stage (below 12q).
+//    Inverse: for q < 2^55 bounds double unreduced through a phase.
 // GB300, N = 2^16, against Shoup butterflies in radix-8 passes with a CTA barrier each: forward of 384 limbs
 // 304 -> 216 us, HMult with rescale of 8 ciphertexts at level 23 3.28 -> 2.30 ms.  The big kernels then issue
 // 0.45 - 0.47 instructions a cycle with the multiply pipe 68 - 78% busy, as the register loop of the
@@ -44,7 +44,7 @@
 namespace hedap {
 
 // ---------------------------------------------------------------- butterflies
-// mont_mul_lazy returns less than 3q.  Forward (Cooley-Tukey), small primes (1.5 2^32 <= q < 2^57): x + t and x - t
+// mont_mul_lazy returns less than 3q.  Forward (Cooley-Tukey), small primes (q < 2^57): x + t and x - t
 // as they are; a stage lowers and raises the bounds by 3q, so the first load adds 3 log2(N) q and the words stay
 // within [0, (9.2 + 6 log2(N)) q) < 2^64.  Seven products and eight additions, 32.9 cycles of a scheduler per warp
 // in a register loop, against 40.3 with x + 3q - t and 37.2 of a Shoup butterfly that reduces x every other stage.
@@ -57,8 +57,8 @@ __device__ __forceinline__ void ct_bfly(u64& x, u64& y, const ulonglong2 w, u64 
   y = SMALL ? x - t : x + q * 3 - t;
   x = x + t;
 }
-__device__ __forceinline__ bool fwd_small(u64 q) { return q >= (3ull << 31) && q < (1ull << 57); }
-__device__ __forceinline__ bool inv_small(u64 q) { return q >= (3ull << 31) && q < (1ull << 55); }
+__device__ __forceinline__ bool fwd_small(u64 q) { return q < (1ull << 57); }
+__device__ __forceinline__ bool inv_small(u64 q) { return q < (1ull << 55); }
 // what the first load of a forward transform adds to every word
 template <int LOGN>
 __device__ __forceinline__ u64 fwd_bias(u64 q) { return fwd_small(q) ? q * (3 * LOGN) : 0; }
@@ -101,7 +101,9 @@ __device__ __forceinline__ void fwd_pass(u64 (&v)[G][1 << K], u64 q, uint32_t nq
 }
 // K inverse (Gentleman-Sande) stages in registers, the mirror image: stage u pairs words 2^u apart, its
 // sub-block mm spans 2^(u+1) words, tw(u', mm) with u' = K - 1 - u as in the forward pass.  SMALL: the
-// bound 2^E q doubles at every stage; otherwise sums are kept below 3q + 2^32 (differences are taken from 4q).
+// bound 2^E q doubles at every stage; otherwise (q >= 2^55) sums are brought back towards 3q and differences are taken from
+// 4q: sub_if_above may leave a sum 2^32 above 3q, two such sums twice as much, so that the excess doubles at every
+// stage of both phases and stays below 2^(32 + 17) < q.
 template <bool SMALL, int E, int K, int G, class TW>
 __device__ __forceinline__ void inv_pass(u64 (&v)[G][1 << K], u64 q, uint32_t nqi, TW tw) {
 #pragma unroll
@@ -903,7 +905,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_ntt_fwd_rows_ksk(Tables T, Lim
 
 // ---------------------------------------------------------------- inverse, row phase
 // The forward row phase mirrored: the 2^K1 consecutive words of a lane's groups first, then the words
-// 2^K1 apart.  Output left lazy (below 2^(L2+1) q for small primes, 3q otherwise).
+// 2^K1 apart.  Output left lazy (below 2^(L2+1) q for small primes, otherwise below 4q, see inv_pass).
 template <bool SMALL, int L2>
 __device__ __forceinline__ void inv_rows_passes(u64 (&v)[1][1 << Phase<L2>::K0], u64* xs, const ulonglong2* tw,
                                                 const PrimeDev& P, int low) {

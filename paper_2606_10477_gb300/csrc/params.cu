@@ -81,6 +81,7 @@ u64 h_mont(u64 w, u64 q) { return (u64)(((u128)w << 32) % q); }
 u64 h_shoup(u64 w, u64 q) { return (u64)(((u128)w << 64) / q); }
 
 PrimeDev h_prime_dev(u64 q) {
+  if (q < kMinPrime) throw Error(HEDAP_ERR_ARG, "prime below 1.5 2^32");
   PrimeDev p;
   p.q = q;
   p.b = 64 - __builtin_clzll(q);
