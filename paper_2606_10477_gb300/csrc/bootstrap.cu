@@ -283,9 +283,8 @@ std::unique_ptr<Ct> mod_raise(Ctx& C, const Ct& a) {
   {
     ProfScope prof_(PROF_ELEMENTWISE, C.stream, (1.0 + (L + 1.0)) * P * N * 8);
     prof_count_launches(1);
-    launch(k_mod_raise_kernel, dim3(grid_for((size_t)P * (L + 1) * N, 256)), dim3(256), 0, C.stream, C.tab.pr, x.p, o->part(0),
-                                                                                      o->part_stride(), P, L + 1,
-                                                                                      C.log_n);
+    launch(k_mod_raise_kernel, dim3(grid_for((size_t)P * (L + 1) * N, 256)), dim3(256), 0, C.stream, C.tab.pr, x.p,
+           o->part(0), o->part_stride(), P, L + 1, C.log_n);
     HEDAP_LAUNCH_CHECK();
   }
   ntt_forward(C.tab, LimbSet{o->part(0), o->part_stride(), P, 0, L + 1, INT_MAX, 0, 0}, C.stream);
@@ -306,7 +305,8 @@ std::unique_ptr<Ct> mul_monomial(Ctx& C, const Ct& a, u64 e) {
   o->scale = a.scale;
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, 2.0 * a.parts() * (a.level + 1) * C.N * 8);
   prof_count_launches(1);
-  launch(k_monomial_kernel, dim3(grid_for((size_t)a.parts() * (a.level + 1) * C.N, 256)), dim3(256), 0, C.stream, C.tab.pr, a.part(0), a.part_stride(), o->part(0), o->part_stride(), a.parts(), a.level + 1, C.log_n, F);
+  launch(k_monomial_kernel, dim3(grid_for((size_t)a.parts() * (a.level + 1) * C.N, 256)), dim3(256), 0, C.stream, C.tab.pr,
+         a.part(0), a.part_stride(), o->part(0), o->part_stride(), a.parts(), a.level + 1, C.log_n, F);
   HEDAP_LAUNCH_CHECK();
   return o;
 }

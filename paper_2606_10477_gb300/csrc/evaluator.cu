@@ -298,28 +298,21 @@ static void ks_moddown(Ctx& C, u64* acc, u64* v, int batch, int l, u64* out, siz
   const int parts = 2 * batch * (R ? R->count : 1);
   const size_t N = C.N, nl = (size_t)l + 1;
   const int K = C.n_p, ext = l + 1 + K;
-  // ModDown: the special-prime limbs to the coefficient domain (ending with N^-1 phinv_k when the
-  // conversion is fused), the conversion into every Q prime fused into the forward NTT's load, and
-  // (acc - v) P^-1 (+ out) fused into its store
-  const bool fuse = K <= 8;
+  // ModDown: the special-prime limbs (at most 8) to the coefficient domain, ending with N^-1 phinv_k, the conversion
+  // into every Q prime fused into the forward NTT's load, and (acc - v) P^-1 (+ out) fused into its store
   NttAux inv{};
-  if (fuse) {
-    inv.post = C.d_moddown2.p;
-    inv.post_add = C.d_moddown2.p + 2 * K + 1;
-  }
+  inv.post = C.d_moddown2.p;
+  inv.post_add = C.d_moddown2.p + 2 * K + 1;
   ntt_inverse(C.tab, LimbSet{acc, (size_t)ext * N, parts, l + 1, K, l + 1, 0, C.n_q}, C.stream, &inv);
-  if (!fuse) k_moddown_spread(C, acc, v, parts, l);
   const u64* Pinv = C.d_moddown2.p + 3 * K + 1 + 2 * (size_t)K * C.n_q;
   NttAux fw{};
-  if (fuse) {
-    fw.pconv = acc + nl * N;
-    fw.pconv_stride = (size_t)ext * N;
-    fw.pconv_K = K;
-    fw.pconv_ld = C.n_q;
-    fw.pconv_phat = C.d_moddown2.p + 3 * K + 1;
-    fw.pconv_phat_b = C.d_moddown2.p + 3 * K + 1 + (size_t)K * C.n_q;
-    fw.pconv_half = C.d_moddown.p + 3 * K + (size_t)K * C.n_q + 2 * (size_t)C.n_q;
-  }
+  fw.pconv = acc + nl * N;
+  fw.pconv_stride = (size_t)ext * N;
+  fw.pconv_K = K;
+  fw.pconv_ld = C.n_q;
+  fw.pconv_phat = C.d_moddown2.p + 3 * K + 1;
+  fw.pconv_phat_b = C.d_moddown2.p + 3 * K + 1 + (size_t)K * C.n_q;
+  fw.pconv_half = C.d_moddown.p + 3 * K + (size_t)K * C.n_q + 2 * (size_t)C.n_q;
   fw.fin_dst = out;
   fw.fin_dst_stride = out_stride;
   fw.fin_c = acc;
@@ -347,8 +340,9 @@ static void ks_inner(Ctx& C, const u64* d, size_t d_stride, int batch, int l, u6
   if (C.tab.small_routes && C.log_n <= 13 && C.alpha <= 3 && ((size_t)batch * (l + 1 + C.n_p) << C.log_n) <= (size_t)1 << 18) {
     // a small ring's few limbs: the digits transformed in one launch, all of them at once, and the inner product in
     // a second; fused, one warp for 256 words would walk the digits one after the other with fewer than 1024
-    // warps on the GPU (N = 2^12, HMult: 12 digits of 3 ciphertexts, 160 K words a digit, 65 against 71 us;
-    // 7 digits of 295 K words 82 against 78 us)
+    // warps on the GPU.  HMult, separate against fused (us), words a digit over the batch: 12 digits, 2^10 27 K
+    // 26.8 36.5, 213 K 56.1 54.4; 2^12 160 K 44.2 50.8, 319 K 73.8 71.2; 2^13 213 K 64.4 65.8, 426 K 104.9 99.5;
+    // 4 digits, 2^11 41 K 28.7 30.5, 328 K 46.3 45.4; 3 digits, 2^12 197 K 37.8 38.1, 786 K 82.5 76.4.
     ks_modup(C, d, d_stride, batch, l, acc, y);
     KskInnerArgs A;
     A.count = 1;
@@ -609,7 +603,7 @@ std::unique_ptr<Ct> ev_mul_lincomb_rescale(Ctx& C, const Ct& a, const Ct& b, dou
   const int l = std::min(a.level, b.level);
   check_batches(a, b);
   const double m = l >= 1 ? std::round(prod_coef * target * (double)C.primes[l] / prod_scale) : 0.0;
-  if (l < 1 || (m != 1.0 && m != -1.0) || l + 1 > kLcLimbs || C.n_p > 8 || terms.size() + 1 > kLcTerms) {
+  if (l < 1 || (m != 1.0 && m != -1.0) || l + 1 > kLcLimbs || terms.size() + 1 > kLcTerms) {
     auto pr = ev_mul_relin(C, a, b);
     pr->scale = prod_scale;
     std::vector<std::pair<const Ct*, double>> all{{pr.get(), prod_coef}};
@@ -645,7 +639,6 @@ std::unique_ptr<Ct> ev_mul_lincomb_rescale(Ctx& C, const Ct& a, const Ct& b, dou
 std::unique_ptr<Ct> ev_mul(Ctx& C, const Ct& a, const Ct& b) {
   const int l = std::min(a.level, b.level);
   if (l < 1) throw Error(HEDAP_ERR_LEVEL, "rescale needs level >= 1");
-  if (C.n_p > 8) return ev_rescale(C, *ev_mul_relin(C, a, b));
   check_batches(a, b);
   const size_t per = (size_t)(l + 1) * C.N;
   auto o = ct_alloc(C, l - 1, a.batch);  // holds d2 first: batch (l + 1) N of its 2 batch l N words

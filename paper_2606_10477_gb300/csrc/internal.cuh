@@ -216,10 +216,6 @@ struct NttAux {
   // with fin_w2 and no fin_e: the same with 0 in its place (a rescale of c times a constant)
   int fin_neg = 0;  // with fin_e: store the negated residues
 };
-// Forward only: the second phase of the ModUp transform of a key switch fused with the key inner
-// product (k_ntt_fwd_rows_ksk): the transformed digits are multiplied by the switching key and summed
-// over the digits instead of being stored.  The LimbSet's parts are (ciphertext k, digit j) = k dn + j
-// (dn = NttAux::own_dn), its limbs the extended limbs t; a digit's own limbs are read from d.
 // Switching keys are stored with the word pairs of each 256-word run permuted: pair p (words 2 p, 2 p + 1) sits at pair
 // key_pair(p), so that a warp whose lanes own 8 consecutive words each reads 512 consecutive bytes per
 // load (k_ntt_fwd_rows_ksk), and one whose lanes own consecutive pairs reads whole 128-byte lines
@@ -242,6 +238,10 @@ __device__ __forceinline__ ulonglong2 galois_pair(const u64* limb, uint32_t s) {
   return s & 1 ? ulonglong2{v.y, v.x} : v;
 }
 #endif
+// Forward only: the second phase of the ModUp transform of a key switch fused with the key inner
+// product (k_ntt_fwd_rows_ksk): the transformed digits are multiplied by the switching key and summed
+// over the digits instead of being stored.  The LimbSet's parts are (ciphertext k, digit j) = k dn + j
+// (dn = NttAux::own_dn), its limbs the extended limbs t; a digit's own limbs are read from d.
 struct KskFuse {
   const u64* d = nullptr;        // NTT-domain inputs: ciphertext k's limb t at d + k d_stride + t N
   size_t d_stride = 0;
@@ -256,8 +256,10 @@ void ntt_forward(const Tables& T, const LimbSet& S, cudaStream_t st, const NttAu
                  const KskFuse* fuse = nullptr);
 void ntt_inverse(const Tables& T, const LimbSet& S, cudaStream_t st, const NttAux* aux = nullptr);
 // whether a transform of `limbs` limbs at N = 2^T.log_n with n_prod products a word in its load runs with a whole limb
-// per cluster (ntt_impl.cuh): up to 2^21 words in all (a rescale of 8 ciphertexts of 21 limbs at N = 2^12, 1.4 M words,
-// 25.7 us against 29.1 us); beyond, the two-launch kernels carry more at a time
+// per cluster (ntt_impl.cuh): up to 2^21 words in all; beyond, the two-launch kernels carry more at a time.  Forward
+// transforms of 0.26 / 1.05 / 2.1 / 4.2 M words, cluster against two launches (us): 2^10 5.4 7.3 / 9.4 11.6 / 15.7 19.0 /
+// 28.7 34.0; 2^12 5.3 7.2 / 11.7 11.1 / 19.2 19.0 / 34.7 34.3; 2^13 6.4 7.3 / 13.6 12.5 / 22.9 20.7 / 40.2 37.2; a rescale
+// of 8 ciphertexts of 21 limbs at 2^12, 1.4 M words, 25.7 against 29.1 us.
 constexpr size_t kWholeLimbWords = (size_t)1 << 21;
 inline bool ntt_whole_limb(const Tables& T, size_t limbs, int n_prod) {
   const int log_n = T.log_n;

@@ -40,8 +40,8 @@ void k_add_sub(const Ctx& C, const u64* a, size_t as, const u64* b, size_t bs, u
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, 3.0 * n_parts * limbs * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * limbs * C.N / 2;
-  launch(k_add_sub_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, a, as, b, bs, o, os, n_parts, limbs,
-                                                              C.log_n, sub);
+  launch(k_add_sub_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, a, as, b, bs, o, os, n_parts,
+         limbs, C.log_n, sub);
   HEDAP_LAUNCH_CHECK();
 }
 
@@ -127,8 +127,8 @@ void k_tensor(const Ctx& C, const u64* a, size_t as, const u64* b, size_t bs, u6
   ProfScope prof_(PROF_TENSOR, C.stream, 7.0 * batch * limbs * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)batch * limbs * C.N / 2;
-  launch(k_tensor_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, a, as, b, bs, o, os, d2, batch, limbs,
-                                                             C.log_n);
+  launch(k_tensor_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, a, as, b, bs, o, os, d2, batch,
+         limbs, C.log_n);
   HEDAP_LAUNCH_CHECK();
 }
 
@@ -154,8 +154,8 @@ void k_mul_limbconst(const Ctx& C, const u64* in, size_t is, u64* out, size_t os
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, 2.0 * n_parts * limbs * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * limbs * C.N / 2;
-  launch(k_mul_limbconst_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, in, is, out, os, n_parts, limbs,
-                                                                   C.log_n, K);
+  launch(k_mul_limbconst_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, in, is, out, os, n_parts,
+         limbs, C.log_n, K);
   HEDAP_LAUNCH_CHECK();
 }
 
@@ -216,8 +216,8 @@ void k_add_limbconst(const Ctx& C, const u64* in, size_t is, u64* out, size_t os
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, 2.0 * n_parts * limbs * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * limbs * C.N / 2;
-  launch(k_add_limbconst_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, in, is, out, os, n_parts, limbs, C.log_n,
-                                                                   K);
+  launch(k_add_limbconst_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, in, is, out, os, n_parts,
+         limbs, C.log_n, K);
   HEDAP_LAUNCH_CHECK();
 }
 // K's words to device memory: w [n], then wsh [n]
@@ -451,12 +451,12 @@ void k_ksk_inner(const Ctx& C, const u64* y, const u64* d, size_t d_stride, cons
   prof_count_launches(1);
   const unsigned tx = 32u * (unsigned)std::max(1, 8 / batch);  // about 256 threads per CTA
   const dim3 block(tx, (unsigned)batch), grid((unsigned)(C.N / 2 / tx), (unsigned)(ext * A.count));
-  launch(k_ksk_inner_kernel, dim3(grid), dim3(block), 0, C.stream, C.tab.pr, y, d, d_stride, A, level, dn, C.alpha, C.n_q, C.n_p,
-                                                   C.log_n, c0, c0_stride, C.d_pmod.p);
+  launch(k_ksk_inner_kernel, dim3(grid), dim3(block), 0, C.stream, C.tab.pr, y, d, d_stride, A, level, dn, C.alpha,
+         C.n_q, C.n_p, C.log_n, c0, c0_stride, C.d_pmod.p);
   HEDAP_LAUNCH_CHECK();
 }
 
-// a batch over Q_l u P: (P c0, P c1) on the Q limbs (P mod q_i by Barrett), 0 on the special limbs
+// a batch over Q_l u P: (P c0, P c1) on the Q limbs, 0 on the special limbs
 __global__ void k_lift_qp_kernel(const PrimeDev* __restrict__ pr, const u64* __restrict__ pmod,
                                  const u64* in, size_t is, u64* out, int n_parts, int l,
                                  int ext, int log_n) {
@@ -473,8 +473,8 @@ void k_lift_qp(const Ctx& C, const u64* in, size_t is, u64* out, int n_parts, in
   ProfScope prof_(PROF_ELEMENTWISE, C.stream, (double)n_parts * (level + 1 + ext) * C.N * 8);
   prof_count_launches(1);
   const size_t work = (size_t)n_parts * ext * C.N;
-  launch(k_lift_qp_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, C.d_pmod.p, in, is, out, n_parts, level,
-                                                                ext, C.log_n);
+  launch(k_lift_qp_kernel, dim3(grid_for(work, 256)), dim3(256), 0, C.stream, C.tab.pr, C.d_pmod.p, in, is, out,
+         n_parts, level, ext, C.log_n);
   HEDAP_LAUNCH_CHECK();
 }
 

@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols(Tables T, LimbSet S, 
 // rescale is fused), the rescale spread the last limb.  A CTA stages the tiles of its TH / 2^K1 columns once
 // (cp.async, straight into shared memory) and runs the column phase of `lpc` consecutive output limbs of one
 // part from there.  One column a thread: with two, the tiles let only 8 warps fit an SM and the passes
-// waited on their own latency (1313 against 960 us, N = 2^16, 8 x 12 digits at level 23).
+// waited on their own latency (1313 against 960 us when it was tried, 770 us since; N = 2^16, 8 x 12 digits at level 23).
 template <int L1, int L2, int TH, int MINB, int KIND>
 __global__ void __launch_bounds__(TH, MINB) k_ntt_fwd_cols_shared(Tables T, LimbSet S, NttAux A, int lpc) {
   using G = ColGeo<L1, TH>;
