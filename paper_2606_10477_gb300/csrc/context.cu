@@ -232,8 +232,15 @@ Ctx* ctx_create(const hedap_params& P, u64 seed, cudaStream_t st) {
   upload(*C, C->d_sk, skr);
   ntt_forward(C->tab, LimbSet{C->d_sk.p, 0, 1, 0, T, nq, 0, nq}, C->stream);
   gen_galois_key(*C, 0);
-  // pick the NTT launch shape for this ring, on as many limbs as a call has that runs in these shapes (ntt_whole_limb)
-  ntt_tune(*C, std::max(8 * C->n_q, C->log_n <= 13 ? (int)(kWholeLimbWords >> C->log_n) + C->n_q : 0), 2, nullptr, nullptr);
+  // pick the NTT launch shape for this ring, on as many limbs as a call has that runs in these shapes (ntt_whole_limb);
+  // on fewer where there is no memory for that
+  const int few = 8 * C->n_q, many = C->log_n <= 13 ? (int)(kWholeLimbWords >> C->log_n) + C->n_q : 0;
+  try {
+    ntt_tune(*C, std::max(few, many), 2, nullptr, nullptr);
+  } catch (const Error& e) {
+    if (e.code != HEDAP_ERR_OOM || many <= few) throw;
+    ntt_tune(*C, few, 2, nullptr, nullptr);
+  }
   HEDAP_CUDA(cudaStreamSynchronize(C->stream));
   return C.release();
 }

@@ -115,3 +115,21 @@ def test_hoisted_rotations_in_short_memory():
     del rot
     g.sync()
     assert p.cu.cuMemPoolDestroy(pool) == 0
+
+
+def test_context_of_a_small_ring_in_short_memory():
+    """The tuner's scratch for a small ring's large batches (16 MiB) is not needed: with room for the rest only (17 of 32 MiB),
+    the context is made, and its products are those of any other."""
+    p = Pools()
+    pool = p.limited(32 << 20)
+    assert p.cu.cuDeviceSetMemPool(p.dev, pool) == 0
+    try:
+        g = hedap.Context(13, [45] * 4, [60], 1, 40.0, 64, 1)
+        x = inputs.random_ciphertext_limbs(5, g.primes(), 3, g.N)
+        got = g.mul(g.ct_import(x, 3, g.scale), g.ct_import(x, 3, g.scale)).limbs()
+        g.sync()
+        g.close()
+    finally:
+        assert p.cu.cuDeviceSetMemPool(p.dev, p.default) == 0
+    h = hedap.Context(13, [45] * 4, [60], 1, 40.0, 64, 1)
+    assert np.array_equal(got, h.mul(h.ct_import(x, 3, h.scale), h.ct_import(x, 3, h.scale)).limbs())
