@@ -103,10 +103,10 @@ def measured_peaks():
 NTT_MUL_SLOTS_PER_BUTTERFLY = 13
 IMAD_LANES_PER_SM = 64
 # DRAM bytes per transformed limb: dram__bytes_read.sum + dram__bytes_write.sum of the transform launches of one
-# batched HMult with rescale at the top level (`--only hmult --batch 8 --profile-region` under ncu: 4528.0 MB for
+# batched HMult with rescale at the top level (`--only hmult --batch 8 --profile-region` under ncu: 4521.9 MB for
 # 2912 limb transforms, the mix of fused ModUp (with the key inner product) and ModDown-rescale transforms of the
 # step), scaled to a launch group by its limbs
-NTT_DRAM_BYTES_PER_LIMB = 1.555e6
+NTT_DRAM_BYTES_PER_LIMB = 1.553e6
 
 
 def ntt_alu_roofline(n, alg_bytes, ms, groups, peaks, slots):

@@ -26,8 +26,8 @@
 //    Inverse: for q < 2^55 bounds double unreduced through a phase.
 // GB300, N = 2^16, against Shoup butterflies in radix-8 passes with a CTA barrier each: forward of 384 limbs
 // 304 -> 216 us, HMult with rescale of 8 ciphertexts at level 23 3.28 -> 2.30 ms.  The big kernels then issue
-// 0.45 - 0.47 instructions a cycle with the multiply pipe 68 - 78% busy, as the register loop of the
-// butterfly itself does (0.48 and 82%): what is left is their instruction count.
+// 0.45 - 0.50 instructions a cycle of a scheduler with the multiply pipe 74 - 81% busy, the register loop of the
+// butterfly alone 0.50 and 88%: what is left is mostly their instruction count.
 // Optional fusions (NttAux): the first phase may read another buffer (out of place) or compute its
 // input as the fast basis conversion of a key-switching digit (ModUp fused into the load),
 // the inverse may end with a per-limb factor other than N^-1, a digit's own limbs may be skipped,
@@ -1281,7 +1281,7 @@ static void allow_smem(Kernel kern, size_t bytes) {
 constexpr int kKskWarps = 4, kKskMinBlocks = 3;
 
 // Output limbs per CTA of the shared-tile column phase: the number that minimises waves x (limbs + 0.3), the 0.3 limb
-// being the staging of the tiles; `ctas` CTAs per group of limbs, `slots` resident at a time.  One ciphertext at
+// being the staging of the tiles (an estimate, not timed apart); `ctas` CTAs per group of limbs, `slots` resident at a time.  One ciphertext at
 // level 23 (N = 2^16): 9 limbs a CTA, 1.9 waves, where a fixed target of four waves gave 4 limbs and 4.4 waves.
 inline int limbs_per_cta(size_t ctas, int limbs, size_t slots) {
   int best = 1;
