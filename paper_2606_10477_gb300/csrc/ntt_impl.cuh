@@ -16,7 +16,7 @@
 //    holding 2^K0 words of a column or a block (2^17: L1 = 9 in three passes of 8 words, ColGeo; L2 stays 8).
 //    The 2^K1 threads of one block lie in one warp: the row phase has no CTA barrier.
 //  * The first pass of the column phase and the last one read and write global memory from
-//    registers (8 adjacent columns a CTA: whole 32-byte sectors).
+//    registers (8 adjacent columns a CTA, 4 at 2^17: whole 32-byte sectors).
 //  * Twiddles are (w 2^32, w 2^64) mod q pairs (mont_mul_lazy), stored per phase and block in the
 //    order in which the lanes of a warp read them (tw_slot): every load is coalesced and
 //    free of bank conflicts, and a block's twiddles are one run of 2^L2 pairs.
